@@ -11,7 +11,7 @@
 //                CTAs complete on the mbarriers of the leader (rank 0) CTA
 //   warp 1       MMA issuer (leader CTA only): tcgen05.mma.cta_group::2, slot release and accumulator
 //                events by tcgen05.commit multicast to both CTAs
-//   warps 2-9    softmax on the CTA's own S rows (TMEM), P written back to TMEM, epilogue of O through
+//   warps 2-9    one-pass softmax on the CTA's own S rows (TMEM), P written back to TMEM, epilogue of O through
 //                swizzled shared-memory tiles and TMA stores; events to the leader's MMA warp by remote arrive
 // Stage stream, TMEM column plan, running-max rule and chunking are those described at the kernel.
 #include <cuda.h>
@@ -31,16 +31,16 @@ constexpr int TTHREADS = 32 * (10 + NPROD - 1);   // warp 1: MMA issuer; warps 2
 constexpr int BOXB = kBoxRows * 128;       // bytes of one box: kBoxRows rows x 128 bytes
 constexpr float RESCALE_GAP = 16.f;        // log2 units a later piece's row max may exceed the running reference
 
-constexpr int NSX = 12;                    // 16 KiB slots of the staging area; a 32 KiB area after it stages the output tiles
+constexpr int NSX = 14;                    // 16 KiB slots of the staging area
 constexpr int NQS = 8;                     // S phase: slots [0, 8) hold the Q slices (all of d, resident for every piece),
-constexpr int NKS = NSX - NQS + 2;         //          slots [8, 14) are the ring of the K stages: the last two are the
-                                           //          output staging area, idle until the first part of O is read out;
-                                           // V phase: slots [0, 12) form the ring of the V stages
+constexpr int NKS = NSX - NQS;             //          slots [8, 14) are the ring of the K stages;
+constexpr int NSV = 10;                    // V phase: slots [0, 10) form the ring of the V stages, slots [10, 14) stage the output: two tiles of
+                                           //          32 rows x 64 columns per warp, so that a tile is written while the one before leaves
 
 struct Ctl {                               // control block at the start of dynamic shared memory
   uint64_t fullQ[NQS];                     // Q slice dk has arrived (used once)
   uint64_t fullK[NKS], emptyK[NKS];        // ring of the K stages
-  uint64_t fullV[NSX], emptyV[NSX];        // ring of the V stages (starts when the S products are complete)
+  uint64_t fullV[NSV], emptyV[NSV];        // ring of the V stages (starts when the S products are complete)
   uint64_t acc_ev[7];                      // MMA -> other warps, one barrier per event, each used once:
                                            //   [pc] S of piece pc is complete   [3 + p] part p of O is complete
   uint64_t cmp_ev[6];                      // compute warps -> MMA, one barrier per event, each used once:
@@ -49,11 +49,11 @@ struct Ctl {                               // control block at the start of dyna
   int32_t merge_here;                      // set for the CTA that finished a multi-chunk tile last
   uint32_t box[NCX / kBoxRows];            // tensor map id << 30 | first row
   uint8_t kmask[NCX];
-  float xch[2][BM];
+  float xch[2][BM];                        // first-slab maxima of the rows, by the two warps that share them
 };
 constexpr int CTLB = 3072;                 // control block bytes; the ring follows (needs a 1024-byte aligned base)
 constexpr int SLOTP = 16384;               // ring slot: every stage of a CTA is at most 16 KiB
-constexpr int SMEM_X = CTLB + NSX * SLOTP + 32768;
+constexpr int SMEM_X = CTLB + NSX * SLOTP;
 static_assert(sizeof(Ctl) <= CTLB, "control block overflow");
 
 __device__ __forceinline__ void mbar_init(uint64_t* b, uint32_t count) {
@@ -68,8 +68,11 @@ __device__ __forceinline__ uint32_t map_to_rank(uint32_t saddr, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
   return r;
 }
+// Arrival on a barrier of the pair for events in tensor memory only (tcgen05.wait and tcgen05.fence::before_thread_sync come
+// before it, tcgen05.fence::after_thread_sync after the wait): relaxed, because a release at cluster scope would also
+// order the thread's ordinary writes, which takes about 900 cycles and which nobody needs here.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 // TMA box copy into this CTA's shared memory; completion is counted on an mbarrier given by its cluster address
 __device__ __forceinline__ void tma_box2(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar_cluster_addr) {
@@ -139,57 +142,69 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
   // the two CTAs of a pair are neighbours in x; pairs take the (sequence, tile) items in the order the plan kernel left
   // (most keys first)
   const int chunk = blockIdx.y;
-  // launched as a programmatic dependent of the tile plan: the CTAs take their places while that kernel's last CTAs
-  // finish, and read nothing before it has completed
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  uint32_t rank;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+  Ctl& sm = *reinterpret_cast<Ctl*>(smem_raw);
+  const uint32_t ring = smem_u32(smem_raw + CTLB);
+  int fail = (smem_u32(smem_raw) & 1023u) ? 1 : 0;             // the swizzled tiles need a 1024-byte aligned base
+  if (tid < (GENERAL ? NMAPS : 14))   // the descriptors of the tensor maps in use are fetched while the plan is read
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&maps) + (uint64_t)tid * sizeof(CUtensorMap)) : "memory");
+  // Barriers, tensor memory and the first half of the pair-wide barrier that announces them.
+  auto set_up = [&]() {
+    if (tid == 0) {
+      for (int i = 0; i < NQS; ++i) mbar_init(&sm.fullQ[i], 1);
+      for (int i = 0; i < NKS; ++i) { mbar_init(&sm.fullK[i], 1); mbar_init(&sm.emptyK[i], 1); }
+      for (int i = 0; i < NSV; ++i) { mbar_init(&sm.fullV[i], 1); mbar_init(&sm.emptyV[i], 1); }
+      for (int i = 0; i < 7; ++i) mbar_init(&sm.acc_ev[i], 1);
+      for (int i = 0; i < 6; ++i) mbar_init(&sm.cmp_ev[i], 16);   // 8 compute warps of each CTA
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&sm.tmem_base)) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+    __syncwarp();
+    cluster_arrive();
+  };
+  // ... and their end, for a pair that finds nothing to do after it has set up
+  auto tear_down = [&]() {
+    fence_before();
+    __syncthreads();
+    cluster_wait();
+    fence_after();
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(sm.tmem_base) : "memory");
+  };
+  // Launched as a programmatic dependent of the tile plan: the CTAs take their places while that kernel's last CTAs
+  // finish, and read nothing of its before it has completed.  The set-up reads nothing at all: the pairs of a tile's first
+  // chunk, which nearly always find work, do it before the wait (later chunks first learn whether they exist).
+  if (chunk == 0) set_up();
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int4 rec = reinterpret_cast<const int4*>(ws + pl.off_order)[blockIdx.x >> 1];   // {tile index, mode, keys, -}: one load
   const int item = rec.x;
   const int b = item / pl.tc_nt, tile = item % pl.tc_nt;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  uint32_t rank;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
   const size_t tix = (size_t)b * pl.tc_nt + tile;
-  if (tid < (GENERAL ? NMAPS : 14))   // the descriptors of the tensor maps in use are fetched while the plan is read
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&maps) + (uint64_t)tid * sizeof(CUtensorMap)) : "memory");
   const size_t rix = (size_t)b * 2 * pl.tc_nt + 2 * tile + rank;  // this CTA's 128-row tile (partials of multi-chunk tiles)
   // every exit below is taken by both CTAs of the pair alike (it depends on the pair's plan only)
-  if (rec.y != 1 && !(GENERAL && rec.y == 2)) return;          // neither a contiguous-run tile nor a gathered one
   const bool gather = GENERAL && rec.y == 2;                              // the key list is a list of row codes (array << 30 | row), not of boxes
-  const int nk = rec.z;
+  const int nk = rec.y == 1 || gather ? rec.z : 0;
   const int rows_seq = s.D * s.H, row0 = tile * PR + (int)rank * BM;           // first of this CTA's rows within the sequence
-  if (nk <= 0) {                                               // flagged sequence or padding-only tile: zeros
-    if (chunk == 0) {
-      uint4* o4 = reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(out_) + ((size_t)b * rows_seq + row0) * DH);
-      for (int i = tid; i < BM * DH / 8; i += TTHREADS)
-        if (row0 + i / (DH / 8) < rows_seq) o4[i] = make_uint4(0, 0, 0, 0);
+  int nch, CL;
+  chunking_x(nk, GENERAL, nch, CL);
+  if (nk <= 0 || chunk >= nch) {
+    if (chunk == 0) {                                          // flagged sequence or padding-only tile: zeros
+      if (rec.y == 1 || gather) {
+        uint4* o4 = reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(out_) + ((size_t)b * rows_seq + row0) * DH);
+        for (int i = tid; i < BM * DH / 8; i += TTHREADS)
+          if (row0 + i / (DH / 8) < rows_seq) o4[i] = make_uint4(0, 0, 0, 0);
+      }
+      tear_down();
     }
     return;
   }
-  int nch, CL;
-  chunking_x(nk, GENERAL, nch, CL);
-  if (chunk >= nch) return;
   const int cbeg = chunk * CL, cend = min(nk, cbeg + CL);
-
-  Ctl& sm = *reinterpret_cast<Ctl*>(smem_raw);
-  const uint32_t ring = smem_u32(smem_raw + CTLB);
-  int fail = (smem_u32(smem_raw) & 1023u) ? 1 : 0;             // the swizzled tiles need a 1024-byte aligned base
-
-  if (tid == 0) {
-    for (int i = 0; i < NQS; ++i) mbar_init(&sm.fullQ[i], 1);
-    for (int i = 0; i < NKS; ++i) { mbar_init(&sm.fullK[i], 1); mbar_init(&sm.emptyK[i], 1); }
-    for (int i = 0; i < NSX; ++i) { mbar_init(&sm.fullV[i], 1); mbar_init(&sm.emptyV[i], 1); }
-    for (int i = 0; i < 7; ++i) mbar_init(&sm.acc_ev[i], 1);
-    for (int i = 0; i < 6; ++i) mbar_init(&sm.cmp_ev[i], 16);   // 8 compute warps of each CTA
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&sm.tmem_base)) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-  }
-  // Pair-wide barrier, first half: this CTA's barriers exist and its tensor memory is allocated (thread 0 and warp 0 arrive
-  // after doing that).  The plan's boxes and key masks are read while the peer gets there; the wait follows below.
-  __syncwarp();
-  cluster_arrive();
+  if (chunk) set_up();
+  // The plan's boxes and key masks are read while the peer sets up; the wait for it follows.
   {
     const int2* box_g = reinterpret_cast<const int2*>(ws + pl.off_box) + tix * (size_t)(pl.tc_maxk / kBoxRows);
     const uint8_t* kmask_g = reinterpret_cast<const uint8_t*>(ws + pl.off_kmask) + tix * pl.tc_maxk;
@@ -284,7 +299,7 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
       int part = 0, kb = pw;
       while (kb >= nvb) { kb -= nvb; ++part; }
       for (int gv = pw; gv < NVST; gv += NPROD) {
-        const int sl = gv % NSX, use = gv / NSX;
+        const int sl = gv % NSV, use = gv / NSV;
         const uint32_t slot = ring + (uint32_t)sl * SLOTP;
         const uint32_t fb_leader = map_to_rank(smem_u32(&sm.fullV[sl]), 0);
         uint4 vcode = make_uint4(0u, 0u, 0u, 0u);                 // (fetched before the wait for the slot)
@@ -358,13 +373,13 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
           const uint64_t vd = dv0 + (uint64_t)(sl * (SLOTP >> 4));
           if (NQ == 2) {          // per CTA: 64 keys x 128 dims = two [64 x 64] tiles
 #pragma unroll
-            for (int ks = 0; ks < 4; ++ks) mma2_ts(tm + OCOL, tm + kb * 32 + ks * 8, vd + ks * (2048 >> 4), idesc_v, (kb | ks) != 0);
+            for (int ks = 0; ks < 4; ++ks) mma2_ts(tm + OCOL, tm + (kb >> 2) * 128 + (kb & 1) * 64 + (kb & 2) * 16 + ks * 8, vd + ks * (2048 >> 4), idesc_v, (kb | ks) != 0);
           } else {                // per CTA: 128 keys x 64 dims = one [128 x 64] tile
 #pragma unroll
-            for (int ks = 0; ks < 8; ++ks) mma2_ts(tm + OCOL, tm + kb * 64 + ks * 8, vd + ks * (2048 >> 4), idesc_v, (kb | ks) != 0);
+            for (int ks = 0; ks < 8; ++ks) mma2_ts(tm + OCOL, tm + (kb >> 1) * 128 + (ks >> 2) * 64 + (kb & 1) * 32 + (ks & 3) * 8, vd + ks * (2048 >> 4), idesc_v, (kb | ks) != 0);
           }
           mma2_commit(&sm.emptyV[sl]);
-          if (++sl == NSX) { sl = 0; ph ^= 1u; }
+          if (++sl == NSV) { sl = 0; ph ^= 1u; }
         }
         mma2_commit(&sm.acc_ev[3 + part]);
       }
@@ -380,152 +395,163 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
     float m_run = -INFINITY;                         // reference max of the row (log2 units)
     float lp[4] = {0.f, 0.f, 0.f, 0.f};              // this thread's share of the row sum, four independent chains
 
-    // The softmax code works on slabs of 32 keys in short loops: the kernel passes through it once per piece, so long
-    // unrolled code would be fetched cold every time.
-    //
-    // Visibility of a slab for this warp's rows, 32 keys per word (bit t = key t of the slab).  The 32 rows of a warp
-    // belong to one node (H >= 32 on this path), so one ballot over the keys' node masks gives the word.
-    auto slab_vis = [&](int pc, int c) { return __ballot_sync(0xffffffffu, sm.kmask[pc * 256 + hh * 128 + c * 32 + lane] & mybit); };
-    // masked maximum of one slab of S (fp32 columns [col, col + 32))
-    auto slab_max = [&](uint32_t col, uint32_t vis, float mx) {
-      uint32_t sv[32];
-      tmem_ld32(col, sv);
-      float mc[4] = {mx, -INFINITY, -INFINITY, -INFINITY};
-      if (vis == 0xffffffffu) {
-#pragma unroll
-        for (int t = 0; t < 32; ++t) mc[t & 3] = fmaxf(mc[t & 3], __uint_as_float(sv[t]));
-      } else {
-#pragma unroll
-        for (int t = 0; t < 32; ++t) if ((vis >> t) & 1u) mc[t & 3] = fmaxf(mc[t & 3], __uint_as_float(sv[t]));
-      }
-      return fmaxf(fmaxf(mc[0], mc[1]), fmaxf(mc[2], mc[3]));
-    };
-    // P of one slab: 32 S values -> 16 bf16 pairs (low half = even key) stored at P columns [pcol, pcol + 16); the row
-    // sum shares go to lp
-    auto slab_exp = [&](const uint32_t* sv, uint32_t vis, float moff, uint32_t pcol) {
-      uint32_t pk[16];
-      if (vis == 0xffffffffu) {
-#pragma unroll
-        for (int t = 0; t < 32; t += 2) {
-          const float p0 = ex2(fmaf(__uint_as_float(sv[t]), scale2, -moff));
-          const float p1 = ex2(fmaf(__uint_as_float(sv[t + 1]), scale2, -moff));
-          lp[(t >> 1) & 3] += p0 + p1;
-          const __nv_bfloat162 h2 = __floats2bfloat162_rn(p0, p1);
-          pk[t >> 1] = *reinterpret_cast<const uint32_t*>(&h2);
-        }
-      } else {
-#pragma unroll
-        for (int t = 0; t < 32; t += 2) {
-          const float p0 = ((vis >> t) & 1u) ? ex2(fmaf(__uint_as_float(sv[t]), scale2, -moff)) : 0.f;
-          const float p1 = ((vis >> (t + 1)) & 1u) ? ex2(fmaf(__uint_as_float(sv[t + 1]), scale2, -moff)) : 0.f;
-          lp[(t >> 1) & 3] += p0 + p1;
-          const __nv_bfloat162 h2 = __floats2bfloat162_rn(p0, p1);
-          pk[t >> 1] = *reinterpret_cast<const uint32_t*>(&h2);
-        }
-      }
-      tmem_st16(pcol, pk);
-    };
     auto p_stored = [&](int pc) {                    // this warp's P of piece pc is in TMEM: tell the leader's MMA warp
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
       fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(map_to_rank(smem_u32(&sm.cmp_ev[pc]), 0));
     };
-    auto block_mine = [&](int pc) { return hh * 128 < min(256, CL - pc * 256); };
-
-    // The pieces arrive one after the other (the tensor core computes S of the next piece meanwhile).  The first piece sets
-    // the reference maximum of the row; a later piece keeps it unless it exceeds it by more than RESCALE_GAP (weights up
-    // to 2^16 are harmless in bf16/fp32), else the P written so far and the sums are rescaled.
+    // The softmax goes over a piece ONCE, in slabs of 32 keys: a slab is read from tensor memory, checked against the row's
+    // reference maximum, exponentiated and stored as P, the next slab's read already on its way.
     //
-    // Where P lands: piece pc -> columns [128 pc, 128 pc + 128), the warps with hh = 0 write the lower 64 (keys of their S
-    // block, the piece's first 128), the warps with hh = 1 the upper 64.  P of pieces 0 and 2 overlays the first half of the
-    // piece's own S: a warp with hh = 0 writes behind its own reads (slab c -> P columns 16 c.. below the 32 c.. it has
-    // read), but the warps with hh = 1 write over S slabs 2 and 3 of their hh = 0 neighbours, so those are read into
-    // registers first; a barrier of the eight warps follows.  P of piece 1 overlays S of piece 0, which every warp
-    // has finished with when it passes the barrier of piece 1's maximum exchange.
+    // Reference: the maximum over the visible keys of the first slab that has any (the two warps of a row, which share
+    // its keys, exchange it once).  bf16 and fp32 have the range for weights above 1, so a later slab changes the reference
+    // only where it exceeds it by more than RESCALE_GAP (then the warp rescales what it has stored, and the two warps settle
+    // on one reference before the PV product: rare).
+    //
+    // Slabs: the warps with hh = 0 take slabs 0, 1, 4, 5 of a piece, those with hh = 1 slabs 2, 3, 6, 7.  P of piece pc lands in
+    // columns [128 pc, 128 pc + 128), a warp's slabs side by side from 64 hh on: P of pieces 0 and 1 overlays S of piece 0, P of
+    // piece 2 overlays S of piece 2, and with this split every column a warp writes held S of its OWN slabs, all read
+    // before: no warp waits for another.  (A two-pass softmax with contiguous halves needed three barriers a piece and
+    // read S twice.)
+    constexpr uint32_t FULL = 0xffffffffu;
+    uint32_t* xch = reinterpret_cast<uint32_t*>(sm.xch);
+    auto pair_sync = [&]() { asm volatile("bar.sync %0, 64;" ::"r"(2 + q4) : "memory"); };     // the two warps of these rows
+    auto slab_of = [&](int i) { return (i & 1) + ((i & 2) << 1) + 2 * hh; };
+    auto masked = [&](const uint32_t* sv, uint32_t vis, float* v) {      // invisible keys as -inf
+      if (vis == FULL) {
+#pragma unroll
+        for (int t = 0; t < 32; ++t) v[t] = __uint_as_float(sv[t]);
+      } else {
+#pragma unroll
+        for (int t = 0; t < 32; ++t) v[t] = ((vis >> t) & 1u) ? __uint_as_float(sv[t]) : -INFINITY;
+      }
+    };
+    auto max32 = [&](const float* v) {
+      float mc[4] = {v[0], v[1], v[2], v[3]};
+#pragma unroll
+      for (int t = 4; t < 32; ++t) mc[t & 3] = fmaxf(mc[t & 3], v[t]);
+      return fmaxf(fmaxf(mc[0], mc[1]), fmaxf(mc[2], mc[3]));
+    };
+    // multiplies this thread's P columns [64 hh of every piece before pc, the first n slabs of piece pc] by f
+    auto rescale_p = [&](int pc, int n, float f) {
+      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+#pragma unroll 1
+      for (int v = 0; v < 4 * pc + n; ++v) {
+        const uint32_t col = tlane + (v >> 2) * 128 + hh * 64 + (v & 3) * 16;
+        uint32_t r[16];
+        tmem_ld16(col, r);
+#pragma unroll
+        for (int t = 0; t < 16; ++t) {
+          const float2 w = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&r[t]));
+          const __nv_bfloat162 h2 = __floats2bfloat162_rn(w.x * f, w.y * f);
+          r[t] = *reinterpret_cast<const uint32_t*>(&h2);
+        }
+        tmem_st16(col, r);
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c) lp[c] *= f;
+    };
+    int moved = 0;                                   // this warp changed its reference after the exchange
+    auto do_slab = [&](const uint32_t* sv, uint32_t vis, int pc, int i) {
+      float v[32];
+      uint32_t pk[16];
+      masked(sv, vis, v);
+      const float mc = max32(v) * scale2;
+      if (__any_sync(FULL, mc > m_run + RESCALE_GAP)) {        // (warp-uniform: tensor-memory accesses are warp-collective)
+        const float to = mc > m_run + RESCALE_GAP ? mc : m_run;
+        rescale_p(pc, i, ex2(m_run - to));
+        m_run = to;
+        moved = 1;
+      }
+#pragma unroll
+      for (int t = 0; t < 32; t += 2) {
+        const float p0 = ex2(fmaf(v[t], scale2, -m_run)), p1 = ex2(fmaf(v[t + 1], scale2, -m_run));
+        lp[(t >> 1) & 3] += p0 + p1;
+        const __nv_bfloat162 h2 = __floats2bfloat162_rn(p0, p1);
+        pk[t >> 1] = *reinterpret_cast<const uint32_t*>(&h2);
+      }
+      tmem_st16(tlane + pc * 128 + hh * 64 + i * 16, pk);
+    };
 #pragma unroll 1
     for (int pc = 0; pc < npc; ++pc) {
+      const int ns = CL - pc * 256 >= 256 ? 4 : 2;   // slabs of this warp
+      // visibility, 32 keys per word: the 32 rows of a warp belong to one node (H >= 32 on this path), so one ballot over the
+      // keys' node masks gives the word
+      uint32_t vis[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) vis[i] = i < ns ? __ballot_sync(FULL, sm.kmask[pc * 256 + slab_of(i) * 32 + lane] & mybit) : 0u;
       if (!fail && !mbar_wait(&sm.acc_ev[pc], 0)) fail = 1;
       fence_after();
-      const bool mine = block_mine(pc);
-      const uint32_t scol = tlane + (pc == 0 ? 0 : 256) + hh * 128, pcol = tlane + pc * 128 + hh * 64;
-      float mx = -INFINITY;
-      if (mine) {
-#pragma unroll 1
-        for (int c = 0; c < 4; ++c) mx = slab_max(scol + c * 32, slab_vis(pc, c), mx);
+      const uint32_t scol = tlane + (pc == 0 ? 0 : 256);
+      uint32_t sv[2][32];
+      if (m_run == -INFINITY) {                      // uniform over the two warps of these rows: no visible key so far
+        const int first = vis[0] ? 0 : vis[1] ? 1 : vis[2] ? 2 : vis[3] ? 3 : -1;
+        float mc = -INFINITY;
+        if (first >= 0) {
+          uint32_t s0[32];
+          const uint32_t w = first == 0 ? vis[0] : first == 1 ? vis[1] : first == 2 ? vis[2] : vis[3];
+          tmem_ld32(scol + slab_of(first) * 32, s0);
+          float v[32];
+          masked(s0, w, v);
+          mc = max32(v);
+        }
+        xch[hh * BM + row] = __float_as_uint(mc);
+        pair_sync();
+        m_run = fmaxf(mc, __uint_as_float(xch[(hh ^ 1) * BM + row])) * scale2;
+        pair_sync();                                 // (the exchange words may be written again)
       }
-      sm.xch[hh][row] = mx;
-      compute_sync();
-      const float m_pass = fmaxf(sm.xch[0][row], sm.xch[1][row]) * scale2;
-      float factor = 1.f;
-      if (m_pass > m_run + RESCALE_GAP || m_run == -INFINITY) {
-        if (m_run != -INFINITY) factor = ex2(m_run - m_pass);
-        m_run = m_pass;
-      }
-      if (pc && __any_sync(0xffffffffu, factor != 1.f)) {  // warp-uniform: tcgen05.ld/st are warp-collective
-#pragma unroll 1
-        for (int v = 0; v < 2 * pc; ++v) {           // this thread's P columns of the earlier pieces
-          const uint32_t qcol = tlane + (v >> 1) * 128 + hh * 64 + (v & 1) * 32;
-          uint32_t r[32];
-          tmem_ld32(qcol, r);
+      const bool any = m_run != -INFINITY;
+      tmem_ld32_nowait(scol + slab_of(0) * 32, sv[0]);
 #pragma unroll
-          for (int t = 0; t < 32; ++t) {
-            float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&r[t]));
-            const __nv_bfloat162 h2 = __floats2bfloat162_rn(f.x * factor, f.y * factor);
-            r[t] = *reinterpret_cast<const uint32_t*>(&h2);
-          }
-          tmem_st16(qcol, r);
-          tmem_st16(qcol + 16, r + 16);
-        }
+      for (int i = 0; i < 4; ++i) {
+        if (i < ns) {
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          tmem_regs_ready(sv[i & 1]);
+          if (i + 1 < ns) tmem_ld32_nowait(scol + slab_of(i + 1) * 32, sv[(i + 1) & 1]);
+          if (any && vis[i]) do_slab(sv[i & 1], vis[i], pc, i);
+          else {
+            uint32_t z[16];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) lp[c] *= factor;
-      }
-      const float moff = (m_run == -INFINITY) ? 0.f : m_run;
-      {
-        uint32_t hold[64];
-        if (hh == 0) {
-          if (mine) {
-            tmem_ld32_nowait(scol + 64, hold);
-            tmem_ld32_nowait(scol + 96, hold + 32);
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            tmem_regs_ready(hold);
-            tmem_regs_ready(hold + 32);
-          }
-          fence_before();
-        }
-        // all eight warps meet: the neighbours' slabs are in registers, and everybody has read the exchanged maxima (the
-        // exchange buffer is written again for the next piece)
-        asm volatile("bar.sync 2, 256;" ::: "memory");
-        if (hh) fence_after();
-        if (mine) {
-          const int nstream = hh == 0 ? 2 : 4;
-#pragma unroll 1
-          for (int c = 0; c < nstream; ++c) {
-            uint32_t sv[32];
-            tmem_ld32(scol + c * 32, sv);
-            slab_exp(sv, slab_vis(pc, c), moff, pcol + c * 16);
-          }
-          if (hh == 0) {
-            slab_exp(hold, slab_vis(pc, 2), moff, pcol + 32);
-            slab_exp(hold + 32, slab_vis(pc, 3), moff, pcol + 48);
+            for (int t = 0; t < 16; ++t) z[t] = 0u;
+            tmem_st16(tlane + pc * 128 + hh * 64 + i * 16, z);
           }
         }
-        // the MMA warp waits for the last piece only (and, with three pieces, for piece 1 before it overwrites that
-        // piece's S columns); the wait for the stores of a later piece covers the earlier ones
-        if (pc == npc - 1 || (npc == 3 && pc == 1)) p_stored(pc);
       }
+      // the MMA warp waits for the last piece only (and, with three pieces, for piece 1 before it overwrites that
+      // piece's S columns); the wait for the stores of a later piece covers the earlier ones
+      if (npc == 3 && pc == 1) p_stored(1);
     }
-    const float l_part = (lp[0] + lp[1]) + (lp[2] + lp[3]);
-    sm.xch[hh][row] = l_part;
-    compute_sync();
-    const float l_row = sm.xch[0][row] + sm.xch[1][row];
+    // The row sums meet (in the output staging area, idle until O is read out); where a warp moved its reference, the two
+    // settle on the larger one first.
+    float l_row = (lp[0] + lp[1]) + (lp[2] + lp[3]);
+    {
+      const uint32_t mine = ring + (uint32_t)NSV * SLOTP + (uint32_t)(warp - 2) * 8192, other = ring + (uint32_t)NSV * SLOTP + (uint32_t)((warp - 2) ^ 4) * 8192;
+      auto put = [&](int w, float v) { asm volatile("st.shared.b32 [%0], %1;" ::"r"(mine + (uint32_t)(w * 128 + lane * 4)), "r"(__float_as_uint(v)) : "memory"); };
+      auto get = [&](int w) { uint32_t v; asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(other + (uint32_t)(w * 128 + lane * 4)) : "memory"); return __uint_as_float(v); };
+      put(0, l_row); put(1, m_run); put(2, moved ? 1.f : 0.f);
+      pair_sync();
+      float l_other = get(0);
+      if (moved || get(2) != 0.f) {                  // warp-uniform, and alike in both warps
+        const float m_other = get(1), to = fmaxf(m_run, m_other);
+        if (to != -INFINITY) {
+          const float f = ex2(m_run - to), fo = ex2(m_other - to);
+          const int last = npc - 1;
+          if (__any_sync(FULL, f != 1.f)) rescale_p(last, CL - last * 256 >= 256 ? 4 : 2, f);
+          l_row *= f; l_other *= fo;
+          m_run = to;
+        }
+      }
+      p_stored(npc - 1);
+      l_row += l_other;
+    }
 
     const bool rowok = row0 + row < rows_seq;
     const bool full_tile = row0 + BM <= rows_seq;     // whole tile inside the sequence: rows may be stored as 32-row boxes
     const float inv = l_row > 0.f ? 1.f / l_row : 0.f;
     const int cw = OW / 2;                            // columns of the part this thread handles: 128 or 64
-    const uint32_t stage = ring + (uint32_t)NSX * SLOTP + (uint32_t)(warp - 2) * 4096;   // this warp's 32 rows x 64 columns (bf16)
-    bool store_pending = false;
+    const uint32_t stage0 = ring + (uint32_t)NSV * SLOTP + (uint32_t)(warp - 2) * 8192;   // this warp's two tiles of 32 rows x 64 columns (bf16)
+    int nstore = 0;
     for (int part = 0; part < NQ; ++part) {
       if (!fail && !mbar_wait(&sm.acc_ev[3 + part], 0)) fail = 1;
       fence_after();
@@ -554,8 +580,9 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
           // stage the 32 x 64 bf16 tile in the 128-byte swizzle pattern and store it with one TMA request: into the output,
           // or (multi-chunk tiles, where a merge kernel follows) into the chunk's tile of normalised partial outputs, which a merge kernel
           // combines with the chunks' (max, sum)
-          if (store_pending) {
-            if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+          const uint32_t stage = stage0 + (uint32_t)(nstore & 1) * 4096;
+          if (nstore >= 2) {                           // the store before the last has read its tile
+            if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
             __syncwarp();
           }
 #pragma unroll
@@ -580,7 +607,7 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
                          ::"l"(reinterpret_cast<uint64_t>(omap)), "r"(col), "r"(orow), "r"(stage) : "memory");
             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
           }
-          store_pending = true;
+          ++nstore;
         } else if (nch == 1) {
           if (rowok) {
             bf16* orow = reinterpret_cast<bf16*>(out_) + ((size_t)b * rows_seq + row0 + row) * DH + col;
@@ -609,7 +636,7 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
       if (nch > 1 && part == 0 && hh == 0)
         reinterpret_cast<float2*>(ws + pl.off_tpml)[(rix * pl.tc_chmax + chunk) * BM + row] = make_float2(m_run, l_row);
     }
-    if (store_pending && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    if (nstore && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     if (!GENERAL && nch > 1) {
       // Tiles of two chunks where nothing longer can occur: each chunk leaves its unnormalised part of O with (max, sum)
       // per row; the CTA that finishes a 128-row tile last merges the parts (fixed order, so the result does not depend
