@@ -31,6 +31,10 @@ __device__ __forceinline__ int tile_keys_estimate(const tsv_shape& s, int L, int
   return min(n_csa, npt * s.topk) + n_hca + win + 3 * nn;
 }
 
+__device__ __forceinline__ void l2_prefetch(const void* p, uint32_t bytes) {       // (16-byte aligned, a multiple of 16 bytes)
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+
 // GENERAL: gathered tiles may occur (see gathered_tiles_possible); the instantiation without them keeps the short
 // latency chain of the contiguous-run plan.
 template <bool GENERAL>
@@ -406,9 +410,19 @@ __global__ void __launch_bounds__(NT) tc_plan_kernel(const tsv_shape s, const Tv
   const bool tile_cta = blockIdx.x < (unsigned)pl.tc_nt;
   const size_t tix = (size_t)blockIdx.y * pl.tc_nt + blockIdx.x;
   if (threadIdx.x == 0) ahead_sm = 0;
+  if (threadIdx.x < 2 && blockIdx.x == 0 && blockIdx.y == 0) reinterpret_cast<int32_t*>(ws + pl.off_sched)[threadIdx.x] = 0;   // the attention kernel's item counters
   if (threadIdx.x < 2 && tile_cta)                      // finished-chunk counters of the tile's two 128-row halves
     reinterpret_cast<int32_t*>(ws + pl.off_tcnt)[tix * 2 + threadIdx.x] = 0;
   tc_plan_tile<GENERAL>(s, pl, c, nd, sc, ws, cmask_sm, est_sm, &ahead_sm);
+  // The tile's queries into L2: the pairs of the attention kernel all start at once, and the first phase of each is bound by
+  // what arrives from HBM, which idles under the kernels before (first operands of 64 short sequences 10 k -> 7.5 k cycles
+  // after the start, last of the first piece 18 k -> 13 k).  At the end of the CTA's own work, which is a chain of loads that
+  // would queue behind these.
+  if (tile_cta && threadIdx.x < 4) {
+    const int rows_seq = s.D * s.H, r0 = blockIdx.x * tc::PR, rows = min(tc::PR, rows_seq - r0), part = (rows + 3) / 4;
+    const int p0 = min(rows, (int)threadIdx.x * part), pn = min(part, rows - p0);
+    if (pn > 0) l2_prefetch(reinterpret_cast<const char*>(nd.q) + ((size_t)blockIdx.y * rows_seq + r0 + p0) * (tc::DH * 2), (uint32_t)pn * (tc::DH * 2));
+  }
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // (at the END of the CTA's work: the attention kernel's CTAs take their places as this kernel's leave)
   // one CTA waits for the selection in any case, so that the completion of this kernel implies that one's
   if (blockIdx.x == 0 && blockIdx.y == 0) asm volatile("griddepcontrol.wait;" ::: "memory");

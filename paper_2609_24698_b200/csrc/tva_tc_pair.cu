@@ -18,6 +18,8 @@
 #include <stdio.h>
 #include <cudaTypedefs.h>
 
+#include <atomic>
+
 #include "tc_common.cuh"
 
 namespace tsv {
@@ -26,29 +28,36 @@ namespace pair {
 
 using namespace tc;
 
-constexpr int NPROD = 2;                    // producer warps: warp 0 and warp 10
-constexpr int TTHREADS = 32 * (10 + NPROD - 1);   // warp 1: MMA issuer; warps 2-9: softmax and epilogue
+// Warps: 0, 3, 12-15 producers; 1 MMA issuer; 2 hands out the items; 4-11 softmax and epilogue.  The service warpgroups give
+// registers to the compute warpgroups: 128 x (80 + 176 + 176 + 80) of the 512 x 128 the CTA is launched with.
+constexpr int TTHREADS = 512;
+constexpr int NPROD = 6;                    // (12 slots: six producers with two each)
+constexpr int REGS_SERVICE = 80, REGS_COMPUTE = 176;
+static_assert(128 * (2 * REGS_SERVICE + 2 * REGS_COMPUTE) <= TTHREADS * 128, "register split beyond what the CTA is launched with");
 constexpr int BOXB = kBoxRows * 128;       // bytes of one box: kBoxRows rows x 128 bytes
 constexpr float RESCALE_GAP = 16.f;        // log2 units a later piece's row max may exceed the running reference
 
 constexpr int NSX = 14;                    // 16 KiB slots of the staging area
-constexpr int NQS = 8;                     // S phase: slots [0, 8) hold the Q slices (all of d, resident for every piece),
-constexpr int NKS = NSX - NQS;             //          slots [8, 14) are the ring of the K stages;
-constexpr int NSV = 10;                    // V phase: slots [0, 10) form the ring of the V stages, slots [10, 14) stage the output: two tiles of
-                                           //          32 rows x 64 columns per warp, so that a tile is written while the one before leaves
+constexpr int NQS = 8;                     // Q slices of an item (all of d, resident for every piece)
+constexpr int NKS = NSX - NQS;             // K stages in flight
+constexpr int NSV = 12;                    // Slots [0, 12) are one FIFO: an item's eight Q slices and its first four K stages take the next twelve
+                                           // places, its V stages (once the S products are complete) the places from the same start on; so
+                                           // the next item's Q slices land where the V stages are released first.  Slots 12, 13: the other
+                                           // two K stages, and, when O is read out, the staging of the output (a 4 KiB tile per warp).
 
-struct Ctl {                               // control block at the start of dynamic shared memory
-  uint64_t fullQ[NQS];                     // Q slice dk has arrived (used once)
+struct Ctl {                               // control block at the start of dynamic shared memory; no barrier is ever re-initialised
+  uint64_t fullQ[NQS];                     // Q slice dk of the item has arrived
   uint64_t fullK[NKS], emptyK[NKS];        // ring of the K stages
   uint64_t fullV[NSV], emptyV[NSV];        // ring of the V stages (starts when the S products are complete)
-  uint64_t acc_ev[7];                      // MMA -> other warps, one barrier per event, each used once:
+  uint64_t acc_ev[7];                      // MMA -> other warps, one barrier per event, at most once per item:
                                            //   [pc] S of piece pc is complete   [3 + p] part p of O is complete
-  uint64_t cmp_ev[6];                      // compute warps -> MMA, one barrier per event, each used once:
+  uint64_t cmp_ev[7];                      // compute warps -> MMA, likewise:
                                            //   [pc] P of piece pc is in TMEM   [3 + p] part p of O has been read out
+  uint64_t stage_free;                     // the item's output tiles have left the staging slots (this CTA's)
+  uint64_t item_ev;                        // the next item has been handed out
   uint32_t tmem_base;
   int32_t merge_here;                      // set for the CTA that finished a multi-chunk tile last
-  uint32_t box[NCX / kBoxRows];            // tensor map id << 30 | first row
-  uint8_t kmask[NCX];
+  alignas(16) int4 item[2];                // the pair's current and next work: {tile index (-1: no more), mode, keys, chunk}
   float xch[2][BM];                        // first-slab maxima of the rows, by the two warps that share them
 };
 constexpr int CTLB = 3072;                 // control block bytes; the ring follows (needs a 1024-byte aligned base)
@@ -101,10 +110,20 @@ __device__ __forceinline__ void mma2_commit(uint64_t* bar) {
 __device__ __forceinline__ uint32_t make_idesc2(int N, int b_mn_major) {      // M = 256 over the pair
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)b_mn_major << 16) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
 }
+// 16 bytes into the shared memory of a CTA of the pair, counted on a barrier of the same CTA (both by cluster address)
+__device__ __forceinline__ void st_async16(uint32_t cluster_addr, const int4& v, uint32_t bar_cluster_addr) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+               ::"r"(cluster_addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(bar_cluster_addr) : "memory");
+}
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 // the two halves of the pair-wide barrier, for work that does not depend on the peer in between
+__device__ __forceinline__ bool elect_one() {           // true in one lane of the (converged) warp
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(r));
+  return r != 0;
+}
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void compute_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
@@ -124,274 +143,435 @@ constexpr uint32_t OOB_BOX = 0x3FFFFF00u;   // map 0, a row beyond every tensor:
 
 }  // namespace pair
 
-// Per CTA (rank r of the pair), for a chunk of CL keys (pieces of 256 keys, the last may hold 128):
+// One item of work: a chunk of CL keys (pieces of 256 keys, the last may hold 128) of one 256-row tile.
+namespace pair {
+struct Item {
+  int tix, b, tile, nk, chunk, nch, CL, cbeg, cend;
+  int npc;                 // S pieces
+  int NQ, OW;              // the PV product is computed in NQ parts of OW columns of d
+  bool gather;             // the key list is a list of row codes (array << 30 | row), not of boxes
+  __device__ __forceinline__ Item(int4 r, const TvaPlan& pl, bool general) {
+    tix = r.x; b = r.x / pl.tc_nt; tile = r.x - b * pl.tc_nt;
+    gather = general && r.y == 2;
+    nk = r.z; chunk = r.w;
+    tc::chunking_x(nk, general, nch, CL);
+    cbeg = chunk * CL; cend = min(nk, cbeg + CL);
+    npc = (CL + 255) / 256;
+    NQ = CL <= 512 ? 2 : 4;
+    OW = tc::DH / NQ;
+  }
+  __device__ __forceinline__ uint32_t acc_used() const { return ((1u << npc) - 1u) | (((1u << NQ) - 1u) << 3); }
+  __device__ __forceinline__ uint32_t cmp_used() const { return (1u << (npc - 1)) | (npc == 3 ? 2u : 0u) | (((1u << NQ) - 1u) << 3); }
+};
+}  // namespace pair
+
+// PERSISTENT: one pair per two SMs walks its share of the items.  What a pair that served one item each lost on every item
+// (start-up of the CTAs and barriers 4 k cycles, the gap between two CTAs on an SM 5 k, the first operands' latency
+// 4-6 k, of 47 k for 512 keys) happens once: barriers and tensor memory live as long as the kernel, the next item's Q
+// slices go into the V slots the last part of O has released, its first K stages follow, and its S products run under the
+// read-out and the stores of the last part of O.
+//
+// Stages per item and CTA (rank r of the pair):
 //   Q slices:  per 64-wide slice dk of d  [this CTA's 128 rows x 64 dims], fetched once, resident for all pieces
 //   K stages:  piece after piece, per slice dk  [this CTA's half of the piece's keys x 64 dims]
 //   V stages (after the last S product): CL <= 512: per half of d, per 64 keys:  [64 keys x this CTA's 128 of the half's 256 dims]
 //                                        else       per quarter of d, per 128 keys: [128 keys x this CTA's 64 of the quarter's 128 dims]
+// TMEM columns (per CTA, its own 128 rows).  S piece 0 -> [0,256), pieces 1 and 2 -> [256,512) (fp32); P piece pc (bf16 pairs) ->
+// [128 pc, 128 pc + 128); O: CL <= 512 in two halves of 256 columns at [256,512), else in four quarters of 128 columns at [384,512).
 //
-// GENERAL: gathered tiles and tiles of more than two chunks may occur.  Shapes whose capacities rule both out (the
-// benchmark's) run the instantiation without that code: the kernel is one long dependency chain per tile and its
-// timing follows the code layout.
+// Every barrier phase is counted by its users: each role keeps, per barrier, the parity of its next use, and a slot's
+// latest release is awaited before it is filled again, across items too.
+//
+// GENERAL: gathered tiles and tiles of more than two chunks may occur (shapes whose capacities rule both out run the
+// instantiation without that code).
 template <bool GENERAL>
 __global__ void __launch_bounds__(pair::TTHREADS, 1)
 tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s,
                     const TvaPlan pl, void* __restrict__ out_, char* __restrict__ ws, int32_t* __restrict__ status) {
   using namespace pair;
   extern __shared__ unsigned char smem_raw[];
-  // the two CTAs of a pair are neighbours in x; pairs take the (sequence, tile) items in the order the plan kernel left
-  // (most keys first)
-  const int chunk = blockIdx.y;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  uint32_t rank;
+  uint32_t rank;                                                // the two CTAs of a pair are neighbours in x
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
   Ctl& sm = *reinterpret_cast<Ctl*>(smem_raw);
   const uint32_t ring = smem_u32(smem_raw + CTLB);
   int fail = (smem_u32(smem_raw) & 1023u) ? 1 : 0;             // the swizzled tiles need a 1024-byte aligned base
   if (tid < (GENERAL ? NMAPS : 14))   // the descriptors of the tensor maps in use are fetched while the plan is read
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&maps) + (uint64_t)tid * sizeof(CUtensorMap)) : "memory");
-  // Barriers, tensor memory and the first half of the pair-wide barrier that announces them.
-  auto set_up = [&]() {
-    if (tid == 0) {
-      for (int i = 0; i < NQS; ++i) mbar_init(&sm.fullQ[i], 1);
-      for (int i = 0; i < NKS; ++i) { mbar_init(&sm.fullK[i], 1); mbar_init(&sm.emptyK[i], 1); }
-      for (int i = 0; i < NSV; ++i) { mbar_init(&sm.fullV[i], 1); mbar_init(&sm.emptyV[i], 1); }
-      for (int i = 0; i < 7; ++i) mbar_init(&sm.acc_ev[i], 1);
-      for (int i = 0; i < 6; ++i) mbar_init(&sm.cmp_ev[i], 16);   // 8 compute warps of each CTA
-      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (warp == 0) {
-      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&sm.tmem_base)) : "memory");
-      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-    }
-    __syncwarp();
-    cluster_arrive();
-  };
-  // ... and their end, for a pair that finds nothing to do after it has set up
-  auto tear_down = [&]() {
+  if (tid == 0) {
+    for (int i = 0; i < NQS; ++i) mbar_init(&sm.fullQ[i], 1);
+    for (int i = 0; i < NKS; ++i) { mbar_init(&sm.fullK[i], 1); mbar_init(&sm.emptyK[i], 1); }
+    for (int i = 0; i < NSV; ++i) { mbar_init(&sm.fullV[i], 1); mbar_init(&sm.emptyV[i], 1); }
+    for (int i = 0; i < 7; ++i) { mbar_init(&sm.acc_ev[i], 1); mbar_init(&sm.cmp_ev[i], 16); }   // 8 compute warps of each CTA
+    mbar_init(&sm.stage_free, 8);
+    mbar_init(&sm.item_ev, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&sm.tmem_base)) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  __syncwarp();
+  cluster_arrive();                                              // this CTA's barriers exist and its tensor memory is allocated
+  auto leave = [&]() {
+    if (fail) for (int b = (int)(blockIdx.x >> 1); b < s.B; b += (int)(gridDim.x >> 1)) atomicOr(status + b, TSV_ST_INTERNAL);   // (an internal error: every sequence is flagged)
     fence_before();
     __syncthreads();
-    cluster_wait();
+    cluster_sync_all();                                          // neither CTA leaves while the other may still signal it or read its memory
     fence_after();
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(sm.tmem_base) : "memory");
   };
-  // Launched as a programmatic dependent of the tile plan: the CTAs take their places while that kernel's last CTAs
-  // finish, and read nothing of its before it has completed.  The set-up reads nothing at all: the pairs of a tile's first
-  // chunk, which nearly always find work, do it before the wait (later chunks first learn whether they exist).
-  if (chunk == 0) set_up();
+  // Launched as a programmatic dependent of the tile plan: the CTAs take their places and set up while that kernel's last
+  // CTAs finish, and read nothing of its before it has completed.
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  const int4 rec = reinterpret_cast<const int4*>(ws + pl.off_order)[blockIdx.x >> 1];   // {tile index, mode, keys, -}: one load
-  const int item = rec.x;
-  const int b = item / pl.tc_nt, tile = item % pl.tc_nt;
-  const size_t tix = (size_t)b * pl.tc_nt + tile;
-  const size_t rix = (size_t)b * 2 * pl.tc_nt + 2 * tile + rank;  // this CTA's 128-row tile (partials of multi-chunk tiles)
-  // every exit below is taken by both CTAs of the pair alike (it depends on the pair's plan only)
-  const bool gather = GENERAL && rec.y == 2;                              // the key list is a list of row codes (array << 30 | row), not of boxes
-  const int nk = rec.y == 1 || gather ? rec.z : 0;
-  const int rows_seq = s.D * s.H, row0 = tile * PR + (int)rank * BM;           // first of this CTA's rows within the sequence
-  int nch, CL;
-  chunking_x(nk, GENERAL, nch, CL);
-  if (nk <= 0 || chunk >= nch) {
-    if (chunk == 0) {                                          // flagged sequence or padding-only tile: zeros
-      if (rec.y == 1 || gather) {
-        uint4* o4 = reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(out_) + ((size_t)b * rows_seq + row0) * DH);
-        for (int i = tid; i < BM * DH / 8; i += TTHREADS)
-          if (row0 + i / (DH / 8) < rows_seq) o4[i] = make_uint4(0, 0, 0, 0);
-      }
-      tear_down();
-    }
-    return;
-  }
-  const int cbeg = chunk * CL, cend = min(nk, cbeg + CL);
-  if (chunk) set_up();
-  // The plan's boxes and key masks are read while the peer sets up; the wait for it follows.
-  {
-    const int2* box_g = reinterpret_cast<const int2*>(ws + pl.off_box) + tix * (size_t)(pl.tc_maxk / kBoxRows);
-    const uint8_t* kmask_g = reinterpret_cast<const uint8_t*>(ws + pl.off_kmask) + tix * pl.tc_maxk;
-    if (tid < NCX / kBoxRows && !gather) {
-      uint32_t v = OOB_BOX;
-      if (cbeg + tid * kBoxRows < cend) { const int2 bx = box_g[cbeg / kBoxRows + tid]; v = ((uint32_t)bx.x << 30) | (uint32_t)bx.y; }
-      sm.box[tid] = v;
-    }
-    for (int i = tid; i < NCX; i += TTHREADS) sm.kmask[i] = (cbeg + i < cend) ? kmask_g[cbeg + i] : (uint8_t)0;
-  }
+  const int4 rec0 = (int)(blockIdx.x >> 1) < s.B * pl.tc_nt ? __ldcg(reinterpret_cast<const int4*>(ws + pl.off_order) + (blockIdx.x >> 1)) : make_int4(-1, 0, 0, 0);
   fence_before();
   __syncthreads();
   cluster_wait();                                                // barriers of both CTAs exist before anyone signals them
   fence_after();
   const uint32_t tm = sm.tmem_base;
+  const int rows_seq = s.D * s.H;
+  // Item n of this pair (tile index -1: no more).  Item 0 is the first chunk of the tile of this pair's rank, which every warp
+  // looks up itself; the others are handed out (warp 2).  The wait is made whatever failed before (a failure skips later
+  // waits, never a step of the protocol, so that no warp is left alone at a barrier), and is longer than any other.
+  const int own = rec0.z > 0 ? 1 : 0;
+  auto next_item = [&](int n) {
+    if (n < own) return make_int4(rec0.x, rec0.y, rec0.z, 0);
+    bool ok = false;
+    for (int i = 0; i < 8 && !ok; ++i) ok = mbar_wait(&sm.item_ev, (uint32_t)(n - own) & 1u);
+    int4 r = sm.item[(n - own) & 1];
+    if (!ok) { r.x = -1; fail = 1; }
+    return r;
+  };
 
-  // TMEM columns (per CTA, its own 128 rows).  S piece 0 -> [0,256), pieces 1 and 2 -> [256,512) (fp32);
-  // P piece pc (bf16 pairs) -> [128 pc, 128 pc + 128).  CL <= 512: O in two halves of 256 columns at [256,512);
-  // CL <= 768: O in four quarters of 128 columns at [384,512).
-  const int npc = (CL + 255) / 256;                 // S pieces
-  const int NQ = CL <= 512 ? 2 : 4;                 // parts of d the PV product is computed in
-  const int OW = DH / NQ;                           // columns of one part
-  const uint32_t OCOL = 512 - OW;
-  const int vkeys = 16384 / OW;                     // keys per V stage: 64 or 128
-  const int nvb = CL / vkeys;                       // V stages per part
-  const int NKST = 8 * npc;                         // K stages: piece after piece, per piece the eight 64-wide slices of d
-  const int NVST = NQ * nvb;                        // V stages
-
-  if (warp == 0 || warp >= 10) {
-    // ------------------------------------------------------------------ producers (both CTAs): stage g is issued by producer g % NPROD
-    const int pw = warp == 0 ? 0 : warp - 9;
-    // consecutive: do the nb boxes starting at list index i0 name consecutive rows of one array?
-    auto consecutive = [&](int i0, int nb) {
-      const uint32_t b0 = sm.box[i0];
-      if ((b0 & 0x3FFFFFFFu) >= (OOB_BOX & 0x3FFFFFFFu)) return false;
-      for (int i = 1; i < nb; ++i) if (sm.box[i0 + i] != b0 + (uint32_t)(i * kBoxRows)) return false;
-      return true;
+  // (the register split dominates each side's code, which the compiler budgets by it)
+  if (warp < 4 || warp >= 12) {
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_SERVICE));
+  if (warp == 0 || warp == 3 || warp >= 12) {
+    // ------------------------------------------------------------------ producers (both CTAs)
+    // Every slot belongs to one producer, which issues all its copies and awaits all its releases in order (a parity wait
+    // is only good for the phase after the last one seen).  Both CTAs' copies complete on the leader's barriers.
+    // (Six warps because of the gathered tiles: a stage is 32 four-row requests there, and a warp takes about 70 cycles to
+    // issue one; boxes would do with two.)
+    const int pw = warp == 0 ? 0 : warp == 3 ? 1 : warp - 10;
+    uint32_t kcnt = 0, kused = 0, vcnt = 0, vused = 0, accb = 0;  // per slot: parity of the number of uses so far, used at all
+    int n_real = 0;                                               // items with keys so far
+    auto slot_wait = [&](uint64_t* empty, uint32_t cnt, uint32_t used, int sl) {      // the slot's latest release
+      if (((used >> sl) & 1u) && !fail && !mbar_wait(&empty[sl], ((cnt >> sl) & 1u) ^ 1u)) fail = 1;
     };
-    // Q slices: producer 0.  K stage gk = 8 pc + dk: producer (gk + 1) & 1, so that the first K stage leaves at the same
-    // time as the first Q slice.  V stage gv: producer gv & 1.  Both CTAs' copies complete on the leader's barriers.
-    auto issue_q = [&](int dk) {
-      if (lane == 0) {
-        if (rank == 0) mbar_expect_tx(&sm.fullQ[dk], 2 * SLOTP);
-        tma_box2(ring + (uint32_t)dk * SLOTP, &maps.q, dk * 64, b * rows_seq + row0, map_to_rank(smem_u32(&sm.fullQ[dk]), 0));
+    // the boxes of a chunk: lane i holds box i of up to NCX / kBoxRows
+    auto load_box = [&](const Item& w) {
+      uint32_t v = OOB_BOX;
+      if (!w.gather && lane < NCX / kBoxRows && w.cbeg + lane * kBoxRows < w.cend) {
+        const int2 bx = __ldg(reinterpret_cast<const int2*>(ws + pl.off_box) + (size_t)w.tix * (pl.tc_maxk / kBoxRows) + w.cbeg / kBoxRows + lane);
+        v = ((uint32_t)bx.x << 30) | (uint32_t)bx.y;
       }
-      __syncwarp();
+      return v;
     };
-    // Gathered tiles: the keys' row codes stay in global memory (the tile plan left them there, four-aligned groups
-    // never mix arrays); lane l fetches the codes of rows 4 l .. 4 l + 3 of a stage itself.  Keys past the end of the list
-    // read row 0 of the first array (they are masked).
-    const uint4* code_g = reinterpret_cast<const uint4*>(reinterpret_cast<const uint32_t*>(ws + pl.off_krow) + tix * (size_t)pl.tc_maxk + cbeg);
-    auto codes_at = [&](int key) { return cbeg + key < cend ? __ldg(code_g + (key >> 2)) : make_uint4(0u, 0u, 0u, 0u); };
-    uint4 kcode = make_uint4(0u, 0u, 0u, 0u);                                // this lane's codes of the current piece's K stages
-    int kcode_pc = -1;
-    auto issue_k = [&](int gk) {
-      const int pc = gk >> 3, dk = gk & 7, sl = gk % NKS, use = gk / NKS;
-      const uint32_t slot = ring + (uint32_t)(NQS + sl) * SLOTP;
-      const uint32_t fb_leader = map_to_rank(smem_u32(&sm.fullK[sl]), 0);
-      const int bytes = min(256, CL - pc * 256) * 64;                        // bytes THIS CTA copies in the stage
-      if (gather && kcode_pc != pc) {                                        // this CTA's half of the piece's keys: bytes / 128 rows
-        kcode_pc = pc;
-        if (lane * 512 < bytes) kcode = codes_at(pc * 256 + (int)rank * (bytes >> 7) + 4 * lane);
-      }
-      if (lane == 0) {
-        if (use > 0 && !fail && !mbar_wait(&sm.emptyK[sl], (uint32_t)(use - 1) & 1u)) fail = 1;
-        if (rank == 0) mbar_expect_tx(&sm.fullK[sl], 2 * bytes);              // bytes of both CTAs
-      }
-      __syncwarp();
-      // this CTA's half of the piece's keys: boxes [rank * nb, rank * nb + nb) of the piece
-      const int nb = bytes / BOXB, i0 = pc * (256 / kBoxRows) + (int)rank * nb;
-      if (gather) {
-        if (lane * 512 < bytes) tma_gather4(slot + lane * 512, &maps.row[kcode.x >> 30], dk * 64, kcode, fb_leader);
-      } else if (consecutive(i0, nb)) {                                             // nb = 4 (128 rows) or 2 (64 rows)
-        if (lane == 0) { const uint32_t bx = sm.box[i0]; tma_box2(slot, &maps.src[bx >> 30][nb == 4 ? 2 : 1], dk * 64, (int)(bx & 0x3FFFFFFFu), fb_leader); }
-      } else if (lane < nb) {
-        const uint32_t bx = sm.box[i0 + lane];
-        tma_box2(slot + lane * BOXB, &maps.src[bx >> 30][0], dk * 64, (int)(bx & 0x3FFFFFFFu), fb_leader);
-      }
-      __syncwarp();
-    };
-    if (pw == 0) {
-      for (int i = 0; i < 4; ++i) { issue_q(2 * i); issue_q(2 * i + 1); issue_k(2 * i + 1); }
-      for (int gk = 9; gk < NKST; gk += 2) issue_k(gk);
-    } else {
-      for (int gk = 0; gk < NKST; gk += 2) issue_k(gk);
-    }
-    // V stages reuse the whole staging area: they start when the last S product is complete (the softmax of the last
-    // piece is still to come, so the ring is full by the time the PV products start)
-    if (lane == 0 && !fail && !mbar_wait(&sm.acc_ev[npc - 1], 0)) fail = 1;
-    __syncwarp();
-    {
-      int part = 0, kb = pw;
-      while (kb >= nvb) { kb -= nvb; ++part; }
-      for (int gv = pw; gv < NVST; gv += NPROD) {
-        const int sl = gv % NSV, use = gv / NSV;
-        const uint32_t slot = ring + (uint32_t)sl * SLOTP;
-        const uint32_t fb_leader = map_to_rank(smem_u32(&sm.fullV[sl]), 0);
-        uint4 vcode = make_uint4(0u, 0u, 0u, 0u);                 // (fetched before the wait for the slot)
-        if (gather) vcode = codes_at(NQ == 2 ? kb * 64 + 4 * (lane & 15) : kb * 128 + 4 * lane);
+    int g0 = 0;                                                   // first place of the item in the FIFO
+#pragma unroll 1
+    for (int it = 0;; ++it) {
+      const int4 r = next_item(it);
+      if (r.x < 0) break;
+      const Item w(r, pl, GENERAL);
+      const uint32_t box = load_box(w);
+      const int CL = w.CL, NQ = w.NQ, row0 = w.tile * PR + (int)rank * BM;
+      const int vkeys = 16384 / w.OW, nvb = CL / vkeys;            // keys per V stage: 64 or 128; V stages per part
+      const int NKST = 8 * w.npc, NVST = NQ * nvb;
+      auto place = [&](int i) { const int p = g0 + i; return p >= NSV ? p - NSV : p; };      // slot of the FIFO's place i after the item's start
+      auto kslot = [&](int sl) { return sl < NSV - NQS ? place(NQS + sl) : NQS + sl; };
+      // (the K stages of an item lie in six slots of six producers; slots 12 and 13 change hands with the item, when
+      // everything before is complete)
+      auto mine = [&](int phys) { return (phys < NSV ? phys : g0 + phys) % NPROD == pw; };
+      // bit i: boxes i and i + 1 name consecutive rows of one array (one request can fetch both)
+      const uint32_t box_up = __shfl_down_sync(0xffffffffu, box, 1);
+      const uint32_t cons = __ballot_sync(0xffffffffu, lane < 31 && (box & 0x3FFFFFFFu) < (OOB_BOX & 0x3FFFFFFFu) && box_up == box + kBoxRows);
+      auto consecutive = [&](int i0, int nb) { return ((~(cons >> i0)) & ((1u << (nb - 1)) - 1u)) == 0u; };
+      // Gathered tiles: the keys' row codes stay in global memory (the tile plan left them there, four-aligned groups
+      // never mix arrays); lane l fetches the codes of rows 4 l .. 4 l + 3 of a stage itself.  Keys past the end of the list
+      // read row 0 of the first array (they are masked).
+      const uint4* code_g = reinterpret_cast<const uint4*>(reinterpret_cast<const uint32_t*>(ws + pl.off_krow) + (size_t)w.tix * pl.tc_maxk + w.cbeg);
+      auto codes_at = [&](int key) { return w.cbeg + key < w.cend ? __ldg(code_g + (key >> 2)) : make_uint4(0u, 0u, 0u, 0u); };
+      uint4 kcode = make_uint4(0u, 0u, 0u, 0u);                                // this lane's codes of the current piece's K stages
+      int kcode_pc = -1;
+      auto issue_q = [&](int dk) {
         if (lane == 0) {
-          if (use > 0 && !fail && !mbar_wait(&sm.emptyV[sl], (uint32_t)(use - 1) & 1u)) fail = 1;
-          if (rank == 0) mbar_expect_tx(&sm.fullV[sl], 2 * SLOTP);
+          slot_wait(sm.emptyV, vcnt, vused, place(dk));            // (a V stage of the item before)
+          if (rank == 0) mbar_expect_tx(&sm.fullQ[dk], 2 * SLOTP);
+          tma_box2(ring + (uint32_t)place(dk) * SLOTP, &maps.q, dk * 64, w.b * rows_seq + row0, map_to_rank(smem_u32(&sm.fullQ[dk]), 0));
         }
         __syncwarp();
-        if (gather) {             // NQ == 2: 16 row groups x 2 slices of 64 dims; else 32 row groups x this CTA's 64 dims
-          if (NQ == 2) tma_gather4(slot + (lane >> 4) * 8192 + (lane & 15) * 512, &maps.row[vcode.x >> 30], (part * 4 + (int)rank * 2 + (lane >> 4)) * 64, vcode, fb_leader);
-          else tma_gather4(slot + lane * 512, &maps.row[vcode.x >> 30], (part * 2 + (int)rank) * 64, vcode, fb_leader);
-        } else if (NQ == 2) {     // 64 keys x this CTA's 128 dims: key boxes i = 0..1, 64-wide slices j = 0..1
-          const int i0 = kb * (64 / kBoxRows);
-          if (consecutive(i0, 2)) {
-            if (lane < 2) { const uint32_t bx = sm.box[i0]; tma_box2(slot + lane * 8192, &maps.src[bx >> 30][1], (part * 4 + (int)rank * 2 + lane) * 64, (int)(bx & 0x3FFFFFFFu), fb_leader); }
-          } else if (lane < 4) {
-            const int i = lane >> 1, j = lane & 1;
-            const uint32_t bx = sm.box[i0 + i];
-            tma_box2(slot + j * 8192 + i * BOXB, &maps.src[bx >> 30][0], (part * 4 + (int)rank * 2 + j) * 64, (int)(bx & 0x3FFFFFFFu), fb_leader);
-          }
-        } else {                  // 128 keys x this CTA's 64 dims: key boxes 0..3
-          const int i0 = kb * (128 / kBoxRows);
-          if (consecutive(i0, 4)) {
-            if (lane == 0) { const uint32_t bx = sm.box[i0]; tma_box2(slot, &maps.src[bx >> 30][2], (part * 2 + (int)rank) * 64, (int)(bx & 0x3FFFFFFFu), fb_leader); }
-          } else if (lane < 4) {
-            const uint32_t bx = sm.box[i0 + lane];
-            tma_box2(slot + lane * BOXB, &maps.src[bx >> 30][0], (part * 2 + (int)rank) * 64, (int)(bx & 0x3FFFFFFFu), fb_leader);
-          }
+      };
+      auto issue_k = [&](int gk) {
+        const int pc = gk >> 3, dk = gk & 7, sl = gk % NKS;
+        const int phys = kslot(sl);
+        const uint32_t slot = ring + (uint32_t)phys * SLOTP;
+        const uint32_t fb_leader = map_to_rank(smem_u32(&sm.fullK[sl]), 0);
+        const int bytes = min(256, CL - pc * 256) * 64;                        // bytes THIS CTA copies in the stage
+        if (w.gather && kcode_pc != pc) {                                      // this CTA's half of the piece's keys: bytes / 128 rows
+          kcode_pc = pc;
+          if (lane * 512 < bytes) kcode = codes_at(pc * 256 + (int)rank * (bytes >> 7) + 4 * lane);
         }
-        kb += NPROD;
-        while (kb >= nvb) { kb -= nvb; ++part; }
+        if (lane == 0) {
+          if (gk < NKS) {                                          // first round of the item: what the item before kept in the slot
+            if (phys < NSV) slot_wait(sm.emptyV, vcnt, vused, phys);
+            else if (n_real > 0 && !fail && !mbar_wait(&sm.stage_free, (uint32_t)(n_real - 1) & 1u)) fail = 1;
+          }
+          slot_wait(sm.emptyK, kcnt, kused, sl);
+          if (rank == 0) mbar_expect_tx(&sm.fullK[sl], 2 * bytes);              // bytes of both CTAs
+        }
+        __syncwarp();
+        // this CTA's half of the piece's keys: boxes [rank * nb, rank * nb + nb) of the piece
+        const int nb = bytes / BOXB, i0 = pc * (256 / kBoxRows) + (int)rank * nb;
+        if (w.gather) {
+          if (lane * 512 < bytes) tma_gather4(slot + lane * 512, &maps.row[kcode.x >> 30], dk * 64, kcode, fb_leader);
+        } else {
+          const bool one = consecutive(i0, nb);                    // nb = 4 (128 rows) or 2 (64 rows)
+          const uint32_t bx = __shfl_sync(0xffffffffu, box, one ? i0 : i0 + (lane & 3));
+          if (one) { if (lane == 0) tma_box2(slot, &maps.src[bx >> 30][nb == 4 ? 2 : 1], dk * 64, (int)(bx & 0x3FFFFFFFu), fb_leader); }
+          else if (lane < nb) tma_box2(slot + lane * BOXB, &maps.src[bx >> 30][0], dk * 64, (int)(bx & 0x3FFFFFFFu), fb_leader);
+        }
+        __syncwarp();
+      };
+      auto count_k = [&](int gk) { kcnt ^= 1u << (gk % NKS); kused |= 1u << (gk % NKS); };     // every stage, whoever issues it
+#pragma unroll 1
+      for (int gk = 0; gk < NKST; ++gk) {
+        if (gk < 8 && mine(place(gk))) issue_q(gk);
+        if (mine(kslot(gk % NKS))) issue_k(gk);
+        count_k(gk);
       }
+      // V stages reuse the whole staging area: they start when the last S product is complete (the softmax of the last
+      // piece is still to come, so the ring is full by the time the PV products start)
+      if (lane == 0 && !fail && !mbar_wait(&sm.acc_ev[w.npc - 1], (accb >> (w.npc - 1)) & 1u)) fail = 1;
+      __syncwarp();
+      {
+        int part = 0, kb = 0, sl = g0;
+#pragma unroll 1
+        for (int gv = 0; gv < NVST; ++gv) {
+          if (mine(sl)) {
+            const uint32_t slot = ring + (uint32_t)sl * SLOTP;
+            const uint32_t fb_leader = map_to_rank(smem_u32(&sm.fullV[sl]), 0);
+            uint4 vcode = make_uint4(0u, 0u, 0u, 0u);               // (fetched before the wait for the slot)
+            if (w.gather) vcode = codes_at(NQ == 2 ? kb * 64 + 4 * (lane & 15) : kb * 128 + 4 * lane);
+            if (lane == 0) {
+              slot_wait(sm.emptyV, vcnt, vused, sl);
+              if (rank == 0) mbar_expect_tx(&sm.fullV[sl], 2 * SLOTP);
+            }
+            __syncwarp();
+            if (w.gather) {           // NQ == 2: 16 row groups x 2 slices of 64 dims; else 32 row groups x this CTA's 64 dims
+              if (NQ == 2) tma_gather4(slot + (lane >> 4) * 8192 + (lane & 15) * 512, &maps.row[vcode.x >> 30], (part * 4 + (int)rank * 2 + (lane >> 4)) * 64, vcode, fb_leader);
+              else tma_gather4(slot + lane * 512, &maps.row[vcode.x >> 30], (part * 2 + (int)rank) * 64, vcode, fb_leader);
+            } else if (NQ == 2) {     // 64 keys x this CTA's 128 dims: key boxes i = 0..1, 64-wide slices j = 0..1
+              const int i0 = kb * (64 / kBoxRows);
+              const bool one = consecutive(i0, 2);
+              const uint32_t bx = __shfl_sync(0xffffffffu, box, one ? i0 : i0 + ((lane >> 1) & 1));
+              if (one) { if (lane < 2) tma_box2(slot + lane * 8192, &maps.src[bx >> 30][1], (part * 4 + (int)rank * 2 + lane) * 64, (int)(bx & 0x3FFFFFFFu), fb_leader); }
+              else if (lane < 4) tma_box2(slot + (lane & 1) * 8192 + (lane >> 1) * BOXB, &maps.src[bx >> 30][0], (part * 4 + (int)rank * 2 + (lane & 1)) * 64, (int)(bx & 0x3FFFFFFFu), fb_leader);
+            } else {                  // 128 keys x this CTA's 64 dims: key boxes 0..3
+              const int i0 = kb * (128 / kBoxRows);
+              const bool one = consecutive(i0, 4);
+              const uint32_t bx = __shfl_sync(0xffffffffu, box, one ? i0 : i0 + (lane & 3));
+              if (one) { if (lane == 0) tma_box2(slot, &maps.src[bx >> 30][2], (part * 2 + (int)rank) * 64, (int)(bx & 0x3FFFFFFFu), fb_leader); }
+              else if (lane < 4) tma_box2(slot + lane * BOXB, &maps.src[bx >> 30][0], (part * 2 + (int)rank) * 64, (int)(bx & 0x3FFFFFFFu), fb_leader);
+            }
+          }
+          vcnt ^= 1u << sl; vused |= 1u << sl;
+          if (++sl == NSV) sl = 0;
+          if (++kb == nvb) { kb = 0; ++part; }
+        }
+      }
+      g0 = (g0 + NVST) % NSV;
+      accb ^= w.acc_used();
+      ++n_real;
+    }
+    // every release has arrived in this CTA before it may leave
+    if (lane == 0) {
+      for (int sl = 0; sl < NKS; ++sl) slot_wait(sm.emptyK, kcnt, kused, sl);
+      for (int sl = 0; sl < NSV; ++sl) slot_wait(sm.emptyV, vcnt, vused, sl);
     }
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer (leader CTA only)
-    if (lane == 0 && rank == 0) {
-      const uint32_t idesc_k256 = make_idesc2(256, 0), idesc_k128 = make_idesc2(128, 0), idesc_v = make_idesc2(OW, 1);
-      auto need_ev = [&](int e) { if (!fail && !mbar_wait(&sm.cmp_ev[e], 0)) fail = 1; };
-      // The issuing thread is the pacemaker of the tensor pipe: stages are walked with counters (no divisions), and the
-      // descriptors of a stage are the slot-0 descriptor plus a multiple of the slot size (the address field counts
-      // 16-byte units and cannot overflow within the ring).
-      const uint64_t dk0 = make_desc(ring, 16, 1024), dv0 = make_desc(ring, NQ == 2 ? 8192 : 16384, 1024);
-      // S, piece after piece (the softmax of a piece runs while the tensor core works on the next one): per piece the
-      // eight slices of d, Q slice from its resident slot, K stage from the ring
-      int sl = 0; uint32_t kph = 0;                      // slot and parity of the next K stage
-      for (int pc = 0; pc < npc; ++pc) {
-        if (pc == 2) need_ev(1);                         // piece 2 reuses the S columns of piece 1
-        const uint32_t scol = tm + (pc == 0 ? 0 : 256);
-        const uint32_t idesc = CL - pc * 256 >= 256 ? idesc_k256 : idesc_k128;
-        for (int dk = 0; dk < 8; ++dk) {
-          if (pc == 0 && !fail && !mbar_wait(&sm.fullQ[dk], 0)) fail = 1;
-          if (!fail && !mbar_wait(&sm.fullK[sl], kph)) fail = 1;
-          fence_after();
-          const uint64_t qd = dk0 + (uint64_t)(dk * (SLOTP >> 4)), kd = dk0 + (uint64_t)((NQS + sl) * (SLOTP >> 4));
+    // The whole warp walks the stages and one elected lane issues: with control flow and indices uniform over the warp the
+    // descriptors are computed in uniform registers, where the instruction wants them.  (Inside a one-lane branch every
+    // operand is moved there first, and the issuing thread was the pacemaker: 175 cycles per 256-wide product.)
+    if (rank == 0) {
+      const uint32_t idesc_k256 = make_idesc2(256, 0), idesc_k128 = make_idesc2(128, 0);
+      uint32_t accb = 0, cmpb = 0, kpar = 0, vpar = 0;    // parities of the next use, per event / slot
+      int g0 = 0, pend = -1;                         // pend: the read-out event of the item before that is still to be awaited
+      uint32_t pend_par = 0;
+      const bool one = elect_one();
+      auto need_ev = [&](int e) { if (!fail && !mbar_wait(&sm.cmp_ev[e], (cmpb >> e) & 1u)) fail = 1; };
+      // the columns [256, 512) of the item before have been read out
+      auto need_pend = [&]() { if (pend >= 0) { if (!fail && !mbar_wait(&sm.cmp_ev[pend], pend_par)) fail = 1; pend = -1; } };
+#pragma unroll 1
+      for (int it = 0;; ++it) {
+        int4 r = next_item(it);
+        r = make_int4(__shfl_sync(0xffffffffu, r.x, 0), __shfl_sync(0xffffffffu, r.y, 0), __shfl_sync(0xffffffffu, r.z, 0), __shfl_sync(0xffffffffu, r.w, 0));
+        if (r.x < 0) break;
+        const Item w(r, pl, GENERAL);
+        const int CL = w.CL, NQ = w.NQ, npc = w.npc, OW = w.OW, nvb = CL * OW / 16384;
+        const uint32_t OCOL = 512 - OW, idesc_v = make_idesc2(OW, 1);
+        // The issuing thread is the pacemaker of the tensor pipe: stages are walked with counters (no divisions), and the
+        // descriptors of a stage are the slot-0 descriptor plus a multiple of the slot size (the address field counts
+        // 16-byte units and cannot overflow within the ring).
+        const uint64_t dk0 = make_desc(ring, 16, 1024), dv0 = make_desc(ring, NQ == 2 ? 8192 : 16384, 1024);
+        // S, piece after piece (the softmax of a piece runs while the tensor core works on the next one): per piece the
+        // eight slices of d, Q slice from its resident slot, K stage from the ring
+        auto place = [&](int i) { const int p = g0 + i; return p >= NSV ? p - NSV : p; };
+        int sl = 0;                                        // ring position of the next K stage
+#pragma unroll 1
+        for (int pc = 0; pc < npc; ++pc) {
+          if (pc == 1) need_pend();                        // piece 1 overwrites the last part of O of the item before
+          if (pc == 2) need_ev(1);                         // piece 2 reuses the S columns of piece 1
+          const uint32_t scol = tm + (pc == 0 ? 0 : 256);
+          const uint32_t idesc = CL - pc * 256 >= 256 ? idesc_k256 : idesc_k128;
+#pragma unroll 1
+          for (int dk = 0; dk < 8; ++dk) {
+            if (pc == 0 && !fail && !mbar_wait(&sm.fullQ[dk], (uint32_t)it & 1u)) fail = 1;
+            if (!fail && !mbar_wait(&sm.fullK[sl], (kpar >> sl) & 1u)) fail = 1;
+            kpar ^= 1u << sl;
+            fence_after();
+            const int kphys = sl < NSV - NQS ? place(NQS + sl) : NQS + sl;
+            const uint64_t qd = dk0 + (uint64_t)(place(dk) * (SLOTP >> 4)), kd = dk0 + (uint64_t)(kphys * (SLOTP >> 4));
 #pragma unroll
-          for (int ks = 0; ks < 4; ++ks) mma2_ss(scol, qd + 2 * ks, kd + 2 * ks, idesc, (dk | ks) != 0);
-          mma2_commit(&sm.emptyK[sl]);
-          if (++sl == NKS) { sl = 0; kph ^= 1u; }
-        }
-        mma2_commit(&sm.acc_ev[pc]);                     // S of the piece is complete
-      }
-      sl = 0;
-      uint32_t ph = 0;                                   // slot and parity of the next V stage
-      for (int part = 0; part < NQ; ++part) {
-        need_ev(part == 0 ? npc - 1 : 3 + part - 1);     // all of P is in TMEM / the previous part of O has been read out
-        for (int kb = 0; kb < nvb; ++kb) {
-          if (!fail && !mbar_wait(&sm.fullV[sl], ph)) fail = 1;
-          fence_after();
-          const uint64_t vd = dv0 + (uint64_t)(sl * (SLOTP >> 4));
-          if (NQ == 2) {          // per CTA: 64 keys x 128 dims = two [64 x 64] tiles
-#pragma unroll
-            for (int ks = 0; ks < 4; ++ks) mma2_ts(tm + OCOL, tm + (kb >> 2) * 128 + (kb & 1) * 64 + (kb & 2) * 16 + ks * 8, vd + ks * (2048 >> 4), idesc_v, (kb | ks) != 0);
-          } else {                // per CTA: 128 keys x 64 dims = one [128 x 64] tile
-#pragma unroll
-            for (int ks = 0; ks < 8; ++ks) mma2_ts(tm + OCOL, tm + (kb >> 1) * 128 + (ks >> 2) * 64 + (kb & 1) * 32 + (ks & 3) * 8, vd + ks * (2048 >> 4), idesc_v, (kb | ks) != 0);
+            for (int ks = 0; ks < 4; ++ks) if (one) mma2_ss(scol, qd + 2 * ks, kd + 2 * ks, idesc, (dk | ks) != 0);
+            if (one) mma2_commit(&sm.emptyK[sl]);
+            if (++sl == NKS) sl = 0;
           }
-          mma2_commit(&sm.emptyV[sl]);
-          if (++sl == NSV) { sl = 0; ph ^= 1u; }
+          if (one) mma2_commit(&sm.acc_ev[pc]);                     // S of the piece is complete
         }
-        mma2_commit(&sm.acc_ev[3 + part]);
+        need_pend();
+        sl = g0;                                           // slot of the next V stage
+#pragma unroll 1
+        for (int part = 0; part < NQ; ++part) {
+          need_ev(part == 0 ? npc - 1 : 3 + part - 1);     // all of P is in TMEM / the previous part of O has been read out
+#pragma unroll 1
+          for (int kb = 0; kb < nvb; ++kb) {
+            if (!fail && !mbar_wait(&sm.fullV[sl], (vpar >> sl) & 1u)) fail = 1;
+            vpar ^= 1u << sl;
+            fence_after();
+            const uint64_t vd = dv0 + (uint64_t)(sl * (SLOTP >> 4));
+            if (NQ == 2) {          // per CTA: 64 keys x 128 dims = two [64 x 64] tiles
+#pragma unroll
+              for (int ks = 0; ks < 4; ++ks) if (one) mma2_ts(tm + OCOL, tm + (kb >> 2) * 128 + (kb & 1) * 64 + (kb & 2) * 16 + ks * 8, vd + ks * (2048 >> 4), idesc_v, (kb | ks) != 0);
+            } else {                // per CTA: 128 keys x 64 dims = one [128 x 64] tile
+#pragma unroll
+              for (int ks = 0; ks < 8; ++ks) if (one) mma2_ts(tm + OCOL, tm + (kb >> 1) * 128 + (ks >> 2) * 64 + (kb & 1) * 32 + (ks & 3) * 8, vd + ks * (2048 >> 4), idesc_v, (kb | ks) != 0);
+            }
+            if (one) mma2_commit(&sm.emptyV[sl]);
+            if (++sl == NSV) sl = 0;
+          }
+          if (one) mma2_commit(&sm.acc_ev[3 + part]);
+        }
+        // P (overwritten by the next item's first piece) is free when the last part is complete
+        if (!fail && !mbar_wait(&sm.acc_ev[3 + NQ - 1], (accb >> (3 + NQ - 1)) & 1u)) fail = 1;
+        pend = 3 + NQ - 1; pend_par = (cmpb >> pend) & 1u;
+        accb ^= w.acc_used(); cmpb ^= w.cmp_used();
+        g0 = sl;
       }
     }
     __syncwarp();
   } else {
+    // ------------------------------------------------------------------ hands out the items
+    // The plan kernel left a record {tile, mode, keys} per tile, most keys first.  The items are the tiles' chunks in that
+    // order; pair p starts with the first chunk of tile p, all others are taken from a counter (items differ in length and in
+    // where their rows come from, so a fixed deal leaves pairs idle: 177 k cycles for the slowest of 74 pairs against a mean
+    // of 125 k on 64 sequences of 1-4 k tokens).  The leader's warp takes the next item when all compute warps have stored
+    // the current one's P: every warp of the pair has seen the current one then, and the producers are about to need the next.
+    const int ntile = s.B * pl.tc_nt, P = gridDim.x >> 1, me = blockIdx.x >> 1;
+    const int4* order = reinterpret_cast<const int4*>(ws + pl.off_order);
+    if (rank == 0) {
+      int32_t* counter = reinterpret_cast<int32_t*>(ws + pl.off_sched);
+      uint32_t cmpb = 0;
+      int base = 0, w0 = -32, q = 0;                    // window: tiles w0 .. w0 + 31, a lane each; base: items before it
+      int4 rec = make_int4(-1, 0, 0, 0);
+      int n = 0, incl = 0, tot = 0;
+#pragma unroll 1
+      for (int it = 0;; ++it) {
+        int4 r = make_int4(rec0.x, rec0.y, rec0.z, 0);
+        if (it >= own) {
+        {
+          int nx = 0x7fffffff;
+          if (lane == 0 && !fail) nx = atomicAdd(counter, 1);
+          q = __shfl_sync(0xffffffffu, nx, 0);
+        }
+        while (q >= base + tot && w0 + 32 < ntile) {
+          base += tot; w0 += 32;
+          n = 0;
+          if (w0 + lane < ntile) {
+            int CL;
+            rec = order[w0 + lane];
+            if (rec.z > 0) { chunking_x(rec.z, GENERAL, n, CL); if (w0 + lane < P) --n; }     // (the first chunks of the first P tiles are given)
+          }
+          incl = n;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += y; }
+          tot = __shfl_sync(0xffffffffu, incl, 31);
+        }
+        r = make_int4(-1, 0, 0, 0);
+        if (q < base + tot) {
+          const uint32_t has = __ballot_sync(0xffffffffu, q - base < incl);
+          const int src = __ffs(has) - 1;
+          r.x = __shfl_sync(0xffffffffu, rec.x, src); r.y = __shfl_sync(0xffffffffu, rec.y, src); r.z = __shfl_sync(0xffffffffu, rec.z, src);
+          r.w = q - base - (__shfl_sync(0xffffffffu, incl, src) - __shfl_sync(0xffffffffu, n, src)) + (w0 + src < P ? 1 : 0);
+        }
+        if (lane < 2) st_async16(map_to_rank(smem_u32(&sm.item[(it - own) & 1]), lane), r, map_to_rank(smem_u32(&sm.item_ev), lane));
+        if (lane == 0) mbar_expect_tx(&sm.item_ev, 16);
+        __syncwarp();
+        }
+        if (r.x < 0) break;
+        const Item w(r, pl, GENERAL);
+        if (!fail && !mbar_wait(&sm.cmp_ev[w.npc - 1], (cmpb >> (w.npc - 1)) & 1u)) fail = 1;
+        cmpb ^= w.cmp_used();
+        fail = __any_sync(0xffffffffu, fail);
+      }
+      // the last pair to run out of items leaves the counters as it found them
+      if (lane == 0 && atomicAdd(counter + 1, 1) == P - 1) { counter[0] = 0; counter[1] = 0; __threadfence(); }
+    } else {
+#pragma unroll 1
+      for (int it = own;; ++it) {
+        if (lane == 0) mbar_expect_tx(&sm.item_ev, 16);
+        __syncwarp();
+        if (next_item(it).x < 0) break;
+      }
+    }
+    // tiles without keys (flagged sequences, padding): zeros, tile t by pair t mod P, each CTA its own rows
+#pragma unroll 1
+    for (int t0 = me; t0 < ntile; t0 += 32 * P) {
+      int4 rz = make_int4(0, 0, 1, 0);
+      if (t0 + lane * P < ntile) rz = order[t0 + lane * P];
+      uint32_t zero = __ballot_sync(0xffffffffu, rz.z <= 0);
+      while (zero) {
+        const int tix = __shfl_sync(0xffffffffu, rz.x, __ffs(zero) - 1), b = tix / pl.tc_nt, row0 = (tix - b * pl.tc_nt) * PR + (int)rank * BM;
+        zero &= zero - 1;
+        uint4* o4 = reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(out_) + ((size_t)b * rows_seq + row0) * DH);
+        const int n16 = min(BM, rows_seq - row0) * (DH / 8);
+#pragma unroll 4
+        for (int i = lane; i < n16; i += 32) o4[i] = make_uint4(0, 0, 0, 0);
+      }
+    }
+  }
+  leave();
+  } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_COMPUTE));
     // ------------------------------------------------------------------ softmax + epilogue (8 warps)
-    const int q4 = warp & 3, hh = (warp - 2) >> 2;
+    const int q4 = warp & 3, hh = (warp - 4) >> 2;
     const int row = q4 * 32 + lane;
     const uint32_t tlane = tm + ((uint32_t)(q4 * 32) << 16);
     const uint32_t mybit = 1u << ((int)rank * (BM / s.H) + row / s.H);      // node of this row within the pair's plan tile
     const float scale2 = s.sm_scale * 1.4426950408889634f;
+    uint32_t accb = 0;                               // parity of the next use of each acc_ev
+#pragma unroll 1
+    for (int it = 0;; ++it) {
+    const int4 rec = next_item(it);
+    if (rec.x < 0) break;
+    const Item w(rec, pl, GENERAL);
+    const int b = w.b, nch = w.nch, CL = w.CL, chunk = w.chunk, npc = w.npc, NQ = w.NQ, OW = w.OW;
+    const int row0 = w.tile * PR + (int)rank * BM;   // first of this CTA's rows within the sequence
+    const size_t rix = (size_t)b * 2 * pl.tc_nt + 2 * w.tile + rank;      // this CTA's 128-row tile (partials of multi-chunk tiles)
+    const uint32_t OCOL = 512 - OW;
+    const uint8_t* kmask_g = reinterpret_cast<const uint8_t*>(ws + pl.off_kmask) + (size_t)w.tix * pl.tc_maxk + w.cbeg;
     float m_run = -INFINITY;                         // reference max of the row (log2 units)
     float lp[4] = {0.f, 0.f, 0.f, 0.f};              // this thread's share of the row sum, four independent chains
 
@@ -443,8 +623,8 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
         tmem_ld16(col, r);
 #pragma unroll
         for (int t = 0; t < 16; ++t) {
-          const float2 w = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&r[t]));
-          const __nv_bfloat162 h2 = __floats2bfloat162_rn(w.x * f, w.y * f);
+          const float2 pv = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&r[t]));
+          const __nv_bfloat162 h2 = __floats2bfloat162_rn(pv.x * f, pv.y * f);
           r[t] = *reinterpret_cast<const uint32_t*>(&h2);
         }
         tmem_st16(col, r);
@@ -480,8 +660,13 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
       // keys' node masks gives the word
       uint32_t vis[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) vis[i] = i < ns ? __ballot_sync(FULL, sm.kmask[pc * 256 + slab_of(i) * 32 + lane] & mybit) : 0u;
-      if (!fail && !mbar_wait(&sm.acc_ev[pc], 0)) fail = 1;
+      for (int i = 0; i < 4; ++i) {
+        const int key = pc * 256 + slab_of(i) * 32 + lane;
+        vis[i] = i < ns && w.cbeg + key < w.cend ? kmask_g[key] : 0u;
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) vis[i] = __ballot_sync(FULL, vis[i] & mybit);
+      if (!fail && !mbar_wait(&sm.acc_ev[pc], (accb >> pc) & 1u)) fail = 1;
       fence_after();
       const uint32_t scol = tlane + (pc == 0 ? 0 : 256);
       uint32_t sv[2][32];
@@ -490,10 +675,10 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
         float mc = -INFINITY;
         if (first >= 0) {
           uint32_t s0[32];
-          const uint32_t w = first == 0 ? vis[0] : first == 1 ? vis[1] : first == 2 ? vis[2] : vis[3];
+          const uint32_t vw = first == 0 ? vis[0] : first == 1 ? vis[1] : first == 2 ? vis[2] : vis[3];
           tmem_ld32(scol + slab_of(first) * 32, s0);
           float v[32];
-          masked(s0, w, v);
+          masked(s0, vw, v);
           mc = max32(v);
         }
         xch[hh * BM + row] = __float_as_uint(mc);
@@ -526,9 +711,9 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
     // settle on the larger one first.
     float l_row = (lp[0] + lp[1]) + (lp[2] + lp[3]);
     {
-      const uint32_t mine = ring + (uint32_t)NSV * SLOTP + (uint32_t)(warp - 2) * 8192, other = ring + (uint32_t)NSV * SLOTP + (uint32_t)((warp - 2) ^ 4) * 8192;
-      auto put = [&](int w, float v) { asm volatile("st.shared.b32 [%0], %1;" ::"r"(mine + (uint32_t)(w * 128 + lane * 4)), "r"(__float_as_uint(v)) : "memory"); };
-      auto get = [&](int w) { uint32_t v; asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(other + (uint32_t)(w * 128 + lane * 4)) : "memory"); return __uint_as_float(v); };
+      const uint32_t mine = ring + (uint32_t)NSV * SLOTP + (uint32_t)(warp - 4) * 4096, other = ring + (uint32_t)NSV * SLOTP + (uint32_t)((warp - 4) ^ 4) * 4096;
+      auto put = [&](int i, float v) { asm volatile("st.shared.b32 [%0], %1;" ::"r"(mine + (uint32_t)(i * 128 + lane * 4)), "r"(__float_as_uint(v)) : "memory"); };
+      auto get = [&](int i) { uint32_t v; asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(other + (uint32_t)(i * 128 + lane * 4)) : "memory"); return __uint_as_float(v); };
       put(0, l_row); put(1, m_run); put(2, moved ? 1.f : 0.f);
       pair_sync();
       float l_other = get(0);
@@ -550,39 +735,33 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
     const bool full_tile = row0 + BM <= rows_seq;     // whole tile inside the sequence: rows may be stored as 32-row boxes
     const float inv = l_row > 0.f ? 1.f / l_row : 0.f;
     const int cw = OW / 2;                            // columns of the part this thread handles: 128 or 64
-    const uint32_t stage0 = ring + (uint32_t)NSV * SLOTP + (uint32_t)(warp - 2) * 8192;   // this warp's two tiles of 32 rows x 64 columns (bf16)
-    int nstore = 0;
+    const uint32_t stage = ring + (uint32_t)NSV * SLOTP + (uint32_t)(warp - 4) * 4096;   // this warp's tile of 32 rows x 64 columns (bf16)
+    bool stored = false;
     for (int part = 0; part < NQ; ++part) {
-      if (!fail && !mbar_wait(&sm.acc_ev[3 + part], 0)) fail = 1;
+      if (!fail && !mbar_wait(&sm.acc_ev[3 + part], (accb >> (3 + part)) & 1u)) fail = 1;
       fence_after();
-      // the thread's columns of the part (128 or 64) go to registers at once, so that the MMA may overwrite the part
-      // while the values are normalised and stored
-      uint32_t ro[128];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) if (c * 32 < cw) tmem_ld32_nowait(tlane + OCOL + hh * cw + c * 32, ro + c * 32);
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-      for (int c = 0; c < 4; ++c) tmem_regs_ready(ro + c * 32);
-      if (part < NQ - 1) {
-        fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(map_to_rank(smem_u32(&sm.cmp_ev[3 + part]), 0));
-      }
-#pragma unroll
-      for (int cg = 0; cg < 2; ++cg) {
-        const int c0 = cg * 64;
-        if (c0 >= cw) break;
-        const uint32_t* r0 = ro + cg * 64;
-        const uint32_t* r1 = ro + cg * 64 + 32;
+      // 64 of the thread's 128 (or 64) columns at a time; when the last are in registers the MMA may overwrite the part
+#pragma unroll 1
+      for (int c0 = 0; c0 < cw; c0 += 64) {
+        uint32_t r0[32], r1[32];
+        tmem_ld32_nowait(tlane + OCOL + hh * cw + c0, r0);
+        tmem_ld32_nowait(tlane + OCOL + hh * cw + c0 + 32, r1);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        tmem_regs_ready(r0);
+        tmem_regs_ready(r1);
+        if (c0 + 64 >= cw) {
+          fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(map_to_rank(smem_u32(&sm.cmp_ev[3 + part]), 0));
+        }
         const int col = part * OW + hh * cw + c0;
         const bool many = GENERAL && nch > 1;
         if ((nch == 1 && full_tile) || many) {
           // stage the 32 x 64 bf16 tile in the 128-byte swizzle pattern and store it with one TMA request: into the output,
           // or (multi-chunk tiles, where a merge kernel follows) into the chunk's tile of normalised partial outputs, which a merge kernel
           // combines with the chunks' (max, sum)
-          const uint32_t stage = stage0 + (uint32_t)(nstore & 1) * 4096;
-          if (nstore >= 2) {                           // the store before the last has read its tile
-            if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+          if (stored) {                                // the store before has read the tile
+            if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
             __syncwarp();
           }
 #pragma unroll
@@ -607,7 +786,7 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
                          ::"l"(reinterpret_cast<uint64_t>(omap)), "r"(col), "r"(orow), "r"(stage) : "memory");
             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
           }
-          ++nstore;
+          stored = true;
         } else if (nch == 1) {
           if (rowok) {
             bf16* orow = reinterpret_cast<bf16*>(out_) + ((size_t)b * rows_seq + row0 + row) * DH + col;
@@ -636,14 +815,18 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
       if (nch > 1 && part == 0 && hh == 0)
         reinterpret_cast<float2*>(ws + pl.off_tpml)[(rix * pl.tc_chmax + chunk) * BM + row] = make_float2(m_run, l_row);
     }
-    if (nstore && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    accb ^= w.acc_used();
+    if (lane == 0) {                                 // the staging slots are free for the next item's K stages
+      asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+      asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&sm.stage_free)) : "memory");
+    }
     if (!GENERAL && nch > 1) {
       // Tiles of two chunks where nothing longer can occur: each chunk leaves its unnormalised part of O with (max, sum)
       // per row; the CTA that finishes a 128-row tile last merges the parts (fixed order, so the result does not depend
       // on who was last).  (In general a merge kernel follows: one CTA would take too long over many chunks.)
       __threadfence();
       compute_sync();
-      if (warp == 2 && lane == 0) {
+      if (warp == 4 && lane == 0) {
         int32_t* cnt = reinterpret_cast<int32_t*>(ws + pl.off_tcnt) + rix;
         const int done = atomicAdd(cnt, 1);
         sm.merge_here = done == nch - 1;
@@ -657,10 +840,10 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
         // One CTA merges a whole 128-row tile, so global latency has to be covered inside the thread: a warp takes 16 rows
         // (w, w + 8, ...), first the rows' reference maxima and sums (lane j < 16 for row w + 8 j, one round of loads), then
         // four rows at a time with all their loads of a chunk pair in flight; a lane owns columns 4 (l + 32 k) .. + 3.
-        const int w = warp - 2;
+        const int wr = warp - 4;
         float m_row = -INFINITY, inv_row = 0.f;
         if (lane < 16) {
-          const int r = w + 8 * lane;
+          const int r = wr + 8 * lane;
           float l = 0.f;
           for (int ch = 0; ch < nch; ++ch) { const float2 ml = __ldcg(pml + ch * BM + r); if (ml.y > 0.f) m_row = fmaxf(m_row, ml.x); }
           for (int ch = 0; ch < nch; ++ch) { const float2 ml = __ldcg(pml + ch * BM + r); if (ml.y > 0.f) l = fmaf(ml.y, exp2f(ml.x - m_row), l); }
@@ -683,7 +866,7 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
             float4 v[4][4];
 #pragma unroll
             for (int jx = 0; jx < 4; ++jx) {
-              const int r = w + 8 * (4 * step + jx);
+              const int r = wr + 8 * (4 * step + jx);
               ml[jx] = __ldcg(pml + ch * BM + r);
               const float4* p4 = reinterpret_cast<const float4*>(po + ((size_t)ch * BM + r) * DH);
 #pragma unroll
@@ -701,7 +884,7 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
           }
 #pragma unroll
           for (int jx = 0; jx < 4; ++jx) {
-            const int r = w + 8 * (4 * step + jx);
+            const int r = wr + 8 * (4 * step + jx);
             if (row0 + r >= rows_seq) continue;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -715,12 +898,10 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
         }
       }
     }
+    }
+    if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    leave();
   }
-  if (fail) atomicOr(status + b, TSV_ST_INTERNAL);
-  fence_before();
-  __syncthreads();
-  cluster_sync_all();                                            // neither CTA leaves while the other may still signal it or read its memory
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(tm) : "memory");
 }
 
 // ------------------------------------------------------------------------------------------------ host side
@@ -786,7 +967,7 @@ int prepare_tva_tc_pair(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c
 int launch_tva_tc_pair(const tsv_shape& s, const TvaPlan& p, const TvaTcPrep& prep, bool general, void* out, char* ws, int32_t* status, cudaStream_t st) {
   const pair::MapSet& ms = *reinterpret_cast<const pair::MapSet*>(prep.maps);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(2 * p.tc_nt * s.B, p.tc_chmax, 1);
+  const int64_t most = (int64_t)p.tc_nt * s.B * p.tc_chmax;                 // items, if every tile had the most chunks
   cfg.blockDim = dim3(pair::TTHREADS, 1, 1);
   cfg.dynamicSmemBytes = pair::SMEM_X;
   cfg.stream = st;
@@ -797,6 +978,16 @@ int launch_tva_tc_pair(const tsv_shape& s, const TvaPlan& p, const TvaTcPrep& pr
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
+  // as many pairs as the device holds at once (asked for once; 74 on a B200), but no more than there can be items
+  static std::atomic<int> resident{0};
+  int pairs = resident.load(std::memory_order_relaxed);
+  if (!pairs) {
+    cfg.gridDim = dim3(2, 1, 1);
+    if (cudaOccupancyMaxActiveClusters(&pairs, tc_attn_pair_kernel<true>, &cfg) != cudaSuccess || pairs < 1) { cudaGetLastError(); pairs = 64; }
+    resident.store(pairs, std::memory_order_relaxed);
+  }
+  if (pairs > most) pairs = (int)most;
+  cfg.gridDim = dim3(2 * pairs, 1, 1);
   const cudaError_t le = general ? cudaLaunchKernelEx(&cfg, tc_attn_pair_kernel<true>, ms, s, p, out, ws, status)
                                  : cudaLaunchKernelEx(&cfg, tc_attn_pair_kernel<false>, ms, s, p, out, ws, status);
   if (le != cudaSuccess) {
