@@ -56,18 +56,30 @@ bool make_tva_plan(const tsv_shape& s, TvaPlan& p) {
   p.off_po = off;     if (p.nsplit > 1) off = up256(off + (size_t)s.B * s.D * s.H * p.nsplit * s.d * sizeof(float));
   p.off_pml = off;    if (p.nsplit > 1) off = up256(off + (size_t)s.B * s.D * s.H * p.nsplit * 2 * sizeof(float));
   p.tc = tva_tc_eligible(s);
-  p.tc_nt = p.tc_maxk = p.tc_chmax = p.tc_misc_rows = 0;
+  p.tc_nt = p.tc_maxk = p.tc_chmax = p.tc_misc_rows = 0; p.tc_split = 1; p.tc_f32 = 0;
   p.off_krow = p.off_kmask = p.off_nkeys = p.off_tpo = p.off_tpml = p.off_box = p.off_mode = p.off_misc = p.off_order = p.off_tcnt = p.off_sched = off;
   p.off_selmask = off;
   p.mask_ld = (p.cand_cap + 15) & ~15;
   if (p.tc) {
     tva_tc_plan_sizes(s, p);
     const size_t tiles = (size_t)s.B * p.tc_nt;
+    const size_t off_pool = p.off_po;
+    // Partial outputs (a slot of 128 rows per 128-row tile and chunk) share their space with those of the CUDA-core path (a
+    // call takes one path or the other): with few tiles that leaves room to cut a tile into more chunks than its length asks
+    // for, up to one per SM pair.
+    const size_t slot = 2 * tiles * 128 * s.d * sizeof(float), slot_ml = 2 * tiles * 128 * 2 * sizeof(float);
+    if (p.tc_chmax > 1) off = up256(up256(off + p.tc_chmax * slot) + p.tc_chmax * slot_ml);
+    const size_t pool = off - off_pool;
+    int64_t ch = kPairsFor / (int64_t)tiles;
+    if (ch > (p.tc_maxk + 127) / 128) ch = (p.tc_maxk + 127) / 128;
+    while (ch > p.tc_chmax && up256((size_t)ch * slot) + up256((size_t)ch * slot_ml) > pool) --ch;
+    if (ch >= 4) p.tc_split = (int32_t)ch; else ch = 1;
+    if (ch > p.tc_chmax) p.tc_chmax = (int32_t)ch;
+    p.off_tpo = off_pool;
+    p.off_tpml = off_pool + up256((size_t)p.tc_chmax * slot);
     p.off_krow = off;  off = up256(off + tiles * p.tc_maxk * sizeof(uint32_t));   // row codes of gathered tiles
     p.off_kmask = off; off = up256(off + tiles * p.tc_maxk);
     p.off_nkeys = off; off = up256(off + tiles * sizeof(int32_t));
-    p.off_tpo = off;   if (p.tc_chmax > 1) off = up256(off + 2 * tiles * p.tc_chmax * 128 * s.d * sizeof(float));
-    p.off_tpml = off;  if (p.tc_chmax > 1) off = up256(off + 2 * tiles * p.tc_chmax * 128 * 2 * sizeof(float));
     p.off_box = off;   off = up256(off + tiles * (p.tc_maxk / 32) * 2 * sizeof(int32_t));
     p.off_mode = off;  off = up256(off + tiles * sizeof(int32_t));
     p.off_misc = off;  off = up256(off + (size_t)s.B * p.tc_misc_rows * s.d * 2);

@@ -45,6 +45,8 @@ struct TvaPlan {
   size_t off_selcnt, off_sel, off_scores, off_po, off_pml, total;
   // tensor-core path (bf16, d = 512): row tiles per sequence, key-list capacity per tile, max chunks per tile
   int32_t tc, tc_nt, tc_maxk, tc_chmax;
+  int32_t tc_split;                  // chunks a tile may be cut into to fill the device (1: tiles enough)
+  int32_t tc_f32;                    // all partial outputs are fp32 (set at the launch)
   int32_t tc_misc_rows;              // rows of the per-sequence packed buffer
   size_t off_krow, off_kmask, off_nkeys, off_tpo, off_tpml, off_box, off_mode, off_misc, off_order, off_tcnt, off_sched;   // off_sched: the paired kernel's item counter, the pairs that have run out of items
   // selection as a byte per candidate (1 = selected), one row of mask_ld bytes per node, written for the nodes that rank:
@@ -52,6 +54,7 @@ struct TvaPlan {
   size_t off_selmask;
   int32_t mask_ld;
 };
+constexpr int kPairsFor = 74;         // SM pairs the splitting of few tiles aims at (a B200 holds 74)
 bool make_tva_plan(const tsv_shape& s, TvaPlan& p);
 
 int launch_bsb(const tsv_shape& s, const tsv_cache& c, const tsv_nodes& nd, const tsv_scratch& sc, int32_t* status, cudaStream_t st);
@@ -86,7 +89,7 @@ bool tva_tc_pair_usable(const tsv_cache& c);
 // Host-side preparation of the tensor-core attention path: everything that can fail on the host (tensor maps, kernel
 // attributes) is done here, before any kernel of the call is enqueued.
 struct TvaTcPrep {
-  alignas(64) unsigned char maps[19 * 128];   // the paired kernel's tensor maps (a CUtensorMap is 128 bytes)
+  alignas(64) unsigned char maps[20 * 128];   // the paired kernel's tensor maps (a CUtensorMap is 128 bytes)
 };
 int prepare_tva_tc_pair(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, const tsv_nodes& nd, void* out, char* ws, TvaTcPrep& prep);
 // general: gathered tiles or tiles of more than two chunks may occur (else the instantiation without that code runs)

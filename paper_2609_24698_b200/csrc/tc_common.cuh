@@ -10,7 +10,8 @@ namespace tc {
 constexpr int DH = 512;             // head dim handled by this path
 constexpr int BM = 128;             // rows per CTA
 constexpr int PR = 256;             // rows per plan tile: two row tiles (one CTA pair) share one key list
-constexpr int NC = 512;             // keys per chunk of a list that is cut into several
+constexpr int NC = 512;             // keys per chunk of a list that is cut into many
+constexpr int NCMIN = 128;          // keys of the shortest chunk worth an SM pair of its own
 constexpr uint32_t WAIT_LIMIT = 1u << 14;   // polls before a wait gives up (then no later wait of the thread is attempted)
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -103,18 +104,27 @@ __device__ __forceinline__ float ex2(float x) {
 
 constexpr int NCX = 768;             // max keys per chunk of the TMA kernel: P (bf16) takes 384 TMEM columns, an O quarter 128
 // Chunking of the TMA kernel: nch chunks of CL keys, CL a multiple of 128 and <= NCX.
-// general = false (shapes whose capacities allow at most two chunks of NCX keys and no gathered tile): as few chunks as
-// possible; the two chunks of a long list are merged inside the kernel.
-// general = true: a list that does not fit one chunk is cut into chunks of at most NC keys: the partial outputs go through
-// the cheap path (bf16 tiles, merge kernel), the PV product of a chunk of <= 512 keys runs in halves of d instead of
-// quarters, and more, shorter work items fill the SM pairs better (measured on 131072-token prefixes: attention stage
-// 142 us with 768-key chunks, 130 with 640, 116 with 512, 135 with 384).
-__device__ __host__ __forceinline__ void chunking_x(int nk, bool general, int& nch, int& CL) {
+// general = false (shapes whose capacities allow at most two chunks of NCX keys and no gathered tile): as few chunks as possible.
+// general = true: a list that does not fit one chunk is cut into chunks of at most NC keys, whose PV product runs in halves of
+// d instead of quarters and which fill the SM pairs better (two chunks of up to NCX instead of three of NC cost 12 % of the
+// attention kernel on 32 paged sequences of 256-4096 tokens, and gained nothing on 64 flat ones).
+// split: chunks a tile may be cut into so that few tiles still use all pairs (1 where there are tiles enough).
+// f32: the partial outputs of the tile are fp32 (a tile that is cut for the sake of parallelism alone is not rounded before
+// the merge); f32_all: all multi-chunk tiles are.
+__device__ __host__ __forceinline__ void chunking_x(int nk, bool general, int split, bool f32_all, int& nch, int& CL, bool& f32) {
   nch = (nk + NCX - 1) / NCX;
   if (general && nch > 1) nch = (nk + NC - 1) / NC;
+  f32 = f32_all || nch <= 1;
+  if (split > 1) {
+    int w = (nk + NCMIN - 1) / NCMIN;
+    if (w > split) w = split;
+    if (w > nch) nch = w;
+  }
   if (nch < 1) nch = 1;
   CL = (((nk + nch - 1) / nch) + 127) / 128 * 128;
   if (CL < 128) CL = 128;
+  nch = (nk + CL - 1) / CL;
+  if (nch < 1) nch = 1;
 }
 
 }  // namespace tc

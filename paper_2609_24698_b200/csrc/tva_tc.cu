@@ -14,6 +14,8 @@
 //                    Each tile CTA leaves its record {tile, mode, keys} at the tile's scheduling position (its rank by
 //                    estimated key count, most first); an extra CTA per sequence packs the small scattered rows.
 //   tc_combine_pair_kernel  merges the chunks of the paired kernel's multi-chunk tiles (fixed order).
+#include <type_traits>
+
 #include "tc_common.cuh"
 
 namespace tsv {
@@ -433,21 +435,26 @@ __global__ void __launch_bounds__(NT) tc_plan_kernel(const tsv_shape s, const Tv
 // the row's (reference max, sum); the row's output is the average of the partial outputs weighted by sum * 2^(max - row max).
 // grid (128-row tiles, sequences, groups of 8 rows): a warp merges one row, a lane owns 16 consecutive columns; the chunks
 // are accumulated in order, four chunks' loads in flight.
+// ANY32: some tiles' partial outputs may be fp32 (else all are bf16, and the kernel keeps its registers low).
+template <bool ANY32>
 __global__ void __launch_bounds__(256) tc_combine_pair_kernel(const tsv_shape s, const TvaPlan pl, void* __restrict__ out_, const char* __restrict__ ws) {
   using namespace tc;
+  asm volatile("griddepcontrol.wait;" ::: "memory");            // launched as a programmatic dependent of the attention kernel
   const int rt = blockIdx.x, tile = rt >> 1, b = blockIdx.y;
   const size_t tix = (size_t)b * pl.tc_nt + tile, rix = (size_t)b * 2 * pl.tc_nt + rt;
   const int mode = reinterpret_cast<const int32_t*>(ws + pl.off_mode)[tix];
   const int nk = reinterpret_cast<const int32_t*>(ws + pl.off_nkeys)[tix];
   if ((mode != 1 && mode != 2) || nk <= 0) return;
   int nch, CL;
-  chunking_x(nk, true, nch, CL);
+  bool f32;
+  chunking_x(nk, true, pl.tc_split, pl.tc_f32, nch, CL, f32);
+  if (!ANY32) f32 = false;                                       // (no tile is split, so one with more than one chunk was too long for one: bf16)
   if (nch <= 1) return;                                          // the paired kernel wrote the output itself
   const int rows_seq = s.D * s.H, row0 = rt * BM;
   const int lane = threadIdx.x & 31, row = blockIdx.z * 8 + (threadIdx.x >> 5);
   if (row >= BM || row0 + row >= rows_seq) return;
   // (a chunk's bf16 tile lies at the start of the chunk's slot of BM x DH floats)
-  const uint4* po = reinterpret_cast<const uint4*>(reinterpret_cast<const bf16*>(ws + pl.off_tpo) + (rix * pl.tc_chmax * 2 * BM + row) * DH) + 2 * lane;
+  const uint4* po = reinterpret_cast<const uint4*>(ws + pl.off_tpo) + (rix * pl.tc_chmax * BM * (DH / 4) + (size_t)row * (DH / (f32 ? 4 : 8))) + (f32 ? 4 : 2) * lane;
   const float2* pml = reinterpret_cast<const float2*>(ws + pl.off_tpml) + rix * pl.tc_chmax * BM + row;
   float m = -INFINITY;
   for (int ch = lane; ch < nch; ch += 32) { const float2 ml = pml[(size_t)ch * BM]; if (ml.y > 0.f) m = fmaxf(m, ml.x); }
@@ -456,28 +463,39 @@ __global__ void __launch_bounds__(256) tc_combine_pair_kernel(const tsv_shape s,
   float l = 0.f, acc[16];
 #pragma unroll
   for (int k = 0; k < 16; ++k) acc[k] = 0.f;
-  for (int c0 = 0; c0 < nch; c0 += 4) {
-    float2 ml[4];
-    uint4 v[4][2];
+  auto merge = [&](auto vec) {                                   // vec: 16-byte pieces of a lane's 16 columns
+    constexpr int V = decltype(vec)::value;
+    for (int c0 = 0; c0 < nch; c0 += 4) {
+      float2 ml[4];
+      uint4 v[4][V];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int ch = c0 + u < nch ? c0 + u : nch - 1;
-      ml[u] = pml[(size_t)ch * BM];
-      v[u][0] = po[(size_t)ch * 2 * BM * (DH / 8)]; v[u][1] = po[(size_t)ch * 2 * BM * (DH / 8) + 1];
-    }
+      for (int u = 0; u < 4; ++u) {
+        const int ch = c0 + u < nch ? c0 + u : nch - 1;
+        ml[u] = pml[(size_t)ch * BM];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      if (c0 + u >= nch || !(ml[u].y > 0.f)) continue;
-      const float w = ml[u].y * exp2f(ml[u].x - m);
-      l += w;
-      const uint32_t wd[8] = {v[u][0].x, v[u][0].y, v[u][0].z, v[u][0].w, v[u][1].x, v[u][1].y, v[u][1].z, v[u][1].w};
+        for (int x = 0; x < V; ++x) v[u][x] = po[(size_t)ch * BM * (DH / 4) + x];
+      }
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        acc[2 * k] = fmaf(__uint_as_float(wd[k] << 16), w, acc[2 * k]);
-        acc[2 * k + 1] = fmaf(__uint_as_float(wd[k] & 0xFFFF0000u), w, acc[2 * k + 1]);
+      for (int u = 0; u < 4; ++u) {
+        if (c0 + u >= nch || !(ml[u].y > 0.f)) continue;
+        const float w = ml[u].y * exp2f(ml[u].x - m);
+        l += w;
+#pragma unroll
+        for (int x = 0; x < V; ++x) {
+          const uint32_t wd[4] = {v[u][x].x, v[u][x].y, v[u][x].z, v[u][x].w};
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            if (V == 4) acc[4 * x + k] = fmaf(__uint_as_float(wd[k]), w, acc[4 * x + k]);
+            else {
+              acc[8 * x + 2 * k] = fmaf(__uint_as_float(wd[k] << 16), w, acc[8 * x + 2 * k]);
+              acc[8 * x + 2 * k + 1] = fmaf(__uint_as_float(wd[k] & 0xFFFF0000u), w, acc[8 * x + 2 * k + 1]);
+            }
+          }
+        }
       }
     }
-  }
+  };
+  if (ANY32 && f32) merge(std::integral_constant<int, 4>()); else merge(std::integral_constant<int, 2>());
   const float inv = l > 0.f ? 1.f / l : 0.f;
   uint32_t o[8];
 #pragma unroll
@@ -540,12 +558,14 @@ int prepare_tva_tc(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, con
   TSV_PREP((tc_plan_kernel<true, 1024>));
   TSV_PREP((tc_plan_kernel<true, 256>));
   TSV_PREP((tc_plan_kernel<false, 256>));
-  TSV_PREP(tc_combine_pair_kernel);
+  TSV_PREP(tc_combine_pair_kernel<true>);
+  TSV_PREP(tc_combine_pair_kernel<false>);
   return prepare_tva_tc_pair(s, p, c, nd, out, ws, prep);
 }
 
-int launch_tva_tc(const tsv_shape& s, const TvaPlan& p, const TvaTcPrep& prep, const tsv_cache& c, const tsv_nodes& nd, const tsv_scratch& sc,
+int launch_tva_tc(const tsv_shape& s, const TvaPlan& p_in, const TvaTcPrep& prep, const tsv_cache& c, const tsv_nodes& nd, const tsv_scratch& sc,
                   void* out, char* ws, int32_t* status, cudaStream_t st, bool with_plan) {
+  TvaPlan p = p_in;
   const bool gathered = gathered_tiles_possible(s, p, c);
   const dim3 pgrid(p.tc_nt + 1, s.B);                                                                              // x: tiles + the packing CTA
   if (with_plan) {
@@ -563,11 +583,19 @@ int launch_tva_tc(const tsv_shape& s, const TvaPlan& p, const TvaTcPrep& prep, c
   count_launch();
   // general: some tile may have more than two chunks of the longest kind, or be gathered; then every multi-chunk tile
   // leaves bf16 partial outputs for the merge kernel
-  const bool general = (p.tc_maxk + tc::NCX - 1) / tc::NCX > 2 || gathered;
+  const bool many = (p.tc_maxk + tc::NCX - 1) / tc::NCX > 2 || gathered, general = many || p.tc_split > 1;
+  p.tc_f32 = !many;                                    // (no more than two long chunks a tile: merged without rounding in either instantiation)
   const int r = launch_tva_tc_pair(s, p, prep, general, out, ws, status, st);
   if (r != TSV_OK) return r;
   if (general && p.tc_chmax > 1) {
-    tc_combine_pair_kernel<<<dim3(2 * p.tc_nt, s.B, tc::BM / 8), 256, 0, st>>>(s, p, out, ws);   // z: groups of 8 rows
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2 * p.tc_nt, s.B, tc::BM / 8); cfg.blockDim = dim3(256, 1, 1); cfg.stream = st;                 // z: groups of 8 rows
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    if (p.tc_split > 1 || p.tc_f32) cudaLaunchKernelEx(&cfg, tc_combine_pair_kernel<true>, s, p, out, (const char*)ws);
+    else cudaLaunchKernelEx(&cfg, tc_combine_pair_kernel<false>, s, p, out, (const char*)ws);
     count_launch();
   }
   return cudaGetLastError() == cudaSuccess ? TSV_OK : TSV_ERR_CUDA;

@@ -29,10 +29,10 @@ namespace pair {
 using namespace tc;
 
 // Warps: 0, 3, 12-15 producers; 1 MMA issuer; 2 hands out the items; 4-11 softmax and epilogue.  The service warpgroups give
-// registers to the compute warpgroups: 128 x (80 + 176 + 176 + 80) of the 512 x 128 the CTA is launched with.
+// registers to the compute warpgroups: 128 x (96 + 160 + 160 + 96) of the 512 x 128 the CTA is launched with.
 constexpr int TTHREADS = 512;
 constexpr int NPROD = 6;                    // (12 slots: six producers with two each)
-constexpr int REGS_SERVICE = 80, REGS_COMPUTE = 176;
+constexpr int REGS_SERVICE = 96, REGS_COMPUTE = 160;
 static_assert(128 * (2 * REGS_SERVICE + 2 * REGS_COMPUTE) <= TTHREADS * 128, "register split beyond what the CTA is launched with");
 constexpr int BOXB = kBoxRows * 128;       // bytes of one box: kBoxRows rows x 128 bytes
 constexpr float RESCALE_GAP = 16.f;        // log2 units a later piece's row max may exceed the running reference
@@ -135,9 +135,10 @@ struct alignas(64) MapSet {
   CUtensorMap out;        // 32-row boxes (stores)
   CUtensorMap src[4][3];  // [csa, hca, window, packed misc][32, 64, 128 rows]
   CUtensorMap row[4];     // the same arrays with one-row boxes: gathers of four rows by index
-  CUtensorMap part;       // normalised partial outputs of tiles of more than two chunks (bf16, 32-row boxes, stores)
+  CUtensorMap part;       // normalised partial outputs of multi-chunk tiles (bf16, 32-row boxes, stores)
+  CUtensorMap part32;     // the same in fp32, 32-column boxes (tiles cut for the sake of parallelism: no rounding before the merge)
 };
-constexpr int NMAPS = 19;
+constexpr int NMAPS = 20;
 
 constexpr uint32_t OOB_BOX = 0x3FFFFF00u;   // map 0, a row beyond every tensor: the box is zero-filled
 
@@ -149,12 +150,13 @@ struct Item {
   int tix, b, tile, nk, chunk, nch, CL, cbeg, cend;
   int npc;                 // S pieces
   int NQ, OW;              // the PV product is computed in NQ parts of OW columns of d
+  bool f32;                // partial outputs are fp32
   bool gather;             // the key list is a list of row codes (array << 30 | row), not of boxes
   __device__ __forceinline__ Item(int4 r, const TvaPlan& pl, bool general) {
     tix = r.x; b = r.x / pl.tc_nt; tile = r.x - b * pl.tc_nt;
     gather = general && r.y == 2;
     nk = r.z; chunk = r.w;
-    tc::chunking_x(nk, general, nch, CL);
+    tc::chunking_x(nk, general, pl.tc_split, pl.tc_f32, nch, CL, f32);
     cbeg = chunk * CL; cend = min(nk, cbeg + CL);
     npc = (CL + 255) / 256;
     NQ = CL <= 512 ? 2 : 4;
@@ -224,6 +226,7 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
   // Launched as a programmatic dependent of the tile plan: the CTAs take their places and set up while that kernel's last
   // CTAs finish, and read nothing of its before it has completed.
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // (the merge kernel, which waits for this one before it does anything)
   const int4 rec0 = (int)(blockIdx.x >> 1) < s.B * pl.tc_nt ? __ldcg(reinterpret_cast<const int4*>(ws + pl.off_order) + (blockIdx.x >> 1)) : make_int4(-1, 0, 0, 0);
   fence_before();
   __syncthreads();
@@ -501,8 +504,9 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
           n = 0;
           if (w0 + lane < ntile) {
             int CL;
+            bool f32;
             rec = order[w0 + lane];
-            if (rec.z > 0) { chunking_x(rec.z, GENERAL, n, CL); if (w0 + lane < P) --n; }     // (the first chunks of the first P tiles are given)
+            if (rec.z > 0) { chunking_x(rec.z, GENERAL, pl.tc_split, pl.tc_f32, n, CL, f32); if (w0 + lane < P) --n; }     // (the first chunks of the first P tiles are given)
           }
           incl = n;
 #pragma unroll
@@ -760,6 +764,32 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
           // stage the 32 x 64 bf16 tile in the 128-byte swizzle pattern and store it with one TMA request: into the output,
           // or (multi-chunk tiles, where a merge kernel follows) into the chunk's tile of normalised partial outputs, which a merge kernel
           // combines with the chunks' (max, sum)
+          if (many && w.f32) {               // fp32: two tiles of 32 columns
+#pragma unroll
+            for (int x = 0; x < 2; ++x) {
+              if (stored) {
+                if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                __syncwarp();
+              }
+              stored = true;
+#pragma unroll
+              for (int v = 0; v < 8; ++v) {
+                float f[4];
+#pragma unroll
+                for (int t = 0; t < 4; ++t) f[t] = __uint_as_float(x ? r1[v * 4 + t] : r0[v * 4 + t]) * inv;
+                asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(stage + lane * 128 + ((v ^ (lane & 7)) << 4)), "f"(f[0]), "f"(f[1]),
+                             "f"(f[2]), "f"(f[3]) : "memory");
+              }
+              asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+              __syncwarp();
+              if (lane == 0) {
+                asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];"
+                             ::"l"(reinterpret_cast<uint64_t>(&maps.part32)), "r"(col + 32 * x), "r"((int)((rix * pl.tc_chmax + chunk) * BM) + q4 * 32), "r"(stage) : "memory");
+                asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+              }
+            }
+            continue;
+          }
           if (stored) {                                // the store before has read the tile
             if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
             __syncwarp();
@@ -837,63 +867,25 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
         bf16* orow0 = reinterpret_cast<bf16*>(out_) + ((size_t)b * rows_seq + row0) * DH;
         const float* po = reinterpret_cast<const float*>(ws + pl.off_tpo) + rix * pl.tc_chmax * BM * DH;
         const float2* pml = reinterpret_cast<const float2*>(ws + pl.off_tpml) + rix * pl.tc_chmax * BM;
-        // One CTA merges a whole 128-row tile, so global latency has to be covered inside the thread: a warp takes 16 rows
-        // (w, w + 8, ...), first the rows' reference maxima and sums (lane j < 16 for row w + 8 j, one round of loads), then
-        // four rows at a time with all their loads of a chunk pair in flight; a lane owns columns 4 (l + 32 k) .. + 3.
+        // A warp takes 16 rows (wr, wr + 8, ...), a lane columns 4 (l + 32 k) .. + 3 of a row.  (Few registers on purpose: the path
+        // is rare and must not cost the kernel around it any.)
         const int wr = warp - 4;
-        float m_row = -INFINITY, inv_row = 0.f;
-        if (lane < 16) {
-          const int r = wr + 8 * lane;
-          float l = 0.f;
-          for (int ch = 0; ch < nch; ++ch) { const float2 ml = __ldcg(pml + ch * BM + r); if (ml.y > 0.f) m_row = fmaxf(m_row, ml.x); }
-          for (int ch = 0; ch < nch; ++ch) { const float2 ml = __ldcg(pml + ch * BM + r); if (ml.y > 0.f) l = fmaf(ml.y, exp2f(ml.x - m_row), l); }
-          inv_row = l > 0.f ? 1.f / l : 0.f;
-        }
 #pragma unroll 1
-        for (int step = 0; step < 4; ++step) {
-          float4 acc[4][4];
-          float mj[4], invj[4];
+        for (int r = wr; r < BM && row0 + r < rows_seq; r += 8) {
+          const float2 a0 = __ldcg(pml + r), a1 = __ldcg(pml + BM + r);
+          const float m = fmaxf(a0.y > 0.f ? a0.x : -INFINITY, a1.y > 0.f ? a1.x : -INFINITY);
+          const float w0 = a0.y > 0.f ? exp2f(a0.x - m) : 0.f, w1 = a1.y > 0.f ? exp2f(a1.x - m) : 0.f, l = a0.y * w0 + a1.y * w1;
+          const float i0 = l > 0.f ? w0 / l : 0.f, i1 = l > 0.f ? w1 / l : 0.f;
+          const float4* p0 = reinterpret_cast<const float4*>(po + (size_t)r * DH);
+          const float4* p1 = reinterpret_cast<const float4*>(po + ((size_t)BM + r) * DH);
 #pragma unroll
-          for (int jx = 0; jx < 4; ++jx) {
-            mj[jx] = __shfl_sync(0xffffffffu, m_row, 4 * step + jx);
-            invj[jx] = __shfl_sync(0xffffffffu, inv_row, 4 * step + jx);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) acc[jx][k] = make_float4(0.f, 0.f, 0.f, 0.f);
-          }
-#pragma unroll 2
-          for (int ch = 0; ch < nch; ++ch) {
-            float2 ml[4];
-            float4 v[4][4];
-#pragma unroll
-            for (int jx = 0; jx < 4; ++jx) {
-              const int r = wr + 8 * (4 * step + jx);
-              ml[jx] = __ldcg(pml + ch * BM + r);
-              const float4* p4 = reinterpret_cast<const float4*>(po + ((size_t)ch * BM + r) * DH);
-#pragma unroll
-              for (int k = 0; k < 4; ++k) v[jx][k] = __ldcg(p4 + lane + 32 * k);
-            }
-#pragma unroll
-            for (int jx = 0; jx < 4; ++jx) {
-              const float wgt = ml[jx].y > 0.f ? exp2f(ml[jx].x - mj[jx]) : 0.f;
-#pragma unroll
-              for (int k = 0; k < 4; ++k) {
-                acc[jx][k].x = fmaf(v[jx][k].x, wgt, acc[jx][k].x); acc[jx][k].y = fmaf(v[jx][k].y, wgt, acc[jx][k].y);
-                acc[jx][k].z = fmaf(v[jx][k].z, wgt, acc[jx][k].z); acc[jx][k].w = fmaf(v[jx][k].w, wgt, acc[jx][k].w);
-              }
-            }
-          }
-#pragma unroll
-          for (int jx = 0; jx < 4; ++jx) {
-            const int r = wr + 8 * (4 * step + jx);
-            if (row0 + r >= rows_seq) continue;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const __nv_bfloat162 lo = __floats2bfloat162_rn(acc[jx][k].x * invj[jx], acc[jx][k].y * invj[jx]);
-              const __nv_bfloat162 hi = __floats2bfloat162_rn(acc[jx][k].z * invj[jx], acc[jx][k].w * invj[jx]);
-              uint2 o2;
-              o2.x = *reinterpret_cast<const uint32_t*>(&lo); o2.y = *reinterpret_cast<const uint32_t*>(&hi);
-              *reinterpret_cast<uint2*>(orow0 + (size_t)r * DH + 4 * (lane + 32 * k)) = o2;
-            }
+          for (int k = 0; k < 4; ++k) {
+            const float4 x = __ldcg(p0 + lane + 32 * k), y = __ldcg(p1 + lane + 32 * k);
+            const __nv_bfloat162 lo = __floats2bfloat162_rn(fmaf(x.x, i0, y.x * i1), fmaf(x.y, i0, y.y * i1));
+            const __nv_bfloat162 hi = __floats2bfloat162_rn(fmaf(x.z, i0, y.z * i1), fmaf(x.w, i0, y.w * i1));
+            uint2 o2;
+            o2.x = *reinterpret_cast<const uint32_t*>(&lo); o2.y = *reinterpret_cast<const uint32_t*>(&hi);
+            *reinterpret_cast<uint2*>(orow0 + (size_t)r * DH + 4 * (lane + 32 * k)) = o2;
           }
         }
       }
@@ -916,15 +908,15 @@ static PFN_cuTensorMapEncodeTiled encode_fn() {
   return fn;
 }
 
-// rows x 512 bf16, row-major; boxes of 32 rows x 64 columns written with the 128-byte swizzle
-static bool make_map(CUtensorMap* m, const void* basep, int64_t rows, int box_rows = kBoxRows) {
+// rows x 512 bf16 (or fp32), row-major; boxes of 32 rows x 128 bytes written with the 128-byte swizzle
+static bool make_map(CUtensorMap* m, const void* basep, int64_t rows, int box_rows = kBoxRows, bool f32 = false) {
   PFN_cuTensorMapEncodeTiled fn = encode_fn();
   if (!fn || rows <= 0 || ((uintptr_t)basep & 15)) return false;
   const cuuint64_t gdim[2] = {(cuuint64_t)tc::DH, (cuuint64_t)rows};
-  const cuuint64_t gstr[1] = {(cuuint64_t)tc::DH * 2};
-  const cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
+  const cuuint64_t gstr[1] = {(cuuint64_t)tc::DH * (f32 ? 4 : 2)};
+  const cuuint32_t box[2] = {f32 ? 32u : 64u, (cuuint32_t)box_rows};
   const cuuint32_t estr[2] = {1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(basep), gdim, gstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+  return fn(m, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(basep), gdim, gstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -949,7 +941,9 @@ int prepare_tva_tc_pair(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c
   // the kernel); the general instantiation stores 128 x 512 bf16 at the start of the slot: as rows of 1 KiB the buffer
   // has 2 x 128 rows per slot
   if (p.tc_chmax > 1) ok = ok && make_map(&ms.part, ws + p.off_tpo, (int64_t)s.B * 2 * p.tc_nt * p.tc_chmax * 2 * tc::BM, 32);
-  else ms.part = ms.out;                                                       // (never used: no tile has more than one chunk)
+  if (p.tc_split > 1) ok = ok && make_map(&ms.part32, ws + p.off_tpo, (int64_t)s.B * 2 * p.tc_nt * p.tc_chmax * tc::BM, 32, true);
+  else ms.part32 = ms.out;
+  if (p.tc_chmax <= 1) ms.part = ms.out;                                                       // (never used: no tile has more than one chunk)
   if (!ok) {
     fprintf(stderr, "tsv: cuTensorMapEncodeTiled failed\n");
     return TSV_ERR_CUDA;
