@@ -3,6 +3,7 @@
 #include <math.h>
 
 #include <atomic>
+#include <mutex>
 
 #include "kernels.h"
 
@@ -10,6 +11,36 @@ namespace tsv {
 
 static std::atomic<uint64_t> g_launches{0};
 void count_launch(int n) { g_launches.fetch_add((uint64_t)n, std::memory_order_relaxed); }
+
+bool ensure_smem(const void* kernel, int bytes) {
+  struct Entry { std::atomic<const void*> kernel{nullptr}; std::atomic<int> dev{-1}, bytes{0}; };
+  static Entry table[256];                              // (kernel, device) pairs, filled from the front
+  static std::mutex m;
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return false; }
+  for (Entry& e : table) {
+    const void* k = e.kernel.load(std::memory_order_acquire);
+    if (!k) break;
+    if (k == kernel && e.dev.load(std::memory_order_relaxed) == dev) {
+      if (e.bytes.load(std::memory_order_acquire) >= bytes) return true;
+      break;
+    }
+  }
+  std::lock_guard<std::mutex> g(m);
+  Entry* hit = nullptr;
+  for (Entry& e : table) {
+    const void* k = e.kernel.load(std::memory_order_relaxed);
+    if (!k || (k == kernel && e.dev.load(std::memory_order_relaxed) == dev)) { hit = &e; break; }
+  }
+  if (hit && hit->kernel.load(std::memory_order_relaxed) && hit->bytes.load(std::memory_order_relaxed) >= bytes) return true;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) { cudaGetLastError(); return false; }
+  if (hit) {
+    hit->dev.store(dev, std::memory_order_relaxed);
+    hit->bytes.store(bytes, std::memory_order_release);
+    hit->kernel.store(kernel, std::memory_order_release);
+  }
+  return true;
+}
 
 static bool shape_ok(const tsv_shape* s) {
   if (!s) return false;

@@ -17,6 +17,10 @@ void count_launch(int n = 1);
     }                                                                                                             \
   } while (0)   // bumps the reporting counter behind tsv_kernel_launches()
 
+// Raises a kernel's dynamic shared-memory limit on the current device where it is below `bytes` (never lowers it: another
+// shape's launches need what they asked for).  The driver is called once per kernel, device and new maximum.
+bool ensure_smem(const void* kernel, int bytes);
+
 // Per-layer pointers accept_and_refresh needs, packed so that a group of layers fits in
 // kernel-parameter space.
 struct AarLayer {
@@ -72,6 +76,11 @@ int launch_tva_select(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, 
 bool topk_fused_applies(const tsv_shape& s, const TvaPlan& p);
 int launch_topk_fused(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, const tsv_nodes& nd, const tsv_scratch& sc,
                       int32_t* topk_idx, char* ws, int32_t* status, cudaStream_t st);
+// top-k of all nodes of a sequence by a thread-block cluster per sequence, or (longer lists, larger trees) scores over all SMs and
+// a CTA per node
+bool topk_seq_applies(const tsv_shape& s, const TvaPlan& p);
+int launch_topk_seq(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, const tsv_nodes& nd, const tsv_scratch& sc,
+                    int32_t* topk_idx, char* ws, int32_t* status, cudaStream_t st);
 // per-node top-k of long candidate lists by a thread-block cluster per node
 bool topk_long_applies(const tsv_shape& s, const TvaPlan& p);
 int launch_topk_long(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, const tsv_nodes& nd, const tsv_scratch& sc,

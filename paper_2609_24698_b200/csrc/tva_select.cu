@@ -541,6 +541,8 @@ __global__ void __launch_bounds__(256) topk_kernel(const tsv_shape s, const TvaP
 int launch_tva_select(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, const tsv_nodes& nd, const tsv_scratch& sc,
                       int32_t* topk_idx, char* ws, int32_t* status, cudaStream_t st) {
   const bool bf = s.dtype == TSV_BF16;
+  if (topk_fused_applies(s, p)) return launch_topk_fused(s, p, c, nd, sc, topk_idx, ws, status, st);
+  if (topk_seq_applies(s, p)) return launch_topk_seq(s, p, c, nd, sc, topk_idx, ws, status, st);
   if (p.need_scores && !p.idx_fused) {
     const int pref_cap = (int)(s.max_L / s.m_csa);
     dim3 grid((pref_cap + 255) / 256, s.B, s.D <= 8 ? s.D : 8);        // z: slabs of nodes, so a ranked sequence is scored by many CTAs
@@ -566,7 +568,6 @@ int launch_tva_select(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, 
     }
   }
   if (topk_long_applies(s, p)) return launch_topk_long(s, p, c, nd, sc, topk_idx, ws, status, st);
-  if (topk_fused_applies(s, p)) return launch_topk_fused(s, p, c, nd, sc, topk_idx, ws, status, st);
   dim3 g2(s.D, s.B);
   const bool paged = c.page_table != nullptr;
   size_t sm2 = p.idx_fused ? (size_t)s.HI * s.di * sizeof(float) : 0;         // the node's indexer queries ...

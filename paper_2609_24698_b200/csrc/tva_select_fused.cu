@@ -1,4 +1,4 @@
-// Per-node top-k for short candidate lists (at most kIdxFusedMax committed entries) with 128-wide bf16 indexer rows (the
+// Per-node top-k for short candidate lists (capacity at most kCands) with 128-wide bf16 indexer rows (the
 // benchmark's): one CTA per (sequence, node) that scores, ranks and selects.  Same result as topk_kernel (the exact k
 // largest scores, ties to the lower index, ascending output); built so that
 //   * nodes that do not rank (nearly all of them) are a short chain and ALL CTAs of the launch are resident at once
@@ -16,10 +16,8 @@ namespace tsv {
 namespace fsel {
 
 constexpr int DI = 128;                       // indexer width (bf16: 256-byte rows)
-// candidates per thread (keys in registers): 3 for lists of up to 768 candidates, else 9 (9 x 256 >= kIdxFusedMax + TSV_MAX_D);
-// two instantiations, so that the short lists of the common shapes do not step through the predicated code of nine
-constexpr int KPT_SHORT = 3, KPT_LONG = 9;
-static_assert(kIdxFusedMax + TSV_MAX_D <= KPT_LONG * 256, "candidate lists must fit the in-register keys");
+// candidates per thread (keys in registers)
+constexpr int KPT = 3, kCands = KPT * 256;
 
 __device__ __forceinline__ void cp16(uint32_t dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
@@ -36,7 +34,7 @@ __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], const uint32_t (&a
 
 // Dynamic shared memory: [4][128] bf16 queries (heads beyond HI zero) | scores [score_cap] fp32 | two buffers of `rows`
 // staged indexer rows of 256 bytes (16-byte pieces XOR-swizzled by the row, so that ldmatrix reads without conflicts).
-template <bool PAGED, int KPT>
+template <bool PAGED>
 __global__ void __launch_bounds__(256, 4) topk_fused_kernel(const tsv_shape s, const TvaPlan pl, const tsv_cache c, const tsv_nodes nd,
                                                             const tsv_scratch sc, int32_t* __restrict__ topk_user, char* __restrict__ ws,
                                                             int32_t* __restrict__ status, const int rows, const int score_cap) {
@@ -283,9 +281,11 @@ __global__ void __launch_bounds__(256, 4) topk_fused_kernel(const tsv_shape s, c
   if (t == 0) *selcnt = k;
 }
 
-// The kernel serves: bf16, 128-wide indexer rows, at most four indexer heads, lists the selection scores itself.
+// bf16, 128-wide indexer rows, at most four indexer heads, three keys per thread: longer lists go to topk_seq_kernel, which reads an
+// indexer row once per sequence instead of once per node (a longer instantiation of this kernel took 18-34 us where that one takes
+// 13-23), while here, where few nodes or none rank, a CTA per node and no cluster is the shorter chain.
 bool topk_fused_applies(const tsv_shape& s, const TvaPlan& p) {
-  return p.need_scores && p.idx_fused && s.dtype == TSV_BF16 && s.di == fsel::DI && s.HI <= 4;
+  return p.need_scores && p.idx_fused && p.cand_cap <= fsel::kCands && s.dtype == TSV_BF16 && s.di == fsel::DI && s.HI <= 4;
 }
 
 // Rows per staging buffer (two buffers) and dynamic shared memory: as many rows (<= 128, a multiple of 16) as let four
@@ -311,15 +311,13 @@ int launch_topk_fused(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, 
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;          // may start under the state build's tail (it waits inside)
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = 1;
-#define TSV_FUSED_LAUNCH(PG_, KPT_)                                                                                                     \
-  do {                                                                                                                                 \
-    TSV_PREP((topk_fused_kernel<PG_, KPT_>));                                                                                          \
-    if (bytes > 40 * 1024) cudaFuncSetAttribute(topk_fused_kernel<PG_, KPT_>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes); \
-    cudaLaunchKernelEx(&cfg, topk_fused_kernel<PG_, KPT_>, s, p, c, nd, sc, topk_idx, ws, status, rows, score_cap);                     \
+#define TSV_FUSED_LAUNCH(PG_)                                                                                                    \
+  do {                                                                                                                          \
+    TSV_PREP(topk_fused_kernel<PG_>);                                                                                           \
+    if (bytes > 40 * 1024 && !ensure_smem((const void*)topk_fused_kernel<PG_>, (int)bytes)) return TSV_ERR_CUDA;                \
+    cudaLaunchKernelEx(&cfg, topk_fused_kernel<PG_>, s, p, c, nd, sc, topk_idx, ws, status, rows, score_cap);                   \
   } while (0)
-  const bool shortl = p.cand_cap <= fsel::KPT_SHORT * 256;
-  if (c.page_table) { if (shortl) TSV_FUSED_LAUNCH(true, fsel::KPT_SHORT); else TSV_FUSED_LAUNCH(true, fsel::KPT_LONG); }
-  else { if (shortl) TSV_FUSED_LAUNCH(false, fsel::KPT_SHORT); else TSV_FUSED_LAUNCH(false, fsel::KPT_LONG); }
+  if (c.page_table) TSV_FUSED_LAUNCH(true); else TSV_FUSED_LAUNCH(false);
 #undef TSV_FUSED_LAUNCH
   count_launch();
   return cudaGetLastError() == cudaSuccess ? TSV_OK : TSV_ERR_CUDA;

@@ -1,0 +1,560 @@
+// Per-node top-k with 128-wide bf16 indexer rows and up to four indexer heads, for lists beyond the short ones.
+//
+// Scoring (both forms): a warp scores sixteen entries at a time for eight nodes and all heads by tensor-core products (16
+// entries x 32 query rows), its rows straight from global memory into the fragments: an inner product does not care for the
+// order of its terms, so lane tq of a row's four takes the 16-byte pieces tq, tq + 4, ... and the queries are read the same
+// way.  An indexer row is read once per sequence (one CTA per node read it once per node, in rounds of 96 rows through
+// shared memory), and no warp waits for another.
+//
+//   topk_seq_kernel   lists of up to kSeqMax entries, trees of up to eight nodes: one cluster of eight CTAs per SEQUENCE.  The
+//                     entries are split over the CTAs; a warp leaves its scores in the lists of the nodes' owners (CTA r owns
+//                     node r) through distributed shared memory, and after one cluster barrier every node's whole list
+//                     lies in its owner's shared memory.
+//   score_rows_kernel + topk_list_kernel   longer lists or larger trees: the scores over all SMs into the workspace, then a
+//                     CTA per node with its list in shared memory.
+//
+// The selection finds the k largest by ONE histogram over equal intervals of [min, max] (the scores of a list share their high
+// bits, so radix digits of the bit pattern take four passes with colliding bins): the interval of the k-th largest holds few
+// candidates, which are ranked against each other exactly (ties to the lower index).  Degenerate lists (more than CAP
+// candidates in that interval: ties, outliers) take four radix passes instead.
+// Same result as topk_kernel: the exact k largest scores, ties to the lower index, ascending output.
+#include "select_common.cuh"
+
+namespace tsv {
+
+namespace ssel {
+
+constexpr int CS = 8;                  // CTAs per cluster = nodes scored together
+constexpr int kSeqMax = 4096;          // longest list of the cluster form
+constexpr int DI = 128, HMAX = 4;      // indexer width, heads (query row 4 n + h, absent ones zero)
+constexpr int QP = 320;                // pitch of a staged query row: conflict-free 16-byte fragment loads
+constexpr int CAP = 256;               // candidates ranked against each other
+
+__device__ __forceinline__ void mma_bf16_16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ uint32_t map_to_rank(uint32_t saddr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+// dynamic shared memory of the cluster form: queries | a step's scores per warp | score list of the owned node | bit per candidate
+struct Layout {
+  uint32_t loc, sc, bits, total;
+  __host__ __device__ Layout(int nw, int cap) {
+    loc = 32 * QP;
+    sc = loc + (uint32_t)nw * 512;
+    bits = sc + (uint32_t)cap * 4;
+    total = bits + ((uint32_t)cap + 31) / 32 * 4;
+  }
+};
+
+// Sixteen entries against the queries of eight nodes.
+struct Scorer {
+  const char* ikb;
+  RowAddr rows;
+  int g, tq, end;
+  float iwr[4][2];                                       // head weights of this lane's columns 8 j + 2 tq, + 1
+  // rows g and g + 8 of the sixteen entries from e on: lane tq's pieces of 16 bytes, four of a row
+  template <bool PAGED>
+  __device__ __forceinline__ void fetch(int e, uint4 (&lo)[4], uint4 (&hi)[4]) const {
+    const int r0 = min(e + g, end - 1), r1 = min(e + g + 8, end - 1);
+    const uint4* p0 = reinterpret_cast<const uint4*>(ikb + (size_t)(PAGED ? rows.rel(r0) : (int64_t)r0) * (DI * 2));
+    const uint4* p1 = reinterpret_cast<const uint4*>(ikb + (size_t)(PAGED ? rows.rel(r1) : (int64_t)r1) * (DI * 2));
+#pragma unroll
+    for (int q = 0; q < 4; ++q) { lo[q] = __ldg(p0 + 4 * q); hi[q] = __ldg(p1 + 4 * q); }
+  }
+  __device__ __forceinline__ void weights(const float* iw, int n0, int D, int HI) {      // iw: [D][HI] of the sequence
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        const int n = n0 + 2 * j + (tq >> 1), h = ((2 * tq) & 3) + x;
+        iwr[j][x] = n < D && h < HI ? __ldg(iw + n * HI + h) : 0.f;
+      }
+  }
+  // scores into buf (this warp's, [8 nodes][16 entries]); qs: the staged queries
+  __device__ __forceinline__ void score(const uint4 (&lo)[4], const uint4 (&hi)[4], const unsigned char* qs, float* buf) const {
+    float acc[4][4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int x = 0; x < 4; ++x) acc[j][x] = 0.f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {                      // column g of tile j = query row 8 j + g
+        const uint4 bv = *reinterpret_cast<const uint4*>(qs + (8 * j + g) * QP + q * 64 + tq * 16);
+        mma_bf16_16816(acc[j], lo[q].x, hi[q].x, lo[q].y, hi[q].y, bv.x, bv.y);
+        mma_bf16_16816(acc[j], lo[q].z, hi[q].z, lo[q].w, hi[q].w, bv.z, bv.w);
+      }
+    }
+    __syncwarp();                                        // (the step before has left the buffer)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      float l = fmaf(iwr[j][1], fmaxf(acc[j][1], 0.f), iwr[j][0] * fmaxf(acc[j][0], 0.f));
+      float h = fmaf(iwr[j][1], fmaxf(acc[j][3], 0.f), iwr[j][0] * fmaxf(acc[j][2], 0.f));
+      l += __shfl_xor_sync(0xffffffffu, l, 1);
+      h += __shfl_xor_sync(0xffffffffu, h, 1);
+      if (!(tq & 1)) { float* o = buf + (2 * j + (tq >> 1)) * 16 + g; o[0] = l; o[8] = h; }
+    }
+    __syncwarp();
+  }
+};
+// queries of nodes n0 .. n0 + 7 of sequence b into shared memory: row 4 (n - n0) + h; absent heads and node slots zero
+__device__ __forceinline__ void stage_queries(unsigned char* qs, const void* iq_, int b, int n0, int D, int HI) {
+  const uint4* iq = reinterpret_cast<const uint4*>(reinterpret_cast<const bf16*>(iq_) + (size_t)b * D * HI * DI);
+  for (int idx = threadIdx.x; idx < 32 * 16; idx += blockDim.x) {
+    const int row = idx >> 4, c16 = idx & 15, n = n0 + (row >> 2), h = row & 3;
+    *reinterpret_cast<uint4*>(qs + row * QP + c16 * 16) = n < D && h < HI ? __ldg(iq + (n * HI + h) * (DI / 8) + c16) : make_uint4(0u, 0u, 0u, 0u);
+  }
+}
+// Lane j = node j: the strict ancestors of node n that close a CSA block (from their positions), root first.  One warp.
+__device__ __forceinline__ void path_of(PathEntries& pe, const TreeMeta& tm, const tsv_shape& s, int n, bool live) {
+  const int t = threadIdx.x & 31;
+  const bool valid = !tm.status && t < tm.nn;
+  const uint32_t strict = live ? tm.anc[n] & ~(1u << n) : 0u;
+  const uint32_t cm = __ballot_sync(0xffffffffu, valid && node_closes(tm.L, tm.depth[t], s.m_csa)) & strict;
+  if ((cm >> t) & 1u) { const int o = __popc(cm & ((1u << t) - 1u)); pe.newc[o] = t; pe.newc_blk[o] = (tm.L + tm.depth[t]) / s.m_csa; }
+  if (t == 0) pe.n_newc = __popc(cm);
+}
+// Scores of the in-tree entries on node n's path (the state build's results): warp w takes entries w, w + nw, ...
+__device__ __forceinline__ void score_extras(float* extra, const PathEntries& pe, const tsv_shape& s, const tsv_nodes& nd, const tsv_scratch& sc, int b, int n) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5, D = s.D, HI = s.HI;
+  const bf16* iq = reinterpret_cast<const bf16*>(nd.iq) + ((size_t)b * D + n) * HI * DI;
+  for (int i = w; i < pe.n_newc; i += nw) {
+    const bf16* ik = reinterpret_cast<const bf16*>(sc.new_csa_ik) + ((size_t)b * D + pe.newc[i]) * DI;
+    float tot = 0.f;
+    for (int h = 0; h < HI; ++h) {
+      float p = 0.f;
+#pragma unroll
+      for (int x = lane; x < DI; x += 32) p = fmaf(to_f(iq[h * DI + x]), to_f(ik[x]), p);
+      p = warp_sum(p);
+      tot = fmaf(nd.iw[((size_t)b * D + n) * HI + h], fmaxf(p, 0.f), tot);
+    }
+    if (lane == 0) extra[i] = tot;
+  }
+}
+// Everything is selected (or nothing: padding, a flagged sequence): the index list, where somebody reads it.
+__device__ __forceinline__ void select_all(int n_cand, int n_csa, const PathEntries& pe, int k, int32_t* sel, int32_t* usr, int32_t* selcnt) {
+  for (int i = threadIdx.x; i < k; i += blockDim.x) {
+    const int v = i < n_cand ? (i < n_csa ? i : pe.newc_blk[i - n_csa]) : -1;
+    sel[i] = v; if (usr) usr[i] = v;
+  }
+  if (threadIdx.x == 0) *selcnt = n_cand;
+}
+
+template <int NT, int NB>
+struct SelectSmem {
+  int hist[NB];                                          // zero at the start of the selection, like cnt
+  float red[2][NT / 32];
+  int wsum[2][NT / 32];
+  int bin, rem, cnt;
+  float cand_s[CAP];
+  int cand_i[CAP];
+};
+
+// Selection of one node by the whole CTA: list (shared memory, n_cand scores, committed entries first), bits (zero).  lists: write
+// the index list; selmask: a byte per candidate for the tile plan, or null.
+template <int NT, int NB>
+__device__ __forceinline__ void select_node(SelectSmem<NT, NB>& sm, const float* list, uint32_t* bits, int n_cand, int n_csa, const PathEntries& pe, int k,
+                                            bool lists, int32_t* sel, int32_t* usr, int32_t* selcnt, uint8_t* selmask) {
+  constexpr int NW = NT / 32;
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  float lo = INFINITY, hi = -INFINITY;
+  for (int i = t; i < n_cand; i += NT) { const float v = list[i]; lo = fminf(lo, v); hi = fmaxf(hi, v); }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) { lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o)); hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o)); }
+  if (lane == 0) { sm.red[0][w] = lo; sm.red[1][w] = hi; }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < NW; ++i) { lo = fminf(lo, sm.red[0][i]); hi = fmaxf(hi, sm.red[1][i]); }
+  // interval of a score: monotone in the score (a rounded subtraction and product are), so intervals order as scores do
+  const float scale = hi > lo ? (float)NB / (hi - lo) : 0.f;
+  const bool regular = scale > 0.f && scale < 1e30f;     // (else: all equal, not finite, or too narrow)
+  auto bin_of = [&](float v) { return min(NB - 1, (int)((v - lo) * scale)); };
+  int m = CAP + 1, bstar = 0, rem = k;
+  if (regular) {
+    for (int i = t; i < n_cand; i += NT) atomicAdd(&sm.hist[bin_of(list[i])], 1);
+    __syncthreads();
+    // thread t holds intervals NB - 1 - t PER .. down: exclusive sum from the top
+    constexpr int PER = NB / NT;
+    int h[PER], tot = 0;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) { h[j] = sm.hist[NB - 1 - (t * PER + j)]; tot += h[j]; }
+    int incl = tot;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += y; }
+    if (lane == 31) sm.wsum[0][w] = incl;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < NW; ++i) if (i < w) incl += sm.wsum[0][i];
+    int cum = incl - tot;
+    if (cum < k && incl >= k) {                          // exactly one thread
+#pragma unroll
+      for (int j = 0; j < PER; ++j) {
+        if (cum + h[j] >= k) { sm.bin = NB - 1 - (t * PER + j); sm.rem = k - cum; break; }
+        cum += h[j];
+      }
+    }
+    __syncthreads();
+    bstar = sm.bin; rem = sm.rem;
+    for (int i = t; i < n_cand; i += NT) {
+      const float v = list[i];
+      if (bin_of(v) == bstar) { const int pos = atomicAdd(&sm.cnt, 1); if (pos < CAP) { sm.cand_s[pos] = v; sm.cand_i[pos] = i; } }
+    }
+    __syncthreads();
+    m = sm.cnt;
+    if (m <= CAP) {
+      for (int x = t; x < m; x += NT) {
+        const float v = sm.cand_s[x];
+        const int ix = sm.cand_i[x];
+        int r = 0;
+        for (int y = 0; y < m; ++y) { const float u = sm.cand_s[y]; r += (u > v || (u == v && sm.cand_i[y] < ix)) ? 1 : 0; }
+        if (r < rem) atomicOr(&bits[ix >> 5], 1u << (ix & 31));
+      }
+      __syncthreads();
+    }
+  }
+  uint32_t thr = 0;
+  const bool radix = m > CAP;
+  if (radix) {                                           // four passes of 8 bits over the order-preserving keys
+    uint32_t mask = 0;
+    rem = k;
+#pragma unroll 1
+    for (int pass = 0; pass < 4; ++pass) {
+      const int shift = 24 - 8 * pass;
+      __syncthreads();
+      for (int i = t; i < 256; i += NT) sm.hist[i] = 0;
+      __syncthreads();
+      for (int i = t; i < n_cand; i += NT) { const uint32_t key = order_key(list[i]); if ((key & mask) == thr) atomicAdd(&sm.hist[(key >> shift) & 255u], 1); }
+      __syncthreads();
+      // every warp finds the interval of the rem-th largest for itself: lane l owns bins 255 - 8 l .. 248 - 8 l
+      int h[8], tot = 0;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) { h[j] = sm.hist[255 - (lane * 8 + j)]; tot += h[j]; }
+      int incl = tot;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += y; }
+      const bool own = incl - tot < rem && incl >= rem;  // exactly one lane
+      int cum = incl - tot, bin = 255 - lane * 8;
+      if (own) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) { if (cum + h[j] >= rem) { bin = 255 - (lane * 8 + j); break; } cum += h[j]; }
+      }
+      const int src = __ffs(__ballot_sync(0xffffffffu, own)) - 1;
+      thr |= (uint32_t)__shfl_sync(0xffffffffu, bin, src) << shift;
+      rem -= __shfl_sync(0xffffffffu, cum, src);
+      mask |= 0xFFu << shift;
+    }
+  }
+  // Warp w owns the candidates [w * part, (w + 1) * part), rows of 32.  above: certainly taken; edge (radix only): equal to the
+  // threshold, of which the first rem in index order are taken.
+  const int part = ((n_cand + NW - 1) / NW + 31) & ~31, beg = min(n_cand, w * part), end = min(n_cand, beg + part);
+  auto classify = [&](int i, bool& above, bool& edge) {
+    above = edge = false;
+    if (i >= end) return;
+    const float v = list[i];
+    if (radix) { const uint32_t key = order_key(v); above = key > thr; edge = key == thr; }
+    else { const int bn = bin_of(v); above = bn > bstar || (bn == bstar && ((bits[i >> 5] >> (i & 31)) & 1u)); }
+  };
+  int pos = 0, eq_base = 0;
+  if (lists || radix) {
+    int ca = 0, ce = 0;
+    for (int i0 = beg; i0 < end; i0 += 32) {
+      bool above, edge;
+      classify(i0 + lane, above, edge);
+      ca += __popc(__ballot_sync(0xffffffffu, above)); ce += __popc(__ballot_sync(0xffffffffu, edge));
+    }
+    __syncthreads();
+    if (lane == 0) { sm.wsum[0][w] = ca; sm.wsum[1][w] = ce; }
+    __syncthreads();
+    for (int i = 0; i < w; ++i) { pos += sm.wsum[0][i]; eq_base += sm.wsum[1][i]; }
+    if (radix) pos += min(rem, eq_base);
+  }
+  const uint32_t lt = (1u << lane) - 1u;
+  for (int i0 = beg; i0 < end; i0 += 32) {
+    const int i = i0 + lane;
+    bool take, edge;
+    classify(i, take, edge);
+    if (radix) {
+      const uint32_t eqm = __ballot_sync(0xffffffffu, edge);
+      take = take || (edge && eq_base + __popc(eqm & lt) < rem);
+      eq_base += __popc(eqm);
+    }
+    if (selmask && i < end) selmask[i] = (uint8_t)take;
+    if (lists) {
+      const uint32_t tkm = __ballot_sync(0xffffffffu, take);
+      if (take) {
+        const int p = pos + __popc(tkm & lt), val = i < n_csa ? i : pe.newc_blk[i - n_csa];
+        sel[p] = val; if (usr) usr[p] = val;
+      }
+      pos += __popc(tkm);
+    }
+  }
+  if (lists && t == 0) *selcnt = k;
+}
+
+}  // namespace ssel
+
+// `cap`: floats of the score list (covers the padded shares of the eight CTAs and the in-tree entries).
+template <bool PAGED>
+__global__ void __launch_bounds__(128, 4) topk_seq_kernel(const tsv_shape s, const TvaPlan pl, const tsv_cache c, const tsv_nodes nd,
+                                                         const tsv_scratch sc, int32_t* __restrict__ topk_user, char* __restrict__ ws,
+                                                         int32_t* __restrict__ status, const int cap) {
+  using namespace ssel;
+  constexpr int NT = 128, NB = 1024, NW = NT / 32;
+  extern __shared__ __align__(128) unsigned char dsm[];
+  __shared__ TreeMeta tm;
+  __shared__ TreeStage tstage;
+  __shared__ PathEntries pe;
+  __shared__ float extra[TSV_MAX_D];
+  __shared__ SelectSmem<NT, NB> sm;
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the tile plan may start its selection-independent part
+  const int rank = blockIdx.x, b = blockIdx.y, D = s.D, k = s.topk, HI = s.HI;
+  const bool lists = !pl.tc || topk_user;               // somebody reads the index lists (the tile plan reads mask rows only)
+  const int L0 = c.L[b];
+  // some node may have more than k candidates (and the rows exist: a sequence of bad length or capacity is flagged below)
+  const bool any_rank = L0 >= 0 && (int64_t)L0 + D <= s.max_L && (L0 + D) / s.m_csa <= c.csa_cap[b] && L0 / s.m_csa + D > k;
+  if (!any_rank && !lists && rank != 0) return;          // (alike in the whole cluster but for CTA 0, which validates the sequence)
+  const Layout lay(NW, cap);
+  const uint32_t smem_s = (uint32_t)__cvta_generic_to_shared(dsm);
+  float* loc = reinterpret_cast<float*>(dsm + lay.loc) + w * 128;
+  float* list = reinterpret_cast<float*>(dsm + lay.sc);
+  uint32_t* bits = reinterpret_cast<uint32_t*>(dsm + lay.bits);
+  if (any_rank) cluster_arrive();                        // (every CTA runs before a peer writes to it; awaited before the first write)
+  // this CTA's entries (a multiple of sixteen but for the end of the list)
+  const int n_ent = any_rank ? L0 / s.m_csa : 0;
+  const int share = ((n_ent + CS - 1) / CS + 15) & ~15, e0 = min(n_ent, rank * share), e1 = min(n_ent, e0 + share);
+  Scorer sco;
+  sco.g = lane >> 2; sco.tq = lane & 3; sco.end = e1;
+  uint4 alo[4], ahi[4];
+  const int first = e0 + 16 * w;
+  if (any_rank) {
+    if (PAGED) sco.rows = csa_rows_of(c, s, b); else { sco.rows.pt = nullptr; sco.rows.per_page = 1; sco.rows.row0 = c.csa_row0[b]; }
+    sco.ikb = reinterpret_cast<const char*>(c.csa_ik) + (size_t)sco.rows.row0 * (DI * 2) + sco.tq * 16;
+    if (first < e1) sco.fetch<PAGED>(first, alo, ahi);
+    stage_queries(dsm, nd.iq, b, 0, D, HI);
+    sco.weights(nd.iw + (size_t)b * D * HI, 0, D, HI);
+    for (int i = t; i < (cap + 31) / 32; i += NT) bits[i] = 0u;
+    for (int i = t; i < NB; i += NT) sm.hist[i] = 0;
+    if (t == 0) sm.cnt = 0;
+  }
+  coop_tree_meta(tm, tstage, s, c.L + b, nd.parent + (size_t)b * D, nd.n_nodes + b, c.csa_cap + b, c.hca_cap + b);
+  if (t == 0 && rank == 0 && tm.status) atomicOr(status + b, tm.status);
+  const int n = rank;                                    // the node this CTA owns
+  const bool live = !tm.status && n < tm.nn;
+  const int n_csa = tm.n_csa;
+  if (t < 32) path_of(pe, tm, s, n, live);
+  __syncthreads();                                       // (the path entries: a warp without entries to score reads them at once)
+  // (a sequence flagged for its tree is scored too -- its rows exist -- and then dropped)
+  if (any_rank) {
+    cluster_wait();                                      // the peers run
+    for (int e = first; e < e1; e += 16 * NW) {
+      uint4 nlo[4], nhi[4];
+      const bool more = e + 16 * NW < e1;
+      if (more) sco.fetch<PAGED>(e + 16 * NW, nlo, nhi);
+      sco.score(alo, ahi, dsm, loc);
+      // lane l: four entries of node l / 4 (up to three past the end of the list: overwritten below or never read)
+      const float4 v = *reinterpret_cast<const float4*>(loc + 4 * lane);
+      if ((lane >> 2) < D && e + 4 * (lane & 3) < e1)
+        asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(map_to_rank(smem_s + lay.sc + (uint32_t)(e + 4 * (lane & 3)) * 4, lane >> 2)),
+                     "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+      if (more) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) { alo[q] = nlo[q]; ahi[q] = nhi[q]; }
+      }
+    }
+    __syncwarp();
+    cluster_arrive();                                    // this CTA's scores are on their way; awaited below
+    // the state build's results: the first thing of that kernel this CTA reads (all of the above may run under its tail)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (live) score_extras(extra, pe, s, nd, sc, b, n);
+    __syncwarp();
+    cluster_wait();                                      // every peer's scores of this node are in the list; nobody touches a peer's memory from here on
+  } else if (rank == 0 && b == 0) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");   // (so that this kernel's completion implies the state build's)
+  }
+  __syncthreads();
+  if (n >= D) return;
+  int32_t* sel = reinterpret_cast<int32_t*>(ws + pl.off_sel) + ((size_t)b * D + n) * k;
+  int32_t* selcnt = reinterpret_cast<int32_t*>(ws + pl.off_selcnt) + (size_t)b * D + n;
+  int32_t* usr = topk_user ? topk_user + ((size_t)b * D + n) * k : nullptr;
+  const int n_cand = live ? n_csa + pe.n_newc : 0;
+  if (n_cand <= k) {
+    if (lists) select_all(n_cand, n_csa, pe, k, sel, usr, selcnt);
+    return;
+  }
+  for (int i = n_csa + t; i < n_cand; i += NT) list[i] = extra[i - n_csa];
+  __syncthreads();
+  uint8_t* selmask = pl.tc ? reinterpret_cast<uint8_t*>(ws + pl.off_selmask) + ((size_t)b * D + n) * pl.mask_ld : nullptr;   // (for the tile plan)
+  select_node(sm, list, bits, n_cand, n_csa, pe, k, lists, sel, usr, selcnt, selmask);
+}
+
+// ------------------------------------------------------------------------------------------------ long lists
+// Scores of all nodes of a sequence into the workspace.  grid (entry blocks, B, groups of eight nodes), four warps, kRowSteps steps
+// of sixteen entries each; reads the caller's data and the committed caches only, so it runs under the state build's tail.
+constexpr int kRowSteps = 4;
+template <bool PAGED>
+__global__ void __launch_bounds__(128) score_rows_kernel(const tsv_shape s, const TvaPlan pl, const tsv_cache c, const tsv_nodes nd, char* __restrict__ ws) {
+  using namespace ssel;
+  __shared__ __align__(16) unsigned char qs[32 * QP];
+  __shared__ __align__(16) float bufs[4][128];
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the selection waits for this kernel before it reads a score
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5, b = blockIdx.y, n0 = 8 * blockIdx.z, D = s.D, HI = s.HI;
+  const int L0 = c.L[b];
+  // (the rows exist: a sequence of bad length or capacity is flagged by the selection)
+  const bool any_rank = L0 >= 0 && (int64_t)L0 + D <= s.max_L && (L0 + D) / s.m_csa <= c.csa_cap[b] && L0 / s.m_csa + D > s.topk;
+  const int n_ent = any_rank ? L0 / s.m_csa : 0;
+  const int first = (blockIdx.x * kRowSteps * 4 + w) * 16;
+  if ((int)(blockIdx.x * kRowSteps * 64) >= n_ent) {
+    if (blockIdx.x == 0 && b == 0 && blockIdx.z == 0) asm volatile("griddepcontrol.wait;" ::: "memory");   // (this kernel's completion implies the state build's)
+    return;
+  }
+  Scorer sco;
+  sco.g = lane >> 2; sco.tq = lane & 3; sco.end = n_ent;
+  if (PAGED) sco.rows = csa_rows_of(c, s, b); else { sco.rows.pt = nullptr; sco.rows.per_page = 1; sco.rows.row0 = c.csa_row0[b]; }
+  sco.ikb = reinterpret_cast<const char*>(c.csa_ik) + (size_t)sco.rows.row0 * (DI * 2) + sco.tq * 16;
+  uint4 alo[4], ahi[4], nlo[4], nhi[4];
+  sco.fetch<PAGED>(min(first, n_ent - 1), alo, ahi);
+  stage_queries(qs, nd.iq, b, n0, D, HI);
+  sco.weights(nd.iw + (size_t)b * D * HI, n0, D, HI);
+  __syncthreads();
+  float* scores = reinterpret_cast<float*>(ws + pl.off_scores) + (size_t)b * D * pl.score_ld;
+  // (the call before on the same workspace may still be read: nothing is written before the kernel before has ended)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+#pragma unroll
+  for (int st = 0; st < kRowSteps; ++st) {
+    const int e = first + st * 64;
+    if (e >= n_ent) break;
+    if (st + 1 < kRowSteps) sco.fetch<PAGED>(min(e + 64, n_ent - 1), nlo, nhi);
+    sco.score(alo, ahi, qs, bufs[w]);
+    const float4 v = *reinterpret_cast<const float4*>(bufs[w] + 4 * lane);
+    const int n = n0 + (lane >> 2), i = e + 4 * (lane & 3);            // (rows of the score array are padded to whole float4)
+    if (n < D && i < n_ent) *reinterpret_cast<float4*>(scores + (size_t)n * pl.score_ld + i) = v;
+    if (st + 1 < kRowSteps) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) { alo[q] = nlo[q]; ahi[q] = nhi[q]; }
+    }
+  }
+}
+
+// Selection of one node from the score array: grid (D, B).  Dynamic shared memory: the list, a bit per candidate.
+constexpr int kListThreads = 1024, kListBins = 2048;
+__global__ void __launch_bounds__(kListThreads) topk_list_kernel(const tsv_shape s, const TvaPlan pl, const tsv_cache c, const tsv_nodes nd,
+                                                                 const tsv_scratch sc, int32_t* __restrict__ topk_user, char* __restrict__ ws,
+                                                                 int32_t* __restrict__ status) {
+  using namespace ssel;
+  extern __shared__ __align__(128) unsigned char dsm[];
+  __shared__ TreeMeta tm;
+  __shared__ TreeStage tstage;
+  __shared__ PathEntries pe;
+  __shared__ float extra[TSV_MAX_D];
+  __shared__ SelectSmem<kListThreads, kListBins> sm;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the tile plan may start its selection-independent part
+  const int t = threadIdx.x, n = blockIdx.x, b = blockIdx.y, D = s.D, k = s.topk;
+  const bool lists = !pl.tc || topk_user;
+  coop_tree_meta(tm, tstage, s, c.L + b, nd.parent + (size_t)b * D, nd.n_nodes + b, c.csa_cap + b, c.hca_cap + b);
+  if (t == 0 && n == 0 && tm.status) atomicOr(status + b, tm.status);
+  const bool live = !tm.status && n < tm.nn;
+  const int n_csa = tm.n_csa;
+  if (t < 32) path_of(pe, tm, s, n, live);
+  for (int i = t; i < kListBins; i += kListThreads) sm.hist[i] = 0;
+  if (t == 0) sm.cnt = 0;
+  __syncthreads();
+  int32_t* sel = reinterpret_cast<int32_t*>(ws + pl.off_sel) + ((size_t)b * D + n) * k;
+  int32_t* selcnt = reinterpret_cast<int32_t*>(ws + pl.off_selcnt) + (size_t)b * D + n;
+  int32_t* usr = topk_user ? topk_user + ((size_t)b * D + n) * k : nullptr;
+  const int n_cand = live ? n_csa + pe.n_newc : 0;
+  if (n_cand <= k) {
+    // (waits too: this kernel's completion implies that of the ones before)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (lists) select_all(n_cand, n_csa, pe, k, sel, usr, selcnt);
+    return;
+  }
+  float* list = reinterpret_cast<float*>(dsm);
+  uint32_t* bits = reinterpret_cast<uint32_t*>(dsm + (((size_t)pl.score_ld + TSV_MAX_D + 3) & ~(size_t)3) * 4);
+  for (int i = t; i < (n_cand + 31) / 32; i += kListThreads) bits[i] = 0u;
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // the scores, and (the scoring kernel waited) the entries closed inside the tree
+  const float4* src = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(ws + pl.off_scores) + ((size_t)b * D + n) * pl.score_ld);
+  const int n4 = (n_csa + 3) >> 2;
+  for (int i0 = t; i0 < n4; i0 += 4 * kListThreads) {
+    float4 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) if (i0 + u * kListThreads < n4) v[u] = __ldcg(src + i0 + u * kListThreads);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) if (i0 + u * kListThreads < n4) reinterpret_cast<float4*>(list)[i0 + u * kListThreads] = v[u];
+  }
+  score_extras(extra, pe, s, nd, sc, b, n);
+  __syncthreads();
+  for (int i = n_csa + t; i < n_cand; i += kListThreads) list[i] = extra[i - n_csa];
+  __syncthreads();
+  uint8_t* selmask = pl.tc ? reinterpret_cast<uint8_t*>(ws + pl.off_selmask) + ((size_t)b * D + n) * pl.mask_ld : nullptr;   // (for the tile plan)
+  select_node(sm, list, bits, n_cand, n_csa, pe, k, lists, sel, usr, selcnt, selmask);
+}
+
+// ------------------------------------------------------------------------------------------------ dispatch
+static int seq_cap(const tsv_shape& s) {                 // padded shares of eight CTAs, the in-tree entries
+  const int ent = (int)(s.max_L / s.m_csa), share = ((ent + ssel::CS - 1) / ssel::CS + 15) & ~15;
+  return (share * ssel::CS + TSV_MAX_D + 127) & ~127;
+}
+static size_t list_bytes(const TvaPlan& p) {
+  const size_t fl = ((size_t)p.score_ld + TSV_MAX_D + 3) & ~(size_t)3;
+  return fl * 4 + (fl + 31) / 32 * 4;
+}
+// The cluster form: its CTAs are small and all resident up to some 70 sequences; beyond kSeqMax entries a node's list is the work of
+// too few threads.
+static bool seq_form(const tsv_shape& s) { return s.D <= ssel::CS && s.max_L / s.m_csa <= ssel::kSeqMax; }
+
+// bf16, 128-wide indexer rows, at most four heads, lists that fit one CTA's shared memory as scores and are too long for
+// topk_fused_kernel (which is the shorter chain while a list is three keys a thread).
+bool topk_seq_applies(const tsv_shape& s, const TvaPlan& p) {
+  return p.need_scores && s.dtype == TSV_BF16 && s.di == ssel::DI && s.HI <= ssel::HMAX && !topk_fused_applies(s, p) &&
+         (seq_form(s) || list_bytes(p) <= 200 * 1024);
+}
+
+int launch_topk_seq(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, const tsv_nodes& nd, const tsv_scratch& sc,
+                    int32_t* topk_idx, char* ws, int32_t* status, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;          // may start under the tail of the kernel before (it waits inside)
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = ssel::CS; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cudaError_t e;
+  if (seq_form(s)) {
+    const int cap = seq_cap(s);
+    const int bytes = (int)ssel::Layout(4, cap).total;
+    cfg.numAttrs = 2;
+    cfg.gridDim = dim3(ssel::CS, s.B, 1); cfg.blockDim = dim3(128, 1, 1); cfg.dynamicSmemBytes = bytes;
+    TSV_PREP(topk_seq_kernel<true>); TSV_PREP(topk_seq_kernel<false>);
+    const void* kern = c.page_table ? (const void*)topk_seq_kernel<true> : (const void*)topk_seq_kernel<false>;
+    if (bytes > 32 * 1024 && !ensure_smem(kern, bytes)) return TSV_ERR_CUDA;
+    e = c.page_table ? cudaLaunchKernelEx(&cfg, topk_seq_kernel<true>, s, p, c, nd, sc, topk_idx, ws, status, cap)
+                     : cudaLaunchKernelEx(&cfg, topk_seq_kernel<false>, s, p, c, nd, sc, topk_idx, ws, status, cap);
+    count_launch();
+  } else {
+    const int bytes = (int)list_bytes(p);
+    if (!ensure_smem((const void*)topk_list_kernel, bytes)) return TSV_ERR_CUDA;
+    cfg.numAttrs = 1;
+    const int ent = (int)(s.max_L / s.m_csa), per = kRowSteps * 64;
+    cfg.gridDim = dim3((ent + per - 1) / per, s.B, (s.D + 7) / 8); cfg.blockDim = dim3(128, 1, 1);
+    TSV_PREP(score_rows_kernel<true>); TSV_PREP(score_rows_kernel<false>); TSV_PREP(topk_list_kernel);
+    e = c.page_table ? cudaLaunchKernelEx(&cfg, score_rows_kernel<true>, s, p, c, nd, ws) : cudaLaunchKernelEx(&cfg, score_rows_kernel<false>, s, p, c, nd, ws);
+    count_launch();
+    if (e != cudaSuccess) { cudaGetLastError(); return TSV_ERR_CUDA; }
+    cfg.gridDim = dim3(s.D, s.B, 1); cfg.blockDim = dim3(kListThreads, 1, 1); cfg.dynamicSmemBytes = bytes;
+    e = cudaLaunchKernelEx(&cfg, topk_list_kernel, s, p, c, nd, sc, topk_idx, ws, status);
+    count_launch();
+  }
+  return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? TSV_OK : TSV_ERR_CUDA;
+}
+
+}  // namespace tsv

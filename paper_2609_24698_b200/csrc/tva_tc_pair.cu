@@ -226,7 +226,9 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
   // Launched as a programmatic dependent of the tile plan: the CTAs take their places and set up while that kernel's last
   // CTAs finish, and read nothing of its before it has completed.
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // (the merge kernel, which waits for this one before it does anything)
+  // The merge kernel, where one follows, may take its places: it waits for this kernel before it does anything.  (Nothing else may
+  // start before this kernel has ended: the next call's tile plan would overwrite what is read here.)
+  if (GENERAL && pl.tc_chmax > 1) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int4 rec0 = (int)(blockIdx.x >> 1) < s.B * pl.tc_nt ? __ldcg(reinterpret_cast<const int4*>(ws + pl.off_order) + (blockIdx.x >> 1)) : make_int4(-1, 0, 0, 0);
   fence_before();
   __syncthreads();
