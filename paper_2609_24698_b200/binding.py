@@ -105,8 +105,18 @@ def _stream(stream) -> int:
     return (torch.cuda.current_stream() if stream is None else stream).cuda_stream
 
 
+class _Versioned:
+    """Counts the assignments to an object's fields, so that what was built from them can tell that it is out of date."""
+    _version = 0
+
+    def __setattr__(self, name, value):
+        d = self.__dict__
+        d[name] = value
+        d["_version"] = d.get("_version", 0) + 1
+
+
 @dataclass
-class LayerCache:
+class LayerCache(_Versioned):
     """Persistent per-layer state (device tensors); rows of sequence b start at *_row0[b]."""
     L: torch.Tensor
     csa_kv: torch.Tensor
@@ -158,7 +168,7 @@ class LayerCache:
 
 
 @dataclass
-class NodeInputs:
+class NodeInputs(_Versioned):
     q: torch.Tensor
     kv: torch.Tensor
     c_csa: torch.Tensor
@@ -176,7 +186,7 @@ class NodeInputs:
 
 
 @dataclass
-class Scratch:
+class Scratch(_Versioned):
     csa_mx: torch.Tensor
     csa_s: torch.Tensor
     csa_acc_kv: torch.Tensor
@@ -312,15 +322,47 @@ def bench_tree_verify_attn_stages(shape: CShape, cache: LayerCache, nodes: NodeI
 
 
 class LayerPack:
-    """Host arrays of per-layer struct pointers for accept_and_refresh, built once and reused."""
+    """Host arrays of per-layer struct pointers for the calls over all layers, built once and reused."""
 
     def __init__(self, caches: List[LayerCache], nodes: List[NodeInputs], scratch: List[Scratch]):
         n = len(caches)
         self.n = n
+        objs = (*caches, *nodes, *scratch)
+        self._ids, self._version = [id(x) for x in objs], sum(x._version for x in objs)
+        self._tensors = [t for x in objs for t in x.__dict__.values() if isinstance(t, torch.Tensor)]
+        self._ptrs = [t.data_ptr() for t in self._tensors]
         self._keep = ([c.struct() for c in caches], [x.struct() for x in nodes], [s.struct() for s in scratch])
         self.caches = (C.POINTER(CCache) * n)(*[C.pointer(x) for x in self._keep[0]])
         self.nodes = (C.POINTER(CNodes) * n)(*[C.pointer(x) for x in self._keep[1]])
         self.scratch = (C.POINTER(CScratch) * n)(*[C.pointer(x) for x in self._keep[2]])
+
+
+    def current(self, caches: List[LayerCache], nodes: List[NodeInputs], scratch: List[Scratch]) -> bool:
+        """Whether the arrays still describe these objects: the same ones, no field assigned since, no tensor's storage
+        exchanged in place."""
+        objs = (*caches, *nodes, *scratch)
+        return (self._version == sum([x._version for x in objs]) and self._ids == [id(x) for x in objs]
+                and self._ptrs == [t.data_ptr() for t in self._tensors])
+
+
+_lib.tsv_verify_cycle.restype = C.c_int
+_lib.tsv_verify_cycle.argtypes = [C.POINTER(CShape), C.c_int32, C.POINTER(C.POINTER(CCache)), C.POINTER(C.POINTER(CNodes)),
+                                  C.POINTER(C.POINTER(CScratch)), C.POINTER(_p), C.POINTER(_p), _p, C.c_size_t, _p, _p, _p, _p, _p, _p, _p]
+
+
+def verify_cycle(shape: CShape, pack: LayerPack, out: Optional[List[torch.Tensor]], topk_idx: List[Optional[torch.Tensor]],
+                 workspace: torch.Tensor, refresh, status: torch.Tensor, stream=None) -> None:
+    """One whole cycle in ONE call (an export of the library outside its public header): status cleared, per layer
+    branch_state_build and (out given) tree_verify_attn, then (refresh = draft, target, accept_len, accept_path, bonus given)
+    accept_and_refresh.  The same kernels in the same order as the separate calls."""
+    n = pack.n
+    wp, wn = _aligned(workspace)
+    outs = (_p * n)(*[t.data_ptr() for t in out]) if out is not None else None
+    topk = (_p * n)(*[_ptr(t) for t in topk_idx]) if any(t is not None for t in topk_idx) else None
+    rf = [t.data_ptr() for t in refresh] if refresh is not None else [None] * 5
+    r = _lib.tsv_verify_cycle(C.byref(shape), n, pack.caches, pack.nodes, pack.scratch, outs, topk, wp, wn, *rf, _ptr(status), _stream(stream))
+    if r:
+        raise TsvError(r, "tsv_verify_cycle")
 
 
 def accept_and_refresh(shape: CShape, pack: LayerPack, draft_tok: torch.Tensor, target_tok: torch.Tensor,

@@ -209,7 +209,7 @@ int branch_state_build(const tsv_shape* shape, const tsv_cache* cache, const tsv
   if (!shape_ok(shape)) return TSV_ERR_SHAPE;
   int r;
   if ((r = check_cache(cache, shape)) || (r = check_nodes(nodes, false)) || (r = check_scratch(scratch))) return r;
-  return launch_bsb(resolved(shape), *cache, *nodes, *scratch, status, (cudaStream_t)stream);
+  return launch_bsb(resolved(shape), *cache, *nodes, *scratch, status, false, (cudaStream_t)stream);
 }
 
 int tree_verify_attn(const tsv_shape* shape, const tsv_cache* cache, const tsv_nodes* nodes, const tsv_scratch* scratch,
@@ -258,6 +258,40 @@ int accept_and_refresh(const tsv_shape* shape, int32_t n_layers, const tsv_cache
     if ((r = check_cache(caches[l], shape)) || (r = check_nodes(nodes[l], false)) || (r = check_scratch(scratch[l]))) return r;
   return launch_aar(resolved(shape), n_layers, caches, nodes, scratch, nodes[0]->parent, nodes[0]->n_nodes, draft_tok, target_tok, accept_len,
                     accept_path, bonus_tok, status, (cudaStream_t)stream);
+}
+
+// Not part of the public interface (not declared in tsv.h): a whole cycle in one call, for a host loop that launches eagerly.
+// Clears `status` (the first layer's state build writes it), then per layer branch_state_build and, unless `out` is NULL,
+// tree_verify_attn, then, unless `draft_tok` is NULL, accept_and_refresh: the kernels of the separate calls in their order.
+// out / topk_idx: HOST arrays of n_layers device pointers (topk_idx, or its entries, may be NULL).
+int tsv_verify_cycle(const tsv_shape* shape, int32_t n_layers, const tsv_cache* const* caches, const tsv_nodes* const* nodes,
+                     const tsv_scratch* const* scratch, void* const* out, int32_t* const* topk_idx, void* workspace, size_t workspace_bytes,
+                     const int32_t* draft_tok, const int32_t* target_tok, int32_t* accept_len, int32_t* accept_path, int32_t* bonus_tok,
+                     int32_t* status, void* stream) {
+  if (!shape || !caches || !nodes || !scratch || !status) return TSV_ERR_NULL;
+  if (draft_tok && (!target_tok || !accept_len || !accept_path || !bonus_tok)) return TSV_ERR_NULL;
+  if (!shape_ok(shape)) return TSV_ERR_SHAPE;
+  if (n_layers < 1 || n_layers > 4096) return TSV_ERR_SHAPE;
+  int r;
+  for (int l = 0; l < n_layers; ++l) {
+    if ((r = check_cache(caches[l], shape)) || (r = check_nodes(nodes[l], out != nullptr)) || (r = check_scratch(scratch[l]))) return r;
+    if (out && !out[l]) return TSV_ERR_NULL;
+    if (out && !al16(out[l])) return TSV_ERR_ALIGN;
+  }
+  const tsv_shape s = resolved(shape);
+  const cudaStream_t st = (cudaStream_t)stream;
+  TvaPlan p;
+  if (out) {
+    make_tva_plan(s, p);
+    if (!workspace || ((uintptr_t)workspace & 255) || workspace_bytes < p.total) return TSV_ERR_WORKSPACE;
+  }
+  for (int l = 0; l < n_layers; ++l) {
+    if ((r = launch_bsb(s, *caches[l], *nodes[l], *scratch[l], status, l == 0, st))) return r;
+    if (out && (r = tva_stages(s, p, *caches[l], *nodes[l], *scratch[l], out[l], topk_idx ? topk_idx[l] : nullptr, (char*)workspace, status, st, 3))) return r;
+  }
+  if (!draft_tok) return TSV_OK;
+  return launch_aar(s, n_layers, caches, nodes, scratch, nodes[0]->parent, nodes[0]->n_nodes, draft_tok, target_tok, accept_len, accept_path,
+                    bonus_tok, status, st);
 }
 
 }  // extern "C"

@@ -39,7 +39,7 @@ constexpr int kBsbThreads = 128;
 // DEFER: the C128-deferred schedule is on (a separate instantiation, so that the timely schedule's code is untouched by it)
 template <typename T, int DMAX, bool DEFER>
 __global__ void __launch_bounds__(kBsbThreads) bsb_kernel(const tsv_shape s, const tsv_cache c, const tsv_nodes nd,
-                                                          const tsv_scratch sc, int32_t* __restrict__ status) {
+                                                          const tsv_scratch sc, int32_t* __restrict__ status, const bool reset_status) {
   extern __shared__ float hist[];                      // [D][kBsbThreads] post-fold value of this thread's element per node
   __shared__ TreeMeta tm;
   __shared__ TreeStage tstage;
@@ -74,7 +74,10 @@ __global__ void __launch_bounds__(kBsbThreads) bsb_kernel(const tsv_shape s, con
   const bool hdef = DEFER && hca_deferred(s, tm.L) && !tm.status;     // (tm.L is 0 for a flagged length: such a sequence commits nothing)
   if (chain < 2) {
     const bool writer = blockIdx.y == 0;
-    if (tm.status && writer && threadIdx.x == 0) atomicOr(status + b, tm.status);
+    if (writer && threadIdx.x == 0) {
+      // (a selection CTA that runs early may have or-ed in what it found: the same bits)
+      if (reset_status) status[b] = tm.status; else if (tm.status) atomicOr(status + b, tm.status);
+    }
     const int nn = tm.status ? 0 : tm.nn, n = lane;
     const bool valid = n < nn;
     const int depth = valid ? tm.depth[n] : -1, par = valid && n ? tm.parent[n] : 0;
@@ -133,7 +136,7 @@ __global__ void __launch_bounds__(kBsbThreads) bsb_kernel(const tsv_shape s, con
   }
 }
 
-int launch_bsb(const tsv_shape& s, const tsv_cache& c, const tsv_nodes& nd, const tsv_scratch& sc, int32_t* status, cudaStream_t st) {
+int launch_bsb(const tsv_shape& s, const tsv_cache& c, const tsv_nodes& nd, const tsv_scratch& sc, int32_t* status, bool reset_status, cudaStream_t st) {
   const int elems = 2 * s.d + s.di;
   const dim3 grid(s.B, (elems + kBsbThreads - 1) / kBsbThreads);
   const size_t sm = (size_t)s.D * kBsbThreads * sizeof(float);
@@ -141,7 +144,7 @@ int launch_bsb(const tsv_shape& s, const tsv_cache& c, const tsv_nodes& nd, cons
 #define TSV_BSB_LAUNCH(T_, DM_, DF_)                                              \
   do {                                                                            \
     TSV_PREP((bsb_kernel<T_, DM_, DF_>));                                         \
-    bsb_kernel<T_, DM_, DF_><<<grid, kBsbThreads, sm, st>>>(s, c, nd, sc, status); \
+    bsb_kernel<T_, DM_, DF_><<<grid, kBsbThreads, sm, st>>>(s, c, nd, sc, status, reset_status); \
   } while (0)
   if (small) {
     if (bf) { if (defer) TSV_BSB_LAUNCH(bf16, 8, true); else TSV_BSB_LAUNCH(bf16, 8, false); }

@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(kItThreads) idx_score_tc_kernel(const tsv_shap
 template <int HI>
 void launch_hi(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, const tsv_nodes& nd, const tsv_scratch& sc, char* ws,
                int32_t* status, cudaStream_t st) {
-  cudaFuncSetAttribute(idx_score_tc_kernel<HI>, cudaFuncAttributeMaxDynamicSharedMemorySize, kItSmem);
+  ensure_smem((const void*)idx_score_tc_kernel<HI>, kItSmem);
   TSV_PREP(idx_score_tc_kernel<HI>);
   const int pref_cap = (int)(s.max_L / s.m_csa);
   const dim3 grid((pref_cap + kTilesPerCta * kItRows - 1) / (kTilesPerCta * kItRows), s.B);

@@ -61,7 +61,8 @@ struct TvaPlan {
 constexpr int kPairsFor = 74;         // SM pairs the splitting of few tiles aims at (a B200 holds 74)
 bool make_tva_plan(const tsv_shape& s, TvaPlan& p);
 
-int launch_bsb(const tsv_shape& s, const tsv_cache& c, const tsv_nodes& nd, const tsv_scratch& sc, int32_t* status, cudaStream_t st);
+// reset_status: status is written (0 for a usable sequence) instead of or-ed into
+int launch_bsb(const tsv_shape& s, const tsv_cache& c, const tsv_nodes& nd, const tsv_scratch& sc, int32_t* status, bool reset_status, cudaStream_t st);
 int launch_aar(const tsv_shape& s, int n_layers, const tsv_cache* const* caches, const tsv_nodes* const* nodes,
                const tsv_scratch* const* scratch, const int32_t* parent, const int32_t* n_nodes,
                const int32_t* draft, const int32_t* target, int32_t* accept_len, int32_t* accept_path,
@@ -98,7 +99,7 @@ bool tva_tc_pair_usable(const tsv_cache& c);
 // Host-side preparation of the tensor-core attention path: everything that can fail on the host (tensor maps, kernel
 // attributes) is done here, before any kernel of the call is enqueued.
 struct TvaTcPrep {
-  alignas(64) unsigned char maps[20 * 128];   // the paired kernel's tensor maps (a CUtensorMap is 128 bytes)
+  const void* maps;     // the paired kernel's tensor maps (kept by the calling thread; copied into the launch's parameters)
 };
 int prepare_tva_tc_pair(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, const tsv_nodes& nd, void* out, char* ws, TvaTcPrep& prep);
 // general: gathered tiles or tiles of more than two chunks may occur (else the instantiation without that code runs)

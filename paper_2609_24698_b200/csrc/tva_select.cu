@@ -556,11 +556,11 @@ int launch_tva_select(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, 
       count_launch();
     } else if (grid.x > 0) {
       if (bf) {
-        cudaFuncSetAttribute(idx_score_kernel<bf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        ensure_smem((const void*)idx_score_kernel<bf16>, (int)sm);
         TSV_PREP(idx_score_kernel<bf16>);
         idx_score_kernel<bf16><<<grid, 256, sm, st>>>(s, p, c, nd, sc, ws);
       } else {
-        cudaFuncSetAttribute(idx_score_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        ensure_smem((const void*)idx_score_kernel<float>, (int)sm);
         TSV_PREP(idx_score_kernel<float>);
         idx_score_kernel<float><<<grid, 256, sm, st>>>(s, p, c, nd, sc, ws);
       }
@@ -575,7 +575,7 @@ int launch_tva_select(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, 
 #define TSV_TOPK_LAUNCH(T_, PG_)                                                                                        \
   do {                                                                                                                  \
     TSV_PREP((topk_kernel<T_, PG_>));                                                                                   \
-    if (sm2 > 48 * 1024) cudaFuncSetAttribute(topk_kernel<T_, PG_>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2); \
+    if (sm2 > 48 * 1024) ensure_smem((const void*)topk_kernel<T_, PG_>, (int)sm2); \
     topk_kernel<T_, PG_><<<g2, 256, sm2, st>>>(s, p, c, nd, sc, topk_idx, ws, status);                                  \
   } while (0)
   if (bf) { if (paged) TSV_TOPK_LAUNCH(bf16, true); else TSV_TOPK_LAUNCH(bf16, false); }

@@ -256,7 +256,7 @@ static int launch_one(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, 
   constexpr int V = Vec<T>::N;
   const int hgroups = (s.H + kHeadsPerCta - 1) / kHeadsPerCta;
   const size_t sm = ((size_t)kHeadsPerCta * s.d + (size_t)kKeyTile * (s.d + V)) * sizeof(T) + kHeadsPerCta * kKeyTile * sizeof(float);
-  if (cudaFuncSetAttribute(attn_simt_kernel<T, NCH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess) return TSV_ERR_CUDA;
+  if (!ensure_smem((const void*)attn_simt_kernel<T, NCH>, (int)sm)) return TSV_ERR_CUDA;
   dim3 grid(p.nsplit, s.D * hgroups, s.B);
   TSV_PREP((attn_simt_kernel<T, NCH>));
   TSV_PREP(attn_combine_kernel<T>);

@@ -549,12 +549,9 @@ static bool gathered_tiles_possible(const tsv_shape& s, const TvaPlan& p, const 
 // Host-side work of the tensor-core path that can fail, before anything of the call is enqueued.
 int prepare_tva_tc(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, const tsv_nodes& nd, void* out, char* ws, TvaTcPrep& prep) {
   const size_t plan_sm = plan_smem_bytes(p);
-  if (plan_sm > 32 * 1024 && (cudaFuncSetAttribute(tc_plan_kernel<true, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan_sm) != cudaSuccess ||
-                              cudaFuncSetAttribute(tc_plan_kernel<true, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan_sm) != cudaSuccess ||
-                              cudaFuncSetAttribute(tc_plan_kernel<false, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan_sm) != cudaSuccess)) {
-    cudaGetLastError();
+  if (plan_sm > 32 * 1024 && !(ensure_smem((const void*)tc_plan_kernel<true, 1024>, (int)plan_sm) && ensure_smem((const void*)tc_plan_kernel<true, 256>, (int)plan_sm) &&
+                               ensure_smem((const void*)tc_plan_kernel<false, 256>, (int)plan_sm)))
     return TSV_ERR_CUDA;
-  }
   TSV_PREP((tc_plan_kernel<true, 1024>));
   TSV_PREP((tc_plan_kernel<true, 256>));
   TSV_PREP((tc_plan_kernel<false, 256>));

@@ -143,21 +143,14 @@ class VerifyEngine:
 
     def _pack(self, inp: InputSet) -> tsv.LayerPack:
         p = self._packs.get(inp)
-        if p is None:
+        if p is None or not p.current(self.caches, inp.layers, self.scratch):
             p = self._packs[inp] = tsv.LayerPack(self.caches, inp.layers, self.scratch)
         return p
 
     def launch_cycle(self, inp: InputSet, attention: bool = True, refresh: bool = True) -> None:
         """Enqueue one verify cycle on the current stream (no host sync)."""
-        self.status.zero_()
-        for l in range(self.n_layers):
-            tsv.branch_state_build(self.cshape, self.caches[l], inp.layers[l], self.scratch[l], self.status)
-            if attention:
-                tsv.tree_verify_attn(self.cshape, self.caches[l], inp.layers[l], self.scratch[l], self.out[l], self.topk_idx[l],
-                                     self.workspace, self.status)
-        if refresh:
-            tsv.accept_and_refresh(self.cshape, self._pack(inp), inp.draft, inp.target, self.accept_len, self.accept_path,
-                                   self.bonus, self.status)
+        tsv.verify_cycle(self.cshape, self._pack(inp), self.out if attention else None, self.topk_idx, self.workspace,
+                         (inp.draft, inp.target, self.accept_len, self.accept_path, self.bonus) if refresh else None, self.status)
 
     def capture(self, inp: InputSet) -> torch.cuda.CUDAGraph:
         """Capture one cycle over `inp` into a CUDA graph (the launch sequence is shape-stable)."""
