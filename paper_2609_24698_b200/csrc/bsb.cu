@@ -45,6 +45,9 @@ __global__ void __launch_bounds__(kBsbThreads) bsb_kernel(const tsv_shape s, con
   __shared__ TreeStage tstage;
   __shared__ FoldCoef fcs[TSV_MAX_D], fhs[TSV_MAX_D];
   const int b = blockIdx.x, D = s.D;
+  // Launched as a programmatic dependent (its CTAs take their places as those of the kernel before leave); waits before it reads or
+  // signals anything, so nothing of this call starts before what came earlier on the stream is complete.
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the selection may start the part of it that does not read this kernel's results
   const int d = s.d, di = s.di;
   const int e = blockIdx.y * kBsbThreads + threadIdx.x;   // element index: [0,d) CSA kv | [d,d+di) CSA indexer key | [d+di,2d+di) HCA kv
@@ -141,10 +144,16 @@ int launch_bsb(const tsv_shape& s, const tsv_cache& c, const tsv_nodes& nd, cons
   const dim3 grid(s.B, (elems + kBsbThreads - 1) / kBsbThreads);
   const size_t sm = (size_t)s.D * kBsbThreads * sizeof(float);
   const bool defer = (s.flags & TSV_FLAG_HCA_DEFERRED) != 0, bf = s.dtype == TSV_BF16, small = s.D <= 8;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = dim3(kBsbThreads, 1, 1); cfg.dynamicSmemBytes = sm; cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
 #define TSV_BSB_LAUNCH(T_, DM_, DF_)                                              \
   do {                                                                            \
     TSV_PREP((bsb_kernel<T_, DM_, DF_>));                                         \
-    bsb_kernel<T_, DM_, DF_><<<grid, kBsbThreads, sm, st>>>(s, c, nd, sc, status, reset_status); \
+    cudaLaunchKernelEx(&cfg, bsb_kernel<T_, DM_, DF_>, s, c, nd, sc, status, reset_status);  \
   } while (0)
   if (small) {
     if (bf) { if (defer) TSV_BSB_LAUNCH(bf16, 8, true); else TSV_BSB_LAUNCH(bf16, 8, false); }
