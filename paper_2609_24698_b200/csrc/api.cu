@@ -170,6 +170,7 @@ static int tva_stages(const tsv_shape& s, const TvaPlan& p_in, const tsv_cache& 
   if ((stages & 1) && (r = launch_tva_select(s, p, c, nd, sc, topk_idx, ws, status, st))) return r;
   if (!(stages & 6)) return TSV_OK;
   if (p.tc) return launch_tva_tc(s, p, prep, c, nd, sc, out, ws, status, st, (stages & 2) != 0);
+  if (tva_f32_applies(s)) return launch_tva_f32(s, p, c, nd, sc, out, ws, st);
   return launch_tva_simt(s, p, c, nd, sc, out, ws, status, st);
 }
 

@@ -86,6 +86,10 @@ int launch_topk_seq(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, co
 bool topk_long_applies(const tsv_shape& s, const TvaPlan& p);
 int launch_topk_long(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, const tsv_nodes& nd, const tsv_scratch& sc,
                      int32_t* topk_idx, char* ws, int32_t* status, cudaStream_t st);
+// fp32 storage, 128-wide rows
+bool tva_f32_applies(const tsv_shape& s);
+int launch_tva_f32(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, const tsv_nodes& nd, const tsv_scratch& sc,
+                   void* out, char* ws, cudaStream_t st);
 int launch_tva_simt(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, const tsv_nodes& nd, const tsv_scratch& sc,
                     void* out, char* ws, int32_t* status, cudaStream_t st);
 

@@ -1,6 +1,6 @@
-// Per-node top-k with 128-wide bf16 indexer rows and up to four indexer heads, for lists beyond the short ones.
+// Per-node top-k with 256-byte indexer rows (128 bf16 or 64 fp32) and up to four indexer heads, for lists beyond the short ones.
 //
-// Scoring (both forms): a warp scores sixteen entries at a time for eight nodes and all heads by tensor-core products (16
+// Scoring (both forms; fp32 storage below): a warp scores sixteen entries at a time for eight nodes and all heads by tensor-core products (16
 // entries x 32 query rows), its rows straight from global memory into the fragments: an inner product does not care for the
 // order of its terms, so lane tq of a row's four takes the 16-byte pieces tq, tq + 4, ... and the queries are read the same
 // way.  An indexer row is read once per sequence (one CTA per node read it once per node, in rounds of 96 rows through
@@ -12,6 +12,9 @@
 //                     lies in its owner's shared memory.
 //   score_rows_kernel + topk_list_kernel   longer lists or larger trees: the scores over all SMs into the workspace, then a
 //                     CTA per node with its list in shared memory.
+//
+// fp32 storage (cluster form only): a lane scores one entry for all nodes and heads, its row in registers, the queries
+// broadcast from shared memory; exact fp32 products in eight interleaved partial sums per inner product.
 //
 // The selection finds the k largest by ONE histogram over equal intervals of [min, max] (the scores of a list share their high
 // bits, so radix digits of the bit pattern take four passes with colliding bins): the interval of the k-th largest holds few
@@ -26,7 +29,8 @@ namespace ssel {
 
 constexpr int CS = 8;                  // CTAs per cluster = nodes scored together
 constexpr int kSeqMax = 4096;          // longest list of the cluster form
-constexpr int DI = 128, HMAX = 4;      // indexer width, heads (query row 4 n + h, absent ones zero)
+constexpr int DI = 128, HMAX = 4;      // indexer width (bf16), heads (query row 4 n + h, absent ones zero)
+constexpr int ROWB = 256;              // bytes of an indexer row
 constexpr int QP = 320;                // pitch of a staged query row: conflict-free 16-byte fragment loads
 constexpr int CAP = 256;               // candidates ranked against each other
 
@@ -107,10 +111,10 @@ struct Scorer {
 };
 // queries of nodes n0 .. n0 + 7 of sequence b into shared memory: row 4 (n - n0) + h; absent heads and node slots zero
 __device__ __forceinline__ void stage_queries(unsigned char* qs, const void* iq_, int b, int n0, int D, int HI) {
-  const uint4* iq = reinterpret_cast<const uint4*>(reinterpret_cast<const bf16*>(iq_) + (size_t)b * D * HI * DI);
+  const uint4* iq = reinterpret_cast<const uint4*>(reinterpret_cast<const char*>(iq_) + (size_t)b * D * HI * ROWB);
   for (int idx = threadIdx.x; idx < 32 * 16; idx += blockDim.x) {
     const int row = idx >> 4, c16 = idx & 15, n = n0 + (row >> 2), h = row & 3;
-    *reinterpret_cast<uint4*>(qs + row * QP + c16 * 16) = n < D && h < HI ? __ldg(iq + (n * HI + h) * (DI / 8) + c16) : make_uint4(0u, 0u, 0u, 0u);
+    *reinterpret_cast<uint4*>(qs + row * QP + c16 * 16) = n < D && h < HI ? __ldg(iq + (n * HI + h) * (ROWB / 16) + c16) : make_uint4(0u, 0u, 0u, 0u);
   }
 }
 // Lane j = node j: the strict ancestors of node n that close a CSA block (from their positions), root first.  One warp.
@@ -123,11 +127,13 @@ __device__ __forceinline__ void path_of(PathEntries& pe, const TreeMeta& tm, con
   if (t == 0) pe.n_newc = __popc(cm);
 }
 // Scores of the in-tree entries on node n's path (the state build's results): warp w takes entries w, w + nw, ...
+template <typename T>
 __device__ __forceinline__ void score_extras(float* extra, const PathEntries& pe, const tsv_shape& s, const tsv_nodes& nd, const tsv_scratch& sc, int b, int n) {
+  constexpr int DI = ROWB / (int)sizeof(T);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5, D = s.D, HI = s.HI;
-  const bf16* iq = reinterpret_cast<const bf16*>(nd.iq) + ((size_t)b * D + n) * HI * DI;
+  const T* iq = reinterpret_cast<const T*>(nd.iq) + ((size_t)b * D + n) * HI * DI;
   for (int i = w; i < pe.n_newc; i += nw) {
-    const bf16* ik = reinterpret_cast<const bf16*>(sc.new_csa_ik) + ((size_t)b * D + pe.newc[i]) * DI;
+    const T* ik = reinterpret_cast<const T*>(sc.new_csa_ik) + ((size_t)b * D + pe.newc[i]) * DI;
     float tot = 0.f;
     for (int h = 0; h < HI; ++h) {
       float p = 0.f;
@@ -302,12 +308,13 @@ __device__ __forceinline__ void select_node(SelectSmem<NT, NB>& sm, const float*
 }  // namespace ssel
 
 // `cap`: floats of the score list (covers the padded shares of the eight CTAs and the in-tree entries).
-template <bool PAGED>
+template <bool PAGED, typename T>
 __global__ void __launch_bounds__(128, 4) topk_seq_kernel(const tsv_shape s, const TvaPlan pl, const tsv_cache c, const tsv_nodes nd,
                                                          const tsv_scratch sc, int32_t* __restrict__ topk_user, char* __restrict__ ws,
                                                          int32_t* __restrict__ status, const int cap) {
   using namespace ssel;
   constexpr int NT = 128, NB = 1024, NW = NT / 32;
+  constexpr bool BF = sizeof(T) == 2;
   extern __shared__ __align__(128) unsigned char dsm[];
   __shared__ TreeMeta tm;
   __shared__ TreeStage tstage;
@@ -337,10 +344,11 @@ __global__ void __launch_bounds__(128, 4) topk_seq_kernel(const tsv_shape s, con
   const int first = e0 + 16 * w;
   if (any_rank) {
     if (PAGED) sco.rows = csa_rows_of(c, s, b); else { sco.rows.pt = nullptr; sco.rows.per_page = 1; sco.rows.row0 = c.csa_row0[b]; }
-    sco.ikb = reinterpret_cast<const char*>(c.csa_ik) + (size_t)sco.rows.row0 * (DI * 2) + sco.tq * 16;
-    if (first < e1) sco.fetch<PAGED>(first, alo, ahi);
+    sco.ikb = reinterpret_cast<const char*>(c.csa_ik) + (size_t)sco.rows.row0 * ROWB + (BF ? sco.tq * 16 : 0);
+    if (BF && first < e1) sco.template fetch<PAGED>(first, alo, ahi);
     stage_queries(dsm, nd.iq, b, 0, D, HI);
-    sco.weights(nd.iw + (size_t)b * D * HI, 0, D, HI);
+    if (BF) sco.weights(nd.iw + (size_t)b * D * HI, 0, D, HI);
+    else if (t < 32) reinterpret_cast<float*>(dsm + lay.loc)[t] = (t >> 2) < D && (t & 3) < HI ? __ldg(nd.iw + ((size_t)b * D + (t >> 2)) * HI + (t & 3)) : 0.f;
     for (int i = t; i < (cap + 31) / 32; i += NT) bits[i] = 0u;
     for (int i = t; i < NB; i += NT) sm.hist[i] = 0;
     if (t == 0) sm.cnt = 0;
@@ -355,10 +363,11 @@ __global__ void __launch_bounds__(128, 4) topk_seq_kernel(const tsv_shape s, con
   // (a sequence flagged for its tree is scored too -- its rows exist -- and then dropped)
   if (any_rank) {
     cluster_wait();                                      // the peers run
+    if constexpr (BF) {
     for (int e = first; e < e1; e += 16 * NW) {
       uint4 nlo[4], nhi[4];
       const bool more = e + 16 * NW < e1;
-      if (more) sco.fetch<PAGED>(e + 16 * NW, nlo, nhi);
+      if (more) sco.template fetch<PAGED>(e + 16 * NW, nlo, nhi);
       sco.score(alo, ahi, dsm, loc);
       // lane l: four entries of node l / 4 (up to three past the end of the list: overwritten below or never read)
       const float4 v = *reinterpret_cast<const float4*>(loc + 4 * lane);
@@ -370,11 +379,38 @@ __global__ void __launch_bounds__(128, 4) topk_seq_kernel(const tsv_shape s, con
         for (int q = 0; q < 4; ++q) { alo[q] = nlo[q]; ahi[q] = nhi[q]; }
       }
     }
+    } else {
+      const float* iws = reinterpret_cast<const float*>(dsm + lay.loc);
+      for (int e = e0 + 32 * w + lane; e < e1; e += 32 * NW) {
+        const float4* row = reinterpret_cast<const float4*>(sco.ikb + (size_t)(PAGED ? sco.rows.rel(e) : (int64_t)e) * ROWB);
+        float4 r[16];
+#pragma unroll
+        for (int x = 0; x < 16; ++x) r[x] = __ldg(row + x);
+#pragma unroll 1
+        for (int n = 0; n < D; ++n) {
+          float tot = 0.f;
+#pragma unroll 1
+          for (int h = 0; h < HI; ++h) {
+            const float4* q = reinterpret_cast<const float4*>(dsm + (4 * n + h) * QP);
+            float p[8];
+#pragma unroll
+            for (int x = 0; x < 8; ++x) {               // partial sum x: pieces x and x + 8 of the row
+              const float4 a = q[x], c2 = q[x + 8];
+              p[x] = fmaf(a.w, r[x].w, fmaf(a.z, r[x].z, fmaf(a.y, r[x].y, a.x * r[x].x)));
+              p[x] = fmaf(c2.w, r[x + 8].w, fmaf(c2.z, r[x + 8].z, fmaf(c2.y, r[x + 8].y, fmaf(c2.x, r[x + 8].x, p[x]))));
+            }
+            const float d = ((p[0] + p[1]) + (p[2] + p[3])) + ((p[4] + p[5]) + (p[6] + p[7]));
+            tot = fmaf(iws[4 * n + h], fmaxf(d, 0.f), tot);
+          }
+          asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(map_to_rank(smem_s + lay.sc + (uint32_t)e * 4, n)), "f"(tot) : "memory");
+        }
+      }
+    }
     __syncwarp();
     cluster_arrive();                                    // this CTA's scores are on their way; awaited below
     // the state build's results: the first thing of that kernel this CTA reads (all of the above may run under its tail)
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (live) score_extras(extra, pe, s, nd, sc, b, n);
+    if (live) score_extras<T>(extra, pe, s, nd, sc, b, n);
     __syncwarp();
     cluster_wait();                                      // every peer's scores of this node are in the list; nobody touches a peer's memory from here on
   } else if (rank == 0 && b == 0) {
@@ -490,7 +526,7 @@ __global__ void __launch_bounds__(kListThreads) topk_list_kernel(const tsv_shape
 #pragma unroll
     for (int u = 0; u < 4; ++u) if (i0 + u * kListThreads < n4) reinterpret_cast<float4*>(list)[i0 + u * kListThreads] = v[u];
   }
-  score_extras(extra, pe, s, nd, sc, b, n);
+  score_extras<bf16>(extra, pe, s, nd, sc, b, n);
   __syncthreads();
   for (int i = n_csa + t; i < n_cand; i += kListThreads) list[i] = extra[i - n_csa];
   __syncthreads();
@@ -511,9 +547,10 @@ static size_t list_bytes(const TvaPlan& p) {
 // too few threads.
 static bool seq_form(const tsv_shape& s) { return s.D <= ssel::CS && s.max_L / s.m_csa <= ssel::kSeqMax; }
 
-// bf16, 128-wide indexer rows, at most four heads, lists that fit one CTA's shared memory as scores and are too long for
+// 256-byte indexer rows, at most four heads.  fp32: the cluster form's lists.  bf16: lists that fit one CTA's shared memory as scores and are too long for
 // topk_fused_kernel (which is the shorter chain while a list is three keys a thread).
 bool topk_seq_applies(const tsv_shape& s, const TvaPlan& p) {
+  if (p.need_scores && s.dtype == TSV_FP32) return s.di * 4 == ssel::ROWB && s.HI <= ssel::HMAX && seq_form(s);
   return p.need_scores && s.dtype == TSV_BF16 && s.di == ssel::DI && s.HI <= ssel::HMAX && !topk_fused_applies(s, p) &&
          (seq_form(s) || list_bytes(p) <= 200 * 1024);
 }
@@ -534,11 +571,13 @@ int launch_topk_seq(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, co
     const int bytes = (int)ssel::Layout(4, cap).total;
     cfg.numAttrs = 2;
     cfg.gridDim = dim3(ssel::CS, s.B, 1); cfg.blockDim = dim3(128, 1, 1); cfg.dynamicSmemBytes = bytes;
-    TSV_PREP(topk_seq_kernel<true>); TSV_PREP(topk_seq_kernel<false>);
-    const void* kern = c.page_table ? (const void*)topk_seq_kernel<true> : (const void*)topk_seq_kernel<false>;
-    if (bytes > 32 * 1024 && !ensure_smem(kern, bytes)) return TSV_ERR_CUDA;
-    e = c.page_table ? cudaLaunchKernelEx(&cfg, topk_seq_kernel<true>, s, p, c, nd, sc, topk_idx, ws, status, cap)
-                     : cudaLaunchKernelEx(&cfg, topk_seq_kernel<false>, s, p, c, nd, sc, topk_idx, ws, status, cap);
+    TSV_PREP((topk_seq_kernel<true, bf16>)); TSV_PREP((topk_seq_kernel<false, bf16>)); TSV_PREP((topk_seq_kernel<true, float>)); TSV_PREP((topk_seq_kernel<false, float>));
+    auto go = [&](auto kern) {
+      if (bytes > 32 * 1024 && !ensure_smem((const void*)kern, bytes)) return cudaErrorInvalidValue;
+      return cudaLaunchKernelEx(&cfg, kern, s, p, c, nd, sc, topk_idx, ws, status, cap);
+    };
+    if (s.dtype == TSV_BF16) e = c.page_table ? go(topk_seq_kernel<true, bf16>) : go(topk_seq_kernel<false, bf16>);
+    else e = c.page_table ? go(topk_seq_kernel<true, float>) : go(topk_seq_kernel<false, float>);
     count_launch();
   } else {
     const int bytes = (int)list_bytes(p);
