@@ -147,10 +147,11 @@ constexpr uint32_t OOB_BOX = 0x3FFFFF00u;   // map 0, a row beyond every tensor:
 
 // One item of work: a chunk of CL keys (pieces of 256 keys, the last may hold 128) of one 256-row tile.
 namespace pair {
+constexpr int NQ = 4, OW = tc::DH / NQ;      // the PV product is computed in NQ parts of OW columns of d
 struct Item {
   int tix, b, tile, nk, chunk, nch, CL, cbeg, cend;
   int npc;                 // S pieces
-  int NQ, OW;              // the PV product is computed in NQ parts of OW columns of d
+  bool dbl;                // two O buffers: a part is computed while the one before is read out
   bool f32;                // partial outputs are fp32
   bool gather;             // the key list is a list of row codes (array << 30 | row), not of boxes
   __device__ __forceinline__ Item(int4 r, const TvaPlan& pl, bool general) {
@@ -160,8 +161,7 @@ struct Item {
     tc::chunking_x(nk, general, pl.tc_split, pl.tc_f32, nch, CL, f32);
     cbeg = chunk * CL; cend = min(nk, cbeg + CL);
     npc = (CL + 255) / 256;
-    NQ = CL <= 512 ? 2 : 4;
-    OW = tc::DH / NQ;
+    dbl = CL <= 512;
   }
   __device__ __forceinline__ uint32_t acc_used() const { return ((1u << npc) - 1u) | (((1u << NQ) - 1u) << 3); }
   __device__ __forceinline__ uint32_t cmp_used() const { return (1u << (npc - 1)) | (npc == 3 ? 2u : 0u) | (((1u << NQ) - 1u) << 3); }
@@ -177,10 +177,11 @@ struct Item {
 // Stages per item and CTA (rank r of the pair):
 //   Q slices:  per 64-wide slice dk of d  [this CTA's 128 rows x 64 dims], fetched once, resident for all pieces
 //   K stages:  piece after piece, per slice dk  [this CTA's half of the piece's keys x 64 dims]
-//   V stages (after the last S product): CL <= 512: per half of d, per 64 keys:  [64 keys x this CTA's 128 of the half's 256 dims]
-//                                        else       per quarter of d, per 128 keys: [128 keys x this CTA's 64 of the quarter's 128 dims]
+//   V stages (after the last S product): per quarter of d, per 128 keys: [128 keys x this CTA's 64 of the quarter's 128 dims]
 // TMEM columns (per CTA, its own 128 rows).  S piece 0 -> [0,256), pieces 1 and 2 -> [256,512) (fp32); P piece pc (bf16 pairs) ->
-// [128 pc, 128 pc + 128); O: CL <= 512 in two halves of 256 columns at [256,512), else in four quarters of 128 columns at [384,512).
+// [128 pc, 128 pc + 128); O, in four quarters of 128 columns: CL <= 512 alternately at [256,384) and [384,512), so that a quarter's
+// products run while the one before is read out (halves of 256 columns left the tensor core idle for 2.4 k cycles of 31 k per
+// 512-key item), else at [384,512).
 //
 // Every barrier phase is counted by its users: each role keeps, per barrier, the parity of its next use, and a slot's
 // latest release is awaited before it is filled again, across items too.
@@ -281,8 +282,8 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
       if (r.x < 0) break;
       const Item w(r, pl, GENERAL);
       const uint32_t box = load_box(w);
-      const int CL = w.CL, NQ = w.NQ, row0 = w.tile * PR + (int)rank * BM;
-      const int vkeys = 16384 / w.OW, nvb = CL / vkeys;            // keys per V stage: 64 or 128; V stages per part
+      const int CL = w.CL, row0 = w.tile * PR + (int)rank * BM;
+      const int nvb = CL / 128;                                    // V stages per part
       const int NKST = 8 * w.npc, NVST = NQ * nvb;
       auto place = [&](int i) { const int p = g0 + i; return p >= NSV ? p - NSV : p; };      // slot of the FIFO's place i after the item's start
       auto kslot = [&](int sl) { return sl < NSV - NQS ? place(NQS + sl) : NQS + sl; };
@@ -358,22 +359,14 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
             const uint32_t slot = ring + (uint32_t)sl * SLOTP;
             const uint32_t fb_leader = map_to_rank(smem_u32(&sm.fullV[sl]), 0);
             uint4 vcode = make_uint4(0u, 0u, 0u, 0u);               // (fetched before the wait for the slot)
-            if (w.gather) vcode = codes_at(NQ == 2 ? kb * 64 + 4 * (lane & 15) : kb * 128 + 4 * lane);
+            if (w.gather) vcode = codes_at(kb * 128 + 4 * lane);
             if (lane == 0) {
               slot_wait(sm.emptyV, vcnt, vused, sl);
               if (rank == 0) mbar_expect_tx(&sm.fullV[sl], 2 * SLOTP);
             }
             __syncwarp();
-            if (w.gather) {           // NQ == 2: 16 row groups x 2 slices of 64 dims; else 32 row groups x this CTA's 64 dims
-              if (NQ == 2) tma_gather4(slot + (lane >> 4) * 8192 + (lane & 15) * 512, &maps.row[vcode.x >> 30], (part * 4 + (int)rank * 2 + (lane >> 4)) * 64, vcode, fb_leader);
-              else tma_gather4(slot + lane * 512, &maps.row[vcode.x >> 30], (part * 2 + (int)rank) * 64, vcode, fb_leader);
-            } else if (NQ == 2) {     // 64 keys x this CTA's 128 dims: key boxes i = 0..1, 64-wide slices j = 0..1
-              const int i0 = kb * (64 / kBoxRows);
-              const bool one = consecutive(i0, 2);
-              const uint32_t bx = __shfl_sync(0xffffffffu, box, one ? i0 : i0 + ((lane >> 1) & 1));
-              if (one) { if (lane < 2) tma_box2(slot + lane * 8192, &maps.src[bx >> 30][1], (part * 4 + (int)rank * 2 + lane) * 64, (int)(bx & 0x3FFFFFFFu), fb_leader); }
-              else if (lane < 4) tma_box2(slot + (lane & 1) * 8192 + (lane >> 1) * BOXB, &maps.src[bx >> 30][0], (part * 4 + (int)rank * 2 + (lane & 1)) * 64, (int)(bx & 0x3FFFFFFFu), fb_leader);
-            } else {                  // 128 keys x this CTA's 64 dims: key boxes 0..3
+            if (w.gather) tma_gather4(slot + lane * 512, &maps.row[vcode.x >> 30], (part * 2 + (int)rank) * 64, vcode, fb_leader);
+            else {                    // key boxes 0..3
               const int i0 = kb * (128 / kBoxRows);
               const bool one = consecutive(i0, 4);
               const uint32_t bx = __shfl_sync(0xffffffffu, box, one ? i0 : i0 + (lane & 3));
@@ -404,24 +397,29 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
     if (rank == 0) {
       const uint32_t idesc_k256 = make_idesc2(256, 0), idesc_k128 = make_idesc2(128, 0);
       uint32_t accb = 0, cmpb = 0, kpar = 0, vpar = 0;    // parities of the next use, per event / slot
-      int g0 = 0, pend = -1;                         // pend: the read-out event of the item before that is still to be awaited
+      int g0 = 0;
+      uint32_t pend = 0;                                  // read-out events of the item before that are still to be awaited
       uint32_t pend_par = 0;
       const bool one = elect_one();
       auto need_ev = [&](int e) { if (!fail && !mbar_wait(&sm.cmp_ev[e], (cmpb >> e) & 1u)) fail = 1; };
       // the columns [256, 512) of the item before have been read out
-      auto need_pend = [&]() { if (pend >= 0) { if (!fail && !mbar_wait(&sm.cmp_ev[pend], pend_par)) fail = 1; pend = -1; } };
+      auto need_pend = [&]() {
+#pragma unroll
+        for (int e = 3 + NQ - 2; e < 3 + NQ; ++e) if (((pend >> e) & 1u) && !fail && !mbar_wait(&sm.cmp_ev[e], (pend_par >> e) & 1u)) fail = 1;
+        pend = 0;
+      };
 #pragma unroll 1
       for (int it = 0;; ++it) {
         int4 r = next_item(it);
         r = make_int4(__shfl_sync(0xffffffffu, r.x, 0), __shfl_sync(0xffffffffu, r.y, 0), __shfl_sync(0xffffffffu, r.z, 0), __shfl_sync(0xffffffffu, r.w, 0));
         if (r.x < 0) break;
         const Item w(r, pl, GENERAL);
-        const int CL = w.CL, NQ = w.NQ, npc = w.npc, OW = w.OW, nvb = CL * OW / 16384;
-        const uint32_t OCOL = 512 - OW, idesc_v = make_idesc2(OW, 1);
+        const int CL = w.CL, npc = w.npc, nvb = CL / 128;
+        const uint32_t idesc_v = make_idesc2(OW, 1);
         // The issuing thread is the pacemaker of the tensor pipe: stages are walked with counters (no divisions), and the
         // descriptors of a stage are the slot-0 descriptor plus a multiple of the slot size (the address field counts
         // 16-byte units and cannot overflow within the ring).
-        const uint64_t dk0 = make_desc(ring, 16, 1024), dv0 = make_desc(ring, NQ == 2 ? 8192 : 16384, 1024);
+        const uint64_t dk0 = make_desc(ring, 16, 1024), dv0 = make_desc(ring, 16384, 1024);
         // S, piece after piece (the softmax of a piece runs while the tensor core works on the next one): per piece the
         // eight slices of d, Q slice from its resident slot, K stage from the ring
         auto place = [&](int i) { const int p = g0 + i; return p >= NSV ? p - NSV : p; };
@@ -451,20 +449,18 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
         sl = g0;                                           // slot of the next V stage
 #pragma unroll 1
         for (int part = 0; part < NQ; ++part) {
-          need_ev(part == 0 ? npc - 1 : 3 + part - 1);     // all of P is in TMEM / the previous part of O has been read out
+          const uint32_t ocol = tm + (w.dbl ? 256 + (part & 1) * OW : 384);
+          if (part == 0) need_ev(npc - 1);                 // all of P is in TMEM
+          else if (!w.dbl || part >= 2) need_ev(3 + part - (w.dbl ? 2 : 1));      // the part before in these columns has been read out
 #pragma unroll 1
           for (int kb = 0; kb < nvb; ++kb) {
             if (!fail && !mbar_wait(&sm.fullV[sl], (vpar >> sl) & 1u)) fail = 1;
             vpar ^= 1u << sl;
             fence_after();
             const uint64_t vd = dv0 + (uint64_t)(sl * (SLOTP >> 4));
-            if (NQ == 2) {          // per CTA: 64 keys x 128 dims = two [64 x 64] tiles
+            // per CTA: 128 keys x 64 dims = one [128 x 64] tile
 #pragma unroll
-              for (int ks = 0; ks < 4; ++ks) if (one) mma2_ts(tm + OCOL, tm + (kb >> 2) * 128 + (kb & 1) * 64 + (kb & 2) * 16 + ks * 8, vd + ks * (2048 >> 4), idesc_v, (kb | ks) != 0);
-            } else {                // per CTA: 128 keys x 64 dims = one [128 x 64] tile
-#pragma unroll
-              for (int ks = 0; ks < 8; ++ks) if (one) mma2_ts(tm + OCOL, tm + (kb >> 1) * 128 + (ks >> 2) * 64 + (kb & 1) * 32 + (ks & 3) * 8, vd + ks * (2048 >> 4), idesc_v, (kb | ks) != 0);
-            }
+            for (int ks = 0; ks < 8; ++ks) if (one) mma2_ts(ocol, tm + (kb >> 1) * 128 + (ks >> 2) * 64 + (kb & 1) * 32 + (ks & 3) * 8, vd + ks * (2048 >> 4), idesc_v, (kb | ks) != 0);
             if (one) mma2_commit(&sm.emptyV[sl]);
             if (++sl == NSV) sl = 0;
           }
@@ -472,7 +468,7 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
         }
         // P (overwritten by the next item's first piece) is free when the last part is complete
         if (!fail && !mbar_wait(&sm.acc_ev[3 + NQ - 1], (accb >> (3 + NQ - 1)) & 1u)) fail = 1;
-        pend = 3 + NQ - 1; pend_par = (cmpb >> pend) & 1u;
+        pend = (w.dbl ? 3u : 2u) << (3 + NQ - 2); pend_par = cmpb;
         accb ^= w.acc_used(); cmpb ^= w.cmp_used();
         g0 = sl;
       }
@@ -574,10 +570,9 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
     const int4 rec = next_item(it);
     if (rec.x < 0) break;
     const Item w(rec, pl, GENERAL);
-    const int b = w.b, nch = w.nch, CL = w.CL, chunk = w.chunk, npc = w.npc, NQ = w.NQ, OW = w.OW;
+    const int b = w.b, nch = w.nch, CL = w.CL, chunk = w.chunk, npc = w.npc;
     const int row0 = w.tile * PR + (int)rank * BM;   // first of this CTA's rows within the sequence
     const size_t rix = (size_t)b * 2 * pl.tc_nt + 2 * w.tile + rank;      // this CTA's 128-row tile (partials of multi-chunk tiles)
-    const uint32_t OCOL = 512 - OW;
     const uint8_t* kmask_g = reinterpret_cast<const uint8_t*>(ws + pl.off_kmask) + (size_t)w.tix * pl.tc_maxk + w.cbeg;
     float m_run = -INFINITY;                         // reference max of the row (log2 units)
     float lp[4] = {0.f, 0.f, 0.f, 0.f};              // this thread's share of the row sum, four independent chains
@@ -741,27 +736,25 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
     const bool rowok = row0 + row < rows_seq;
     const bool full_tile = row0 + BM <= rows_seq;     // whole tile inside the sequence: rows may be stored as 32-row boxes
     const float inv = l_row > 0.f ? 1.f / l_row : 0.f;
-    const int cw = OW / 2;                            // columns of the part this thread handles: 128 or 64
+    constexpr int cw = OW / 2;                        // columns of the part this thread handles
     const uint32_t stage = ring + (uint32_t)NSV * SLOTP + (uint32_t)(warp - 4) * 4096;   // this warp's tile of 32 rows x 64 columns (bf16)
     bool stored = false;
+#pragma unroll 1
     for (int part = 0; part < NQ; ++part) {
       if (!fail && !mbar_wait(&sm.acc_ev[3 + part], (accb >> (3 + part)) & 1u)) fail = 1;
       fence_after();
-      // 64 of the thread's 128 (or 64) columns at a time; when the last are in registers the MMA may overwrite the part
-#pragma unroll 1
-      for (int c0 = 0; c0 < cw; c0 += 64) {
+      do {
         uint32_t r0[32], r1[32];
-        tmem_ld32_nowait(tlane + OCOL + hh * cw + c0, r0);
-        tmem_ld32_nowait(tlane + OCOL + hh * cw + c0 + 32, r1);
+        const uint32_t ocol = tlane + (w.dbl ? 256 + (part & 1) * OW : 384) + hh * cw;
+        tmem_ld32_nowait(ocol, r0);
+        tmem_ld32_nowait(ocol + 32, r1);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
         tmem_regs_ready(r0);
         tmem_regs_ready(r1);
-        if (c0 + 64 >= cw) {
-          fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive_cluster(map_to_rank(smem_u32(&sm.cmp_ev[3 + part]), 0));
-        }
-        const int col = part * OW + hh * cw + c0;
+        fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(map_to_rank(smem_u32(&sm.cmp_ev[3 + part]), 0));   // in registers: the columns may be overwritten
+        const int col = part * OW + hh * cw;
         const bool many = GENERAL && nch > 1;
         if ((nch == 1 && full_tile) || many) {
           // stage the 32 x 64 bf16 tile in the 128-byte swizzle pattern and store it with one TMA request: into the output,
@@ -844,7 +837,7 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
                                                                       __uint_as_float(r1[v * 4 + 2]), __uint_as_float(r1[v * 4 + 3]));
           }
         }
-      }
+      } while (0);
       if (nch > 1 && part == 0 && hh == 0)
         reinterpret_cast<float2*>(ws + pl.off_tpml)[(rix * pl.tc_chmax + chunk) * BM + row] = make_float2(m_run, l_row);
     }
