@@ -23,14 +23,18 @@ namespace tsv {
 
 // ------------------------------------------------------------------------------------------------ plan
 constexpr int kRankTilesMax = 2048;                    // beyond that many tiles they keep their natural order
-// Estimated number of keys a tile of a sequence stages, from its committed length and node count alone (for tiles on the
+// Estimated length of a tile's work items: the keys it stages, from its committed length and node count alone (for tiles on the
 // contiguous-run path it is exact up to the entries closed inside the tree; only the order of the tiles depends on it).
 __device__ __forceinline__ int tile_keys_estimate(const tsv_shape& s, int L, int nn, int tile, int npt) {
   if (L < 0 || (int64_t)L + s.D > s.max_L || nn < 1 || nn > s.D || tile * npt >= nn) return 0;
   auto r32 = [](int x) { return (x + kBoxRows - 1) / kBoxRows * kBoxRows; };
   const int n_csa = L / s.m_csa, n_hca = L / s.m_hca, nh_in = n_hca <= kHcaMiscMax ? n_hca : 0, win = min(L, s.window);
-  if (n_csa <= 2 * s.topk) return r32(n_csa) + (n_hca > kHcaMiscMax ? r32(n_hca) : 0) + r32(win) + r32(nh_in + nn);
-  return min(n_csa, npt * s.topk) + n_hca + win + 3 * nn;
+  const int nk = n_csa <= 2 * s.topk ? r32(n_csa) + (n_hca > kHcaMiscMax ? r32(n_hca) : 0) + r32(win) + r32(nh_in + nn)
+                                     : min(n_csa, npt * s.topk) + n_hca + win + 3 * nn;
+  // The order is by the length of the work items (chunks), longest first: the pairs take them in that order, and an item of 600-768
+  // keys (a whole tile) taken last would leave one pair working alone (64 sequences of 1-4 k tokens: the slowest pair ended at
+  // 132 k cycles against a mean of 107 k when the order was by the tile's keys).
+  return nk <= tc::NCX ? nk : min(nk, tc::NC);
 }
 
 __device__ __forceinline__ void l2_prefetch(const void* p, uint32_t bytes) {       // (16-byte aligned, a multiple of 16 bytes)
