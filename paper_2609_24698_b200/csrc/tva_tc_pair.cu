@@ -655,6 +655,17 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
       }
       tmem_st16(tlane + pc * 128 + hh * 64 + i * 16, pk);
     };
+    // Node masks of this lane's keys of a piece, a byte per slab; fetched a piece ahead (fetched when needed they cost the chain a
+    // memory latency, 1.3 k cycles per piece after the first).
+    uint8_t km[4];
+    auto fetch_masks = [&](int pc) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int key = pc * 256 + slab_of(i) * 32 + lane;
+        km[i] = key < CL && w.cbeg + key < w.cend ? __ldg(kmask_g + key) : (uint8_t)0;
+      }
+    };
+    fetch_masks(0);
 #pragma unroll 1
     for (int pc = 0; pc < npc; ++pc) {
       const int ns = CL - pc * 256 >= 256 ? 4 : 2;   // slabs of this warp
@@ -662,12 +673,8 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
       // keys' node masks gives the word
       uint32_t vis[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int key = pc * 256 + slab_of(i) * 32 + lane;
-        vis[i] = i < ns && w.cbeg + key < w.cend ? kmask_g[key] : 0u;
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i) vis[i] = __ballot_sync(FULL, vis[i] & mybit);
+      for (int i = 0; i < 4; ++i) vis[i] = __ballot_sync(FULL, km[i] & mybit);
+      if (pc + 1 < npc) fetch_masks(pc + 1);
       if (!fail && !mbar_wait(&sm.acc_ev[pc], (accb >> pc) & 1u)) fail = 1;
       fence_after();
       const uint32_t scol = tlane + (pc == 0 ? 0 : 256);
