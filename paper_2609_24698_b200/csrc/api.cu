@@ -90,7 +90,7 @@ bool make_tva_plan(const tsv_shape& s, TvaPlan& p) {
   p.tc_nt = p.tc_maxk = p.tc_chmax = p.tc_misc_rows = 0; p.tc_split = 1; p.tc_f32 = 0;
   p.off_krow = p.off_kmask = p.off_nkeys = p.off_tpo = p.off_tpml = p.off_box = p.off_mode = p.off_misc = p.off_order = p.off_tcnt = p.off_sched = off;
   p.off_selmask = off;
-  p.mask_ld = (p.cand_cap + 15) & ~15;
+  p.mask_ld = ((p.cand_cap + 31) / 32 + 3) & ~3;
   if (p.tc) {
     tva_tc_plan_sizes(s, p);
     const size_t tiles = (size_t)s.B * p.tc_nt;
@@ -117,7 +117,7 @@ bool make_tva_plan(const tsv_shape& s, TvaPlan& p) {
     p.off_order = off; off = up256(off + tiles * 4 * sizeof(int32_t));
     p.off_tcnt = off;  off = up256(off + 2 * tiles * sizeof(int32_t));     // finished chunks per 128-row tile (paired kernel)
     p.off_sched = off; off = up256(off + 2 * sizeof(int32_t));
-    p.off_selmask = off; if (p.need_scores) off = up256(off + (size_t)s.B * s.D * p.mask_ld);
+    p.off_selmask = off; if (p.need_scores) off = up256(off + (size_t)s.B * s.D * p.mask_ld * sizeof(uint32_t));
   }
   p.total = off;
   return true;

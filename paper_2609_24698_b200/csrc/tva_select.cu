@@ -450,7 +450,7 @@ __global__ void __launch_bounds__(256) topk_kernel(const tsv_shape s, const TvaP
   }
   const uint32_t thr = sh_prefix;       // key of the k-th largest score
   const int r = sh_remaining;           // how many of the scores equal to it are taken (lowest indices)
-  uint8_t* selmask = pl.tc ? reinterpret_cast<uint8_t*>(ws + pl.off_selmask) + ((size_t)b * D + n) * pl.mask_ld : nullptr;   // the selection as a byte per candidate (for the tile plan)
+  uint32_t* selmask = pl.tc ? reinterpret_cast<uint32_t*>(ws + pl.off_selmask) + ((size_t)b * D + n) * pl.mask_ld : nullptr;   // the selection as a bit per candidate (for the tile plan)
   if (!in_regs) {
     // Long lists: warp w owns a contiguous share of the candidates (whole 128-candidate steps: a lane holds four
     // consecutive candidates of a step) and walks it twice, eight steps per round: first counting the
@@ -500,12 +500,17 @@ __global__ void __launch_bounds__(256) topk_kernel(const tsv_shape s, const TvaP
         for (int j = 0; j < 4; ++j) { pos += __popc(tkm[j] & lt); ntk += __popc(tkm[j]); }
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          if (selmask && (full || ib + j < end)) selmask[ib + j] = (uint8_t)take[j];
           if (take[j]) {
             const int i = ib + j, v = i < n_csa ? i : pe.newc_blk[i - n_csa];
             sel[pos] = v; if (usr) usr[pos] = v;
             ++pos;
           }
+        }
+        if (selmask) {                                 // eight lanes' four candidates make a word
+          uint32_t word = ((uint32_t)take[0] | (uint32_t)take[1] << 1 | (uint32_t)take[2] << 2 | (uint32_t)take[3] << 3) << (4 * (lane & 7));
+#pragma unroll
+          for (int o = 1; o < 8; o <<= 1) word |= __shfl_xor_sync(0xffffffffu, word, o);
+          if (!(lane & 7) && ib < end) selmask[ib >> 5] = word;
         }
         eq_base += neq; out_base += ntk;
       }
@@ -528,7 +533,8 @@ __global__ void __launch_bounds__(256) topk_kernel(const tsv_shape s, const TvaP
     const int eq_rank = eq_base + block_excl_scan_256(eq, wsum, tot_eq);
     const int take = gt || (eq && eq_rank < r);
     const int pos = out_base + block_excl_scan_256(take, wsum, tot_take);
-    if (selmask && i < n_cand) selmask[i] = (uint8_t)take;
+    const uint32_t tkm = __ballot_sync(0xffffffffu, take);
+    if (selmask && !(threadIdx.x & 31) && i < n_cand) selmask[i >> 5] = tkm;
     if (take) {
       const int v = i < n_csa ? i : pe.newc_blk[i - n_csa];
       sel[pos] = v; if (usr) usr[pos] = v;

@@ -165,10 +165,10 @@ struct SelectSmem {
 };
 
 // Selection of one node by the whole CTA: list (shared memory, n_cand scores, committed entries first), bits (zero).  lists: write
-// the index list; selmask: a byte per candidate for the tile plan, or null.
+// the index list; selmask: a bit per candidate for the tile plan, or null.
 template <int NT, int NB>
 __device__ __forceinline__ void select_node(SelectSmem<NT, NB>& sm, const float* list, uint32_t* bits, int n_cand, int n_csa, const PathEntries& pe, int k,
-                                            bool lists, int32_t* sel, int32_t* usr, int32_t* selcnt, uint8_t* selmask) {
+                                            bool lists, int32_t* sel, int32_t* usr, int32_t* selcnt, uint32_t* selmask) {
   constexpr int NW = NT / 32;
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   float lo = INFINITY, hi = -INFINITY;
@@ -292,9 +292,9 @@ __device__ __forceinline__ void select_node(SelectSmem<NT, NB>& sm, const float*
       take = take || (edge && eq_base + __popc(eqm & lt) < rem);
       eq_base += __popc(eqm);
     }
-    if (selmask && i < end) selmask[i] = (uint8_t)take;
+    const uint32_t tkm = __ballot_sync(0xffffffffu, take);
+    if (selmask && lane == 0) selmask[i0 >> 5] = tkm;
     if (lists) {
-      const uint32_t tkm = __ballot_sync(0xffffffffu, take);
       if (take) {
         const int p = pos + __popc(tkm & lt), val = i < n_csa ? i : pe.newc_blk[i - n_csa];
         sel[p] = val; if (usr) usr[p] = val;
@@ -428,7 +428,7 @@ __global__ void __launch_bounds__(128, 4) topk_seq_kernel(const tsv_shape s, con
   }
   for (int i = n_csa + t; i < n_cand; i += NT) list[i] = extra[i - n_csa];
   __syncthreads();
-  uint8_t* selmask = pl.tc ? reinterpret_cast<uint8_t*>(ws + pl.off_selmask) + ((size_t)b * D + n) * pl.mask_ld : nullptr;   // (for the tile plan)
+  uint32_t* selmask = pl.tc ? reinterpret_cast<uint32_t*>(ws + pl.off_selmask) + ((size_t)b * D + n) * pl.mask_ld : nullptr;   // (for the tile plan)
   select_node(sm, list, bits, n_cand, n_csa, pe, k, lists, sel, usr, selcnt, selmask);
 }
 
@@ -530,7 +530,7 @@ __global__ void __launch_bounds__(kListThreads) topk_list_kernel(const tsv_shape
   __syncthreads();
   for (int i = n_csa + t; i < n_cand; i += kListThreads) list[i] = extra[i - n_csa];
   __syncthreads();
-  uint8_t* selmask = pl.tc ? reinterpret_cast<uint8_t*>(ws + pl.off_selmask) + ((size_t)b * D + n) * pl.mask_ld : nullptr;   // (for the tile plan)
+  uint32_t* selmask = pl.tc ? reinterpret_cast<uint32_t*>(ws + pl.off_selmask) + ((size_t)b * D + n) * pl.mask_ld : nullptr;   // (for the tile plan)
   select_node(sm, list, bits, n_cand, n_csa, pe, k, lists, sel, usr, selcnt, selmask);
 }
 

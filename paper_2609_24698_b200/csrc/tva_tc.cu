@@ -6,7 +6,7 @@
 // a per-key bitmask applied to the S fragment after it is read back from tensor memory.
 //
 //   tc_plan_kernel   per (sequence, plan tile): the keys visible to at least one node of the tile, as four runs {CSA
-//                    entries, HCA entries, window ring, packed misc rows} padded to 32 rows, with a node mask per key.
+//                    entries, HCA entries, window ring, packed misc rows} padded to 32 rows, the CSA entries last, with a node mask per key.
 //                    Contiguous-run tiles (every node selects all CSA candidates, or the CSA slab is at most 2 x topk
 //                    rows): the runs as 32-row TMA boxes.  Gathered tiles (selection far from dense, or a paged pool
 //                    whose pages do not hold whole boxes): the first run holds only the entries some node of the tile
@@ -43,14 +43,16 @@ __device__ __forceinline__ void l2_prefetch(const void* p, uint32_t bytes) {    
 
 // GENERAL: gathered tiles may occur (see gathered_tiles_possible); the instantiation without them keeps the short
 // latency chain of the contiguous-run plan.
-template <bool GENERAL>
+template <bool GENERAL, int PARTS>
 __device__ __forceinline__ void tc_plan_tile(const tsv_shape& s, const TvaPlan& pl, const tsv_cache& c, const tsv_nodes& nd,
-                                             const tsv_scratch& sc, char* __restrict__ ws, uint8_t* cmask, int* est, int* ahead_sm) {
+                                             const tsv_scratch& sc, char* __restrict__ ws, uint32_t* words, int* est, int* ahead_sm) {
   __shared__ TreeMeta tm;
   __shared__ TreeStage tstage;
   __shared__ int n_cand[8], win_lo[8];
   __shared__ int dense;
-  const int tile = blockIdx.x, b = blockIdx.y, D = s.D, H = s.H;
+  // PARTS CTAs per tile (part 0 does everything but its share of a long list's compaction), then the packing CTA
+  const int tile = blockIdx.x / PARTS, part = PARTS > 1 ? blockIdx.x % PARTS : 0, b = blockIdx.y, D = s.D, H = s.H;
+  const bool packer = tile >= pl.tc_nt;
   const int npt = tc::PR / H, n0 = tile * npt;
   const size_t tix = (size_t)b * pl.tc_nt + tile;
   uint32_t* krow = reinterpret_cast<uint32_t*>(ws + pl.off_krow) + tix * pl.tc_maxk;    // gathered tiles: array << 30 | row per key
@@ -62,7 +64,7 @@ __device__ __forceinline__ void tc_plan_tile(const tsv_shape& s, const TvaPlan& 
   __shared__ int64_t row0_sm[2];
   // (the length and node count of "its" tile's sequence, for the ranking of the tiles: requested now, used after the tree's loads)
   const int ntile = s.B * pl.tc_nt;
-  const bool ranked_order = ntile <= kRankTilesMax && blockIdx.x < (unsigned)pl.tc_nt;
+  const bool ranked_order = ntile <= kRankTilesMax && !packer && part == 0;
   int eL = -1, enn = 0;
   if (ranked_order && (int)threadIdx.x < ntile) { eL = c.L[threadIdx.x / pl.tc_nt]; enn = nd.n_nodes[threadIdx.x / pl.tc_nt]; }
   if (threadIdx.x == 40) row0_sm[0] = c.page_table ? 0 : c.csa_row0[b];
@@ -107,8 +109,8 @@ __device__ __forceinline__ void tc_plan_tile(const tsv_shape& s, const TvaPlan& 
   csa_row.row0 = row0_sm[0]; hca_row.row0 = row0_sm[1];
   // runs of consecutive rows exist in a paged pool only where a page holds whole 32-row boxes of the layer
   const bool csa_runs = !c.page_table || (csa_row.per_page % kBoxRows == 0 && c.page_tokens % kBoxRows == 0), hca_runs = !c.page_table || hca_row.per_page % kBoxRows == 0;
-  if (blockIdx.x >= (unsigned)pl.tc_nt) {
-    // The extra CTA of the sequence (grid x = tiles + 1): rows that are small and scattered (few HCA entries, tree nodes,
+  if (packer) {
+    // The extra CTA of the sequence (the last in grid x): rows that are small and scattered (few HCA entries, tree nodes,
     // entries closed inside the tree) are packed into one contiguous per-sequence buffer so that TMA boxes can fetch
     // them.  Kept off the tile CTAs: the copy is a chain of its own (addresses, loads, stores).
     if (tm.status) return;
@@ -184,219 +186,167 @@ __device__ __forceinline__ void tc_plan_tile(const tsv_shape& s, const TvaPlan& 
     if (lane == 0) dense = over == 0;
   }
   __syncthreads();
-  if (tm.status || n0 >= tm.nn) { if (threadIdx.x == 0) leave_record(0, 1); return; }
+  if (tm.status || n0 >= tm.nn) { if (threadIdx.x == 0 && part == 0) leave_record(0, 1); return; }
   const int nvalid = min(npt, tm.nn - n0);
   const uint32_t validbits = (1u << nvalid) - 1u;
   const int n_csa = tm.n_csa;
-  // Ranked nodes: node bits per committed CSA entry (cmask) and, per node, which blocks closed inside the tree are in
-  // its selection (bit = block index - n_csa).  The selection kernel left, for every node that ranks, a byte per
-  // candidate (1 = selected): the rows of the tile's nodes are combined sixteen entries at a time (coalesced 16-byte
-  // loads; the tile CTA of a ranked sequence is on the critical path of the whole stage).
-  //
-  // Where gathered tiles may occur the array is padded by one word after every `per` entries (per: the power of two that
-  // spreads the entries over the CTA's threads): the compaction below gives a thread `per` consecutive entries, and
-  // without the padding the threads of a warp would all read the same bank.
-  __shared__ uint32_t newc_bits[8];
-  int psh = 3;                                         // log2(per)
-  if (GENERAL) while (((int)blockDim.x << psh) < n_csa) ++psh;
-  auto phys = [&](int i) { return GENERAL ? i + ((i >> psh) << 2) : i; };
-  // Contiguous-run tiles with ranking nodes (`late`): everything that does not depend on the selection -- boxes, the masks of
-  // the HCA, window and packed runs -- is written before the wait; after it only the masks of the committed CSA run (the
-  // combined mask rows, stored straight into the key masks) and of the entries closed inside the tree.
+  // Four runs of keys, each padded to whole boxes: HCA entries (when too many for the packed rows), the window ring, the packed
+  // rows, and last the committed CSA entries, the only run that depends on the selection: everything else is written before the
+  // CTA waits for it.
+  //   contiguous-run tiles: every run as TMA boxes; ranked nodes still take this path while the CSA run is at most twice the
+  //     selection size: all committed entries are staged and the unselected ones are masked per node
+  //   gathered tiles (a longer CSA run, or a paged pool whose pages do not hold whole boxes): the CSA run holds only the entries
+  //     some node of the tile selected, and every key is named by its row (array << 30 | row) for four-row TMA gathers
   const bool runs_ok = !GENERAL || ((dense || n_csa <= 2 * s.topk) && csa_runs && (hca_runs || tm.n_hca <= kHcaMiscMax));
-  const bool late = !dense && runs_ok;
-  uint32_t allbits = 0, rankbits = 0;                  // nodes that take every committed entry / nodes that rank
+  if (PARTS > 1 && part && (dense || runs_ok)) return;   // (the parts share the compaction of a ranked gathered tile only)
+  uint32_t rankbits = 0;                               // nodes that rank (the others take every committed entry)
 #pragma unroll 1
-  for (int nl = 0; nl < nvalid; ++nl) { if (n_cand[nl] <= s.topk) allbits |= 1u << nl; else rankbits |= 1u << nl; }
-  const uint8_t* mrow = reinterpret_cast<const uint8_t*>(ws + pl.off_selmask) + ((size_t)b * D + n0) * pl.mask_ld;
-  // In-tree entries: candidate n_csa + o of a node is the block closed at the o-th of its strict ancestors that closed one.
-  // Warp nl looks at node n0 + nl, lane a at ancestor a: one load per lane, all in flight together (the caller synchronises).
-  auto fetch_newc_bits = [&]() {
-    const int nl = threadIdx.x >> 5, a = threadIdx.x & 31;
-    if (nl < 8) {
-      const uint32_t closed = __ballot_sync(0xffffffffu, a < D && cdone[a]);
-      uint32_t v = 0;
-      if (nl < nvalid && ((rankbits >> nl) & 1u)) {
-        const uint32_t up = tm.anc[n0 + nl] & closed & ((1u << (n0 + nl)) - 1u);     // strict ancestors that closed a block
-        if ((up >> a) & 1u) {
-          const int o = __popc(up & ((1u << a) - 1u));
-          const int dblk = (tm.L + tm.depth[a]) / s.m_csa - n_csa;
-          if (mrow[(size_t)nl * pl.mask_ld + n_csa + o] && dblk >= 0 && dblk < 32) v = 1u << dblk;
-        }
-      }
-      v = __reduce_or_sync(0xffffffffu, v);
-      if (a == 0) newc_bits[nl] = v;
-    }
+  for (int nl = 0; nl < nvalid; ++nl) if (n_cand[nl] > s.topk) rankbits |= 1u << nl;
+  // The selection kernel left, for every node that ranks, a bit per candidate.
+  const uint32_t* mrow = reinterpret_cast<const uint32_t*>(ws + pl.off_selmask) + ((size_t)b * D + n0) * pl.mask_ld;
+  const int nwords = (n_csa + 31) >> 5, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+  // word wi of node n0 + nl: entries [32 wi, 32 wi + 32), those that do not exist cleared
+  auto node_word = [&](int nl, int wi) -> uint32_t {
+    const int left = n_csa - 32 * wi;
+    return (((rankbits >> nl) & 1u) ? __ldcg(mrow + (size_t)nl * pl.mask_ld + wi) : 0xffffffffu) & (left >= 32 ? 0xffffffffu : (1u << left) - 1u);
   };
-  // sixteen committed entries from entry i: the node bits of each as four words of four mask bytes
-  auto combine16 = [&](int i, uint32_t acc[4]) {
-    const uint32_t all4 = 0x01010101u * allbits;
-    acc[0] = acc[1] = acc[2] = acc[3] = all4;
-#pragma unroll
-    for (int nl = 0; nl < 8; ++nl) {
-      if ((rankbits >> nl) & 1u) {
-        const uint4 v = __ldcg(reinterpret_cast<const uint4*>(mrow + (size_t)nl * pl.mask_ld + i));
-        acc[0] |= (v.x & 0x01010101u) << nl; acc[1] |= (v.y & 0x01010101u) << nl;
-        acc[2] |= (v.z & 0x01010101u) << nl; acc[3] |= (v.w & 0x01010101u) << nl;
-      }
-    }
-  };
-  if (!dense && !runs_ok) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");  // the selection's mask rows
-    fetch_newc_bits();
-    uint32_t* cm32 = reinterpret_cast<uint32_t*>(cmask);
-#pragma unroll 2
-    for (int i = 16 * threadIdx.x; i < n_csa; i += 16 * blockDim.x) {
-      uint32_t acc[4];
-      combine16(i, acc);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) cm32[phys(i + 4 * q) >> 2] = acc[q];      // (bytes past n_csa are never read)
-    }
-    __syncthreads();
-  }
-  // is the entry closed at node a (a strict ancestor of node n0 + nl) among that node's selected CSA entries?
-  auto newc_selected = [&](int nl, int a) {
-    if (n_cand[nl] <= s.topk) return true;
-    const int dblk = (tm.L + tm.depth[a]) / s.m_csa - n_csa;
-    return dblk >= 0 && dblk < 32 && ((newc_bits[nl] >> dblk) & 1u);
-  };
-  {
-    // the packed per-sequence rows (written by the sequence's extra CTA): few HCA entries, tree nodes, entries closed in the tree
-    const int nh_in = tm.n_hca <= kHcaMiscMax ? tm.n_hca : 0;
-    int ncd = 0, nhd = 0;
+  // the packed per-sequence rows (written by the sequence's extra CTA): few HCA entries, tree nodes, entries closed in the tree
+  const int nh_in = tm.n_hca <= kHcaMiscMax ? tm.n_hca : 0;
+  int ncd = 0, nhd = 0;
 #pragma unroll 1
-    for (int j = 0; j < tm.nn; ++j) { ncd += cdone[j] != 0; nhd += hdone[j] != 0; }
-    const int n_misc = nh_in + tm.nn + ncd + nhd;
-    // Ranked nodes still take the contiguous-run path while the run is at most twice the selection size: all committed
-    // entries are staged and the unselected ones are masked per node.  Beyond that (or where a paged pool's pages do not
-    // hold whole boxes) the tile is GATHERED: the same four runs, but the first holds only the committed entries some node
-    // of the tile selected, and every key is named by its row (array << 30 | row) for four-row TMA gathers.
-    int n_uni = n_csa;                                 // keys of the first run
-    __shared__ int uni_tot;
-    if (!runs_ok) {
-      // Ordered compaction of the selected entries: a thread owns `per` consecutive entries, counts its selected ones
-      // (four mask bytes per word), one block scan, then writes its rows and masks at consecutive positions.
-      __shared__ int wsum_c[33];
-      const uint32_t* cm32 = reinterpret_cast<const uint32_t*>(cmask);
-      const int per = 1 << psh, beg = min(n_csa, (int)threadIdx.x << psh), end = min(n_csa, beg + per);
-      const uint32_t* mine = cm32 + (phys(beg) >> 2);  // this thread's words (its share starts on a word: per is a multiple of 8)
-      const uint32_t dmask = dense ? validbits : 0u;   // (a dense tile comes here only from a paged pool with odd pages)
-      int cnt = 0;
-      for (int i = beg; i < end; i += 4) {
-        uint32_t w = dense ? 0x01010101u * dmask : mine[(i - beg) >> 2];
-        if (end - i < 4) w &= (1u << (8 * (end - i))) - 1u;
-        cnt += (w & 0xFFu ? 1 : 0) + (w & 0xFF00u ? 1 : 0) + (w & 0xFF0000u ? 1 : 0) + (w & 0xFF000000u ? 1 : 0);
-      }
-      int total;
-      int pos = block_excl_scan(cnt, wsum_c, total);
-      if (threadIdx.x == 0) uni_tot = total;
-      for (int i = beg; i < end; i += 4) {
-        uint32_t w = dense ? 0x01010101u * dmask : mine[(i - beg) >> 2];
-        if (end - i < 4) w &= (1u << (8 * (end - i))) - 1u;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const uint32_t m = (w >> (8 * j)) & 0xFFu;
-          if (m) { krow[pos] = (uint32_t)csa_row(i + j); kmask[pos] = (uint8_t)m; ++pos; }
-        }
-      }
-      __syncthreads();
-      n_uni = uni_tot;
-    }
-    {
+  for (int j = 0; j < tm.nn; ++j) { ncd += cdone[j] != 0; nhd += hdone[j] != 0; }
+  const int n_misc = nh_in + tm.nn + ncd + nhd;
+  // the window: the ring in slot order, or (paged pool) the positions from the 32-aligned start of the box that holds the oldest
+  // window position up to L - 1 (the positions before the window are masked like every position a node cannot see)
+  const int win_a = c.page_table ? (max(0, tm.L - s.window) & ~(kBoxRows - 1)) : 0;
+  auto r32 = [](int x) { return (x + kBoxRows - 1) / kBoxRows * kBoxRows; };
+  const int c1 = tm.n_hca > kHcaMiscMax ? tm.n_hca : 0, c2 = c.page_table ? tm.L - win_a : min(tm.L, s.window), c3 = n_misc;
+  const int k2 = r32(c1), k3 = k2 + r32(c2), k4 = k3 + r32(c3);        // first keys of the window, the packed rows, the CSA run
+  // row of key i of run g (g = 0: the whole CSA slab)
+  auto run_row = [&](int g, int i) -> int64_t {
+    return g == 0 ? csa_row(i) : g == 1 ? hca_row(i) : g == 3 ? (int64_t)b * pl.tc_misc_rows + i
+                  : c.page_table ? tok_row_of(c, s, b, win_a + i) : (int64_t)b * s.window + i;
+  };
+  auto run_of = [&](int k) { return k >= k4 ? 0 : k >= k3 ? 3 : k >= k2 ? 2 : 1; };
+  auto run_first = [&](int g) { return g == 0 ? k4 : g == 3 ? k3 : g == 2 ? k2 : 0; };
+  const int newc0 = nh_in + tm.nn;                     // first packed row of the CSA entries closed inside the tree
+  // node a that closed the ord-th CSA (HCA) block of the tree
+  auto closer = [&](const uint8_t* dn, int ord) {
+    int a = 0;
+#pragma unroll 1
+    for (int j = 0; j < tm.nn; ++j) if (dn[j]) { if (ord == 0) { a = j; break; } --ord; }
+    return a;
+  };
+  if (part == 0) {
+    const int kb = dense || runs_ok ? k4 + r32(n_csa) : k4;
+    if (runs_ok) {
       int2* box = reinterpret_cast<int2*>(ws + pl.off_box) + tix * (size_t)(pl.tc_maxk / kBoxRows);
-      // four runs, each padded to whole boxes: committed CSA entries, HCA entries (when too many for the packed rows),
-      // the window ring, the packed rows.  One pass over all keys: a thread finds the run of its key by comparison, so
-      // the runs' (short, latency-bound) mask computations overlap instead of following each other.
-      // the window: the ring in slot order, or (paged pool) the positions from the 32-aligned start of the box that holds
-      // the oldest window position up to L - 1 (the positions before the window are masked like every position a node
-      // cannot see)
-      const int win_a = c.page_table ? (max(0, tm.L - s.window) & ~(kBoxRows - 1)) : 0;
-      const int cnt[4] = {n_uni, tm.n_hca > kHcaMiscMax ? tm.n_hca : 0, c.page_table ? tm.L - win_a : min(tm.L, s.window), n_misc};
-      const int64_t start[4] = {0, 0, (int64_t)b * s.window, (int64_t)b * pl.tc_misc_rows};
-      int k0[5];                                       // first key of each run
-      k0[0] = 0;
-#pragma unroll
-      for (int g = 0; g < 4; ++g) k0[g + 1] = k0[g] + (cnt[g] + kBoxRows - 1) / kBoxRows * kBoxRows;
-      const int kb = k0[4];
-      // row of key i of run g (g >= 1, or the whole CSA slab as run 0 of a contiguous-run tile)
-      auto run_row = [&](int g, int i) -> int64_t {
-        return g == 0 ? csa_row(i) : g == 1 ? hca_row(i) : (g == 2 && c.page_table) ? tok_row_of(c, s, b, win_a + i) : start[g] + i;
-      };
-      if (runs_ok) {
-        for (int bi = threadIdx.x; bi < kb / kBoxRows; bi += blockDim.x) {
-          const int k = bi * kBoxRows;
-          const int g = k >= k0[3] ? 3 : (k >= k0[2] ? 2 : (k >= k0[1] ? 1 : 0));
-          // (a box of a cache run never crosses a page: it starts on a multiple of 32 entries and per_page is one too)
-          box[bi] = make_int2(g, (int)run_row(g, k - k0[g]));
-        }
+#pragma unroll 1
+      for (int bi = threadIdx.x; bi < kb / kBoxRows; bi += blockDim.x) {
+        const int k = bi * kBoxRows, g = run_of(k);
+        // (a box of a cache run never crosses a page: it starts on a multiple of 32 entries and per_page is one too)
+        box[bi] = make_int2(g, (int)run_row(g, k - run_first(g)));
       }
-      // (gathered tiles: the compaction above has written the keys of the first run already)
-#pragma unroll 1
-      for (int k = (runs_ok ? 0 : n_uni) + threadIdx.x; k < kb; k += blockDim.x) {
-        const int g = k >= k0[3] ? 3 : (k >= k0[2] ? 2 : (k >= k0[1] ? 1 : 0));
-        const int i = k - k0[g];
-        uint32_t m = 0;
-        if (late && (g == 0 || (g == 3 && i >= nh_in + tm.nn && i < nh_in + tm.nn + ncd))) continue;   // after the wait, below
-        if (i < cnt[g]) {
-          if (g == 0) m = validbits;                                 // (dense contiguous-run tiles only: see the loop's start and the line above)
-          else if (g == 1) m = validbits;
-          else if (g == 2) {
-            const int pos = c.page_table ? win_a + i : tm.L - 1 - ((tm.L - 1 - i) % s.window);
-#pragma unroll 1
-            for (int nl = 0; nl < nvalid; ++nl) if (pos >= win_lo[nl]) m |= 1u << nl;
-          } else if (i < nh_in) m = validbits;
-          else if (i < nh_in + tm.nn) {
-            const int j = i - nh_in;
-#pragma unroll 1
-            for (int nl = 0; nl < nvalid; ++nl) if ((tm.anc[n0 + nl] >> j) & 1u) m |= 1u << nl;
-          } else {
-            int ord = i - nh_in - tm.nn;
-            const bool isc = ord < ncd;
-            if (!isc) ord -= ncd;
-            const uint8_t* dn = isc ? cdone : hdone;
-            int a = 0;
-#pragma unroll 1
-            for (int j = 0; j < tm.nn; ++j) if (dn[j]) { if (ord == 0) { a = j; break; } --ord; }
-#pragma unroll 1
-            for (int nl = 0; nl < nvalid; ++nl)
-              if (a != n0 + nl && ((tm.anc[n0 + nl] >> a) & 1u) && (!isc || newc_selected(nl, a))) m |= 1u << nl;
-          }
-        }
-        kmask[k] = (uint8_t)m;
-        // gathered tiles: the key's row; the padding of a run repeats the run's first row (masked)
-        if (!runs_ok) krow[k] = ((uint32_t)g << 30) | (uint32_t)(cnt[g] ? run_row(g, i < cnt[g] ? i : 0) : 0);
-      }
-      if (threadIdx.x == 0) leave_record(kb, runs_ok ? 1 : 2);
-      if (late) {
-        asm volatile("griddepcontrol.wait;" ::: "memory");  // the selection's mask rows
-        fetch_newc_bits();
-        // the committed CSA run (its first key is key 0 of the tile): sixteen key masks per store; the run's padding is zero
-        uint4* km4 = reinterpret_cast<uint4*>(kmask);
-        for (int i = 16 * threadIdx.x; i < k0[1]; i += 16 * blockDim.x) {
-          uint32_t acc[4] = {0u, 0u, 0u, 0u};
-          if (i < n_csa) combine16(i, acc);             // (a mask row holds a multiple of 16 bytes that covers n_csa)
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const int left = n_csa - (i + 4 * q);
-            if (left < 4) acc[q] = left <= 0 ? 0u : acc[q] & ((1u << (8 * left)) - 1u);
-          }
-          km4[i >> 4] = make_uint4(acc[0], acc[1], acc[2], acc[3]);
-        }
-        __syncthreads();
-        // the CSA entries closed inside the tree (ncd keys of the packed run)
-        if ((int)threadIdx.x < ncd) {
-          int ord = threadIdx.x, a = 0;
-#pragma unroll 1
-          for (int j = 0; j < tm.nn; ++j) if (cdone[j]) { if (ord == 0) { a = j; break; } --ord; }
-          uint32_t m = 0;
-#pragma unroll 1
-          for (int nl = 0; nl < nvalid; ++nl)
-            if (a != n0 + nl && ((tm.anc[n0 + nl] >> a) & 1u) && newc_selected(nl, a)) m |= 1u << nl;
-          kmask[k0[3] + nh_in + tm.nn + threadIdx.x] = (uint8_t)m;
-        }
-      }
-      return;
     }
+    // One pass over all keys: a thread finds the run of its key by comparison, so the runs' (short, latency-bound) mask
+    // computations overlap instead of following each other.
+#pragma unroll 1
+    for (int k = threadIdx.x; k < (dense ? kb : k4); k += blockDim.x) {
+      const int g = run_of(k), i = k - run_first(g), cg = g == 0 ? n_csa : g == 1 ? c1 : g == 2 ? c2 : c3;
+      uint32_t m = 0;
+      if (i < cg) {
+        if (g < 2 || (g == 3 && i < nh_in)) m = validbits;
+        else if (g == 2) {
+          const int pos = c.page_table ? win_a + i : tm.L - 1 - ((tm.L - 1 - i) % s.window);
+#pragma unroll 1
+          for (int nl = 0; nl < nvalid; ++nl) if (pos >= win_lo[nl]) m |= 1u << nl;
+        } else {
+          // a tree node (visible to itself and its descendants) or an entry closed at one (to its strict descendants; a CSA
+          // entry to those that selected it: ranked tiles write these masks after the wait)
+          const bool own = i < newc0, isc = !own && i < newc0 + ncd;
+          const int a = own ? i - nh_in : isc ? closer(cdone, i - newc0) : closer(hdone, i - newc0 - ncd);
+#pragma unroll 1
+          for (int nl = 0; nl < nvalid; ++nl) if (((tm.anc[n0 + nl] >> a) & 1u) && (own || a != n0 + nl)) m |= 1u << nl;
+        }
+      }
+      if (dense || !(g == 3 && i >= newc0 && i < newc0 + ncd)) kmask[k] = (uint8_t)m;
+      // gathered tiles: the key's row; the padding of a run repeats the run's first row (masked)
+      if (!runs_ok) krow[k] = ((uint32_t)g << 30) | (uint32_t)(cg ? run_row(g, i < cg ? i : 0) : 0);
+    }
+    if ((dense || runs_ok) && threadIdx.x == 0) leave_record(kb, runs_ok ? 1 : 2);
+  }
+  if (dense) return;
+  asm volatile("griddepcontrol.wait;" ::: "memory");    // the selection's mask rows
+  // In-tree entries: candidate n_csa + o of a node is the block closed at the o-th of its strict ancestors that closed one.
+  // Thread i: the i-th closed entry of the tree, its mask over the tile's nodes.
+  if (part == 0 && (int)threadIdx.x >= (int)blockDim.x - 32 && lane < ncd) {
+    const int a = closer(cdone, lane);
+    uint32_t closed = 0, m = 0;
+#pragma unroll 1
+    for (int j = 0; j < tm.nn; ++j) closed |= (uint32_t)(cdone[j] != 0) << j;
+#pragma unroll 1
+    for (int nl = 0; nl < nvalid; ++nl) {
+      const uint32_t up = tm.anc[n0 + nl] & ((1u << (n0 + nl)) - 1u);      // strict ancestors
+      if (!((up >> a) & 1u)) continue;
+      const int cand = n_csa + __popc(up & closed & ((1u << a) - 1u));
+      if (!((rankbits >> nl) & 1u) || ((__ldcg(mrow + (size_t)nl * pl.mask_ld + (cand >> 5)) >> (cand & 31)) & 1u)) m |= 1u << nl;
+    }
+    kmask[k3 + newc0 + lane] = (uint8_t)m;
+  }
+  if (runs_ok) {
+    // the committed CSA run, a word of 32 entries per warp and step (its padding is zero): lane nl fetches node nl's word
+#pragma unroll 2
+    for (int wi = warp; wi < nwords; wi += nwarp) {
+      const uint32_t v = lane < nvalid ? node_word(lane, wi) : 0u;
+      uint32_t m = 0;
+#pragma unroll
+      for (int nl = 0; nl < 8; ++nl) m |= ((__shfl_sync(0xffffffffu, v, nl) >> lane) & 1u) << nl;
+      kmask[k4 + 32 * wi + lane] = (uint8_t)m;
+    }
+    return;
+  }
+  if (!GENERAL) return;
+  // Gathered: ordered compaction of the entries some node selected.  A thread counts those of a word of 32 entries, one block scan
+  // gives each word its place, then a warp writes a word's entries (lane = entry: consecutive places, coalesced stores).  Over
+  // long lists (PARTS > 1) several CTAs do the count each for itself and share the writing, which is bound by the issue slots of
+  // one SM (32768 entries: 22 us by one CTA).
+  __shared__ int wsum_c[33];
+  const int wld = (pl.cand_cap + 31) >> 5;             // words: [wld] place of the word's first entry, then [wld] per node
+  int* place = reinterpret_cast<int*>(words);
+  int n_uni = 0;
+#pragma unroll 1
+  for (int w0 = 0; w0 < nwords; w0 += blockDim.x) {
+    const int wi = w0 + threadIdx.x;
+    uint32_t u = 0u;
+    if (wi < nwords) {
+      uint32_t v[8];
+#pragma unroll
+      for (int nl = 0; nl < 8; ++nl) v[nl] = nl < nvalid ? node_word(nl, wi) : 0u;
+#pragma unroll
+      for (int nl = 0; nl < 8; ++nl) if (nl < nvalid) { u |= v[nl]; words[(1 + nl) * wld + wi] = v[nl]; }
+    }
+    int total;
+    const int at = block_excl_scan(__popc(u), wsum_c, total);
+    if (wi < nwords) place[wi] = n_uni + at;
+    n_uni += total;
+  }
+  if (part == 0 && threadIdx.x == 0) leave_record(k4 + r32(n_uni), 2);
+  __syncthreads();
+#pragma unroll 1
+  for (int wi = warp * PARTS + part; wi < nwords; wi += nwarp * PARTS) {
+    uint32_t m = 0;
+#pragma unroll
+    for (int nl = 0; nl < 8; ++nl) if (nl < nvalid) m |= ((words[(1 + nl) * wld + wi] >> lane) & 1u) << nl;
+    const uint32_t u = __ballot_sync(0xffffffffu, m != 0);
+    if (m) {
+      const int p = k4 + place[wi] + __popc(u & ((1u << lane) - 1u));
+      krow[p] = (uint32_t)csa_row(32 * wi + lane);
+      kmask[p] = (uint8_t)m;
+    }
+  }
+  if (part == 0 && threadIdx.x < kBoxRows) {            // the run's padding (masked)
+    const int p = k4 + n_uni + threadIdx.x;
+    if (p < k4 + r32(n_uni)) { krow[p] = (uint32_t)csa_row(0); kmask[p] = 0; }
   }
 }
 
@@ -407,25 +357,28 @@ __device__ __forceinline__ void tc_plan_tile(const tsv_shape& s, const TvaPlan& 
 // ranks is planned from the caller's inputs alone: its CTA never waits for the kernels before this one.
 // NT threads per CTA: 256, or 1024 for gathered tiles over long candidate lists (the union of a tile's selections over tens
 // of thousands of entries is the work of ONE CTA, alone on its SM).
+constexpr int kPlanParts = 8;                          // CTAs per tile over long candidate lists
 template <bool GENERAL, int NT>
 __global__ void __launch_bounds__(NT) tc_plan_kernel(const tsv_shape s, const TvaPlan pl, const tsv_cache c, const tsv_nodes nd,
                                                                          const tsv_scratch sc, char* __restrict__ ws) {
-  extern __shared__ uint8_t cmask_sm[];                // [cand_cap] node bits per committed CSA entry (ranked case only)
+  extern __shared__ uint32_t words_sm[];               // gathered tiles: per word of 32 entries its place and the nodes' selections
   __shared__ int est_sm[kRankTilesMax];
   __shared__ int ahead_sm;
-  const bool tile_cta = blockIdx.x < (unsigned)pl.tc_nt;
-  const size_t tix = (size_t)blockIdx.y * pl.tc_nt + blockIdx.x;
+  constexpr int PARTS = NT > 256 ? kPlanParts : 1;
+  const int tile = blockIdx.x / PARTS;
+  const bool tile_cta = tile < pl.tc_nt && blockIdx.x % PARTS == 0;
+  const size_t tix = (size_t)blockIdx.y * pl.tc_nt + tile;
   if (threadIdx.x == 0) ahead_sm = 0;
   if (threadIdx.x < 2 && blockIdx.x == 0 && blockIdx.y == 0) reinterpret_cast<int32_t*>(ws + pl.off_sched)[threadIdx.x] = 0;   // the attention kernel's item counters
   if (threadIdx.x < 2 && tile_cta)                      // finished-chunk counters of the tile's two 128-row halves
     reinterpret_cast<int32_t*>(ws + pl.off_tcnt)[tix * 2 + threadIdx.x] = 0;
-  tc_plan_tile<GENERAL>(s, pl, c, nd, sc, ws, cmask_sm, est_sm, &ahead_sm);
+  tc_plan_tile<GENERAL, PARTS>(s, pl, c, nd, sc, ws, words_sm, est_sm, &ahead_sm);
   // The tile's queries into L2: the pairs of the attention kernel all start at once, and the first phase of each is bound by
   // what arrives from HBM, which idles under the kernels before (first operands of 64 short sequences 10 k -> 7.5 k cycles
   // after the start, last of the first piece 18 k -> 13 k).  At the end of the CTA's own work, which is a chain of loads that
   // would queue behind these.
   if (tile_cta && threadIdx.x < 4) {
-    const int rows_seq = s.D * s.H, r0 = blockIdx.x * tc::PR, rows = min(tc::PR, rows_seq - r0), part = (rows + 3) / 4;
+    const int rows_seq = s.D * s.H, r0 = tile * tc::PR, rows = min(tc::PR, rows_seq - r0), part = (rows + 3) / 4;
     const int p0 = min(rows, (int)threadIdx.x * part), pn = min(part, rows - p0);
     if (pn > 0) l2_prefetch(reinterpret_cast<const char*>(nd.q) + ((size_t)blockIdx.y * rows_seq + r0 + p0) * (tc::DH * 2), (uint32_t)pn * (tc::DH * 2));
   }
@@ -537,7 +490,10 @@ void tva_tc_plan_sizes(const tsv_shape& s, TvaPlan& p) {
   p.tc_chmax = (p.tc_maxk + tc::NC - 1) / tc::NC;
 }
 
-static size_t plan_smem_bytes(const TvaPlan& p) { return p.need_scores ? (((size_t)p.cand_cap + 3) & ~(size_t)3) + 4 * 1024 + 16 : 0; }   // node bits per entry, cleared by words (+ the padding words)
+// (only where gathered tiles may occur)
+static size_t plan_smem_bytes(const tsv_shape& s, const TvaPlan& p, bool gathered) {
+  return gathered ? (((size_t)p.cand_cap + 31) / 32) * 4 * (1 + (size_t)(tc::PR / s.H)) : 0;
+}
 // Can the plan kernel produce a gathered tile for these capacities?  (A committed CSA run longer than twice the
 // selection size, or a paged pool whose pages do not hold whole 32-row boxes of a layer.)
 static bool gathered_tiles_possible(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c) {
@@ -552,7 +508,7 @@ static bool gathered_tiles_possible(const tsv_shape& s, const TvaPlan& p, const 
 
 // Host-side work of the tensor-core path that can fail, before anything of the call is enqueued.
 int prepare_tva_tc(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, const tsv_nodes& nd, void* out, char* ws, TvaTcPrep& prep) {
-  const size_t plan_sm = plan_smem_bytes(p);
+  const size_t plan_sm = plan_smem_bytes(s, p, gathered_tiles_possible(s, p, c));
   if (plan_sm > 32 * 1024 && !(ensure_smem((const void*)tc_plan_kernel<true, 1024>, (int)plan_sm) && ensure_smem((const void*)tc_plan_kernel<true, 256>, (int)plan_sm) &&
                                ensure_smem((const void*)tc_plan_kernel<false, 256>, (int)plan_sm)))
     return TSV_ERR_CUDA;
@@ -572,7 +528,7 @@ int launch_tva_tc(const tsv_shape& s, const TvaPlan& p_in, const TvaTcPrep& prep
   if (with_plan) {
     cudaLaunchConfig_t cfg = {};
     const bool wide = gathered && p.cand_cap > 8192;    // long candidate lists: the CTA's passes over all entries want many threads
-    cfg.gridDim = pgrid; cfg.blockDim = dim3(wide ? 1024 : 256, 1, 1); cfg.dynamicSmemBytes = plan_smem_bytes(p); cfg.stream = st;
+    cfg.gridDim = wide ? dim3(p.tc_nt * kPlanParts + 1, s.B) : pgrid; cfg.blockDim = dim3(wide ? 1024 : 256, 1, 1); cfg.dynamicSmemBytes = plan_smem_bytes(s, p, gathered); cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;        // may start under the selection kernel's tail (it waits inside)
     attr[0].val.programmaticStreamSerializationAllowed = 1;
