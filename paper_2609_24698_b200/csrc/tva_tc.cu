@@ -388,14 +388,18 @@ __global__ void __launch_bounds__(NT) tc_plan_kernel(const tsv_shape s, const Tv
 }
 
 // ------------------------------------------------------------------------------------------------ merge
-// Merge of the paired kernel's multi-chunk tiles (launched with its general instantiation): every chunk left its NORMALISED partial output (bf16) with
-// the row's (reference max, sum); the row's output is the average of the partial outputs weighted by sum * 2^(max - row max).
-// grid (128-row tiles, sequences, groups of 8 rows): a warp merges one row, a lane owns 16 consecutive columns; the chunks
-// are accumulated in order, four chunks' loads in flight.
+// Merge of the paired kernel's multi-chunk tiles (launched with its general instantiation): every chunk left its NORMALISED partial output with
+// the row's (reference max, sum); the row's output is the average of the partial outputs weighted by sum * 2^(max - row max), the
+// chunks accumulated in order.
+// grid (128-row tiles, sequences, groups of 8 * rpw rows): a warp merges rpw rows one after the other, a lane owns 16 columns as 16-byte
+// pieces of the row (coalesced).  The traffic is L2's (67 MB at 64 sequences of 1-4 k tokens), so what counts is latency: a row's (max,
+// sum) and its first four chunks are requested together (after the maxima had been reduced they cost a third latency), and a CTA
+// lives for several rows instead of starting anew for each.
 // ANY32: some tiles' partial outputs may be fp32 (else all are bf16, and the kernel keeps its registers low).
 template <bool ANY32>
-__global__ void __launch_bounds__(256) tc_combine_pair_kernel(const tsv_shape s, const TvaPlan pl, void* __restrict__ out_, const char* __restrict__ ws) {
+__global__ void __launch_bounds__(256) tc_combine_pair_kernel(const tsv_shape s, const TvaPlan pl, void* __restrict__ out_, const char* __restrict__ ws, const int rpw) {
   using namespace tc;
+  constexpr uint32_t FULL = 0xffffffffu;
   asm volatile("griddepcontrol.wait;" ::: "memory");            // launched as a programmatic dependent of the attention kernel
   const int rt = blockIdx.x, tile = rt >> 1, b = blockIdx.y;
   const size_t tix = (size_t)b * pl.tc_nt + tile, rix = (size_t)b * 2 * pl.tc_nt + rt;
@@ -407,62 +411,82 @@ __global__ void __launch_bounds__(256) tc_combine_pair_kernel(const tsv_shape s,
   chunking_x(nk, true, pl.tc_split, pl.tc_f32, nch, CL, f32);
   if (!ANY32) f32 = false;                                       // (no tile is split, so one with more than one chunk was too long for one: bf16)
   if (nch <= 1) return;                                          // the paired kernel wrote the output itself
-  const int rows_seq = s.D * s.H, row0 = rt * BM;
-  const int lane = threadIdx.x & 31, row = blockIdx.z * 8 + (threadIdx.x >> 5);
-  if (row >= BM || row0 + row >= rows_seq) return;
-  // (a chunk's bf16 tile lies at the start of the chunk's slot of BM x DH floats)
-  const uint4* po = reinterpret_cast<const uint4*>(ws + pl.off_tpo) + (rix * pl.tc_chmax * BM * (DH / 4) + (size_t)row * (DH / (f32 ? 4 : 8))) + (f32 ? 4 : 2) * lane;
-  const float2* pml = reinterpret_cast<const float2*>(ws + pl.off_tpml) + rix * pl.tc_chmax * BM + row;
-  float m = -INFINITY;
-  for (int ch = lane; ch < nch; ch += 32) { const float2 ml = pml[(size_t)ch * BM]; if (ml.y > 0.f) m = fmaxf(m, ml.x); }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  float l = 0.f, acc[16];
-#pragma unroll
-  for (int k = 0; k < 16; ++k) acc[k] = 0.f;
+  const int rows_seq = s.D * s.H, row0 = rt * BM, lane = threadIdx.x & 31;
+  const int first = blockIdx.z * 8 * rpw + (threadIdx.x >> 5), last = min(min(BM, rows_seq - row0), (int)(blockIdx.z + 1) * 8 * rpw);
+  const float2* pml = reinterpret_cast<const float2*>(ws + pl.off_tpml) + rix * pl.tc_chmax * BM;
   auto merge = [&](auto vec) {                                   // vec: 16-byte pieces of a lane's 16 columns
     constexpr int V = decltype(vec)::value;
-    for (int c0 = 0; c0 < nch; c0 += 4) {
-      float2 ml[4];
+    // (a chunk's bf16 tile lies at the start of the chunk's slot of BM x DH floats)
+    const uint4* po = reinterpret_cast<const uint4*>(ws + pl.off_tpo) + rix * pl.tc_chmax * BM * (DH / 4) + lane;
+#pragma unroll 1
+    for (int row = first; row < last; row += 8) {
+      const uint4* pr = po + (size_t)row * (DH / (V == 4 ? 4 : 8));
+      float2 x = lane < nch ? pml[(size_t)lane * BM + row] : make_float2(-INFINITY, 0.f);
       uint4 v[4][V];
+      auto fetch = [&](int c0) {
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int ch = c0 + u < nch ? c0 + u : nch - 1;
-        ml[u] = pml[(size_t)ch * BM];
+        for (int u = 0; u < 4; ++u)
+          if (c0 + u < nch) {
 #pragma unroll
-        for (int x = 0; x < V; ++x) v[u][x] = po[(size_t)ch * BM * (DH / 4) + x];
-      }
+            for (int q = 0; q < V; ++q) v[u][q] = __ldcg(pr + (size_t)(c0 + u) * BM * (DH / 4) + 32 * q);
+          }
+      };
+      fetch(0);
+      float m = x.y > 0.f ? x.x : -INFINITY;
+#pragma unroll 1
+      for (int ch = lane + 32; ch < nch; ch += 32) { const float2 y = pml[(size_t)ch * BM + row]; if (y.y > 0.f) m = fmaxf(m, y.x); }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (c0 + u >= nch || !(ml[u].y > 0.f)) continue;
-        const float w = ml[u].y * exp2f(ml[u].x - m);
-        l += w;
+      for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(FULL, m, o));
+      float wt = x.y > 0.f ? x.y * exp2f(x.x - m) : 0.f;         // lane c: weight of chunk c (of the 32 chunks at hand)
+      float l = 0.f, acc[16];
 #pragma unroll
-        for (int x = 0; x < V; ++x) {
-          const uint32_t wd[4] = {v[u][x].x, v[u][x].y, v[u][x].z, v[u][x].w};
+      for (int k = 0; k < 16; ++k) acc[k] = 0.f;
+#pragma unroll 1
+      for (int c0 = 0; c0 < nch; c0 += 4) {
+        if (c0) {
+          fetch(c0);
+          if ((c0 & 31) == 0) {                                  // (lists of more than 32 chunks)
+            x = c0 + lane < nch ? pml[(size_t)(c0 + lane) * BM + row] : make_float2(-INFINITY, 0.f);
+            wt = x.y > 0.f ? x.y * exp2f(x.x - m) : 0.f;
+          }
+        }
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            if (V == 4) acc[4 * x + k] = fmaf(__uint_as_float(wd[k]), w, acc[4 * x + k]);
-            else {
-              acc[8 * x + 2 * k] = fmaf(__uint_as_float(wd[k] << 16), w, acc[8 * x + 2 * k]);
-              acc[8 * x + 2 * k + 1] = fmaf(__uint_as_float(wd[k] & 0xFFFF0000u), w, acc[8 * x + 2 * k + 1]);
+        for (int u = 0; u < 4; ++u) {
+          const float w = __shfl_sync(FULL, wt, (c0 + u) & 31);
+          if (c0 + u >= nch) continue;
+          l += w;
+#pragma unroll
+          for (int q = 0; q < V; ++q) {
+            const uint32_t wd[4] = {v[u][q].x, v[u][q].y, v[u][q].z, v[u][q].w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              if (V == 4) acc[4 * q + k] = fmaf(__uint_as_float(wd[k]), w, acc[4 * q + k]);
+              else {
+                acc[8 * q + 2 * k] = fmaf(__uint_as_float(wd[k] << 16), w, acc[8 * q + 2 * k]);
+                acc[8 * q + 2 * k + 1] = fmaf(__uint_as_float(wd[k] & 0xFFFF0000u), w, acc[8 * q + 2 * k + 1]);
+              }
             }
           }
         }
       }
+      const float inv = l > 0.f ? 1.f / l : 0.f;
+      uint32_t o[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const __nv_bfloat162 h2 = __floats2bfloat162_rn(acc[2 * k] * inv, acc[2 * k + 1] * inv);
+        o[k] = *reinterpret_cast<const uint32_t*>(&h2);
+      }
+      bf16* orow = reinterpret_cast<bf16*>(out_) + ((size_t)b * rows_seq + row0 + row) * DH;
+      if (V == 4) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) reinterpret_cast<uint2*>(orow)[lane + 32 * q] = make_uint2(o[2 * q], o[2 * q + 1]);
+      } else {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) reinterpret_cast<uint4*>(orow)[lane + 32 * q] = make_uint4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
+      }
     }
   };
   if (ANY32 && f32) merge(std::integral_constant<int, 4>()); else merge(std::integral_constant<int, 2>());
-  const float inv = l > 0.f ? 1.f / l : 0.f;
-  uint32_t o[8];
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const __nv_bfloat162 h2 = __floats2bfloat162_rn(acc[2 * k] * inv, acc[2 * k + 1] * inv);
-    o[k] = *reinterpret_cast<const uint32_t*>(&h2);
-  }
-  uint4* orow = reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(out_) + ((size_t)b * rows_seq + row0 + row) * DH) + 2 * lane;
-  orow[0] = make_uint4(o[0], o[1], o[2], o[3]);
-  orow[1] = make_uint4(o[4], o[5], o[6], o[7]);
 }
 
 bool tva_tc_eligible(const tsv_shape& s) {
@@ -546,13 +570,16 @@ int launch_tva_tc(const tsv_shape& s, const TvaPlan& p_in, const TvaTcPrep& prep
   if (r != TSV_OK) return r;
   if (general && p.tc_chmax > 1) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2 * p.tc_nt, s.B, tc::BM / 8); cfg.blockDim = dim3(256, 1, 1); cfg.stream = st;                 // z: groups of 8 rows
+    // rows a warp takes: one while that leaves SMs idle otherwise, up to four
+    const int64_t groups = (int64_t)2 * p.tc_nt * s.B * (tc::BM / 8);
+    const int rpw = groups <= 4 * 148 ? 1 : groups <= 8 * 148 ? 2 : 4;
+    cfg.gridDim = dim3(2 * p.tc_nt, s.B, tc::BM / 8 / rpw); cfg.blockDim = dim3(256, 1, 1); cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
-    if (p.tc_split > 1 || p.tc_f32) cudaLaunchKernelEx(&cfg, tc_combine_pair_kernel<true>, s, p, out, (const char*)ws);
-    else cudaLaunchKernelEx(&cfg, tc_combine_pair_kernel<false>, s, p, out, (const char*)ws);
+    if (p.tc_split > 1 || p.tc_f32) cudaLaunchKernelEx(&cfg, tc_combine_pair_kernel<true>, s, p, out, (const char*)ws, rpw);
+    else cudaLaunchKernelEx(&cfg, tc_combine_pair_kernel<false>, s, p, out, (const char*)ws, rpw);
     count_launch();
   }
   return cudaGetLastError() == cudaSuccess ? TSV_OK : TSV_ERR_CUDA;
