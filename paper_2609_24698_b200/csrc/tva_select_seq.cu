@@ -11,7 +11,7 @@
 //                     node r) through distributed shared memory, and after one cluster barrier every node's whole list
 //                     lies in its owner's shared memory.
 //   score_rows_kernel + topk_list_kernel   longer lists or larger trees: the scores over all SMs into the workspace, then a
-//                     CTA per node with its list in shared memory.
+//                     cluster of eight CTAs per node with the list in shared memory.
 //
 // fp32 storage (cluster form only): a lane scores one entry for all nodes and heads, its row in registers, the queries
 // broadcast from shared memory; exact fp32 products in eight interleaved partial sums per inner product.
@@ -480,58 +480,224 @@ __global__ void __launch_bounds__(128) score_rows_kernel(const tsv_shape s, cons
   }
 }
 
-// Selection of one node from the score array: grid (D, B).  Dynamic shared memory: the list, a bit per candidate.
-constexpr int kListThreads = 1024, kListBins = 2048;
-__global__ void __launch_bounds__(kListThreads) topk_list_kernel(const tsv_shape s, const TvaPlan pl, const tsv_cache c, const tsv_nodes nd,
+// Selection of one node from the score array by a cluster of eight CTAs: grid (8 D, B).  A CTA keeps its share of the list in
+// shared memory; what the CTAs need of one another (extrema, histogram, the candidates of one interval) each leaves in its own
+// shared memory and pulls from the others' after a cluster barrier.  (One CTA per node took 20 us over 32768 candidates.)
+constexpr int kListThreads = 512, kListBins = 1024;
+struct ListSmem {
+  int hist[2][kListBins];                                // [0] the intervals; both: the digits of the radix passes
+  float2 ext;
+  int cnt[2];                                            // candidates; (entries certainly taken, entries equal to the threshold)
+  int eqs;
+  float cand_s[ssel::CAP];
+  int cand_i[ssel::CAP];
+  float all_s[ssel::CAP];
+  int all_i[ssel::CAP];
+  float red[2][kListThreads / 32];
+  int wsum[2][kListThreads / 32];
+  int bin, rem;
+};
+__global__ void __launch_bounds__(kListThreads, 2) topk_list_kernel(const tsv_shape s, const TvaPlan pl, const tsv_cache c, const tsv_nodes nd,
                                                                  const tsv_scratch sc, int32_t* __restrict__ topk_user, char* __restrict__ ws,
                                                                  int32_t* __restrict__ status) {
   using namespace ssel;
+  constexpr int NT = kListThreads, NW = NT / 32, NB = kListBins;
   extern __shared__ __align__(128) unsigned char dsm[];
   __shared__ TreeMeta tm;
   __shared__ TreeStage tstage;
   __shared__ PathEntries pe;
   __shared__ float extra[TSV_MAX_D];
-  __shared__ SelectSmem<kListThreads, kListBins> sm;
+  __shared__ __align__(16) ListSmem sm;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the tile plan may start its selection-independent part
-  const int t = threadIdx.x, n = blockIdx.x, b = blockIdx.y, D = s.D, k = s.topk;
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5, rank = blockIdx.x % CS, n = blockIdx.x / CS, b = blockIdx.y, D = s.D, k = s.topk;
   const bool lists = !pl.tc || topk_user;
   coop_tree_meta(tm, tstage, s, c.L + b, nd.parent + (size_t)b * D, nd.n_nodes + b, c.csa_cap + b, c.hca_cap + b);
-  if (t == 0 && n == 0 && tm.status) atomicOr(status + b, tm.status);
+  if (t == 0 && n == 0 && rank == 0 && tm.status) atomicOr(status + b, tm.status);
   const bool live = !tm.status && n < tm.nn;
   const int n_csa = tm.n_csa;
   if (t < 32) path_of(pe, tm, s, n, live);
-  for (int i = t; i < kListBins; i += kListThreads) sm.hist[i] = 0;
-  if (t == 0) sm.cnt = 0;
+  for (int i = t; i < NB; i += NT) { sm.hist[0][i] = 0; sm.hist[1][i] = 0; }
+  if (t == 0) { sm.cnt[0] = sm.cnt[1] = 0; sm.eqs = 0; }
   __syncthreads();
   int32_t* sel = reinterpret_cast<int32_t*>(ws + pl.off_sel) + ((size_t)b * D + n) * k;
   int32_t* selcnt = reinterpret_cast<int32_t*>(ws + pl.off_selcnt) + (size_t)b * D + n;
   int32_t* usr = topk_user ? topk_user + ((size_t)b * D + n) * k : nullptr;
   const int n_cand = live ? n_csa + pe.n_newc : 0;
+  // (every exit is taken by the whole cluster alike)
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // the scores, and (the scoring kernel waited) the entries closed inside the tree
   if (n_cand <= k) {
-    // (waits too: this kernel's completion implies that of the ones before)
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (lists) select_all(n_cand, n_csa, pe, k, sel, usr, selcnt);
+    if (lists && rank == 0) select_all(n_cand, n_csa, pe, k, sel, usr, selcnt);
     return;
   }
+  // this CTA's candidates [c0, c1), a multiple of 32 but for the end of the list
+  const int per = ((n_cand + CS - 1) / CS + 31) & ~31, c0 = min(n_cand, rank * per), c1 = min(n_cand, c0 + per), len = c1 - c0;
   float* list = reinterpret_cast<float*>(dsm);
-  uint32_t* bits = reinterpret_cast<uint32_t*>(dsm + (((size_t)pl.score_ld + TSV_MAX_D + 3) & ~(size_t)3) * 4);
-  for (int i = t; i < (n_cand + 31) / 32; i += kListThreads) bits[i] = 0u;
-  asm volatile("griddepcontrol.wait;" ::: "memory");   // the scores, and (the scoring kernel waited) the entries closed inside the tree
-  const float4* src = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(ws + pl.off_scores) + ((size_t)b * D + n) * pl.score_ld);
-  const int n4 = (n_csa + 3) >> 2;
-  for (int i0 = t; i0 < n4; i0 += 4 * kListThreads) {
-    float4 v[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) if (i0 + u * kListThreads < n4) v[u] = __ldcg(src + i0 + u * kListThreads);
-#pragma unroll
-    for (int u = 0; u < 4; ++u) if (i0 + u * kListThreads < n4) reinterpret_cast<float4*>(list)[i0 + u * kListThreads] = v[u];
+  uint32_t* bits = reinterpret_cast<uint32_t*>(list + (((pl.score_ld + TSV_MAX_D + CS - 1) / CS + 63) & ~31));
+  for (int i = t; i < (len + 31) / 32; i += NT) bits[i] = 0u;
+  const float4* src = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(ws + pl.off_scores) + ((size_t)b * D + n) * pl.score_ld + c0);
+  const int n4 = (min(c1, n_csa) - c0 + 3) >> 2;       // (negative: none)
+  for (int i = t; i < n4; i += NT) reinterpret_cast<float4*>(list)[i] = __ldcg(src + i);
+  if (c1 > n_csa) {
+    score_extras<bf16>(extra, pe, s, nd, sc, b, n);
+    __syncthreads();
+    for (int i = max(n_csa, c0) + t; i < c1; i += NT) list[i - c0] = extra[i - n_csa];
   }
-  score_extras<bf16>(extra, pe, s, nd, sc, b, n);
   __syncthreads();
-  for (int i = n_csa + t; i < n_cand; i += kListThreads) list[i] = extra[i - n_csa];
+  float lo = INFINITY, hi = -INFINITY;
+  for (int i = t; i < len; i += NT) { const float v = list[i]; lo = fminf(lo, v); hi = fmaxf(hi, v); }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) { lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o)); hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o)); }
+  if (lane == 0) { sm.red[0][w] = lo; sm.red[1][w] = hi; }
   __syncthreads();
+  if (t == 0) {
+    for (int i = 0; i < NW; ++i) { lo = fminf(lo, sm.red[0][i]); hi = fmaxf(hi, sm.red[1][i]); }
+    sm.ext = make_float2(lo, hi);
+  }
+  auto peer = [&](const void* p, int r) { return map_to_rank((uint32_t)__cvta_generic_to_shared(p), r); };
+  auto peer_i = [&](const int* p, int r) { int v; asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(peer(p, r))); return v; };
+  auto peer_f = [&](const float* p, int r) { float v; asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(peer(p, r))); return v; };
+  auto meet = [&]() { __syncthreads(); cluster_arrive(); cluster_wait(); };
+  meet();
+  {
+    const int r = lane & 7;
+    lo = peer_f(&sm.ext.x, r); hi = peer_f(&sm.ext.y, r);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) { lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o)); hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o)); }
+  }
+  const float scale = hi > lo ? (float)NB / (hi - lo) : 0.f;
+  const bool regular = scale > 0.f && scale < 1e30f;     // (else: all equal, not finite, or too narrow)
+  auto bin_of = [&](float v) { return min(NB - 1, (int)((v - lo) * scale)); };
+  // the interval (of nb in h, over the whole cluster) of the rem-th largest: its number, and what of rem is left in it
+  auto locate = [&](const int* h, int nb, int rem, int& bin, int& left) {
+    int v[2] = {0, 0};
+    const int hi2 = nb - 2 - 2 * t;                      // thread t: intervals nb - 1 - 2 t and nb - 2 - 2 t
+    if (hi2 >= 0) {
+      int x[CS], y[CS];
+#pragma unroll
+      for (int r = 0; r < CS; ++r) asm volatile("ld.shared::cluster.v2.s32 {%0, %1}, [%2];" : "=r"(x[r]), "=r"(y[r]) : "r"(peer(h + hi2, r)));
+#pragma unroll
+      for (int r = 0; r < CS; ++r) { v[0] += y[r]; v[1] += x[r]; }
+    }
+    int incl = v[0] + v[1];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += y; }
+    if (lane == 31) sm.wsum[0][w] = incl;
+    __syncthreads();
+#pragma unroll 1
+    for (int i = 0; i < w; ++i) incl += sm.wsum[0][i];
+    const int excl = incl - v[0] - v[1];
+    if (excl < rem && incl >= rem) {                     // exactly one thread
+      const bool first = excl + v[0] >= rem;
+      sm.bin = hi2 + (first ? 1 : 0); sm.rem = rem - excl - (first ? 0 : v[0]);
+    }
+    __syncthreads();
+    bin = sm.bin; left = sm.rem;
+  };
+  int m = CAP + 1, bstar = 0, rem = k;
+  if (regular) {
+    for (int i = t; i < len; i += NT) atomicAdd(&sm.hist[0][bin_of(list[i])], 1);
+    meet();
+    locate(sm.hist[0], NB, k, bstar, rem);
+    for (int i = t; i < len; i += NT) {
+      const float v = list[i];
+      if (bin_of(v) == bstar) { const int pos = atomicAdd(&sm.cnt[0], 1); if (pos < CAP) { sm.cand_s[pos] = v; sm.cand_i[pos] = c0 + i; } }
+    }
+    meet();
+    int base[CS + 1];
+    base[0] = 0;
+#pragma unroll
+    for (int r = 0; r < CS; ++r) base[r + 1] = base[r] + peer_i(&sm.cnt[0], r);
+    m = base[CS];
+    if (m <= CAP) {
+      for (int x = t; x < m; x += NT) {
+        int r = 0, at = x;
+#pragma unroll
+        for (int q = 1; q < CS; ++q) if (x >= base[q]) { r = q; at = x - base[q]; }
+        sm.all_s[x] = peer_f(&sm.cand_s[at], r); sm.all_i[x] = peer_i(&sm.cand_i[at], r);
+      }
+      __syncthreads();
+      const int own = sm.cnt[0];
+      for (int x = t; x < own; x += NT) {
+        const float v = sm.cand_s[x];
+        const int ix = sm.cand_i[x];
+        int r = 0;
+        for (int y = 0; y < m; ++y) { const float u = sm.all_s[y]; r += (u > v || (u == v && sm.all_i[y] < ix)) ? 1 : 0; }
+        if (r < rem) atomicOr(&bits[(ix - c0) >> 5], 1u << (ix & 31));
+      }
+      __syncthreads();
+    }
+  }
+  uint32_t thr = 0;
+  const bool radix = m > CAP;                            // (alike in the cluster)
+  if (radix) {                                           // four passes of 8 bits over the order-preserving keys
+    uint32_t mask = 0;
+    rem = k;
+    meet();                                              // (everyone has pulled the intervals)
+    for (int i = t; i < 256; i += NT) { sm.hist[0][i] = 0; sm.hist[1][i] = 0; }
+    __syncthreads();
+#pragma unroll 1
+    for (int pass = 0; pass < 4; ++pass) {
+      const int shift = 24 - 8 * pass, buf = pass & 1;
+      for (int i = t; i < len; i += NT) { const uint32_t key = order_key(list[i]); if ((key & mask) == thr) atomicAdd(&sm.hist[buf][(key >> shift) & 255u], 1); }
+      meet();
+      for (int i = t; i < 256; i += NT) sm.hist[buf ^ 1][i] = 0;       // (pulled by everyone before this barrier)
+      int bin;
+      locate(sm.hist[buf], 256, rem, bin, rem);
+      thr |= (uint32_t)bin << shift;
+      mask |= 0xFFu << shift;
+    }
+  }
+  // Warp w owns the candidates [w * part, (w + 1) * part) of the share, rows of 32.  above: certainly taken; edge (radix only): equal
+  // to the threshold, of which the first rem in index order are taken.
+  const int part = ((len + NW - 1) / NW + 31) & ~31, beg = min(len, w * part), end = min(len, beg + part);
+  auto classify = [&](int i, bool& above, bool& edge) {
+    above = edge = false;
+    if (i >= end) return;
+    const float v = list[i];
+    if (radix) { const uint32_t key = order_key(v); above = key > thr; edge = key == thr; }
+    else { const int bn = bin_of(v); above = bn > bstar || (bn == bstar && ((bits[i >> 5] >> (i & 31)) & 1u)); }
+  };
+  int pos = 0, eq_base = 0;
+  if (lists || radix) {
+    int ca = 0, ce = 0;
+    for (int i0 = beg; i0 < end; i0 += 32) {
+      bool above, edge;
+      classify(i0 + lane, above, edge);
+      ca += __popc(__ballot_sync(0xffffffffu, above)); ce += __popc(__ballot_sync(0xffffffffu, edge));
+    }
+    __syncthreads();
+    if (lane == 0) { sm.wsum[0][w] = ca; sm.wsum[1][w] = ce; }
+    __syncthreads();
+    if (t == 0) { int a = 0, e = 0; for (int i = 0; i < NW; ++i) { a += sm.wsum[0][i]; e += sm.wsum[1][i]; } sm.cnt[1] = a; sm.eqs = e; }
+    meet();
+    for (int r = 0; r < rank; ++r) { pos += peer_i(&sm.cnt[1], r); eq_base += peer_i(&sm.eqs, r); }
+    for (int i = 0; i < w; ++i) { pos += sm.wsum[0][i]; eq_base += sm.wsum[1][i]; }
+    if (radix) pos += min(rem, eq_base);
+  }
   uint32_t* selmask = pl.tc ? reinterpret_cast<uint32_t*>(ws + pl.off_selmask) + ((size_t)b * D + n) * pl.mask_ld : nullptr;   // (for the tile plan)
-  select_node(sm, list, bits, n_cand, n_csa, pe, k, lists, sel, usr, selcnt, selmask);
+  const uint32_t lt = (1u << lane) - 1u;
+  for (int i0 = beg; i0 < end; i0 += 32) {
+    const int i = i0 + lane;
+    bool take, edge;
+    classify(i, take, edge);
+    if (radix) {
+      const uint32_t eqm = __ballot_sync(0xffffffffu, edge);
+      take = take || (edge && eq_base + __popc(eqm & lt) < rem);
+      eq_base += __popc(eqm);
+    }
+    const uint32_t tkm = __ballot_sync(0xffffffffu, take);
+    if (selmask && lane == 0) selmask[(c0 + i0) >> 5] = tkm;
+    if (lists) {
+      if (take) {
+        const int p = pos + __popc(tkm & lt), val = c0 + i < n_csa ? c0 + i : pe.newc_blk[c0 + i - n_csa];
+        sel[p] = val; if (usr) usr[p] = val;
+      }
+      pos += __popc(tkm);
+    }
+  }
+  if (lists && rank == 0 && t == 0) *selcnt = k;
+  cluster_arrive();                                      // no CTA leaves while a peer may still read its memory
+  cluster_wait();
 }
 
 // ------------------------------------------------------------------------------------------------ dispatch
@@ -539,15 +705,15 @@ static int seq_cap(const tsv_shape& s) {                 // padded shares of eig
   const int ent = (int)(s.max_L / s.m_csa), share = ((ent + ssel::CS - 1) / ssel::CS + 15) & ~15;
   return (share * ssel::CS + TSV_MAX_D + 127) & ~127;
 }
-static size_t list_bytes(const TvaPlan& p) {
-  const size_t fl = ((size_t)p.score_ld + TSV_MAX_D + 3) & ~(size_t)3;
+static size_t list_bytes(const TvaPlan& p) {             // a share of the list, a bit per candidate of it
+  const size_t fl = (((size_t)p.score_ld + TSV_MAX_D + ssel::CS - 1) / ssel::CS + 63) & ~(size_t)31;
   return fl * 4 + (fl + 31) / 32 * 4;
 }
 // The cluster form: its CTAs are small and all resident up to some 70 sequences; beyond kSeqMax entries a node's list is the work of
 // too few threads.
 static bool seq_form(const tsv_shape& s) { return s.D <= ssel::CS && s.max_L / s.m_csa <= ssel::kSeqMax; }
 
-// 256-byte indexer rows, at most four heads.  fp32: the cluster form's lists.  bf16: lists that fit one CTA's shared memory as scores and are too long for
+// 256-byte indexer rows, at most four heads.  fp32: the cluster form's lists.  bf16: lists that fit the cluster's shared memory as scores and are too long for
 // topk_fused_kernel (which is the shorter chain while a list is three keys a thread).
 bool topk_seq_applies(const tsv_shape& s, const TvaPlan& p) {
   if (p.need_scores && s.dtype == TSV_FP32) return s.di * 4 == ssel::ROWB && s.HI <= ssel::HMAX && seq_form(s);
@@ -581,7 +747,7 @@ int launch_topk_seq(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, co
     count_launch();
   } else {
     const int bytes = (int)list_bytes(p);
-    if (!ensure_smem((const void*)topk_list_kernel, bytes)) return TSV_ERR_CUDA;
+    if (bytes > 24 * 1024 && !ensure_smem((const void*)topk_list_kernel, bytes)) return TSV_ERR_CUDA;
     cfg.numAttrs = 1;
     const int ent = (int)(s.max_L / s.m_csa), per = kRowSteps * 64;
     cfg.gridDim = dim3((ent + per - 1) / per, s.B, (s.D + 7) / 8); cfg.blockDim = dim3(128, 1, 1);
@@ -589,7 +755,7 @@ int launch_topk_seq(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, co
     e = c.page_table ? cudaLaunchKernelEx(&cfg, score_rows_kernel<true>, s, p, c, nd, ws) : cudaLaunchKernelEx(&cfg, score_rows_kernel<false>, s, p, c, nd, ws);
     count_launch();
     if (e != cudaSuccess) { cudaGetLastError(); return TSV_ERR_CUDA; }
-    cfg.gridDim = dim3(s.D, s.B, 1); cfg.blockDim = dim3(kListThreads, 1, 1); cfg.dynamicSmemBytes = bytes;
+    cfg.gridDim = dim3(ssel::CS * s.D, s.B, 1); cfg.blockDim = dim3(kListThreads, 1, 1); cfg.dynamicSmemBytes = bytes; cfg.numAttrs = 2;
     e = cudaLaunchKernelEx(&cfg, topk_list_kernel, s, p, c, nd, sc, topk_idx, ws, status);
     count_launch();
   }
