@@ -87,7 +87,7 @@ bool make_tva_plan(const tsv_shape& s, TvaPlan& p) {
   p.off_po = off;     if (p.nsplit > 1) off = up256(off + (size_t)s.B * s.D * s.H * p.nsplit * s.d * sizeof(float));
   p.off_pml = off;    if (p.nsplit > 1) off = up256(off + (size_t)s.B * s.D * s.H * p.nsplit * 2 * sizeof(float));
   p.tc = tva_tc_eligible(s);
-  p.tc_nt = p.tc_maxk = p.tc_chmax = p.tc_misc_rows = 0; p.tc_split = 1; p.tc_f32 = 0;
+  p.tc_nt = p.tc_maxk = p.tc_chmax = p.tc_misc_rows = 0; p.tc_split = 1; p.tc_f32 = p.tc_packed = 0;
   p.off_krow = p.off_kmask = p.off_nkeys = p.off_tpo = p.off_tpml = p.off_box = p.off_mode = p.off_misc = p.off_order = p.off_tcnt = p.off_sched = off;
   p.off_selmask = off;
   p.mask_ld = ((p.cand_cap + 31) / 32 + 3) & ~3;
@@ -210,7 +210,7 @@ int branch_state_build(const tsv_shape* shape, const tsv_cache* cache, const tsv
   if (!shape_ok(shape)) return TSV_ERR_SHAPE;
   int r;
   if ((r = check_cache(cache, shape)) || (r = check_nodes(nodes, false)) || (r = check_scratch(scratch))) return r;
-  return launch_bsb(resolved(shape), *cache, *nodes, *scratch, status, false, (cudaStream_t)stream);
+  return launch_bsb(resolved(shape), *cache, *nodes, *scratch, status, false, nullptr, 0, (cudaStream_t)stream);
 }
 
 int tree_verify_attn(const tsv_shape* shape, const tsv_cache* cache, const tsv_nodes* nodes, const tsv_scratch* scratch,
@@ -281,13 +281,15 @@ int tsv_verify_cycle(const tsv_shape* shape, int32_t n_layers, const tsv_cache* 
   }
   const tsv_shape s = resolved(shape);
   const cudaStream_t st = (cudaStream_t)stream;
-  TvaPlan p;
+  TvaPlan p = {};
   if (out) {
     make_tva_plan(s, p);
     if (!workspace || ((uintptr_t)workspace & 255) || workspace_bytes < p.total) return TSV_ERR_WORKSPACE;
   }
   for (int l = 0; l < n_layers; ++l) {
-    if ((r = launch_bsb(s, *caches[l], *nodes[l], *scratch[l], status, l == 0, st))) return r;
+    p.tc_packed = out && p.tc && tva_tc_pair_usable(*caches[l]);       // the attention that follows finds the new entries packed
+    if ((r = launch_bsb(s, *caches[l], *nodes[l], *scratch[l], status, l == 0, p.tc_packed ? (char*)workspace + p.off_misc : nullptr,
+                        p.tc_misc_rows, st))) return r;
     if (out && (r = tva_stages(s, p, *caches[l], *nodes[l], *scratch[l], out[l], topk_idx ? topk_idx[l] : nullptr, (char*)workspace, status, st, 3))) return r;
   }
   if (!draft_tok) return TSV_OK;

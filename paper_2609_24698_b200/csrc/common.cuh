@@ -127,15 +127,23 @@ __device__ inline void build_tree_meta(TreeMeta& tm, const tsv_shape& s, int32_t
 // Cooperative front end of build_tree_meta: the first threads of the CTA fetch the parent array and the per-sequence
 // scalars in parallel (one memory latency instead of a chain of dependent loads), then warp 0 derives the tree facts.
 // Must be called by all threads of the CTA (contains two barriers); needs blockDim.x >= 64.
+// In two parts for a caller that has other loads to request behind the tree's.
 struct TreeStage { int32_t parent[TSV_MAX_D]; int32_t scal[4]; };
-__device__ __forceinline__ void coop_tree_meta(TreeMeta& tm, TreeStage& st, const tsv_shape& s, const int32_t* L_b, const int32_t* parent_b,
-                                               const int32_t* nn_b, const int32_t* csa_cap_b, const int32_t* hca_cap_b) {
+struct TreeFetch { int32_t parent, scal; };             // what this thread fetched: a node's parent; a scalar of the sequence
+__device__ __forceinline__ TreeFetch fetch_tree(const tsv_shape& s, const int32_t* L_b, const int32_t* parent_b,
+                                                const int32_t* nn_b, const int32_t* csa_cap_b, const int32_t* hca_cap_b) {
   const int t = threadIdx.x;
-  if (t < s.D) st.parent[t] = parent_b[t];
-  if (t == 32) st.scal[0] = *L_b;
-  if (t == 33) st.scal[1] = *nn_b;
-  if (t == 34 && csa_cap_b) st.scal[2] = *csa_cap_b;
-  if (t == 35 && hca_cap_b) st.scal[3] = *hca_cap_b;
+  TreeFetch f = {0, 0};
+  if (t < s.D) f.parent = parent_b[t];
+  const int32_t* p = t == 32 ? L_b : t == 33 ? nn_b : t == 34 ? csa_cap_b : t == 35 ? hca_cap_b : nullptr;
+  if (p) f.scal = *p;
+  return f;
+}
+__device__ __forceinline__ void derive_tree_meta(TreeMeta& tm, TreeStage& st, const tsv_shape& s, const TreeFetch& f,
+                                                 const bool csa_cap_b, const bool hca_cap_b) {   // (false: capacity unchecked)
+  const int t = threadIdx.x;
+  if (t < s.D) st.parent[t] = f.parent;
+  if (t >= 32 && t < 36) st.scal[t - 32] = f.scal;
   __syncthreads();
   if (t < 32) {
     // Same facts as build_tree_meta, lane n deriving node n: ancestors by walking up the staged parent array (a valid
@@ -165,6 +173,11 @@ __device__ __forceinline__ void coop_tree_meta(TreeMeta& tm, TreeStage& st, cons
     }
   }
   __syncthreads();
+}
+__device__ __forceinline__ void coop_tree_meta(TreeMeta& tm, TreeStage& st, const tsv_shape& s, const int32_t* L_b, const int32_t* parent_b,
+                                               const int32_t* nn_b, const int32_t* csa_cap_b, const int32_t* hca_cap_b) {
+  const TreeFetch f = fetch_tree(s, L_b, parent_b, nn_b, csa_cap_b, hca_cap_b);
+  derive_tree_meta(tm, st, s, f, csa_cap_b != nullptr, hca_cap_b != nullptr);
 }
 
 // Does the node at depth `depth` of a sequence of committed length L close a block of m tokens?  (What the state build

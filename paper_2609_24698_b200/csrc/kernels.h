@@ -52,6 +52,7 @@ struct TvaPlan {
   int32_t tc_split;                  // chunks a tile may be cut into to fill the device (1: tiles enough)
   int32_t tc_f32;                    // all partial outputs are fp32 (set at the launch)
   int32_t tc_misc_rows;              // rows of the per-sequence packed buffer
+  int32_t tc_packed;                 // the state build has put the entries closed inside the tree into that buffer (set at the launch)
   size_t off_krow, off_kmask, off_nkeys, off_tpo, off_tpml, off_box, off_mode, off_misc, off_order, off_tcnt, off_sched;   // off_sched: the paired kernel's item counter, the pairs that have run out of items
   // selection as a bit per candidate, one row of mask_ld words per node, written for the nodes that rank: the tile plan combines
   // the rows of a tile's nodes into its per-key node masks (bits, not bytes: the CTA that plans a tile of a long list reads them all)
@@ -62,7 +63,9 @@ constexpr int kPairsFor = 74;         // SM pairs the splitting of few tiles aim
 bool make_tva_plan(const tsv_shape& s, TvaPlan& p);
 
 // reset_status: status is written (0 for a usable sequence) instead of or-ed into
-int launch_bsb(const tsv_shape& s, const tsv_cache& c, const tsv_nodes& nd, const tsv_scratch& sc, int32_t* status, bool reset_status, cudaStream_t st);
+// misc: the attention's packed buffer of misc_rows rows per sequence, which then gets the entries closed inside the tree too (or NULL)
+int launch_bsb(const tsv_shape& s, const tsv_cache& c, const tsv_nodes& nd, const tsv_scratch& sc, int32_t* status, bool reset_status,
+               void* misc, int misc_rows, cudaStream_t st);
 int launch_aar(const tsv_shape& s, int n_layers, const tsv_cache* const* caches, const tsv_nodes* const* nodes,
                const tsv_scratch* const* scratch, const int32_t* parent, const int32_t* n_nodes,
                const int32_t* draft, const int32_t* target, int32_t* accept_len, int32_t* accept_path,

@@ -112,7 +112,8 @@ __device__ __forceinline__ void tc_plan_tile(const tsv_shape& s, const TvaPlan& 
   if (packer) {
     // The extra CTA of the sequence (the last in grid x): rows that are small and scattered (few HCA entries, tree nodes,
     // entries closed inside the tree) are packed into one contiguous per-sequence buffer so that TMA boxes can fetch
-    // them.  Kept off the tile CTAs: the copy is a chain of its own (addresses, loads, stores).
+    // them.  Kept off the tile CTAs: the copy is a chain of its own (addresses, loads, stores).  Within a cycle launched by one
+    // call the state build has put the entries closed inside the tree here already: no wait for them then, and no copy.
     if (tm.status) return;
     const size_t rowb = (size_t)s.d * 2;
     const int nh_in = tm.n_hca <= kHcaMiscMax ? tm.n_hca : 0;
@@ -133,7 +134,7 @@ __device__ __forceinline__ void tc_plan_tile(const tsv_shape& s, const TvaPlan& 
       const char* src = nullptr;
       if (r < nh_in) src = (const char*)c.hca_kv + (size_t)hca_row(r) * rowb;
       else if (r < nh_in + tm.nn) src = (const char*)nd.kv + ((size_t)b * D + (r - nh_in)) * rowb;
-      else if (r < n_misc) {
+      else if (r < n_misc && !pl.tc_packed) {
         int ord = r - nh_in - tm.nn;
         const bool isc = ord < ncd;
         if (!isc) ord -= ncd;
@@ -150,7 +151,7 @@ __device__ __forceinline__ void tc_plan_tile(const tsv_shape& s, const TvaPlan& 
 #pragma unroll 1
     for (int phase = 0; phase < 2; ++phase) {
       if (phase) {
-        if (n_misc == first) break;
+        if (n_misc == first || pl.tc_packed) break;
         asm volatile("griddepcontrol.wait;" ::: "memory");   // the entries closed inside the tree
       }
       const int lo = phase ? first * CPR : 0, hi = phase ? n_misc * CPR : rows_out * CPR;
