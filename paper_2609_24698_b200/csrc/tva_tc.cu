@@ -277,6 +277,7 @@ __device__ __forceinline__ void tc_plan_tile(const tsv_shape& s, const TvaPlan& 
     if ((dense || runs_ok) && threadIdx.x == 0) leave_record(kb, runs_ok ? 1 : 2);
   }
   if (dense) return;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");    // the selection's mask rows
   // In-tree entries: candidate n_csa + o of a node is the block closed at the o-th of its strict ancestors that closed one.
   // Thread i: the i-th closed entry of the tree, its mask over the tile's nodes.
@@ -374,6 +375,11 @@ __global__ void __launch_bounds__(NT) tc_plan_kernel(const tsv_shape s, const Tv
   if (threadIdx.x < 2 && tile_cta)                      // finished-chunk counters of the tile's two 128-row halves
     reinterpret_cast<int32_t*>(ws + pl.off_tcnt)[tix * 2 + threadIdx.x] = 0;
   tc_plan_tile<GENERAL, PARTS>(s, pl, c, nd, sc, ws, words_sm, est_sm, &ahead_sm);
+  // Signalled here, and by a tile that waits for the selection before that wait: the attention kernel's CTAs take their places as the
+  // CTAs of the small kernels leave (64 grown sequences 842 -> 830 us per pass of eight layers against after the wait).  At the start
+  // of the CTA it is worse (865 -> 901 us): then all pairs begin at the same instant, and their first instructions queue behind
+  // everyone's first operands.
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // The tile's queries into L2: the pairs of the attention kernel all start at once, and the first phase of each is bound by
   // what arrives from HBM, which idles under the kernels before (first operands of 64 short sequences 10 k -> 7.5 k cycles
   // after the start, last of the first piece 18 k -> 13 k).  At the end of the CTA's own work, which is a chain of loads that
@@ -383,7 +389,6 @@ __global__ void __launch_bounds__(NT) tc_plan_kernel(const tsv_shape s, const Tv
     const int p0 = min(rows, (int)threadIdx.x * part), pn = min(part, rows - p0);
     if (pn > 0) l2_prefetch(reinterpret_cast<const char*>(nd.q) + ((size_t)blockIdx.y * rows_seq + r0 + p0) * (tc::DH * 2), (uint32_t)pn * (tc::DH * 2));
   }
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // (at the END of the CTA's work: the attention kernel's CTAs take their places as this kernel's leave)
   // one CTA waits for the selection in any case, so that the completion of this kernel implies that one's
   if (blockIdx.x == 0 && blockIdx.y == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
