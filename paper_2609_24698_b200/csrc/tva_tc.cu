@@ -397,28 +397,48 @@ __global__ void __launch_bounds__(NT) tc_plan_kernel(const tsv_shape s, const Tv
 // Merge of the paired kernel's multi-chunk tiles (launched with its general instantiation): every chunk left its NORMALISED partial output with
 // the row's (reference max, sum); the row's output is the average of the partial outputs weighted by sum * 2^(max - row max), the
 // chunks accumulated in order.
-// grid (128-row tiles, sequences, groups of 8 * rpw rows): a warp merges rpw rows one after the other, a lane owns 16 columns as 16-byte
-// pieces of the row (coalesced).  The traffic is L2's (67 MB at 64 sequences of 1-4 k tokens), so what counts is latency: a row's (max,
-// sum) and its first four chunks are requested together (after the maxima had been reduced they cost a third latency), and a CTA
-// lives for several rows instead of starting anew for each.
+// 1-d grid (scheduling position of the tile, its two 128-row halves, groups of 8 * rpw rows): a warp merges rpw rows one after the
+// other, a lane owns 16 columns as 16-byte pieces of the row (coalesced).  Bound by latency and by the L2 and HBM traffic (67 MB read
+// and 34 MB written at 64 sequences of 1-4 k tokens, 15 us): a row's (max, sum) and its first four chunks are requested together
+// (after the maxima had been reduced they cost a third latency), and a CTA lives for several rows (rpw: 1, 2 or 4).
+// The CTAs take the places of the attention kernel's as those run out of items, and a tile is merged as soon as all warps of its
+// chunks have said that their rows are stored (it is looked for in the order in which the tiles are worked on), the rest when
+// that kernel has ended: at those 64 sequences a pass of eight layers takes 798 instead of 830 us.  Tiles cut to fill the device
+// all end with that kernel, and looking earlier loses 0.4 us a layer: there the merge waits for it at once.
 // ANY32: some tiles' partial outputs may be fp32 (else all are bf16, and the kernel keeps its registers low).
+constexpr int kMergePolls = 256;       // times a warp looks for its tile's chunks (0.3 us each) before it waits for the whole attention kernel
 template <bool ANY32>
 __global__ void __launch_bounds__(256) tc_combine_pair_kernel(const tsv_shape s, const TvaPlan pl, void* __restrict__ out_, const char* __restrict__ ws, const int rpw) {
   using namespace tc;
   constexpr uint32_t FULL = 0xffffffffu;
-  asm volatile("griddepcontrol.wait;" ::: "memory");            // launched as a programmatic dependent of the attention kernel
-  const int rt = blockIdx.x, tile = rt >> 1, b = blockIdx.y;
-  const size_t tix = (size_t)b * pl.tc_nt + tile, rix = (size_t)b * 2 * pl.tc_nt + rt;
-  const int mode = reinterpret_cast<const int32_t*>(ws + pl.off_mode)[tix];
-  const int nk = reinterpret_cast<const int32_t*>(ws + pl.off_nkeys)[tix];
-  if ((mode != 1 && mode != 2) || nk <= 0) return;
+  const int lg = 31 - __clz(BM / 8 / rpw), pos = blockIdx.x >> (lg + 1), half = (blockIdx.x >> lg) & 1, group = blockIdx.x & ((1 << lg) - 1);
+  // Launched as a programmatic dependent of the attention kernel, when all CTAs of that have started: the tile plan is complete.
+  const int4 rec = __ldcg(reinterpret_cast<const int4*>(ws + pl.off_order) + pos);     // {tile, mode, keys}
+  // (What other kernels wrote is read past the L1.)  One CTA waits for that kernel in any case, so that the completion of this one
+  // implies that one's.
+  const bool early = pl.tc_split == 1;
+  if (blockIdx.x == 0 || !early) asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int nk = rec.z, b = (uint32_t)rec.x / (uint32_t)pl.tc_nt, rt = (rec.x - b * pl.tc_nt) * 2 + half;
+  const size_t rix = (size_t)rec.x * 2 + half;
+  if (nk <= 0) return;
   int nch, CL;
   bool f32;
   chunking_x(nk, true, pl.tc_split, pl.tc_f32, nch, CL, f32);
   if (!ANY32) f32 = false;                                       // (no tile is split, so one with more than one chunk was too long for one: bf16)
   if (nch <= 1) return;                                          // the paired kernel wrote the output itself
   const int rows_seq = s.D * s.H, row0 = rt * BM, lane = threadIdx.x & 31;
-  const int first = blockIdx.z * 8 * rpw + (threadIdx.x >> 5), last = min(min(BM, rows_seq - row0), (int)(blockIdx.z + 1) * 8 * rpw);
+  const int first = group * 8 * rpw + (threadIdx.x >> 5), last = min(min(BM, rows_seq - row0), (group + 1) * 8 * rpw);
+  if (first >= last) return;
+  if (early) {
+    const int32_t* cnt = reinterpret_cast<const int32_t*>(ws + pl.off_tcnt) + rix;
+    int done = 0;
+    for (int i = 0; i < kMergePolls; ++i) {                      // (every lane reads it: one request a warp)
+      asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(done) : "l"(cnt) : "memory");
+      if (done >= 8 * nch) break;
+      __nanosleep(200);
+    }
+    if (done < 8 * nch) asm volatile("griddepcontrol.wait;" ::: "memory");
+  }
   const float2* pml = reinterpret_cast<const float2*>(ws + pl.off_tpml) + rix * pl.tc_chmax * BM;
   auto merge = [&](auto vec) {                                   // vec: 16-byte pieces of a lane's 16 columns
     constexpr int V = decltype(vec)::value;
@@ -427,7 +447,7 @@ __global__ void __launch_bounds__(256) tc_combine_pair_kernel(const tsv_shape s,
 #pragma unroll 1
     for (int row = first; row < last; row += 8) {
       const uint4* pr = po + (size_t)row * (DH / (V == 4 ? 4 : 8));
-      float2 x = lane < nch ? pml[(size_t)lane * BM + row] : make_float2(-INFINITY, 0.f);
+      float2 x = lane < nch ? __ldcg(pml + (size_t)lane * BM + row) : make_float2(-INFINITY, 0.f);
       uint4 v[4][V];
       auto fetch = [&](int c0) {
 #pragma unroll
@@ -440,7 +460,7 @@ __global__ void __launch_bounds__(256) tc_combine_pair_kernel(const tsv_shape s,
       fetch(0);
       float m = x.y > 0.f ? x.x : -INFINITY;
 #pragma unroll 1
-      for (int ch = lane + 32; ch < nch; ch += 32) { const float2 y = pml[(size_t)ch * BM + row]; if (y.y > 0.f) m = fmaxf(m, y.x); }
+      for (int ch = lane + 32; ch < nch; ch += 32) { const float2 y = __ldcg(pml + (size_t)ch * BM + row); if (y.y > 0.f) m = fmaxf(m, y.x); }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(FULL, m, o));
       float wt = x.y > 0.f ? x.y * exp2f(x.x - m) : 0.f;         // lane c: weight of chunk c (of the 32 chunks at hand)
@@ -452,7 +472,7 @@ __global__ void __launch_bounds__(256) tc_combine_pair_kernel(const tsv_shape s,
         if (c0) {
           fetch(c0);
           if ((c0 & 31) == 0) {                                  // (lists of more than 32 chunks)
-            x = c0 + lane < nch ? pml[(size_t)(c0 + lane) * BM + row] : make_float2(-INFINITY, 0.f);
+            x = c0 + lane < nch ? __ldcg(pml + (size_t)(c0 + lane) * BM + row) : make_float2(-INFINITY, 0.f);
             wt = x.y > 0.f ? x.y * exp2f(x.x - m) : 0.f;
           }
         }
@@ -579,7 +599,7 @@ int launch_tva_tc(const tsv_shape& s, const TvaPlan& p_in, const TvaTcPrep& prep
     // rows a warp takes: one while that leaves SMs idle otherwise, up to four
     const int64_t groups = (int64_t)2 * p.tc_nt * s.B * (tc::BM / 8);
     const int rpw = groups <= 4 * 148 ? 1 : groups <= 8 * 148 ? 2 : 4;
-    cfg.gridDim = dim3(2 * p.tc_nt, s.B, tc::BM / 8 / rpw); cfg.blockDim = dim3(256, 1, 1); cfg.stream = st;
+    cfg.gridDim = dim3(2 * p.tc_nt * s.B * (tc::BM / 8 / rpw)); cfg.blockDim = dim3(256, 1, 1); cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;

@@ -565,6 +565,18 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
     const uint32_t mybit = 1u << ((int)rank * (BM / s.H) + row / s.H);      // node of this row within the pair's plan tile
     const float scale2 = s.sm_scale * 1.4426950408889634f;
     uint32_t accb = 0;                               // parity of the next use of each acc_ev
+    // The merge kernel is told, per warp, that an item's rows are stored.  It costs nothing half an item later, when the stores are
+    // long complete (right after them it is a wait of a memory latency), and the pair's last item is signalled at the end.  Not where
+    // tiles are cut to fill the device: all items end at about the same time there.
+    int stored_rix = -1;
+    auto signal_stored = [&]() {
+      if (GENERAL && stored_rix >= 0 && lane == 0) {
+        asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+        asm volatile("fence.proxy.async.global;" ::: "memory");
+        asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(reinterpret_cast<int32_t*>(ws + pl.off_tcnt) + stored_rix) : "memory");
+      }
+      stored_rix = -1;
+    };
 #pragma unroll 1
     for (int it = 0;; ++it) {
     const int4 rec = next_item(it);
@@ -716,6 +728,7 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
       // piece's S columns); the wait for the stores of a later piece covers the earlier ones
       if (npc == 3 && pc == 1) p_stored(1);
     }
+    signal_stored();
     // The row sums meet (in the output staging area, idle until O is read out); where a warp moved its reference, the two
     // settle on the larger one first.
     float l_row = (lp[0] + lp[1]) + (lp[2] + lp[3]);
@@ -853,6 +866,7 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
       asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
       asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&sm.stage_free)) : "memory");
     }
+    if (GENERAL && nch > 1 && pl.tc_split == 1) stored_rix = (int)rix;
     if (!GENERAL && nch > 1) {
       // Tiles of two chunks where nothing longer can occur: each chunk leaves its unnormalised part of O with (max, sum)
       // per row; the CTA that finishes a 128-row tile last merges the parts (fixed order, so the result does not depend
@@ -895,6 +909,7 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
     }
     }
     if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    signal_stored();
     leave();
   }
 }
