@@ -196,6 +196,19 @@ struct SelectSmem {
 // Selection of one node by the whole CTA, in two parts.  list: shared memory, the scores of the n_csa committed entries first, then
 // those of the in-tree ones.  First part: the range and the histogram of the committed entries, which need nothing of the state build
 // (the in-tree entries are added to it as they are scored; the intervals at either end take what lies beyond).
+// (All passes over the list fetch several scores before they use one: one shared-memory latency for them all, where a pass that
+// writes in between would take one for each.)
+template <int NT, typename F>
+__device__ __forceinline__ void each_score(const float* list, int n, F f) {
+  constexpr int U = 8;
+  for (int i0 = threadIdx.x; i0 < n; i0 += U * NT) {
+    float v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) v[u] = i0 + u * NT < n ? list[i0 + u * NT] : 0.f;
+#pragma unroll
+    for (int u = 0; u < U; ++u) if (i0 + u * NT < n) f(i0 + u * NT, v[u]);
+  }
+}
 struct ScoreBins {
   float lo, scale;
   bool regular;                                          // (else: all equal, not finite, or too narrow)
@@ -205,9 +218,9 @@ struct ScoreBins {
 template <int NT, int NB>
 __device__ __forceinline__ ScoreBins count_committed(SelectSmem<NT, NB>& sm, const float* list, int n_csa) {
   constexpr int NW = NT / 32;
-  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   float lo = INFINITY, hi = -INFINITY;
-  for (int i = t; i < n_csa; i += NT) { const float v = list[i]; lo = fminf(lo, v); hi = fmaxf(hi, v); }
+  each_score<NT>(list, n_csa, [&](int, float v) { lo = fminf(lo, v); hi = fmaxf(hi, v); });
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) { lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o)); hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o)); }
   if (lane == 0) { sm.red[0][w] = lo; sm.red[1][w] = hi; }
@@ -218,7 +231,7 @@ __device__ __forceinline__ ScoreBins count_committed(SelectSmem<NT, NB>& sm, con
   bins.lo = lo;
   bins.scale = hi > lo ? (float)NB / (hi - lo) : 0.f;
   bins.regular = bins.scale > 0.f && bins.scale < 1e30f;
-  if (bins.regular) for (int i = t; i < n_csa; i += NT) atomicAdd(&sm.hist[bins.of<NB>(list[i])], 1);
+  if (bins.regular) each_score<NT>(list, n_csa, [&](int, float v) { atomicAdd(&sm.hist[bins.of<NB>(v)], 1); });
   return bins;
 }
 
@@ -254,10 +267,9 @@ __device__ __forceinline__ void select_node(SelectSmem<NT, NB>& sm, const ScoreB
     }
     __syncthreads();
     bstar = sm.bin; rem = sm.rem;
-    for (int i = t; i < n_cand; i += NT) {
-      const float v = list[i];
+    each_score<NT>(list, n_cand, [&](int i, float v) {
       if (bin_of(v) == bstar) { const int pos = atomicAdd(&sm.cnt, 1); if (pos < CAP) { sm.cand_s[pos] = v; sm.cand_i[pos] = i; } }
-    }
+    });
     __syncthreads();
     m = sm.cnt;
     if (m <= CAP) {
@@ -306,20 +318,31 @@ __device__ __forceinline__ void select_node(SelectSmem<NT, NB>& sm, const ScoreB
   // Warp w owns the candidates [w * part, (w + 1) * part), rows of 32.  above: certainly taken; edge (radix only): equal to the
   // threshold, of which the first rem in index order are taken.
   const int part = ((n_cand + NW - 1) / NW + 31) & ~31, beg = min(n_cand, w * part), end = min(n_cand, beg + part);
-  auto classify = [&](int i, bool& above, bool& edge) {
-    above = edge = false;
-    if (i >= end) return;
-    const float v = list[i];
-    if (radix) { const uint32_t key = order_key(v); above = key > thr; edge = key == thr; }
-    else { const int bn = bin_of(v); above = bn > bstar || (bn == bstar && ((bits[i >> 5] >> (i & 31)) & 1u)); }
+  constexpr int U = 4;                                   // rows of 32 candidates taken together
+  auto classify = [&](int i0, bool (&above)[U], bool (&edge)[U]) {
+    float v[U];
+    uint32_t word[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i = i0 + 32 * u + lane;
+      v[u] = i < end ? list[i] : 0.f;
+      word[u] = i0 + 32 * u < end ? bits[(i0 >> 5) + u] : 0u;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (radix) { const uint32_t key = order_key(v[u]); above[u] = key > thr; edge[u] = key == thr; }
+      else { const int bn = bin_of(v[u]); above[u] = bn > bstar || (bn == bstar && ((word[u] >> lane) & 1u)); edge[u] = false; }
+      if (i0 + 32 * u + lane >= end) above[u] = edge[u] = false;
+    }
   };
   int pos = 0, eq_base = 0;
   if (lists || radix) {
     int ca = 0, ce = 0;
-    for (int i0 = beg; i0 < end; i0 += 32) {
-      bool above, edge;
-      classify(i0 + lane, above, edge);
-      ca += __popc(__ballot_sync(0xffffffffu, above)); ce += __popc(__ballot_sync(0xffffffffu, edge));
+    for (int i0 = beg; i0 < end; i0 += 32 * U) {
+      bool above[U], edge[U];
+      classify(i0, above, edge);
+#pragma unroll
+      for (int u = 0; u < U; ++u) { ca += __popc(__ballot_sync(0xffffffffu, above[u])); ce += __popc(__ballot_sync(0xffffffffu, edge[u])); }
     }
     __syncthreads();
     if (lane == 0) { sm.wsum[0][w] = ca; sm.wsum[1][w] = ce; }
@@ -328,23 +351,28 @@ __device__ __forceinline__ void select_node(SelectSmem<NT, NB>& sm, const ScoreB
     if (radix) pos += min(rem, eq_base);
   }
   const uint32_t lt = (1u << lane) - 1u;
-  for (int i0 = beg; i0 < end; i0 += 32) {
-    const int i = i0 + lane;
-    bool take, edge;
-    classify(i, take, edge);
-    if (radix) {
-      const uint32_t eqm = __ballot_sync(0xffffffffu, edge);
-      take = take || (edge && eq_base + __popc(eqm & lt) < rem);
-      eq_base += __popc(eqm);
-    }
-    const uint32_t tkm = __ballot_sync(0xffffffffu, take);
-    if (selmask && lane == 0) selmask[i0 >> 5] = tkm;
-    if (lists) {
-      if (take) {
-        const int p = pos + __popc(tkm & lt), val = i < n_csa ? i : pe.newc_blk[i - n_csa];
-        sel[p] = val; if (usr) usr[p] = val;
+  for (int i0 = beg; i0 < end; i0 += 32 * U) {
+    bool above[U], edge[U];
+    classify(i0, above, edge);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int r0 = i0 + 32 * u, i = r0 + lane;
+      if (r0 >= end) break;                              // (uniform in the warp)
+      bool take = above[u];
+      if (radix) {
+        const uint32_t eqm = __ballot_sync(0xffffffffu, edge[u]);
+        take = take || (edge[u] && eq_base + __popc(eqm & lt) < rem);
+        eq_base += __popc(eqm);
       }
-      pos += __popc(tkm);
+      const uint32_t tkm = __ballot_sync(0xffffffffu, take);
+      if (selmask && lane == 0) selmask[r0 >> 5] = tkm;
+      if (lists) {
+        if (take) {
+          const int p = pos + __popc(tkm & lt), val = i < n_csa ? i : pe.newc_blk[i - n_csa];
+          sel[p] = val; if (usr) usr[p] = val;
+        }
+        pos += __popc(tkm);
+      }
     }
   }
   if (lists && t == 0) *selcnt = k;
@@ -369,7 +397,10 @@ __global__ void __launch_bounds__(128, 4) topk_seq_kernel(const tsv_shape s, con
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the tile plan may start its selection-independent part
   const int rank = blockIdx.x, b = blockIdx.y, D = s.D, k = s.topk, HI = s.HI;
   const bool lists = !pl.tc || topk_user;               // somebody reads the index lists (the tile plan reads mask rows only)
+  // (all that depends on the sequence alone is requested together: one memory latency)
+  const TreeFetch tf = fetch_tree(s, c.L + b, nd.parent + (size_t)b * D, nd.n_nodes + b, c.csa_cap + b, c.hca_cap + b);
   const int L0 = c.L[b];
+  const int64_t row0 = PAGED ? 0 : c.csa_row0[b];
   // some node may have more than k candidates (and the rows exist: a sequence of bad length or capacity is flagged below)
   const bool any_rank = L0 >= 0 && (int64_t)L0 + D <= s.max_L && (L0 + D) / s.m_csa <= c.csa_cap[b] && L0 / s.m_csa + D > k;
   if (!any_rank && !lists && rank != 0) return;          // (alike in the whole cluster but for CTA 0, which validates the sequence)
@@ -387,7 +418,7 @@ __global__ void __launch_bounds__(128, 4) topk_seq_kernel(const tsv_shape s, con
   uint4 alo[4], ahi[4];
   const int first = e0 + 16 * w;
   if (any_rank) {
-    if (PAGED) sco.rows = csa_rows_of(c, s, b); else { sco.rows.pt = nullptr; sco.rows.per_page = 1; sco.rows.row0 = c.csa_row0[b]; }
+    if (PAGED) sco.rows = csa_rows_of(c, s, b); else { sco.rows.pt = nullptr; sco.rows.per_page = 1; sco.rows.row0 = row0; }
     sco.ikb = reinterpret_cast<const char*>(c.csa_ik) + (size_t)sco.rows.row0 * ROWB + (BF ? sco.tq * 16 : 0);
     if (BF && first < e1) sco.template fetch<PAGED>(first, alo, ahi);
     stage_queries(dsm, nd.iq, b, 0, D, HI);
@@ -397,7 +428,7 @@ __global__ void __launch_bounds__(128, 4) topk_seq_kernel(const tsv_shape s, con
     for (int i = t; i < NB; i += NT) sm.hist[i] = 0;
     if (t == 0) sm.cnt = 0;
   }
-  coop_tree_meta(tm, tstage, s, c.L + b, nd.parent + (size_t)b * D, nd.n_nodes + b, c.csa_cap + b, c.hca_cap + b);
+  derive_tree_meta(tm, tstage, s, tf, true, true);
   if (t == 0 && rank == 0 && tm.status) atomicOr(status + b, tm.status);
   const int n = rank;                                    // the node this CTA owns
   const bool live = !tm.status && n < tm.nn;
