@@ -15,11 +15,13 @@
  *     work is enqueued on `stream` and the call returns.  Between calls it keeps nothing of the
  *     caller's data; what it does keep per process is set-up it does once (kernel attributes,
  *     the number of CTA pairs a device holds, the driver entry point for tensor maps), the
- *     launch counter behind tsv_kernel_launches(), and for tree_verify_attn_static the
- *     address of its built-in array.
- *   - Stream order: the calls of a layer run in the order given above on one stream.  Some kernels of
- *     tree_verify_attn are launched as PROGRAMMATIC DEPENDENTS of the kernel before them on the stream: the part
- *     of them that reads only the call's inputs (tsv_nodes, the committed tsv_cache) may run before that kernel
+ *     launch counter behind tsv_kernel_launches(), for tree_verify_attn_static the
+ *     address of its built-in array, and per calling thread a bounded number of encoded tensor
+ *     maps, found again by the addresses and sizes they were made from.
+ *   - Stream order: the calls of a layer run in the order given above on one stream.  The kernels are
+ *     launched as programmatic dependents; those of branch_state_build and accept_and_refresh wait for
+ *     all earlier work before they do anything.  Some kernels of tree_verify_attn start earlier: the part
+ *     of them that reads only the call's inputs (tsv_nodes, the committed tsv_cache) may run before the kernel before them
  *     has finished, and that part already writes the call's workspace, topk_idx and status; they wait for
  *     it before they read anything the library's own kernels write.  For the caller this matters in one
  *     case only: a kernel of the caller's that is enqueued directly before tree_verify_attn and itself

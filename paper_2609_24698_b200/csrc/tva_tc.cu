@@ -5,14 +5,14 @@
 // SAME staged key rows (key == value, MQA), so S = Q K^T and O = P K are dense contractions.  Which node sees which key is
 // a per-key bitmask applied to the S fragment after it is read back from tensor memory.
 //
-//   tc_plan_kernel   per (sequence, plan tile): the keys visible to at least one node of the tile, as four runs {CSA
-//                    entries, HCA entries, window ring, packed misc rows} padded to 32 rows, the CSA entries last, with a node mask per key.
+//   tc_plan_kernel   per (sequence, plan tile): the keys visible to at least one node of the tile, as four runs {HCA
+//                    entries, window ring, packed misc rows, CSA entries} padded to 32 rows, with a node mask per key.
 //                    Contiguous-run tiles (every node selects all CSA candidates, or the CSA slab is at most 2 x topk
 //                    rows): the runs as 32-row TMA boxes.  Gathered tiles (selection far from dense, or a paged pool
-//                    whose pages do not hold whole boxes): the first run holds only the entries some node of the tile
+//                    whose pages do not hold whole boxes): the CSA run holds only the entries some node of the tile
 //                    selected, and every key is named by array << 30 | row for four-row TMA gathers.
 //                    Each tile CTA leaves its record {tile, mode, keys} at the tile's scheduling position (its rank by
-//                    estimated key count, most first); an extra CTA per sequence packs the small scattered rows.
+//                    estimated length of its work items, longest first); an extra CTA per sequence packs the small scattered rows.
 //   tc_combine_pair_kernel  merges the chunks of the paired kernel's multi-chunk tiles (fixed order).
 #include <type_traits>
 

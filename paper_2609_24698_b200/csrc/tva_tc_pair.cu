@@ -7,11 +7,13 @@
 // -- the staged key rows -- is split between the two shared memories, so each SM fetches only HALF of
 // the K tile (S = Q K^T: half of the keys) and half of the V tile (O = P K: half of the columns of d).
 // That halves the bytes each SM pulls from L2.
-//   warps 0, 10  producers: TMA boxes (cp.async.bulk.tensor, 128-byte swizzle) into 16 KiB slots; the copies of BOTH
-//                CTAs complete on the mbarriers of the leader (rank 0) CTA
+// The pairs are persistent (one per two SMs): they take (tile, chunk of keys) items from a counter until none is left.
+//   warps 0, 3, 12-15  producers: TMA boxes or four-row gathers (cp.async.bulk.tensor, 128-byte swizzle) into 16 KiB slots, each
+//                slot owned by one producer; the copies of BOTH CTAs complete on the mbarriers of the leader (rank 0) CTA
 //   warp 1       MMA issuer (leader CTA only): tcgen05.mma.cta_group::2, slot release and accumulator
 //                events by tcgen05.commit multicast to both CTAs
-//   warps 2-9    one-pass softmax on the CTA's own S rows (TMEM), P written back to TMEM, epilogue of O through
+//   warp 2       hands out the items (leader's counter, both CTAs told)
+//   warps 4-11   one-pass softmax on the CTA's own S rows (TMEM), P written back to TMEM, epilogue of O through
 //                swizzled shared-memory tiles and TMA stores; events to the leader's MMA warp by remote arrive
 // Stage stream, TMEM column plan, running-max rule and chunking are those described at the kernel.
 #include <cuda.h>
