@@ -31,7 +31,7 @@ import numpy as np  # noqa: E402
 # attention stage with the bytes of ONE of its launches (one layer), and, where captured, the sum over all kernels of one
 # verify cycle.  The captures are summarised under profiles/; workloads without a capture report null.
 NCU_DRAM = {
-    "cfg4": {"kernel": "tc_attn_pair_kernel", "launch_bytes": 66_239_168, "cycle_bytes": None},   # 65.48 MB read + 0.76 MB written
+    "cfg4": {"kernel": "tc_attn_pair_kernel", "launch_bytes": 64_300_000, "cycle_bytes": None},   # 63.6 MB read + 0.7 MB written
     # cfg5: tc_attn_pair_kernel 61.11 MB read + 1.70 MB written; all kernels of one cycle 138.1 MB (cold cache per kernel)
     "cfg5": {"kernel": "tc_attn_pair_kernel", "launch_bytes": 62_808_320, "cycle_bytes": 138_081_792},
 }
