@@ -24,8 +24,12 @@ __device__ inline void path_entries(PathEntries& pe, const TreeMeta& tm, const t
   }
 }
 
-__device__ __forceinline__ uint32_t order_key(float f) {       // larger float -> larger key
-  const uint32_t u = __float_as_uint(f);
+// Larger float -> larger key; a total order of the bit patterns (a positive NaN above everything).  The bits are taken by an opaque
+// move: of a plain reinterpretation the compiler makes float operations in some places (the sign bit set as -|f|), which turn a NaN
+// into another pattern there than elsewhere, and a selection that counts a key in one pass and misses it in the next is short of it.
+__device__ __forceinline__ uint32_t order_key(float f) {
+  uint32_t u;
+  asm("mov.b32 %0, %1;" : "=r"(u) : "f"(f));
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 

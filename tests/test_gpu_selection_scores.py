@@ -1,0 +1,79 @@
+"""Selections over lists with scores at which a float compare and a total order differ, in every selection form: exactly topk
+entries whatever the values, nothing written past a node's row.  The scores are exact small numbers, so that the expected selection
+is one sort on the host."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2609_24698_b200 import synth
+
+pytestmark = pytest.mark.gpu
+
+# dtype, nodes, committed entries, topk.  One CTA per node (short lists); a cluster per sequence, bf16 and fp32; scores over all SMs
+# and a cluster per node, for more than eight nodes and for a long list; the general kernels (other indexer widths): keys in registers,
+# a cluster per node, a list read again in every pass
+FORMS = [("bf16", 8, 600, 512), ("bf16", 8, 900, 800), ("fp32", 8, 600, 512), ("bf16", 12, 900, 800), ("bf16", 7, 4300, 4200),
+         ("fp32", 8, 900, 800, 16), ("bf16", 8, 2500, 2400, 16), ("fp32", 5, 66000, 65800, 8)]
+
+
+def _select(form, HI, ik, tree_ik, iq, iw):
+    """topk_idx of a chain of D nodes (blocks of two tokens: nodes 1, 3, ... close one) after n committed entries with the indexer
+    keys ik [n][di]; every closed entry has the key tree_ik.  The list buffer is followed by a guard."""
+    from paper_2609_24698_b200 import harness as hz
+    dtype, D, n, k = form[:4]
+    di = ik.shape[1]
+    sh = synth.Shape(dtype, 1, D, 4, 16, 2, k, HI, di, 64, 64)
+    ccap, hcap = hz.capacities(sh, [2 * n], 2 * D)
+    eng = hz.VerifyEngine(sh, 1, ccap, hcap, 2 * n + 2 * D, want_topk=True)
+    guard = torch.full((D * k + 64,), -2, dtype=torch.int32, device="cuda")
+    eng.topk_idx = [guard[:D * k].view(1, D, k)]
+    eng.caches[0].L.fill_(2 * n)
+    eng.caches[0].csa_ik[:n] = torch.from_numpy(ik).cuda()
+    inp = hz.InputSet.empty(sh, 1)
+    nd = inp.layers[0]
+    nd.parent.copy_(torch.arange(-1, D - 1).view(1, D)); nd.n_nodes.fill_(D)
+    nd.ikc[:] = torch.from_numpy(tree_ik).cuda()
+    nd.iq[:] = torch.from_numpy(iq).cuda(); nd.iw[:] = torch.from_numpy(iw).cuda()
+    eng.launch_cycle(inp, refresh=False)
+    torch.cuda.synchronize()
+    assert int(eng.status.sum()) == 0
+    got = guard.cpu().numpy()
+    assert (got[D * k:] == -2).all(), "written past the last node's row"
+    return got[:D * k].reshape(D, k)
+
+
+def _check(got, form, scores, tree_score):
+    """scores: of the committed entries, tree_score: of every closed one; NaN above everything, ties to the lower index."""
+    for node, row in enumerate(got):
+        s = np.concatenate([scores, np.full(node // 2, tree_score)])
+        order = np.lexsort((np.arange(len(s)), -np.where(np.isnan(s), np.inf, s)))
+        assert np.array_equal(row, np.sort(order[:form[3]])), (node, len(set(row.tolist())))
+
+
+@pytest.mark.parametrize("form", FORMS)
+@pytest.mark.parametrize("where", ["committed", "tree"])
+@pytest.mark.parametrize("spare", [300])
+def test_nan_scores_select_exactly_topk(form, where, spare):
+    """NaN scores (an overflowed inner product of a head whose weight is zero) in a list whose topk-th score lies among equal ones at
+    the bottom of the range: among so many that the radix passes decide (spare 300)."""
+    dtype, D, n, k = form[:4]
+    di = form[4] if len(form) > 4 else 128 if dtype == "bf16" else 64
+    rng = np.random.default_rng(n)
+    a = rng.integers(1, 200, n).astype(np.float32)
+    zero = rng.permutation(n)[: n - k + spare]                  # relu leaves nothing of them: the topk-th score is theirs
+    a[zero] = -1
+    ik, tree_ik = np.zeros((n, di), np.float32), np.zeros(di, np.float32)
+    ik[:, 0] = a
+    scores, tree_score = np.maximum(a, 0).astype(np.float64), 0.0
+    if where == "committed":
+        ik[zero[:3], 1] = 1e38
+        scores[zero[:3]] = np.nan
+    else:
+        tree_ik[1] = 1e38
+        tree_score = np.nan
+    HI = 2
+    iq = np.zeros((D, HI, di), np.float32)
+    iq[:, 0, 0], iq[:, 1, 1] = 1, 3e38
+    iw = np.zeros((D, HI), np.float32)
+    iw[:, 0] = 2.0 ** np.arange(D)
+    _check(_select(form, HI, ik, tree_ik, iq, iw), form, scores, tree_score)
