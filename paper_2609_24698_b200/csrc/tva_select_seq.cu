@@ -19,7 +19,8 @@
 // The selection finds the k largest by ONE histogram over equal intervals of [min, max] (the scores of a list share their high
 // bits, so radix digits of the bit pattern take four passes with colliding bins): the interval of the k-th largest holds few
 // candidates, which are ranked against each other exactly (ties to the lower index).  Degenerate lists (more than CAP
-// candidates in that interval: ties, outliers) take four radix passes instead.
+// candidates in that interval: ties, outliers; a score that is infinite or NaN) take four radix passes instead: the interval code
+// compares floats, under which a NaN has no place, the radix digits are a total order of the bit patterns.
 // Same result as topk_kernel: the exact k largest scores, ties to the lower index, ascending output.
 #include "select_common.cuh"
 
@@ -211,22 +212,28 @@ __device__ __forceinline__ void each_score(const float* list, int n, F f) {
 }
 struct ScoreBins {
   float lo, scale;
-  bool regular;                                          // (else: all equal, not finite, or too narrow)
+  bool regular;                                          // (else: all equal, not finite, a NaN among them, or too narrow)
   // interval of a score: monotone in the score (a rounded subtraction and product are), so intervals order as scores do
   template <int NB> __device__ __forceinline__ int of(float v) const { return min(NB - 1, max(0, (int)((v - lo) * scale))); }
 };
+// Minimum that a NaN on either side makes NaN.  A list's range is NaN then, its scale 0, and the list not regular.
+__device__ __forceinline__ float min_or_nan(float a, float b) {
+  float r;
+  asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
 template <int NT, int NB>
 __device__ __forceinline__ ScoreBins count_committed(SelectSmem<NT, NB>& sm, const float* list, int n_csa) {
   constexpr int NW = NT / 32;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   float lo = INFINITY, hi = -INFINITY;
-  each_score<NT>(list, n_csa, [&](int, float v) { lo = fminf(lo, v); hi = fmaxf(hi, v); });
+  each_score<NT>(list, n_csa, [&](int, float v) { lo = min_or_nan(lo, v); hi = fmaxf(hi, v); });
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) { lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o)); hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o)); }
+  for (int o = 16; o > 0; o >>= 1) { lo = min_or_nan(lo, __shfl_xor_sync(0xffffffffu, lo, o)); hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o)); }
   if (lane == 0) { sm.red[0][w] = lo; sm.red[1][w] = hi; }
   __syncthreads();
 #pragma unroll
-  for (int i = 0; i < NW; ++i) { lo = fminf(lo, sm.red[0][i]); hi = fmaxf(hi, sm.red[1][i]); }
+  for (int i = 0; i < NW; ++i) { lo = min_or_nan(lo, sm.red[0][i]); hi = fmaxf(hi, sm.red[1][i]); }
   ScoreBins bins;
   bins.lo = lo;
   bins.scale = hi > lo ? (float)NB / (hi - lo) : 0.f;
@@ -498,6 +505,7 @@ __global__ void __launch_bounds__(128, 4) topk_seq_kernel(const tsv_shape s, con
     if (ranks)
       ex.score(pe, s, sc, b, [&](int i, float v) {
         list[n_csa + i] = v;
+        if (v != v) atomicAdd(&sm.cnt, CAP + 1);         // (a NaN: the selection finds its interval overfull and takes the radix passes)
         if (bins.regular) atomicAdd(&sm.hist[bins.of<NB>(v)], 1);
       });
   } else if (rank == 0 && b == 0) {
@@ -630,13 +638,13 @@ __global__ void __launch_bounds__(kListThreads, 2) topk_list_kernel(const tsv_sh
   }
   __syncthreads();
   float lo = INFINITY, hi = -INFINITY;
-  for (int i = t; i < len; i += NT) { const float v = list[i]; lo = fminf(lo, v); hi = fmaxf(hi, v); }
+  for (int i = t; i < len; i += NT) { const float v = list[i]; lo = min_or_nan(lo, v); hi = fmaxf(hi, v); }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) { lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o)); hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o)); }
+  for (int o = 16; o > 0; o >>= 1) { lo = min_or_nan(lo, __shfl_xor_sync(0xffffffffu, lo, o)); hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o)); }
   if (lane == 0) { sm.red[0][w] = lo; sm.red[1][w] = hi; }
   __syncthreads();
   if (t == 0) {
-    for (int i = 0; i < NW; ++i) { lo = fminf(lo, sm.red[0][i]); hi = fmaxf(hi, sm.red[1][i]); }
+    for (int i = 0; i < NW; ++i) { lo = min_or_nan(lo, sm.red[0][i]); hi = fmaxf(hi, sm.red[1][i]); }
     sm.ext = make_float2(lo, hi);
   }
   auto peer = [&](const void* p, int r) { return map_to_rank((uint32_t)__cvta_generic_to_shared(p), r); };
@@ -648,10 +656,10 @@ __global__ void __launch_bounds__(kListThreads, 2) topk_list_kernel(const tsv_sh
     const int r = lane & 7;
     lo = peer_f(&sm.ext.x, r); hi = peer_f(&sm.ext.y, r);
 #pragma unroll
-    for (int o = 4; o > 0; o >>= 1) { lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o)); hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o)); }
+    for (int o = 4; o > 0; o >>= 1) { lo = min_or_nan(lo, __shfl_xor_sync(0xffffffffu, lo, o)); hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o)); }
   }
   const float scale = hi > lo ? (float)NB / (hi - lo) : 0.f;
-  const bool regular = scale > 0.f && scale < 1e30f;     // (else: all equal, not finite, or too narrow)
+  const bool regular = scale > 0.f && scale < 1e30f;     // (else: all equal, not finite, a NaN among them, or too narrow)
   auto bin_of = [&](float v) { return min(NB - 1, (int)((v - lo) * scale)); };
   // the interval (of nb in h, over the whole cluster) of the rem-th largest: its number, and what of rem is left in it
   auto locate = [&](const int* h, int nb, int rem, int& bin, int& left) {
