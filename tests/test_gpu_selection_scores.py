@@ -77,3 +77,21 @@ def test_nan_scores_select_exactly_topk(form, where, spare):
     iw = np.zeros((D, HI), np.float32)
     iw[:, 0] = 2.0 ** np.arange(D)
     _check(_select(form, HI, ik, tree_ik, iq, iw), form, scores, tree_score)
+
+
+@pytest.mark.parametrize("form", FORMS)
+def test_zeros_of_either_sign_tie(form):
+    """All heads of negative weight: the best score is a zero, negative where a product of the two leaves it, positive for an entry
+    closed inside the tree.  They tie, and the lower indices win: the committed ones."""
+    dtype, D, n, k = form[:4]
+    di = form[4] if len(form) > 4 else 128 if dtype == "bf16" else 64
+    rng = np.random.default_rng(n + 1)
+    HI = 4
+    ik = np.zeros((n, di), np.float32)
+    ik[:, :HI] = -rng.integers(1, 100, (n, HI))
+    worse = rng.permutation(n)[: (n - k) // 2]               # the others, more than topk, all score zero
+    ik[worse, 2] = rng.integers(1, 100, len(worse))
+    iq = np.zeros((D, HI, di), np.float32)
+    iq[:, range(HI), range(HI)] = 1
+    iw = np.full((D, HI), -1, np.float32)
+    _check(_select(form, HI, ik, np.zeros(di, np.float32), iq, iw), form, -np.maximum(ik, 0).max(1).astype(np.float64), 0.0)
