@@ -9,6 +9,7 @@ from __future__ import annotations
 import ctypes as C
 import os
 from dataclasses import dataclass
+from operator import attrgetter
 from typing import List, Optional, Sequence
 
 import torch
@@ -56,6 +57,10 @@ class CScratch(C.Structure):
     _fields_ = [(n, _p) for n in ("csa_mx", "csa_s", "csa_acc_kv", "csa_acc_ik", "hca_mx", "hca_s", "hca_acc_kv",
                                   "new_csa_kv", "new_csa_ik", "new_hca_kv", "csa_done", "hca_done")]
 
+
+_CACHE_FIELDS = attrgetter(*CACHE_TENSORS)
+_NODE_FIELDS = attrgetter(*[n for n, _ in CNodes._fields_])
+_SCRATCH_FIELDS = attrgetter(*[n for n, _ in CScratch._fields_])
 
 _lib.tsv_version.restype = C.c_int
 _lib.tsv_kernel_launches.restype = C.c_uint64
@@ -105,18 +110,15 @@ def _stream(stream) -> int:
     return (torch.cuda.current_stream() if stream is None else stream).cuda_stream
 
 
-class _Versioned:
-    """Counts the assignments to an object's fields, so that what was built from them can tell that it is out of date."""
-    _version = 0
-
-    def __setattr__(self, name, value):
-        d = self.__dict__
-        d[name] = value
-        d["_version"] = d.get("_version", 0) + 1
+def _pointers(get, obj) -> List[Optional[int]]:
+    """Device pointers of the tensors that `get` (an attrgetter) takes from obj, as they are now."""
+    return [None if t is None else t.data_ptr() for t in get(obj)]
 
 
+# The device structs of a layer.  words() gives the values of the C struct's fields, read from the tensors as they are at that
+# moment; struct() makes the struct from them.
 @dataclass
-class LayerCache(_Versioned):
+class LayerCache:
     """Persistent per-layer state (device tensors); rows of sequence b start at *_row0[b]."""
     L: torch.Tensor
     csa_kv: torch.Tensor
@@ -137,11 +139,14 @@ class LayerCache(_Versioned):
     page_table: Optional[torch.Tensor] = None      # [B, max_pages] int32: paged pool (csa_row0 / hca_row0 unused then)
     page_tokens: int = 0
 
-    def struct(self) -> CCache:
+    def words(self) -> list:
+        w = _pointers(_CACHE_FIELDS, self)
         pt = self.page_table
-        return CCache(*[_ptr(getattr(self, n)) for n in CACHE_TENSORS], int(self.csa_kv.shape[0]), int(self.hca_kv.shape[0]),
-                      _ptr(pt), int(self.page_tokens), 0 if pt is None else int(pt.shape[1]),
-                      0 if pt is None else int(self.win_kv.shape[0]))
+        w += [self.csa_kv.shape[0], self.hca_kv.shape[0]]
+        return w + ([None, int(self.page_tokens), 0, 0] if pt is None else [pt.data_ptr(), int(self.page_tokens), pt.shape[1], self.win_kv.shape[0]])
+
+    def struct(self) -> CCache:
+        return CCache(*self.words())
 
     def clone(self) -> "LayerCache":
         return LayerCache(*[getattr(self, n).clone() for n in CACHE_TENSORS], page_table=self.page_table, page_tokens=self.page_tokens)
@@ -168,7 +173,7 @@ class LayerCache(_Versioned):
 
 
 @dataclass
-class NodeInputs(_Versioned):
+class NodeInputs:
     q: torch.Tensor
     kv: torch.Tensor
     c_csa: torch.Tensor
@@ -181,12 +186,15 @@ class NodeInputs(_Versioned):
     parent: torch.Tensor
     n_nodes: torch.Tensor
 
+    def words(self) -> list:
+        return _pointers(_NODE_FIELDS, self)
+
     def struct(self) -> CNodes:
-        return CNodes(*[_ptr(getattr(self, n)) for n, _ in CNodes._fields_])
+        return CNodes(*self.words())
 
 
 @dataclass
-class Scratch(_Versioned):
+class Scratch:
     csa_mx: torch.Tensor
     csa_s: torch.Tensor
     csa_acc_kv: torch.Tensor
@@ -200,8 +208,11 @@ class Scratch(_Versioned):
     csa_done: torch.Tensor
     hca_done: torch.Tensor
 
+    def words(self) -> list:
+        return _pointers(_SCRATCH_FIELDS, self)
+
     def struct(self) -> CScratch:
-        return CScratch(*[_ptr(getattr(self, n)) for n, _ in CScratch._fields_])
+        return CScratch(*self.words())
 
 
 def alloc_cache(shape: synth.Shape, csa_caps: Sequence[int], hca_caps: Sequence[int], device="cuda") -> LayerCache:
@@ -327,22 +338,16 @@ class LayerPack:
     def __init__(self, caches: List[LayerCache], nodes: List[NodeInputs], scratch: List[Scratch]):
         n = len(caches)
         self.n = n
-        objs = (*caches, *nodes, *scratch)
-        self._ids, self._version = [id(x) for x in objs], sum(x._version for x in objs)
-        self._tensors = [t for x in objs for t in x.__dict__.values() if isinstance(t, torch.Tensor)]
-        self._ptrs = [t.data_ptr() for t in self._tensors]
+        self._words = [x.words() for x in (*caches, *nodes, *scratch)]
         self._keep = ([c.struct() for c in caches], [x.struct() for x in nodes], [s.struct() for s in scratch])
         self.caches = (C.POINTER(CCache) * n)(*[C.pointer(x) for x in self._keep[0]])
         self.nodes = (C.POINTER(CNodes) * n)(*[C.pointer(x) for x in self._keep[1]])
         self.scratch = (C.POINTER(CScratch) * n)(*[C.pointer(x) for x in self._keep[2]])
 
-
     def current(self, caches: List[LayerCache], nodes: List[NodeInputs], scratch: List[Scratch]) -> bool:
-        """Whether the arrays still describe these objects: the same ones, no field assigned since, no tensor's storage
-        exchanged in place."""
-        objs = (*caches, *nodes, *scratch)
-        return (self._version == sum([x._version for x in objs]) and self._ids == [id(x) for x in objs]
-                and self._ptrs == [t.data_ptr() for t in self._tensors])
+        """Whether the arrays describe these objects as they are now (compared by value: an object may stand at the address of
+        one that is gone)."""
+        return self._words == [x.words() for x in (*caches, *nodes, *scratch)]
 
 
 _lib.tsv_verify_cycle.restype = C.c_int

@@ -29,3 +29,16 @@ def test_layer_pack_follows_its_objects():
     assert not pack.current(caches, inp.layers, scratch)
     pack = tsv.LayerPack(caches, inp.layers, scratch)
     assert not pack.current(caches, inp.layers, [tsv.alloc_scratch(sh, "cpu")])      # another object
+
+
+def test_layer_pack_notices_an_object_at_the_address_of_another():
+    from paper_2609_24698_b200 import binding as tsv, harness as hz
+    sh = synth.Shape("fp32", 2, 5, 4, 16, 2, 4, 1, 8, 4, 8)
+    scratch, inp = [tsv.alloc_scratch(sh, "cpu")], hz.InputSet.empty(sh, 1, "cpu")
+    caches = [tsv.alloc_cache(sh, [8, 8], [4, 4], "cpu")]
+    for _ in range(20):
+        pack = tsv.LayerPack(caches, inp.layers, scratch)
+        tensors = {n: getattr(caches[0], n).clone() for n in tsv.CACHE_TENSORS}
+        caches.clear()
+        caches.append(tsv.LayerCache(**tensors))             # (takes the place the allocator has just got back)
+        assert not pack.current(caches, inp.layers, scratch)
