@@ -15,9 +15,8 @@
  *     work is enqueued on `stream` and the call returns.  Between calls it keeps nothing of the
  *     caller's data; what it does keep per process is set-up it does once (kernel attributes,
  *     the number of CTA pairs a device holds, the driver entry point for tensor maps), the
- *     launch counter behind tsv_kernel_launches(), for tree_verify_attn_static the
- *     address of its built-in array, and per calling thread a bounded number of encoded tensor
- *     maps, found again by the addresses and sizes they were made from.
+ *     launch counter behind tsv_kernel_launches(), and for tree_verify_attn_static the
+ *     address of its built-in array.
  *   - Stream order: the calls of a layer run in the order given above on one stream.  The kernels are
  *     launched as programmatic dependents; those of branch_state_build and accept_and_refresh wait for
  *     all earlier work before they do anything.  Some kernels of tree_verify_attn start earlier: the part

@@ -18,7 +18,6 @@
 // Stage stream, TMEM column plan, running-max rule and chunking are those described at the kernel.
 #include <cuda.h>
 #include <stdio.h>
-#include <string.h>
 #include <cudaTypedefs.h>
 
 #include <atomic>
@@ -950,20 +949,8 @@ int prepare_tva_tc_pair(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c
   const bool has_hca = c.hca_rows > 0 && c.hca_kv;
   const void* bases[4] = {c.csa_kv, has_hca ? c.hca_kv : c.csa_kv, c.win_kv, ws + p.off_misc};
   const int64_t rows[4] = {c.csa_rows, has_hca ? c.hca_rows : c.csa_rows, c.page_table ? c.tok_rows : (int64_t)s.B * s.window, (int64_t)s.B * p.tc_misc_rows};
-  // The maps depend on these words alone.  A program calls with the same few sets (a layer, an input slot) over and over, and
-  // encoding twenty maps costs a call 5 us of host time: the last sets are kept, per thread, a small fixed number of them.
-  const uint64_t key[14] = {(uint64_t)bases[0], (uint64_t)bases[1], (uint64_t)bases[2], (uint64_t)bases[3], (uint64_t)rows[0], (uint64_t)rows[1], (uint64_t)rows[2],
-                            (uint64_t)rows[3], (uint64_t)nd.q, (uint64_t)out, (uint64_t)(ws + p.off_tpo), (uint64_t)s.B << 32 | (uint32_t)(s.D * s.H),
-                            (uint64_t)p.tc_nt << 32 | (uint32_t)p.tc_chmax, (uint64_t)p.tc_split};
-  struct Kept { uint64_t key[14]; bool valid; alignas(64) pair::MapSet maps; };
-  constexpr int kKept = 32;
-  static thread_local Kept kept[kKept];
-  uint64_t hash = 0;
-  for (uint64_t v : key) { hash = (hash ^ v) * 0x9E3779B97F4A7C15ull; hash ^= hash >> 29; }
-  Kept& slot = kept[hash % kKept];
-  if (slot.valid && memcmp(slot.key, key, sizeof(key)) == 0) { prep.maps = &slot.maps; return TSV_OK; }
-  slot.valid = false;
-  pair::MapSet& ms = slot.maps;
+  static_assert(sizeof(pair::MapSet) == sizeof(prep.maps), "TvaTcPrep holds a MapSet");
+  pair::MapSet& ms = *reinterpret_cast<pair::MapSet*>(prep.maps);
   bool ok = make_map(&ms.q, nd.q, (int64_t)s.B * s.D * s.H, 128) && make_map(&ms.out, out, (int64_t)s.B * s.D * s.H, 32);
   for (int a = 0; a < 4 && ok; ++a) {
     for (int k = 0; k < 3 && ok; ++k) ok = make_map(&ms.src[a][k], bases[a], rows[a], 32 << k);
@@ -986,14 +973,11 @@ int prepare_tva_tc_pair(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c
   }
   TSV_PREP(tc_attn_pair_kernel<true>);
   TSV_PREP(tc_attn_pair_kernel<false>);
-  memcpy(slot.key, key, sizeof(key));
-  slot.valid = true;
-  prep.maps = &slot.maps;
   return TSV_OK;
 }
 
 int launch_tva_tc_pair(const tsv_shape& s, const TvaPlan& p, const TvaTcPrep& prep, bool general, void* out, char* ws, int32_t* status, cudaStream_t st) {
-  const pair::MapSet& ms = *static_cast<const pair::MapSet*>(prep.maps);
+  const pair::MapSet& ms = *reinterpret_cast<const pair::MapSet*>(prep.maps);
   cudaLaunchConfig_t cfg = {};
   const int64_t most = (int64_t)p.tc_nt * s.B * p.tc_chmax;                 // items, if every tile had the most chunks
   cfg.blockDim = dim3(pair::TTHREADS, 1, 1);
