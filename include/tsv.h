@@ -7,6 +7,8 @@
  *     for every layer:  branch_state_build(...)  ->  tree_verify_attn(...)
  *     then once:        accept_and_refresh(all layers)
  *
+ * tree_verify_layer(...) is the first two in one call.
+ *
  * Conventions
  *   - Every `void*` / typed pointer inside the structs is a DEVICE pointer unless the
  *     comment says HOST.  The structs themselves and `tsv_shape` live in HOST memory and
@@ -19,7 +21,8 @@
  *     address of its built-in array.
  *   - Stream order: the calls of a layer run in the order given above on one stream.  The kernels are
  *     launched as programmatic dependents; those of branch_state_build and accept_and_refresh wait for
- *     all earlier work before they do anything.  Some kernels of tree_verify_attn start earlier: the part
+ *     all earlier work before they do anything (tree_verify_layer begins with branch_state_build's).  Some kernels of
+ *     tree_verify_attn start earlier: the part
  *     of them that reads only the call's inputs (tsv_nodes, the committed tsv_cache) may run before the kernel before them
  *     has finished, and that part already writes the call's workspace, topk_idx and status; they wait for
  *     it before they read anything the library's own kernels write.  For the caller this matters in one
@@ -39,14 +42,15 @@
  *   - Node n of sequence b sits at depth delta_n (root = node 0 = depth 0) and at position
  *     p_n = L[b] + delta_n.  n_csa = L / m_csa and n_hca = L / m_hca committed entries.
  *   - Return value: 0 or a negative TSV_ERR_* for problems the host can see BEFORE any
- *     launch (nothing is enqueued then: argument checks, tensor-map encoding and kernel
- *     attributes all precede the first launch).  Only a failing kernel launch itself
- *     (TSV_ERR_CUDA out of cudaLaunchKernel) can leave earlier kernels of the same call
+ *     launch (nothing is enqueued then: argument checks, and on the tensor-core path the tensor maps
+ *     and the attributes of its kernels, all precede the first launch).  Only TSV_ERR_CUDA out of a
+ *     kernel launch itself, or out of a later kernel's attributes, can leave earlier kernels of the same call
  *     enqueued; skip accept_and_refresh for that cycle then.  Problems only the device can see (bad parent
  *     array, node count, capacity, length) are reported per sequence in `status[b]`
  *     (bit-or of TSV_ST_*): that sequence's outputs are zero-filled and
  *     accept_and_refresh commits nothing for it (L unchanged).  `status` is or-ed into, never
- *     cleared: zero it at the start of a cycle.  No kernel traps or waits without a bound.
+ *     cleared: zero it at the start of a cycle
+ *     (or let tree_verify_layer of the first layer do it).  No kernel traps or waits without a bound.
  */
 #ifndef TSV_H_
 #define TSV_H_
@@ -238,6 +242,17 @@ int branch_state_build(const tsv_shape *shape, const tsv_cache *cache, const tsv
 int tree_verify_attn(const tsv_shape *shape, const tsv_cache *cache, const tsv_nodes *nodes,
                      const tsv_scratch *scratch, void *out, int32_t *topk_idx,
                      void *workspace, size_t workspace_bytes, int32_t *status, void *stream);
+
+/*
+ * tree_verify_layer -- branch_state_build and then tree_verify_attn of one layer in one call: the call of a model's layer.
+ * Arguments, results and status handling are theirs; and what the two calls cannot know of each other is used: on the
+ * tensor-core path the state build leaves the entries closed inside the tree in `workspace` as the attention reads them too.
+ * first     non-zero for the first layer of a cycle: `status` is written (0 for a usable sequence) instead of or-ed into, so
+ *           that the caller need not zero it.
+ */
+int tree_verify_layer(const tsv_shape *shape, const tsv_cache *cache, const tsv_nodes *nodes,
+                      const tsv_scratch *scratch, void *out, int32_t *topk_idx,
+                      void *workspace, size_t workspace_bytes, int32_t first, int32_t *status, void *stream);
 
 /*
  * accept_and_refresh -- accepted-path state refresh (Sections "Compressed-State Consistency and

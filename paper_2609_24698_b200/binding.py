@@ -74,8 +74,10 @@ _lib.tree_verify_attn.restype = C.c_int
 _lib.tree_verify_attn.argtypes = [C.POINTER(CShape), C.POINTER(CCache), C.POINTER(CNodes), C.POINTER(CScratch),
                                   _p, _p, _p, C.c_size_t, _p, _p]
 _lib.accept_and_refresh.restype = C.c_int
-_lib.accept_and_refresh.argtypes = [C.POINTER(CShape), C.c_int32, C.POINTER(C.POINTER(CCache)), C.POINTER(C.POINTER(CNodes)),
-                                    C.POINTER(C.POINTER(CScratch)), _p, _p, _p, _p, _p, _p, _p]
+_lib.accept_and_refresh.argtypes = [C.POINTER(CShape), C.c_int32, _p, _p, _p, _p, _p, _p, _p, _p, _p, _p]      # (three HOST arrays of struct pointers)
+_lib.tree_verify_layer.restype = C.c_int
+_lib.tree_verify_layer.argtypes = [C.POINTER(CShape), C.POINTER(CCache), C.POINTER(CNodes), C.POINTER(CScratch),
+                                   _p, _p, _p, C.c_size_t, C.c_int32, _p, _p]
 
 
 class TsvError(RuntimeError):
@@ -313,6 +315,30 @@ def tree_verify_attn(shape: CShape, cache: LayerCache, nodes: NodeInputs, scratc
         raise TsvError(r, "tree_verify_attn")
 
 
+class LayerStructs:
+    """The C structs of a layer's cache and scratch pad, made once and used until their tensors change."""
+
+    def __init__(self):
+        self._words = None
+
+    def update(self, cache: LayerCache, scratch: Scratch) -> "LayerStructs":
+        words = cache.words() + scratch.words()
+        if words != self._words:
+            self.cache, self.scratch = cache.struct(), scratch.struct()
+            self._words = words
+        return self
+
+
+def tree_verify_layer(shape: CShape, layer: LayerStructs, nodes: CNodes, out: torch.Tensor, topk_idx: Optional[torch.Tensor],
+                      workspace: torch.Tensor, first: bool, status: torch.Tensor, stream=None) -> None:
+    """branch_state_build and tree_verify_attn of one layer in one call; first: `status` is cleared by it."""
+    wp, wn = _aligned(workspace)
+    r = _lib.tree_verify_layer(C.byref(shape), C.byref(layer.cache), C.byref(nodes), C.byref(layer.scratch), _ptr(out), _ptr(topk_idx), wp, wn,
+                               first, _ptr(status), _stream(stream))
+    if r:
+        raise TsvError(r, "tree_verify_layer")
+
+
 _lib.tsv_bench_tree_verify_attn_stages.restype = C.c_int
 _lib.tsv_bench_tree_verify_attn_stages.argtypes = [C.POINTER(CShape), C.POINTER(CCache), C.POINTER(CNodes), C.POINTER(CScratch),
                                                    _p, _p, _p, C.c_size_t, _p, _p, C.c_int]
@@ -333,41 +359,27 @@ def bench_tree_verify_attn_stages(shape: CShape, cache: LayerCache, nodes: NodeI
 
 
 class LayerPack:
-    """Host arrays of per-layer struct pointers for the calls over all layers, built once and reused."""
+    """Host arrays of per-layer struct pointers for accept_and_refresh."""
 
     def __init__(self, caches: List[LayerCache], nodes: List[NodeInputs], scratch: List[Scratch]):
-        n = len(caches)
-        self.n = n
         self._words = [x.words() for x in (*caches, *nodes, *scratch)]
-        self._keep = ([c.struct() for c in caches], [x.struct() for x in nodes], [s.struct() for s in scratch])
-        self.caches = (C.POINTER(CCache) * n)(*[C.pointer(x) for x in self._keep[0]])
-        self.nodes = (C.POINTER(CNodes) * n)(*[C.pointer(x) for x in self._keep[1]])
-        self.scratch = (C.POINTER(CScratch) * n)(*[C.pointer(x) for x in self._keep[2]])
+        self._set([c.struct() for c in caches], [x.struct() for x in nodes], [s.struct() for s in scratch])
+
+    @classmethod
+    def of_structs(cls, layers: List["LayerStructs"], nodes: List[CNodes]) -> "LayerPack":
+        p = cls.__new__(cls)
+        p._words = None
+        p._set([x.cache for x in layers], nodes, [x.scratch for x in layers])
+        return p
+
+    def _set(self, *structs) -> None:
+        self.n, self._keep = len(structs[0]), structs
+        self.caches, self.nodes, self.scratch = [(_p * self.n)(*map(C.addressof, x)) for x in structs]
 
     def current(self, caches: List[LayerCache], nodes: List[NodeInputs], scratch: List[Scratch]) -> bool:
         """Whether the arrays describe these objects as they are now (compared by value: an object may stand at the address of
         one that is gone)."""
         return self._words == [x.words() for x in (*caches, *nodes, *scratch)]
-
-
-_lib.tsv_verify_cycle.restype = C.c_int
-_lib.tsv_verify_cycle.argtypes = [C.POINTER(CShape), C.c_int32, C.POINTER(C.POINTER(CCache)), C.POINTER(C.POINTER(CNodes)),
-                                  C.POINTER(C.POINTER(CScratch)), C.POINTER(_p), C.POINTER(_p), _p, C.c_size_t, _p, _p, _p, _p, _p, _p, _p]
-
-
-def verify_cycle(shape: CShape, pack: LayerPack, out: Optional[List[torch.Tensor]], topk_idx: List[Optional[torch.Tensor]],
-                 workspace: torch.Tensor, refresh, status: torch.Tensor, stream=None) -> None:
-    """One whole cycle in ONE call (an export of the library outside its public header): status cleared, per layer
-    branch_state_build and (out given) tree_verify_attn, then (refresh = draft, target, accept_len, accept_path, bonus given)
-    accept_and_refresh.  The same kernels in the same order as the separate calls."""
-    n = pack.n
-    wp, wn = _aligned(workspace)
-    outs = (_p * n)(*[t.data_ptr() for t in out]) if out is not None else None
-    topk = (_p * n)(*[_ptr(t) for t in topk_idx]) if any(t is not None for t in topk_idx) else None
-    rf = [t.data_ptr() for t in refresh] if refresh is not None else [None] * 5
-    r = _lib.tsv_verify_cycle(C.byref(shape), n, pack.caches, pack.nodes, pack.scratch, outs, topk, wp, wn, *rf, _ptr(status), _stream(stream))
-    if r:
-        raise TsvError(r, "tsv_verify_cycle")
 
 
 def accept_and_refresh(shape: CShape, pack: LayerPack, draft_tok: torch.Tensor, target_tok: torch.Tensor,

@@ -158,15 +158,20 @@ static int check_scratch(const tsv_scratch* s) {
   return TSV_OK;
 }
 
-// tree_verify_attn after validation.  All host work that can fail (tensor maps, kernel attributes) comes before the
-// first launch, so a negative return means that nothing was enqueued by this call, unless a launch itself fails.
+// tree_verify_attn after validation, with the layer's state build in front of it where `build` asks for it.  The tensor maps and
+// attributes of the tensor-core path come before the first launch.
+enum class Build { none, any_layer, first_layer };    // first_layer: the state build writes the status, others or into it
 static int tva_stages(const tsv_shape& s, const TvaPlan& p_in, const tsv_cache& c, const tsv_nodes& nd, const tsv_scratch& sc, void* out,
-                      int32_t* topk_idx, char* ws, int32_t* status, cudaStream_t st, int stages) {
+                      int32_t* topk_idx, char* ws, int32_t* status, cudaStream_t st, int stages, Build build = Build::none) {
   int r;
   TvaTcPrep prep;
   TvaPlan p = p_in;
   if (p.tc && !tva_tc_pair_usable(c)) p.tc = 0;       // no row counts for the tensor maps: the CUDA-core path (same workspace)
   if (p.tc && (stages & 6) && (r = prepare_tva_tc(s, p, c, nd, out, ws, prep))) return r;
+  if (build != Build::none) {
+    p.tc_packed = p.tc;                               // the attention that follows finds the new entries packed
+    if ((r = launch_bsb(s, c, nd, sc, status, build == Build::first_layer, p.tc_packed ? ws + p.off_misc : nullptr, p.tc_misc_rows, st))) return r;
+  }
   if ((stages & 1) && (r = launch_tva_select(s, p, c, nd, sc, topk_idx, ws, status, st))) return r;
   if (!(stages & 6)) return TSV_OK;
   if (p.tc) return launch_tva_tc(s, p, prep, c, nd, sc, out, ws, status, st, (stages & 2) != 0);
@@ -213,8 +218,8 @@ int branch_state_build(const tsv_shape* shape, const tsv_cache* cache, const tsv
   return launch_bsb(resolved(shape), *cache, *nodes, *scratch, status, false, nullptr, 0, (cudaStream_t)stream);
 }
 
-int tree_verify_attn(const tsv_shape* shape, const tsv_cache* cache, const tsv_nodes* nodes, const tsv_scratch* scratch,
-                     void* out, int32_t* topk_idx, void* workspace, size_t workspace_bytes, int32_t* status, void* stream) {
+static int checked_stages(const tsv_shape* shape, const tsv_cache* cache, const tsv_nodes* nodes, const tsv_scratch* scratch, void* out,
+                          int32_t* topk_idx, void* workspace, size_t workspace_bytes, int32_t* status, void* stream, int stages, Build build) {
   if (!shape || !status || !out) return TSV_ERR_NULL;
   if (!shape_ok(shape)) return TSV_ERR_SHAPE;
   int r;
@@ -224,7 +229,18 @@ int tree_verify_attn(const tsv_shape* shape, const tsv_cache* cache, const tsv_n
   TvaPlan p;
   make_tva_plan(s, p);
   if (!workspace || ((uintptr_t)workspace & 255) || workspace_bytes < p.total) return TSV_ERR_WORKSPACE;
-  return tva_stages(s, p, *cache, *nodes, *scratch, out, topk_idx, (char*)workspace, status, (cudaStream_t)stream, 3);
+  return tva_stages(s, p, *cache, *nodes, *scratch, out, topk_idx, (char*)workspace, status, (cudaStream_t)stream, stages, build);
+}
+
+int tree_verify_attn(const tsv_shape* shape, const tsv_cache* cache, const tsv_nodes* nodes, const tsv_scratch* scratch,
+                     void* out, int32_t* topk_idx, void* workspace, size_t workspace_bytes, int32_t* status, void* stream) {
+  return checked_stages(shape, cache, nodes, scratch, out, topk_idx, workspace, workspace_bytes, status, stream, 3, Build::none);
+}
+
+int tree_verify_layer(const tsv_shape* shape, const tsv_cache* cache, const tsv_nodes* nodes, const tsv_scratch* scratch,
+                      void* out, int32_t* topk_idx, void* workspace, size_t workspace_bytes, int32_t first, int32_t* status, void* stream) {
+  return checked_stages(shape, cache, nodes, scratch, out, topk_idx, workspace, workspace_bytes, status, stream, 3,
+                        first ? Build::first_layer : Build::any_layer);
 }
 
 // Not part of the public interface (not declared in tsv.h): tree_verify_attn restricted to some of its stages, for
@@ -235,16 +251,7 @@ int tree_verify_attn(const tsv_shape* shape, const tsv_cache* cache, const tsv_n
 int tsv_bench_tree_verify_attn_stages(const tsv_shape* shape, const tsv_cache* cache, const tsv_nodes* nodes, const tsv_scratch* scratch,
                                       void* out, int32_t* topk_idx, void* workspace, size_t workspace_bytes, int32_t* status, void* stream,
                                       int stages) {
-  if (!shape || !status || !out) return TSV_ERR_NULL;
-  if (!shape_ok(shape)) return TSV_ERR_SHAPE;
-  int r;
-  if ((r = check_cache(cache, shape)) || (r = check_nodes(nodes, true)) || (r = check_scratch(scratch))) return r;
-  if (!al16(out)) return TSV_ERR_ALIGN;
-  const tsv_shape s = resolved(shape);
-  TvaPlan p;
-  make_tva_plan(s, p);
-  if (!workspace || ((uintptr_t)workspace & 255) || workspace_bytes < p.total) return TSV_ERR_WORKSPACE;
-  return tva_stages(s, p, *cache, *nodes, *scratch, out, topk_idx, (char*)workspace, status, (cudaStream_t)stream, stages & 7);
+  return checked_stages(shape, cache, nodes, scratch, out, topk_idx, workspace, workspace_bytes, status, stream, stages & 7, Build::none);
 }
 
 int accept_and_refresh(const tsv_shape* shape, int32_t n_layers, const tsv_cache* const* caches, const tsv_nodes* const* nodes,
@@ -259,42 +266,6 @@ int accept_and_refresh(const tsv_shape* shape, int32_t n_layers, const tsv_cache
     if ((r = check_cache(caches[l], shape)) || (r = check_nodes(nodes[l], false)) || (r = check_scratch(scratch[l]))) return r;
   return launch_aar(resolved(shape), n_layers, caches, nodes, scratch, nodes[0]->parent, nodes[0]->n_nodes, draft_tok, target_tok, accept_len,
                     accept_path, bonus_tok, status, (cudaStream_t)stream);
-}
-
-// Not part of the public interface (not declared in tsv.h): a whole cycle in one call, for a host loop that launches eagerly.
-// Clears `status` (the first layer's state build writes it), then per layer branch_state_build and, unless `out` is NULL,
-// tree_verify_attn, then, unless `draft_tok` is NULL, accept_and_refresh: the kernels of the separate calls in their order.
-// out / topk_idx: HOST arrays of n_layers device pointers (topk_idx, or its entries, may be NULL).
-int tsv_verify_cycle(const tsv_shape* shape, int32_t n_layers, const tsv_cache* const* caches, const tsv_nodes* const* nodes,
-                     const tsv_scratch* const* scratch, void* const* out, int32_t* const* topk_idx, void* workspace, size_t workspace_bytes,
-                     const int32_t* draft_tok, const int32_t* target_tok, int32_t* accept_len, int32_t* accept_path, int32_t* bonus_tok,
-                     int32_t* status, void* stream) {
-  if (!shape || !caches || !nodes || !scratch || !status) return TSV_ERR_NULL;
-  if (draft_tok && (!target_tok || !accept_len || !accept_path || !bonus_tok)) return TSV_ERR_NULL;
-  if (!shape_ok(shape)) return TSV_ERR_SHAPE;
-  if (n_layers < 1 || n_layers > 4096) return TSV_ERR_SHAPE;
-  int r;
-  for (int l = 0; l < n_layers; ++l) {
-    if ((r = check_cache(caches[l], shape)) || (r = check_nodes(nodes[l], out != nullptr)) || (r = check_scratch(scratch[l]))) return r;
-    if (out && !out[l]) return TSV_ERR_NULL;
-    if (out && !al16(out[l])) return TSV_ERR_ALIGN;
-  }
-  const tsv_shape s = resolved(shape);
-  const cudaStream_t st = (cudaStream_t)stream;
-  TvaPlan p = {};
-  if (out) {
-    make_tva_plan(s, p);
-    if (!workspace || ((uintptr_t)workspace & 255) || workspace_bytes < p.total) return TSV_ERR_WORKSPACE;
-  }
-  for (int l = 0; l < n_layers; ++l) {
-    p.tc_packed = out && p.tc && tva_tc_pair_usable(*caches[l]);       // the attention that follows finds the new entries packed
-    if ((r = launch_bsb(s, *caches[l], *nodes[l], *scratch[l], status, l == 0, p.tc_packed ? (char*)workspace + p.off_misc : nullptr,
-                        p.tc_misc_rows, st))) return r;
-    if (out && (r = tva_stages(s, p, *caches[l], *nodes[l], *scratch[l], out[l], topk_idx ? topk_idx[l] : nullptr, (char*)workspace, status, st, 3))) return r;
-  }
-  if (!draft_tok) return TSV_OK;
-  return launch_aar(s, n_layers, caches, nodes, scratch, nodes[0]->parent, nodes[0]->n_nodes, draft_tok, target_tok, accept_len, accept_path,
-                    bonus_tok, status, st);
 }
 
 }  // extern "C"

@@ -1,13 +1,12 @@
 """Verify-cycle driver over the C-ABI binding: device buffers, stream-ordered calls, graph replay.
 
 Nothing here computes anything of the method; it owns tensors and issues, per cycle,
-    for each layer: branch_state_build -> tree_verify_attn
+    for each layer: tree_verify_layer (branch_state_build -> tree_verify_attn)
     then:           accept_and_refresh(all layers)
 on one CUDA stream with no host synchronisation in between.
 """
 from __future__ import annotations
 
-import weakref
 from typing import Dict, List, Optional, Sequence
 
 import numpy as np
@@ -137,24 +136,33 @@ class VerifyEngine:
         self.accept_len = torch.zeros(B, **i32)
         self.accept_path = torch.zeros(B, D, **i32)
         self.bonus = torch.zeros(B, **i32)
-        # pointer packs per input set; weak keys: an entry must die with its input set (an id() key could be reused by a
-        # later input set and hand accept_and_refresh the pointers of freed tensors)
-        self._packs = weakref.WeakKeyDictionary()
+        self._structs = [tsv.LayerStructs() for _ in range(n_layers)]
+
+    def _layer(self, l: int) -> tsv.LayerStructs:
+        return self._structs[l].update(self.caches[l], self.scratch[l])
 
     def _pack(self, inp: InputSet) -> tsv.LayerPack:
-        p = self._packs.get(inp)
-        if p is None or not p.current(self.caches, inp.layers, self.scratch):
-            p = self._packs[inp] = tsv.LayerPack(self.caches, inp.layers, self.scratch)
-        return p
+        return tsv.LayerPack.of_structs([self._layer(l) for l in range(self.n_layers)], [nd.struct() for nd in inp.layers])
 
     def launch_cycle(self, inp: InputSet, attention: bool = True, refresh: bool = True) -> None:
         """Enqueue one verify cycle on the current stream (no host sync)."""
-        tsv.verify_cycle(self.cshape, self._pack(inp), self.out if attention else None, self.topk_idx, self.workspace,
-                         (inp.draft, inp.target, self.accept_len, self.accept_path, self.bonus) if refresh else None, self.status)
+        stream = torch.cuda.current_stream()
+        if not attention:
+            self.status.zero_()
+        layers, nodes = [], []
+        for l in range(self.n_layers):                  # (a layer's structs just before its call: the first kernels run meanwhile)
+            layers.append(self._layer(l))
+            nodes.append(inp.layers[l].struct())
+            if attention:
+                tsv.tree_verify_layer(self.cshape, layers[l], nodes[l], self.out[l], self.topk_idx[l], self.workspace, l == 0, self.status, stream)
+            else:
+                tsv.branch_state_build(self.cshape, self.caches[l], inp.layers[l], self.scratch[l], self.status, stream)
+        if refresh:
+            tsv.accept_and_refresh(self.cshape, tsv.LayerPack.of_structs(layers, nodes), inp.draft, inp.target, self.accept_len, self.accept_path,
+                                   self.bonus, self.status, stream)
 
     def capture(self, inp: InputSet) -> torch.cuda.CUDAGraph:
         """Capture one cycle over `inp` into a CUDA graph (the launch sequence is shape-stable)."""
-        self._pack(inp)
         s = torch.cuda.Stream()
         s.wait_stream(torch.cuda.current_stream())
         g = torch.cuda.CUDAGraph()

@@ -20,3 +20,14 @@ def test_library_keeps_no_tables_per_thread():
     nothing, has next to none (tensor maps were kept there once, 90 KB, found again by the addresses of a call's inputs)."""
     from paper_2609_24698_b200.build import build_library
     assert _tls_bytes(build_library()) <= 4096
+
+
+def test_every_exported_call_is_declared():
+    """What a caller can reach stands in tsv.h, but for the benchmark's stage timer."""
+    import subprocess
+    from paper_2609_24698_b200.build import build_library
+    from tests.test_abi import declared_functions
+    out = subprocess.run(["nm", "-D", "--defined-only", build_library()], capture_output=True, text=True, check=True).stdout
+    exported = {line.split()[-1] for line in out.splitlines() if " T " in line}
+    c_names = {n for n in exported if not n.startswith("_")}
+    assert c_names - set(declared_functions()) == {"tsv_bench_tree_verify_attn_stages"}
