@@ -10,7 +10,8 @@ import ctypes as C
 import os
 from dataclasses import dataclass
 from operator import attrgetter
-from typing import List, Optional, Sequence
+from struct import Struct
+from typing import List, Optional, Sequence, Tuple
 
 import torch
 
@@ -61,6 +62,7 @@ class CScratch(C.Structure):
 _CACHE_FIELDS = attrgetter(*CACHE_TENSORS)
 _NODE_FIELDS = attrgetter(*[n for n, _ in CNodes._fields_])
 _SCRATCH_FIELDS = attrgetter(*[n for n, _ in CScratch._fields_])
+_fill_nodes = Struct(f"{len(CNodes._fields_)}P").pack_into
 
 _lib.tsv_version.restype = C.c_int
 _lib.tsv_kernel_launches.restype = C.c_uint64
@@ -74,10 +76,9 @@ _lib.tree_verify_attn.restype = C.c_int
 _lib.tree_verify_attn.argtypes = [C.POINTER(CShape), C.POINTER(CCache), C.POINTER(CNodes), C.POINTER(CScratch),
                                   _p, _p, _p, C.c_size_t, _p, _p]
 _lib.accept_and_refresh.restype = C.c_int
-_lib.accept_and_refresh.argtypes = [C.POINTER(CShape), C.c_int32, _p, _p, _p, _p, _p, _p, _p, _p, _p, _p]      # (three HOST arrays of struct pointers)
+_lib.accept_and_refresh.argtypes = [_p, C.c_int32, _p, _p, _p, _p, _p, _p, _p, _p, _p, _p]      # (three HOST arrays of struct pointers)
 _lib.tree_verify_layer.restype = C.c_int
-_lib.tree_verify_layer.argtypes = [C.POINTER(CShape), C.POINTER(CCache), C.POINTER(CNodes), C.POINTER(CScratch),
-                                   _p, _p, _p, C.c_size_t, C.c_int32, _p, _p]
+_lib.tree_verify_layer.argtypes = [_p, _p, _p, _p, _p, _p, _p, C.c_size_t, C.c_int32, _p, _p]
 
 
 class TsvError(RuntimeError):
@@ -112,9 +113,15 @@ def _stream(stream) -> int:
     return (torch.cuda.current_stream() if stream is None else stream).cuda_stream
 
 
-def _pointers(get, obj) -> List[Optional[int]]:
-    """Device pointers of the tensors that `get` (an attrgetter) takes from obj, as they are now."""
-    return [None if t is None else t.data_ptr() for t in get(obj)]
+_data_ptr = torch.Tensor.data_ptr
+
+
+def _pointers(tensors) -> List[int]:
+    """Device pointers of the tensors, as they are now."""
+    try:
+        return list(map(_data_ptr, tensors))
+    except TypeError:                                  # (an optional one is None)
+        return [0 if t is None else t.data_ptr() for t in tensors]
 
 
 # The device structs of a layer.  words() gives the values of the C struct's fields, read from the tensors as they are at that
@@ -142,10 +149,10 @@ class LayerCache:
     page_tokens: int = 0
 
     def words(self) -> list:
-        w = _pointers(_CACHE_FIELDS, self)
+        w = _pointers(_CACHE_FIELDS(self))
         pt = self.page_table
         w += [self.csa_kv.shape[0], self.hca_kv.shape[0]]
-        return w + ([None, int(self.page_tokens), 0, 0] if pt is None else [pt.data_ptr(), int(self.page_tokens), pt.shape[1], self.win_kv.shape[0]])
+        return w + ([0, int(self.page_tokens), 0, 0] if pt is None else [pt.data_ptr(), int(self.page_tokens), pt.shape[1], self.win_kv.shape[0]])
 
     def struct(self) -> CCache:
         return CCache(*self.words())
@@ -189,7 +196,7 @@ class NodeInputs:
     n_nodes: torch.Tensor
 
     def words(self) -> list:
-        return _pointers(_NODE_FIELDS, self)
+        return _pointers(_NODE_FIELDS(self))
 
     def struct(self) -> CNodes:
         return CNodes(*self.words())
@@ -211,7 +218,7 @@ class Scratch:
     hca_done: torch.Tensor
 
     def words(self) -> list:
-        return _pointers(_SCRATCH_FIELDS, self)
+        return _pointers(_SCRATCH_FIELDS(self))
 
     def struct(self) -> CScratch:
         return CScratch(*self.words())
@@ -315,26 +322,14 @@ def tree_verify_attn(shape: CShape, cache: LayerCache, nodes: NodeInputs, scratc
         raise TsvError(r, "tree_verify_attn")
 
 
-class LayerStructs:
-    """The C structs of a layer's cache and scratch pad, made once and used until their tensors change."""
-
-    def __init__(self):
-        self._words = None
-
-    def update(self, cache: LayerCache, scratch: Scratch) -> "LayerStructs":
-        words = cache.words() + scratch.words()
-        if words != self._words:
-            self.cache, self.scratch = cache.struct(), scratch.struct()
-            self._words = words
-        return self
-
-
-def tree_verify_layer(shape: CShape, layer: LayerStructs, nodes: CNodes, out: torch.Tensor, topk_idx: Optional[torch.Tensor],
+def tree_verify_layer(shape: CShape, cache: CCache, nodes: CNodes, scratch: CScratch, out: torch.Tensor, topk_idx: Optional[torch.Tensor],
                       workspace: torch.Tensor, first: bool, status: torch.Tensor, stream=None) -> None:
-    """branch_state_build and tree_verify_attn of one layer in one call; first: `status` is cleared by it."""
+    """branch_state_build and tree_verify_attn of one layer in one call (over the C structs, which a loop keeps); first: `status` is
+    cleared by it."""
     wp, wn = _aligned(workspace)
-    r = _lib.tree_verify_layer(C.byref(shape), C.byref(layer.cache), C.byref(nodes), C.byref(layer.scratch), _ptr(out), _ptr(topk_idx), wp, wn,
-                               first, _ptr(status), _stream(stream))
+    at = C.addressof
+    r = _lib.tree_verify_layer(at(shape), at(cache), at(nodes), at(scratch), _ptr(out), _ptr(topk_idx), wp, wn, first, _ptr(status),
+                               _stream(stream))
     if r:
         raise TsvError(r, "tree_verify_layer")
 
@@ -359,33 +354,42 @@ def bench_tree_verify_attn_stages(shape: CShape, cache: LayerCache, nodes: NodeI
 
 
 class LayerPack:
-    """Host arrays of per-layer struct pointers for accept_and_refresh."""
+    """The C structs of a stack's layers, and the host arrays of their addresses that the call over all layers takes.  update() makes
+    a layer's again: those of the cache and the scratch pad where their pointers or sizes have changed (compared by value: an object
+    may stand at the address of one that is gone), those of a cycle's inputs always (in place: the library reads them during a call)."""
 
     def __init__(self, caches: List[LayerCache], nodes: List[NodeInputs], scratch: List[Scratch]):
-        self._words = [x.words() for x in (*caches, *nodes, *scratch)]
-        self._set([c.struct() for c in caches], [x.struct() for x in nodes], [s.struct() for s in scratch])
+        self.n = n = len(caches)
+        self.structs = [[None, CNodes(), None] for _ in range(n)]                        # cache, nodes, scratch per layer
+        self._words = [[None, None, None] for _ in range(n)]
+        self.caches, self.nodes, self.scratch = (_p * n)(), (_p * n)(), (_p * n)()
+        for l in range(n):
+            self.nodes[l] = C.addressof(self.structs[l][1])
+            self.update(l, caches[l], nodes[l], scratch[l])
 
-    @classmethod
-    def of_structs(cls, layers: List["LayerStructs"], nodes: List[CNodes]) -> "LayerPack":
-        p = cls.__new__(cls)
-        p._words = None
-        p._set([x.cache for x in layers], nodes, [x.scratch for x in layers])
-        return p
-
-    def _set(self, *structs) -> None:
-        self.n, self._keep = len(structs[0]), structs
-        self.caches, self.nodes, self.scratch = [(_p * self.n)(*map(C.addressof, x)) for x in structs]
+    def update(self, l: int, cache: LayerCache, nodes: NodeInputs, scratch: Scratch) -> Tuple[CCache, CNodes, CScratch]:
+        st, words = self.structs[l], self._words[l]
+        w = cache.words()
+        if w != words[0]:
+            words[0], st[0] = w, cache.struct()
+            self.caches[l] = C.addressof(st[0])
+        w = scratch.words()
+        if w != words[2]:
+            words[2], st[2] = w, scratch.struct()
+            self.scratch[l] = C.addressof(st[2])
+        words[1] = nodes.words()
+        _fill_nodes(st[1], 0, *words[1])
+        return st
 
     def current(self, caches: List[LayerCache], nodes: List[NodeInputs], scratch: List[Scratch]) -> bool:
-        """Whether the arrays describe these objects as they are now (compared by value: an object may stand at the address of
-        one that is gone)."""
-        return self._words == [x.words() for x in (*caches, *nodes, *scratch)]
+        """Whether the arrays describe these objects as they are now."""
+        return self._words == [[x.words() for x in layer] for layer in zip(caches, nodes, scratch)]
 
 
 def accept_and_refresh(shape: CShape, pack: LayerPack, draft_tok: torch.Tensor, target_tok: torch.Tensor,
                        accept_len: torch.Tensor, accept_path: torch.Tensor, bonus_tok: torch.Tensor,
                        status: torch.Tensor, stream=None) -> None:
-    r = _lib.accept_and_refresh(C.byref(shape), pack.n, pack.caches, pack.nodes, pack.scratch, _ptr(draft_tok), _ptr(target_tok),
+    r = _lib.accept_and_refresh(C.addressof(shape), pack.n, pack.caches, pack.nodes, pack.scratch, _ptr(draft_tok), _ptr(target_tok),
                                 _ptr(accept_len), _ptr(accept_path), _ptr(bonus_tok), _ptr(status), _stream(stream))
     if r:
         raise TsvError(r, "accept_and_refresh")

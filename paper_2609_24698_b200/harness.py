@@ -136,30 +136,27 @@ class VerifyEngine:
         self.accept_len = torch.zeros(B, **i32)
         self.accept_path = torch.zeros(B, D, **i32)
         self.bonus = torch.zeros(B, **i32)
-        self._structs = [tsv.LayerStructs() for _ in range(n_layers)]
-
-    def _layer(self, l: int) -> tsv.LayerStructs:
-        return self._structs[l].update(self.caches[l], self.scratch[l])
+        self._kept: Optional[tsv.LayerPack] = None       # launch_cycle's structs of the caches and scratch pads
 
     def _pack(self, inp: InputSet) -> tsv.LayerPack:
-        return tsv.LayerPack.of_structs([self._layer(l) for l in range(self.n_layers)], [nd.struct() for nd in inp.layers])
+        return tsv.LayerPack(self.caches, inp.layers, self.scratch)
 
     def launch_cycle(self, inp: InputSet, attention: bool = True, refresh: bool = True) -> None:
         """Enqueue one verify cycle on the current stream (no host sync)."""
         stream = torch.cuda.current_stream()
+        pack = self._kept
+        if pack is None:
+            pack = self._kept = self._pack(inp)
         if not attention:
             self.status.zero_()
-        layers, nodes = [], []
         for l in range(self.n_layers):                  # (a layer's structs just before its call: the first kernels run meanwhile)
-            layers.append(self._layer(l))
-            nodes.append(inp.layers[l].struct())
+            cache, nodes, scratch = pack.update(l, self.caches[l], inp.layers[l], self.scratch[l])
             if attention:
-                tsv.tree_verify_layer(self.cshape, layers[l], nodes[l], self.out[l], self.topk_idx[l], self.workspace, l == 0, self.status, stream)
+                tsv.tree_verify_layer(self.cshape, cache, nodes, scratch, self.out[l], self.topk_idx[l], self.workspace, l == 0, self.status, stream)
             else:
                 tsv.branch_state_build(self.cshape, self.caches[l], inp.layers[l], self.scratch[l], self.status, stream)
         if refresh:
-            tsv.accept_and_refresh(self.cshape, tsv.LayerPack.of_structs(layers, nodes), inp.draft, inp.target, self.accept_len, self.accept_path,
-                                   self.bonus, self.status, stream)
+            tsv.accept_and_refresh(self.cshape, pack, inp.draft, inp.target, self.accept_len, self.accept_path, self.bonus, self.status, stream)
 
     def capture(self, inp: InputSet) -> torch.cuda.CUDAGraph:
         """Capture one cycle over `inp` into a CUDA graph (the launch sequence is shape-stable)."""
