@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(kItThreads) idx_score_tc_kernel(const tsv_shap
   unsigned char* base = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   ItCtl& sm = *reinterpret_cast<ItCtl*>(base);
   const uint32_t bq = smem_u32(base + kItCtl), a0 = bq + kItB;
-  coop_tree_meta(sm.tm, sm.tstage, s, c.L + b, nd.parent + (size_t)b * D, nd.n_nodes + b, nullptr, nullptr);
+  coop_tree_meta(sm.tm, sm.tstage, s, c.L + b, nd.parent + (size_t)b * D, nd.n_nodes + b, c.csa_cap + b, nullptr);
   if (tid == 0) {   // nodes that rank: committed entries + blocks closed at strict ancestors exceed topk
     uint32_t m = 0;
     if (!sm.tm.status)

@@ -25,7 +25,7 @@ __global__ void __launch_bounds__(256) idx_score_kernel(const tsv_shape s, const
     const int L0 = c.L[b];
     if (L0 < 0 || L0 / s.m_csa + D <= s.topk || (int)(blockIdx.x * blockDim.x) >= L0 / s.m_csa) return;
   }
-  coop_tree_meta(tm, tstage, s, c.L + b, nd.parent + (size_t)b * D, nd.n_nodes + b, nullptr, nullptr);
+  coop_tree_meta(tm, tstage, s, c.L + b, nd.parent + (size_t)b * D, nd.n_nodes + b, c.csa_cap + b, nullptr);
   if (threadIdx.x == 0) {
     uint32_t m = 0;
     if (!tm.status)
@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(256) idx_score_rows256_kernel(const tsv_shape 
     const int L0 = c.L[b];
     if (L0 < 0 || L0 / s.m_csa + D <= s.topk || (int)(blockIdx.x * kRows256PerCta) >= L0 / s.m_csa) return;
   }
-  coop_tree_meta(tm, tstage, s, c.L + b, nd.parent + (size_t)b * D, nd.n_nodes + b, nullptr, nullptr);
+  coop_tree_meta(tm, tstage, s, c.L + b, nd.parent + (size_t)b * D, nd.n_nodes + b, c.csa_cap + b, nullptr);
   if (tm.status || n >= tm.nn || (int)(blockIdx.x * kRows256PerCta) >= tm.n_csa) return;
   {   // does this node rank?  candidates = committed entries + blocks closed at its strict ancestors
     int extra = 0;

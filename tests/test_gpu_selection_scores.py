@@ -16,18 +16,21 @@ FORMS = [("bf16", 8, 600, 512), ("bf16", 8, 900, 800), ("fp32", 8, 600, 512), ("
          ("fp32", 8, 900, 800, 16), ("bf16", 8, 2500, 2400, 16), ("fp32", 5, 66000, 65800, 8)]
 
 
-def _select(form, HI, ik, tree_ik, iq, iw):
+def _select(form, HI, ik, tree_ik, iq, iw, room=None, cap=None, status=0):
     """topk_idx of a chain of D nodes (blocks of two tokens: nodes 1, 3, ... close one) after n committed entries with the indexer
-    keys ik [n][di]; every closed entry has the key tree_ik.  The list buffer is followed by a guard."""
+    keys ik [n][di]; every closed entry has the key tree_ik.  The list buffer is followed by a guard.  room: tokens the shape is
+    sized for; cap: entries the cache says it has room for; status: what the device has to report."""
     from paper_2609_24698_b200 import harness as hz
     dtype, D, n, k = form[:4]
     di = ik.shape[1]
     sh = synth.Shape(dtype, 1, D, 4, 16, 2, k, HI, di, 64, 64)
     ccap, hcap = hz.capacities(sh, [2 * n], 2 * D)
-    eng = hz.VerifyEngine(sh, 1, ccap, hcap, 2 * n + 2 * D, want_topk=True)
+    eng = hz.VerifyEngine(sh, 1, ccap, hcap, room or 2 * n + 2 * D, want_topk=True)
     guard = torch.full((D * k + 64,), -2, dtype=torch.int32, device="cuda")
     eng.topk_idx = [guard[:D * k].view(1, D, k)]
     eng.caches[0].L.fill_(2 * n)
+    if cap is not None:
+        eng.caches[0].csa_cap.fill_(cap)
     eng.caches[0].csa_ik[:n] = torch.from_numpy(ik).cuda()
     inp = hz.InputSet.empty(sh, 1)
     nd = inp.layers[0]
@@ -36,7 +39,7 @@ def _select(form, HI, ik, tree_ik, iq, iw):
     nd.iq[:] = torch.from_numpy(iq).cuda(); nd.iw[:] = torch.from_numpy(iw).cuda()
     eng.launch_cycle(inp, refresh=False)
     torch.cuda.synchronize()
-    assert int(eng.status.sum()) == 0
+    assert int(eng.status.sum()) == status
     got = guard.cpu().numpy()
     assert (got[D * k:] == -2).all(), "written past the last node's row"
     return got[:D * k].reshape(D, k)
@@ -95,3 +98,16 @@ def test_zeros_of_either_sign_tie(form):
     iq[:, range(HI), range(HI)] = 1
     iw = np.full((D, HI), -1, np.float32)
     _check(_select(form, HI, ik, np.zeros(di, np.float32), iq, iw), form, -np.maximum(ik, 0).max(1).astype(np.float64), 0.0)
+
+
+@pytest.mark.parametrize("form", FORMS + [("bf16", 4, 2500, 2400)])
+def test_no_room_for_closed_entries_selects_nothing(form):
+    """A sequence whose slab cannot hold what its tree may close is flagged by every form, the scoring kernels among them: none of its
+    rows are read beyond what it says it has, and its lists are empty."""
+    from paper_2609_24698_b200 import binding as tsv
+    dtype, D, n, k = form[:4]
+    di = form[4] if len(form) > 4 else 128 if dtype == "bf16" else 64
+    HI = 8 if D == 4 else 2
+    ones = np.ones((D, HI, di), np.float32)
+    got = _select(form, HI, np.ones((n, di), np.float32), np.zeros(di, np.float32), ones, ones[:, :, 0], cap=n, status=tsv.ST_CSA_CAP)
+    assert (got == -1).all()
