@@ -383,9 +383,9 @@ def test_long_candidate_lists_generic_scoring(dtype):
 
 @pytest.mark.parametrize("D,HI", [(4, 8), (6, 2), (7, 1), (8, 4)])
 def test_long_candidate_lists_tensor_core_scoring(D, HI):
-    """More than 2048 candidates per node with 128-wide bf16 indexer rows: the scores of all nodes and heads come from
-    the tcgen05 scoring kernel (every head count it is built for; ragged last tiles, sequences on both sides of the
-    2304-candidate switch of the selection's key paths)."""
+    """More than 2048 candidates per node with 128-wide bf16 indexer rows: eight heads from the tcgen05 scoring kernel, fewer
+    from the cluster form's warp products (ragged last tiles).  The other shapes of the tcgen05 kernel:
+    test_gpu_selection_scores.py."""
     cfg = synth.small_config(name=f"long_lists_tc_d{D}_hi{HI}", dtype="bf16", B=3, D=D, H=4, d=16, m_csa=2, topk=24, HI=HI,
                              di=128, m_hca=32, window=16, L_min=4200, L_max=5200, layers=1, seed=78 + HI, cfg_id=73)
     lockstep(cfg, cycles=2)

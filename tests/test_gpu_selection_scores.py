@@ -48,7 +48,7 @@ def _select(form, HI, ik, tree_ik, iq, iw, room=None, cap=None, status=0):
 def _check(got, form, scores, tree_score):
     """scores: of the committed entries, tree_score: of every closed one; NaN above everything, ties to the lower index."""
     for node, row in enumerate(got):
-        s = np.concatenate([scores, np.full(node // 2, tree_score)])
+        s = np.concatenate([scores, np.full(node // 2, tree_score) if np.isscalar(tree_score) else tree_score])
         order = np.lexsort((np.arange(len(s)), -np.where(np.isnan(s), np.inf, s)))
         assert np.array_equal(row, np.sort(order[:form[3]])), (node, len(set(row.tolist())))
 
@@ -111,3 +111,20 @@ def test_no_room_for_closed_entries_selects_nothing(form):
     ones = np.ones((D, HI, di), np.float32)
     got = _select(form, HI, np.ones((n, di), np.float32), np.zeros(di, np.float32), ones, ones[:, :, 0], cap=n, status=tsv.ST_CSA_CAP)
     assert (got == -1).all()
+
+
+# The tcgen05 scoring kernel takes the lists that are left to it: eight heads with up to four nodes, and, of fewer heads, capacities
+# beyond the clusters' (room: a list that is short in a cache sized for 450 k entries).  Lists at the edges of its tiles of 128 entries
+# and CTAs of four of them; selected by a cluster of CTAs per node, or by one that reads the scores again in every pass.
+@pytest.mark.parametrize("D,HI,room", [(4, 8, None), (1, 8, None), (8, 1, 900_000), (8, 4, 900_000), (7, 2, 900_000), (3, 8, 900_000)])
+@pytest.mark.parametrize("n", [129, 511, 513, 2688])
+def test_tensor_core_scores(D, HI, room, n):
+    rng = np.random.default_rng(n + D)
+    ik = rng.integers(-3, 4, (n, 128)).astype(np.float32)    # (small integers: exact in bf16, their sums exact in fp32)
+    iq = rng.integers(-2, 3, (D, HI, 128)).astype(np.float32)
+    iw = rng.integers(1, 4, (D, HI)).astype(np.float32)
+    form = ("bf16", D, n, n // 3)
+    got = _select(form, HI, ik, np.zeros(128, np.float32), iq, iw, room=room or 5000 + 2 * n)
+    scores = np.einsum("dhe,dh->de", np.maximum(np.einsum("ed,nhd->nhe", ik, iq), 0), iw)
+    for node in range(D):
+        _check(got[node:node + 1], form, scores[node], np.full(node // 2, 0.0))
