@@ -35,7 +35,7 @@ NCU_DRAM = {
     # cfg5: tc_attn_pair_kernel 61.11 MB read + 1.70 MB written; all kernels of one cycle 138.1 MB (cold cache per kernel)
     "cfg5": {"kernel": "tc_attn_pair_kernel", "launch_bytes": 62_808_320, "cycle_bytes": 138_081_792},
 }
-ATTN_KERNEL = {"cfg1": "attn_simt_kernel (fp32 CUDA-core path)", "cfg2": "tc_attn_pair_kernel + tc_combine_pair_kernel",
+ATTN_KERNEL = {"cfg1": "attn_f32_kernel (fp32, CUDA cores)", "cfg2": "tc_attn_pair_kernel + tc_combine_pair_kernel",
                "cfg2_chain": "tc_attn_pair_kernel + tc_combine_pair_kernel",
                "cfg3": "tc_attn_pair_kernel (contiguous-run and gathered tiles) + tc_combine_pair_kernel", "cfg4": "tc_attn_pair_kernel",
                "cfg5": "tc_attn_pair_kernel (gathered tiles) + tc_combine_pair_kernel"}

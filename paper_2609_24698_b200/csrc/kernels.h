@@ -4,7 +4,7 @@
 
 namespace tsv {
 
-void count_launch(int n = 1);
+void count_launch(int n = 1);         // bumps the reporting counter behind tsv_kernel_launches()
 
 // Every kernel of the library asks for the same (maximal) shared-memory carve-out: consecutive kernels with different
 // carve-outs make the SMs drain and reconfigure between launches, which costs far more than these kernels run.
@@ -15,7 +15,7 @@ void count_launch(int n = 1);
       cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared); \
       done_ = true;                                                                                               \
     }                                                                                                             \
-  } while (0)   // bumps the reporting counter behind tsv_kernel_launches()
+  } while (0)
 
 // Raises a kernel's dynamic shared-memory limit on the current device where it is below `bytes` (never lowers it: another
 // shape's launches need what they asked for).  The driver is called once per kernel, device and new maximum.

@@ -105,8 +105,8 @@ __device__ __forceinline__ float ex2(float x) {
 constexpr int NCX = 768;             // max keys per chunk of the TMA kernel: P (bf16) takes 384 TMEM columns, an O quarter 128
 // Chunking of the TMA kernel: nch chunks of CL keys, CL a multiple of 128 and <= NCX.
 // general = false (shapes whose capacities allow at most two chunks of NCX keys and no gathered tile): as few chunks as possible.
-// general = true: a list that does not fit one chunk is cut into chunks of at most NC keys, whose PV product runs in halves of
-// d instead of quarters and which fill the SM pairs better (two chunks of up to NCX instead of three of NC cost 12 % of the
+// general = true: a list that does not fit one chunk is cut into chunks of at most NC keys, whose quarters of O go through two
+// buffers instead of one and which fill the SM pairs better (two chunks of up to NCX instead of three of NC cost 12 % of the
 // attention kernel on 32 paged sequences of 256-4096 tokens, and gained nothing on 64 flat ones).
 // split: chunks a tile may be cut into so that few tiles still use all pairs (1 where there are tiles enough).
 // f32: the partial outputs of the tile are fp32 (a tile that is cut for the sake of parallelism alone is not rounded before
