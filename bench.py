@@ -32,8 +32,8 @@ import numpy as np  # noqa: E402
 # verify cycle.  The captures are summarised under profiles/; workloads without a capture report null.
 NCU_DRAM = {
     "cfg4": {"kernel": "tc_attn_pair_kernel", "launch_bytes": 64_300_000, "cycle_bytes": None},   # 63.6 MB read + 0.7 MB written
-    # cfg5: tc_attn_pair_kernel 61.11 MB read + 1.70 MB written; all kernels of one cycle 138.1 MB (cold cache per kernel)
-    "cfg5": {"kernel": "tc_attn_pair_kernel", "launch_bytes": 62_808_320, "cycle_bytes": 138_081_792},
+    # cfg5: tc_attn_pair_kernel 60.48 MB read + 1.75 MB written; all kernels of one cycle 138.6 MB (cold cache per kernel)
+    "cfg5": {"kernel": "tc_attn_pair_kernel", "launch_bytes": 62_226_432, "cycle_bytes": 138_580_736},
 }
 ATTN_KERNEL = {"cfg1": "attn_f32_kernel (fp32, CUDA cores)", "cfg2": "tc_attn_pair_kernel + tc_combine_pair_kernel",
                "cfg2_chain": "tc_attn_pair_kernel + tc_combine_pair_kernel",
