@@ -25,7 +25,7 @@ __device__ inline void path_entries(PathEntries& pe, const TreeMeta& tm, const t
 }
 
 // Larger float -> larger key, the two zeros (a head of negative weight leaves -0 where relu leaves nothing) the same key; a total
-// order (a positive NaN above everything).  The bits are taken by an opaque
+// order (a NaN above everything).  The bits are taken by an opaque
 // move: of a plain reinterpretation the compiler makes float operations in some places (the sign bit set as -|f|), which turn a NaN
 // into another pattern there than elsewhere, and a selection that counts a key in one pass and misses it in the next is short of it.
 __device__ __forceinline__ uint32_t order_key(float f) {
