@@ -37,10 +37,6 @@ __device__ __forceinline__ int tile_keys_estimate(const tsv_shape& s, int L, int
   return nk <= tc::NCX ? nk : min(nk, tc::NC);
 }
 
-__device__ __forceinline__ void l2_prefetch(const void* p, uint32_t bytes) {       // (16-byte aligned, a multiple of 16 bytes)
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
-
 // GENERAL: gathered tiles may occur (see gathered_tiles_possible); the instantiation without them keeps the short
 // latency chain of the contiguous-run plan.
 template <bool GENERAL, int PARTS>
@@ -380,15 +376,6 @@ __global__ void __launch_bounds__(NT) tc_plan_kernel(const tsv_shape s, const Tv
   // of the CTA it is worse (865 -> 901 us): then all pairs begin at the same instant, and their first instructions queue behind
   // everyone's first operands.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  // The tile's queries into L2: the pairs of the attention kernel all start at once, and the first phase of each is bound by
-  // what arrives from HBM, which idles under the kernels before (first operands of 64 short sequences 10 k -> 7.5 k cycles
-  // after the start, last of the first piece 18 k -> 13 k).  At the end of the CTA's own work, which is a chain of loads that
-  // would queue behind these.
-  if (tile_cta && threadIdx.x < 4) {
-    const int rows_seq = s.D * s.H, r0 = tile * tc::PR, rows = min(tc::PR, rows_seq - r0), part = (rows + 3) / 4;
-    const int p0 = min(rows, (int)threadIdx.x * part), pn = min(part, rows - p0);
-    if (pn > 0) l2_prefetch(reinterpret_cast<const char*>(nd.q) + ((size_t)blockIdx.y * rows_seq + r0 + p0) * (tc::DH * 2), (uint32_t)pn * (tc::DH * 2));
-  }
   // one CTA waits for the selection in any case, so that the completion of this kernel implies that one's
   if (blockIdx.x == 0 && blockIdx.y == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
@@ -592,7 +579,7 @@ int launch_tva_tc(const tsv_shape& s, const TvaPlan& p_in, const TvaTcPrep& prep
   // leaves bf16 partial outputs for the merge kernel
   const bool many = (p.tc_maxk + tc::NCX - 1) / tc::NCX > 2 || gathered, general = many || p.tc_split > 1;
   p.tc_f32 = !many;                                    // (no more than two long chunks a tile: merged without rounding in either instantiation)
-  const int r = launch_tva_tc_pair(s, p, prep, general, out, ws, status, st);
+  const int r = launch_tva_tc_pair(s, p, prep, general, nd.q, out, ws, status, st);
   if (r != TSV_OK) return r;
   if (general && p.tc_chmax > 1) {
     cudaLaunchConfig_t cfg = {};

@@ -66,6 +66,8 @@ constexpr int CTLB = 3072;                 // control block bytes; the ring foll
 constexpr int SLOTP = 16384;               // ring slot: every stage of a CTA is at most 16 KiB
 constexpr int SMEM_X = CTLB + NSX * SLOTP;
 static_assert(sizeof(Ctl) <= CTLB, "control block overflow");
+constexpr int NBAR = NQS + 2 * NKS + 2 * NSV + 7 + 7 + 2;      // barriers, at the start of the block
+static_assert(offsetof(Ctl, tmem_base) == NBAR * 8 && NBAR <= 64, "the barriers are initialised by a thread each");
 
 __device__ __forceinline__ void mbar_init(uint64_t* b, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count));
@@ -192,7 +194,7 @@ struct Item {
 template <bool GENERAL>
 __global__ void __launch_bounds__(pair::TTHREADS, 1)
 tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s,
-                    const TvaPlan pl, void* __restrict__ out_, char* __restrict__ ws, int32_t* __restrict__ status) {
+                    const TvaPlan pl, const void* __restrict__ q, void* __restrict__ out_, char* __restrict__ ws, int32_t* __restrict__ status) {
   using namespace pair;
   extern __shared__ unsigned char smem_raw[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -201,22 +203,21 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
   Ctl& sm = *reinterpret_cast<Ctl*>(smem_raw);
   const uint32_t ring = smem_u32(smem_raw + CTLB);
   int fail = (smem_u32(smem_raw) & 1023u) ? 1 : 0;             // the swizzled tiles need a 1024-byte aligned base
-  if (tid < (GENERAL ? NMAPS : 14))   // the descriptors of the tensor maps in use are fetched while the plan is read
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&maps) + (uint64_t)tid * sizeof(CUtensorMap)) : "memory");
-  if (tid == 0) {
-    for (int i = 0; i < NQS; ++i) mbar_init(&sm.fullQ[i], 1);
-    for (int i = 0; i < NKS; ++i) { mbar_init(&sm.fullK[i], 1); mbar_init(&sm.emptyK[i], 1); }
-    for (int i = 0; i < NSV; ++i) { mbar_init(&sm.fullV[i], 1); mbar_init(&sm.emptyV[i], 1); }
-    for (int i = 0; i < 7; ++i) { mbar_init(&sm.acc_ev[i], 1); mbar_init(&sm.cmp_ev[i], 16); }   // 8 compute warps of each CTA
-    mbar_init(&sm.stage_free, 8);
-    mbar_init(&sm.item_ev, 1);
+  // Set-up, a warp for each part of it: one thread that initialised the sixty barriers before it allocated tensor memory took 1.7 us
+  // from the CTA's start to the wait below, of the 25 us a layer of one short sequence takes.
+  if (tid < NBAR) {
+    mbar_init(&sm.fullQ[0] + tid, tid >= offsetof(Ctl, cmp_ev) / 8 && tid < offsetof(Ctl, cmp_ev) / 8 + 7 ? 16       // 8 compute warps of each CTA
+                                  : tid == offsetof(Ctl, stage_free) / 8 ? 8 : 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 0) {
+  if (warp == 2) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&sm.tmem_base)) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
+  if (warp == 3 && lane < (GENERAL ? NMAPS : 14))   // the descriptors of the tensor maps in use are fetched while the plan is read
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&maps) + (uint64_t)lane * sizeof(CUtensorMap)) : "memory");
   __syncwarp();
+  fence_before();
   cluster_arrive();                                              // this CTA's barriers exist and its tensor memory is allocated
   auto leave = [&]() {
     if (fail) for (int b = (int)(blockIdx.x >> 1); b < s.B; b += (int)(gridDim.x >> 1)) atomicOr(status + b, TSV_ST_INTERNAL);   // (an internal error: every sequence is flagged)
@@ -226,6 +227,14 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
     fence_after();
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(sm.tmem_base) : "memory");
   };
+  // The queries of tile p by pair p into L2 (its first item is another tile: the longest ones go first, but all pairs' first phase
+  // is bound by what arrives from HBM).  Here, and not by the tile plan's CTAs, which do not end before the copies they have asked
+  // for: of 64 sequences the wait below ended 2.6 us sooner.  Before that wait: the queries are the caller's.
+  if (warp == 2 && lane == 0) {
+    const int p = blockIdx.x >> 1, b = p / pl.tc_nt, r0 = (p - b * pl.tc_nt) * PR + (int)rank * BM, rows = min(BM, s.D * s.H - r0);
+    if (b < s.B && rows > 0)
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(reinterpret_cast<const char*>(q) + ((size_t)b * s.D * s.H + r0) * (DH * 2)), "r"(rows * DH * 2) : "memory");
+  }
   // Launched as a programmatic dependent of the tile plan: the CTAs take their places and set up while that kernel's last
   // CTAs finish, and read nothing of its before it has completed.
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -233,8 +242,6 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
   // start before this kernel has ended: the next call's tile plan would overwrite what is read here.)
   if (GENERAL && pl.tc_chmax > 1) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int4 rec0 = (int)(blockIdx.x >> 1) < s.B * pl.tc_nt ? __ldcg(reinterpret_cast<const int4*>(ws + pl.off_order) + (blockIdx.x >> 1)) : make_int4(-1, 0, 0, 0);
-  fence_before();
-  __syncthreads();
   cluster_wait();                                                // barriers of both CTAs exist before anyone signals them
   fence_after();
   const uint32_t tm = sm.tmem_base;
@@ -976,7 +983,7 @@ int prepare_tva_tc_pair(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c
   return TSV_OK;
 }
 
-int launch_tva_tc_pair(const tsv_shape& s, const TvaPlan& p, const TvaTcPrep& prep, bool general, void* out, char* ws, int32_t* status, cudaStream_t st) {
+int launch_tva_tc_pair(const tsv_shape& s, const TvaPlan& p, const TvaTcPrep& prep, bool general, const void* q, void* out, char* ws, int32_t* status, cudaStream_t st) {
   const pair::MapSet& ms = *reinterpret_cast<const pair::MapSet*>(prep.maps);
   cudaLaunchConfig_t cfg = {};
   const int64_t most = (int64_t)p.tc_nt * s.B * p.tc_chmax;                 // items, if every tile had the most chunks
@@ -1000,8 +1007,8 @@ int launch_tva_tc_pair(const tsv_shape& s, const TvaPlan& p, const TvaTcPrep& pr
   }
   if (pairs > most) pairs = (int)most;
   cfg.gridDim = dim3(2 * pairs, 1, 1);
-  const cudaError_t le = general ? cudaLaunchKernelEx(&cfg, tc_attn_pair_kernel<true>, ms, s, p, out, ws, status)
-                                 : cudaLaunchKernelEx(&cfg, tc_attn_pair_kernel<false>, ms, s, p, out, ws, status);
+  const cudaError_t le = general ? cudaLaunchKernelEx(&cfg, tc_attn_pair_kernel<true>, ms, s, p, q, out, ws, status)
+                                 : cudaLaunchKernelEx(&cfg, tc_attn_pair_kernel<false>, ms, s, p, q, out, ws, status);
   if (le != cudaSuccess) {
     int ncl = -1;
     cudaOccupancyMaxActiveClusters(&ncl, tc_attn_pair_kernel<true>, &cfg);
