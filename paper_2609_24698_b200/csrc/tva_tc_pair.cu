@@ -42,10 +42,16 @@ constexpr float RESCALE_GAP = 16.f;        // log2 units a later piece's row max
 constexpr int NSX = 14;                    // 16 KiB slots of the staging area
 constexpr int NQS = 8;                     // Q slices of an item (all of d, resident for every piece)
 constexpr int NKS = NSX - NQS;             // K stages in flight
-constexpr int NSV = 12;                    // Slots [0, 12) are one FIFO: an item's eight Q slices and its first four K stages take the next twelve
+constexpr int NSV = 12;                    // Slots [0, 12) are one FIFO: an item's first six Q slices and its ring of six K stages take the next twelve
                                            // places, its V stages (once the S products are complete) the places from the same start on; so
-                                           // the next item's Q slices land where the V stages are released first.  Slots 12, 13: the other
-                                           // two K stages, and, when O is read out, the staging of the output (a 4 KiB tile per warp).
+                                           // the next item's operands land where the V stages are released first.  Slots 12, 13: the last
+                                           // two Q slices, and, when O is read out, the staging of the output (a 4 KiB tile per warp).
+// The FIFO's places of an item, about in the order in which the S products want them: Q0 K0 Q1 K1 Q2 K2 K3 Q3 K4 Q4 K5 Q5 (of places
+// p and p + 6, which are one producer's, one is a Q slice, the other a K stage).  Six stages of operands are requested before the item
+// before is done with; with all of Q and four K stages in the FIFO, and the ring's other two stages waiting for the output's staging,
+// the products waited for the fifth stage, requested when the first product was complete: 512-key items 14.8 us.
+__device__ __forceinline__ int q_place(int dk) { return dk < 3 ? 2 * dk : 2 * dk + 1; }         // dk < 6; slices 6 and 7 are in slots 12 and 13
+__device__ __forceinline__ int k_place(int pos) { return pos < 3 ? 2 * pos + 1 : 2 * pos; }     // pos: stage modulo NKS
 
 struct Ctl {                               // control block at the start of dynamic shared memory; no barrier is ever re-initialised
   uint64_t fullQ[NQS];                     // Q slice dk of the item has arrived
@@ -91,6 +97,10 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
 __device__ __forceinline__ void tma_box2(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar_cluster_addr) {
   asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
                ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar_cluster_addr) : "memory");
+}
+// the same box into L2 only
+__device__ __forceinline__ void tma_box_l2(const CUtensorMap* map, int x, int y) {
+  asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y) : "memory");
 }
 // four rows of a 2D tensor, given by their row indices, as four consecutive 128-byte lines of this CTA's shared memory
 __device__ __forceinline__ void tma_gather4(uint32_t dst, const CUtensorMap* map, int x, const uint4& code, uint32_t bar_cluster_addr) {
@@ -268,11 +278,14 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
     // is only good for the phase after the last one seen).  Both CTAs' copies complete on the leader's barriers.
     // (Six warps because of the gathered tiles: a stage is 32 four-row requests there, and a warp takes about 70 cycles to
     // issue one; boxes would do with two.)
+    // A producer steps from one of its own stages to the next: going over all stages of the item and picking out its own took it 1.1 us
+    // from one copy to the next, longer than the slots were in use (512-key items 17.2 us, see k_ring).
     const int pw = warp == 0 ? 0 : warp == 3 ? 1 : warp - 10;
-    uint32_t kcnt = 0, kused = 0, vcnt = 0, vused = 0, accb = 0;  // per slot: parity of the number of uses so far, used at all
+    uint32_t kcnt = 0, accb = 0;                                  // parities of the uses so far: ring positions of the K stages; events
+    uint32_t vcnt = 0, vused = 0;                                 // of this producer's FIFO slots pw and pw + 6 (bits 0, 1): parity of the V stages so far, any
     int n_real = 0;                                               // items with keys so far
-    auto slot_wait = [&](uint64_t* empty, uint32_t cnt, uint32_t used, int sl) {      // the slot's latest release
-      if (((used >> sl) & 1u) && !fail && !mbar_wait(&empty[sl], ((cnt >> sl) & 1u) ^ 1u)) fail = 1;
+    auto v_wait = [&](int h) {                                    // the release of the latest V stage in FIFO slot pw + 6 h
+      if (((vused >> h) & 1u) && !fail && !mbar_wait(&sm.emptyV[pw + NPROD * h], ((vcnt >> h) & 1u) ^ 1u)) fail = 1;
     };
     // the boxes of a chunk: lane i holds box i of up to NCX / kBoxRows
     auto load_box = [&](const Item& w) {
@@ -283,7 +296,7 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
       }
       return v;
     };
-    int g0 = 0;                                                   // first place of the item in the FIFO
+    int g0 = 0;                                                   // slot of the item's first place in the FIFO
 #pragma unroll 1
     for (int it = 0;; ++it) {
       const int4 r = next_item(it);
@@ -293,14 +306,12 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
       const int CL = w.CL, row0 = w.tile * PR + (int)rank * BM;
       const int nvb = CL / 128;                                    // V stages per part
       const int NKST = 8 * w.npc, NVST = NQ * nvb;
-      auto place = [&](int i) { const int p = g0 + i; return p >= NSV ? p - NSV : p; };      // slot of the FIFO's place i after the item's start
-      auto kslot = [&](int sl) { return sl < NSV - NQS ? place(NQS + sl) : NQS + sl; };
-      // (the K stages of an item lie in six slots of six producers; slots 12 and 13 change hands with the item, when
-      // everything before is complete)
-      auto mine = [&](int phys) { return (phys < NSV ? phys : g0 + phys) % NPROD == pw; };
+      // This producer's places of the item are u and u + 6: slots pw + 6 h0 and pw + 6 (1 - h0).
+      const int u = (pw + 2 * NPROD - g0) % NPROD, h0 = (g0 + u) % NSV >= NPROD ? 1 : 0;
+      const int kpos = (u & 1) ? u >> 1 : 3 + (u >> 1);            // its ring position of the K stages
+      const int khalf = (u & 1) ? h0 : h0 ^ 1, kphys = pw + NPROD * khalf;
       // bit i: boxes i and i + 1 name consecutive rows of one array (one request can fetch both)
-      const uint32_t box_up = __shfl_down_sync(0xffffffffu, box, 1);
-      const uint32_t cons = __ballot_sync(0xffffffffu, lane < 31 && (box & 0x3FFFFFFFu) < (OOB_BOX & 0x3FFFFFFFu) && box_up == box + kBoxRows);
+      uint32_t cons = 0;
       auto consecutive = [&](int i0, int nb) { return ((~(cons >> i0)) & ((1u << (nb - 1)) - 1u)) == 0u; };
       // Gathered tiles: the keys' row codes stay in global memory (the tile plan left them there, four-aligned groups
       // never mix arrays); lane l fetches the codes of rows 4 l .. 4 l + 3 of a stage itself.  Keys past the end of the list
@@ -309,32 +320,33 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
       auto codes_at = [&](int key) { return w.cbeg + key < w.cend ? __ldg(code_g + (key >> 2)) : make_uint4(0u, 0u, 0u, 0u); };
       uint4 kcode = make_uint4(0u, 0u, 0u, 0u);                                // this lane's codes of the current piece's K stages
       int kcode_pc = -1;
-      auto issue_q = [&](int dk) {
+      auto issue_q = [&](int dk, int slot) {
         if (lane == 0) {
-          slot_wait(sm.emptyV, vcnt, vused, place(dk));            // (a V stage of the item before)
+          if (slot < NSV) v_wait(slot >= NPROD);                   // (a V stage of the item before)
+          else if (n_real && !fail && !mbar_wait(&sm.stage_free, (uint32_t)(n_real - 1) & 1u)) fail = 1;
           if (rank == 0) mbar_expect_tx(&sm.fullQ[dk], 2 * SLOTP);
-          tma_box2(ring + (uint32_t)place(dk) * SLOTP, &maps.q, dk * 64, w.b * rows_seq + row0, map_to_rank(smem_u32(&sm.fullQ[dk]), 0));
+          tma_box2(ring + (uint32_t)slot * SLOTP, &maps.q, dk * 64, w.b * rows_seq + row0, map_to_rank(smem_u32(&sm.fullQ[dk]), 0));
+          if (n_real && dk < 2) tma_box_l2(&maps.q, (dk + 6) * 64, w.b * rows_seq + row0);     // (the slots of slices 6 and 7 are free last)
         }
         __syncwarp();
       };
+      uint32_t kc = (kcnt >> kpos) & 1u;
+      bool kuse = n_real > 0, kfirst = true;                           // the position has been used; the item's first use is still to come
       auto issue_k = [&](int gk) {
-        const int pc = gk >> 3, dk = gk & 7, sl = gk % NKS;
-        const int phys = kslot(sl);
-        const uint32_t slot = ring + (uint32_t)phys * SLOTP;
-        const uint32_t fb_leader = map_to_rank(smem_u32(&sm.fullK[sl]), 0);
+        const int pc = gk >> 3, dk = gk & 7;
+        const uint32_t slot = ring + (uint32_t)kphys * SLOTP;
+        const uint32_t fb_leader = map_to_rank(smem_u32(&sm.fullK[kpos]), 0);
         const int bytes = min(256, CL - pc * 256) * 64;                        // bytes THIS CTA copies in the stage
         if (w.gather && kcode_pc != pc) {                                      // this CTA's half of the piece's keys: bytes / 128 rows
           kcode_pc = pc;
           if (lane * 512 < bytes) kcode = codes_at(pc * 256 + (int)rank * (bytes >> 7) + 4 * lane);
         }
         if (lane == 0) {
-          if (gk < NKS) {                                          // first round of the item: what the item before kept in the slot
-            if (phys < NSV) slot_wait(sm.emptyV, vcnt, vused, phys);
-            else if (n_real > 0 && !fail && !mbar_wait(&sm.stage_free, (uint32_t)(n_real - 1) & 1u)) fail = 1;
-          }
-          slot_wait(sm.emptyK, kcnt, kused, sl);
-          if (rank == 0) mbar_expect_tx(&sm.fullK[sl], 2 * bytes);              // bytes of both CTAs
+          if (kfirst) v_wait(khalf);                               // (a V stage of the item before)
+          if (kuse && !fail && !mbar_wait(&sm.emptyK[kpos], kc ^ 1u)) fail = 1;
+          if (rank == 0) mbar_expect_tx(&sm.fullK[kpos], 2 * bytes);            // bytes of both CTAs
         }
+        kfirst = false; kuse = true; kc ^= 1u;
         __syncwarp();
         // this CTA's half of the piece's keys: boxes [rank * nb, rank * nb + nb) of the piece
         const int nb = bytes / BOXB, i0 = pc * (256 / kBoxRows) + (int)rank * nb;
@@ -343,48 +355,61 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
         } else {
           const bool one = consecutive(i0, nb);                    // nb = 4 (128 rows) or 2 (64 rows)
           const uint32_t bx = __shfl_sync(0xffffffffu, box, one ? i0 : i0 + (lane & 3));
-          if (one) { if (lane == 0) tma_box2(slot, &maps.src[bx >> 30][nb == 4 ? 2 : 1], dk * 64, (int)(bx & 0x3FFFFFFFu), fb_leader); }
-          else if (lane < nb) tma_box2(slot + lane * BOXB, &maps.src[bx >> 30][0], dk * 64, (int)(bx & 0x3FFFFFFFu), fb_leader);
+          // (the stage of this piece that takes its place has to wait for its product: its rows come from L2 then)
+          const bool ahead = gk < 8 - NKS && n_real;
+          if (one) {
+            const CUtensorMap* map = &maps.src[bx >> 30][nb == 4 ? 2 : 1];
+            if (lane == 0) {
+              tma_box2(slot, map, dk * 64, (int)(bx & 0x3FFFFFFFu), fb_leader);
+              if (ahead) tma_box_l2(map, (dk + NKS) * 64, (int)(bx & 0x3FFFFFFFu));
+            }
+          } else if (lane < nb) {
+            tma_box2(slot + lane * BOXB, &maps.src[bx >> 30][0], dk * 64, (int)(bx & 0x3FFFFFFFu), fb_leader);
+            if (ahead) tma_box_l2(&maps.src[bx >> 30][0], (dk + NKS) * 64, (int)(bx & 0x3FFFFFFFu));
+          }
         }
         __syncwarp();
       };
-      auto count_k = [&](int gk) { kcnt ^= 1u << (gk % NKS); kused |= 1u << (gk % NKS); };     // every stage, whoever issues it
-#pragma unroll 1
-      for (int gk = 0; gk < NKST; ++gk) {
-        if (gk < 8 && mine(place(gk))) issue_q(gk);
-        if (mine(kslot(gk % NKS))) issue_k(gk);
-        count_k(gk);
+      if (!(u & 1)) issue_q(u >> 1, pw + NPROD * h0);
+      {
+        const uint32_t box_up = __shfl_down_sync(0xffffffffu, box, 1);
+        cons = __ballot_sync(0xffffffffu, lane < 31 && (box & 0x3FFFFFFFu) < (OOB_BOX & 0x3FFFFFFFu) && box_up == box + kBoxRows);
       }
+      issue_k(kpos);
+      if (u & 1) issue_q(3 + (u >> 1), pw + NPROD * (h0 ^ 1));
+      if (u == 2 || u == 4) issue_q(5 + (u >> 1), NSV - 1 + (u >> 1));       // (slots 12 and 13 change hands with the item, when everything before is complete)
+#pragma unroll 1
+      for (int gk = kpos + NKS; gk < NKST; gk += NKS) issue_k(gk);
+      kcnt ^= w.npc == 1 ? 0x3Cu : w.npc == 2 ? 0x0Fu : 0u;        // (8, 16 or 24 stages over six positions)
       // V stages reuse the whole staging area: they start when the last S product is complete (the softmax of the last
       // piece is still to come, so the ring is full by the time the PV products start)
       if (lane == 0 && !fail && !mbar_wait(&sm.acc_ev[w.npc - 1], (accb >> (w.npc - 1)) & 1u)) fail = 1;
       __syncwarp();
       {
-        int part = 0, kb = 0, sl = g0;
+        int part = 0, kb = u, h = h0;
 #pragma unroll 1
-        for (int gv = 0; gv < NVST; ++gv) {
-          if (mine(sl)) {
-            const uint32_t slot = ring + (uint32_t)sl * SLOTP;
-            const uint32_t fb_leader = map_to_rank(smem_u32(&sm.fullV[sl]), 0);
-            uint4 vcode = make_uint4(0u, 0u, 0u, 0u);               // (fetched before the wait for the slot)
-            if (w.gather) vcode = codes_at(kb * 128 + 4 * lane);
-            if (lane == 0) {
-              slot_wait(sm.emptyV, vcnt, vused, sl);
-              if (rank == 0) mbar_expect_tx(&sm.fullV[sl], 2 * SLOTP);
-            }
-            __syncwarp();
-            if (w.gather) tma_gather4(slot + lane * 512, &maps.row[vcode.x >> 30], (part * 2 + (int)rank) * 64, vcode, fb_leader);
-            else {                    // key boxes 0..3
-              const int i0 = kb * (128 / kBoxRows);
-              const bool one = consecutive(i0, 4);
-              const uint32_t bx = __shfl_sync(0xffffffffu, box, one ? i0 : i0 + (lane & 3));
-              if (one) { if (lane == 0) tma_box2(slot, &maps.src[bx >> 30][2], (part * 2 + (int)rank) * 64, (int)(bx & 0x3FFFFFFFu), fb_leader); }
-              else if (lane < 4) tma_box2(slot + lane * BOXB, &maps.src[bx >> 30][0], (part * 2 + (int)rank) * 64, (int)(bx & 0x3FFFFFFFu), fb_leader);
-            }
+        for (int gv = u; gv < NVST; gv += NPROD) {
+          while (kb >= nvb) { kb -= nvb; ++part; }
+          const int sl = pw + NPROD * h;
+          const uint32_t slot = ring + (uint32_t)sl * SLOTP;
+          const uint32_t fb_leader = map_to_rank(smem_u32(&sm.fullV[sl]), 0);
+          uint4 vcode = make_uint4(0u, 0u, 0u, 0u);                 // (fetched before the wait for the slot)
+          if (w.gather) vcode = codes_at(kb * 128 + 4 * lane);
+          if (lane == 0) {
+            v_wait(h);
+            if (rank == 0) mbar_expect_tx(&sm.fullV[sl], 2 * SLOTP);
           }
-          vcnt ^= 1u << sl; vused |= 1u << sl;
-          if (++sl == NSV) sl = 0;
-          if (++kb == nvb) { kb = 0; ++part; }
+          __syncwarp();
+          if (w.gather) tma_gather4(slot + lane * 512, &maps.row[vcode.x >> 30], (part * 2 + (int)rank) * 64, vcode, fb_leader);
+          else {                    // key boxes 0..3
+            const int i0 = kb * (128 / kBoxRows);
+            const bool one = consecutive(i0, 4);
+            const uint32_t bx = __shfl_sync(0xffffffffu, box, one ? i0 : i0 + (lane & 3));
+            if (one) { if (lane == 0) tma_box2(slot, &maps.src[bx >> 30][2], (part * 2 + (int)rank) * 64, (int)(bx & 0x3FFFFFFFu), fb_leader); }
+            else if (lane < 4) tma_box2(slot + lane * BOXB, &maps.src[bx >> 30][0], (part * 2 + (int)rank) * 64, (int)(bx & 0x3FFFFFFFu), fb_leader);
+          }
+          vcnt ^= 1u << h; vused |= 1u << h;
+          h ^= 1; kb += NPROD;
         }
       }
       g0 = (g0 + NVST) % NSV;
@@ -393,8 +418,8 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
     }
     // every release has arrived in this CTA before it may leave
     if (lane == 0) {
-      for (int sl = 0; sl < NKS; ++sl) slot_wait(sm.emptyK, kcnt, kused, sl);
-      for (int sl = 0; sl < NSV; ++sl) slot_wait(sm.emptyV, vcnt, vused, sl);
+      if (n_real) for (int sl = 0; sl < NKS; ++sl) if (!fail && !mbar_wait(&sm.emptyK[sl], ((kcnt >> sl) & 1u) ^ 1u)) fail = 1;
+      v_wait(0); v_wait(1);
     }
     __syncwarp();
   } else if (warp == 1) {
@@ -444,8 +469,8 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
             if (!fail && !mbar_wait(&sm.fullK[sl], (kpar >> sl) & 1u)) fail = 1;
             kpar ^= 1u << sl;
             fence_after();
-            const int kphys = sl < NSV - NQS ? place(NQS + sl) : NQS + sl;
-            const uint64_t qd = dk0 + (uint64_t)(place(dk) * (SLOTP >> 4)), kd = dk0 + (uint64_t)(kphys * (SLOTP >> 4));
+            const int kphys = place(k_place(sl)), qphys = dk < NKS ? place(q_place(dk)) : NSV - NKS + dk;
+            const uint64_t qd = dk0 + (uint64_t)(qphys * (SLOTP >> 4)), kd = dk0 + (uint64_t)(kphys * (SLOTP >> 4));
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks) if (one) mma2_ss(scol, qd + 2 * ks, kd + 2 * ks, idesc, (dk | ks) != 0);
             if (one) mma2_commit(&sm.emptyK[sl]);
@@ -493,19 +518,14 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
     const int4* order = reinterpret_cast<const int4*>(ws + pl.off_order);
     if (rank == 0) {
       int32_t* counter = reinterpret_cast<int32_t*>(ws + pl.off_sched);
-      uint32_t cmpb = 0;
-      int base = 0, w0 = -32, q = 0;                    // window: tiles w0 .. w0 + 31, a lane each; base: items before it
+      uint32_t cmpb = 0, accb = 0;
+      int base = 0, w0 = -32;                           // window: tiles w0 .. w0 + 31, a lane each; base: items before it
       int4 rec = make_int4(-1, 0, 0, 0);
       int n = 0, incl = 0, tot = 0;
-#pragma unroll 1
-      for (int it = 0;; ++it) {
-        int4 r = make_int4(rec0.x, rec0.y, rec0.z, 0);
-        if (it >= own) {
-        {
-          int nx = 0x7fffffff;
-          if (lane == 0 && !fail) nx = atomicAdd(counter, 1);
-          q = __shfl_sync(0xffffffffu, nx, 0);
-        }
+      auto take = [&]() {                               // the next item of the device
+        int q = 0x7fffffff;
+        if (lane == 0 && !fail) q = atomicAdd(counter, 1);
+        q = __shfl_sync(0xffffffffu, q, 0);
         while (q >= base + tot && w0 + 32 < ntile) {
           base += tot; w0 += 32;
           n = 0;
@@ -520,22 +540,32 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
           for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += y; }
           tot = __shfl_sync(0xffffffffu, incl, 31);
         }
-        r = make_int4(-1, 0, 0, 0);
+        int4 r = make_int4(-1, 0, 0, 0);
         if (q < base + tot) {
           const uint32_t has = __ballot_sync(0xffffffffu, q - base < incl);
           const int src = __ffs(has) - 1;
           r.x = __shfl_sync(0xffffffffu, rec.x, src); r.y = __shfl_sync(0xffffffffu, rec.y, src); r.z = __shfl_sync(0xffffffffu, rec.z, src);
           r.w = q - base - (__shfl_sync(0xffffffffu, incl, src) - __shfl_sync(0xffffffffu, n, src)) + (w0 + src < P ? 1 : 0);
         }
-        if (lane < 2) st_async16(map_to_rank(smem_u32(&sm.item[(it - own) & 1]), lane), r, map_to_rank(smem_u32(&sm.item_ev), lane));
-        if (lane == 0) mbar_expect_tx(&sm.item_ev, 16);
-        __syncwarp();
+        return r;
+      };
+      int4 r = own ? make_int4(rec0.x, rec0.y, rec0.z, 0) : take();
+#pragma unroll 1
+      for (int it = 0;; ++it) {
+        if (it >= own) {
+          if (lane < 2) st_async16(map_to_rank(smem_u32(&sm.item[(it - own) & 1]), lane), r, map_to_rank(smem_u32(&sm.item_ev), lane));
+          if (lane == 0) mbar_expect_tx(&sm.item_ev, 16);
+          __syncwarp();
         }
         if (r.x < 0) break;
         const Item w(r, pl, GENERAL);
-        if (!fail && !mbar_wait(&sm.cmp_ev[w.npc - 1], (cmpb >> (w.npc - 1)) & 1u)) fail = 1;
-        cmpb ^= w.cmp_used();
+        const int last = w.npc - 1;
+        if (!fail && !mbar_wait(&sm.acc_ev[last], (accb >> last) & 1u)) fail = 1;
+        const int4 next = take();
+        if (!fail && !mbar_wait(&sm.cmp_ev[last], (cmpb >> last) & 1u)) fail = 1;
+        accb ^= w.acc_used(); cmpb ^= w.cmp_used();
         fail = __any_sync(0xffffffffu, fail);
+        r = next;
       }
       // the last pair to run out of items leaves the counters as it found them
       if (lane == 0 && atomicAdd(counter + 1, 1) == P - 1) { counter[0] = 0; counter[1] = 0; __threadfence(); }
