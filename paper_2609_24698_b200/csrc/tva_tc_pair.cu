@@ -49,7 +49,7 @@ constexpr int NSV = 12;                    // Slots [0, 12) are one FIFO: an ite
 // The FIFO's places of an item, about in the order in which the S products want them: Q0 K0 Q1 K1 Q2 K2 K3 Q3 K4 Q4 K5 Q5 (of places
 // p and p + 6, which are one producer's, one is a Q slice, the other a K stage).  Six stages of operands are requested before the item
 // before is done with; with all of Q and four K stages in the FIFO, and the ring's other two stages waiting for the output's staging,
-// the products waited for the fifth stage, requested when the first product was complete: 512-key items 14.8 us.
+// the products waited for the fifth stage, requested when the first product was complete (640-key items 20.2 us, now 19.4).
 __device__ __forceinline__ int q_place(int dk) { return dk < 3 ? 2 * dk : 2 * dk + 1; }         // dk < 6; slices 6 and 7 are in slots 12 and 13
 __device__ __forceinline__ int k_place(int pos) { return pos < 3 ? 2 * pos + 1 : 2 * pos; }     // pos: stage modulo NKS
 
@@ -173,6 +173,7 @@ struct Item {
     nk = r.z; chunk = r.w;
     tc::chunking_x(nk, general, pl.tc_split, pl.tc_f32, nch, CL, f32);
     cbeg = chunk * CL; cend = min(nk, cbeg + CL);
+    CL = max(128, (cend - cbeg + 127) & ~127);           // (the tile's last chunk is as long as what is left)
     npc = (CL + 255) / 256;
     dbl = CL <= 512;
   }
