@@ -87,7 +87,7 @@ bool make_tva_plan(const tsv_shape& s, TvaPlan& p) {
   p.off_po = off;     if (p.nsplit > 1) off = up256(off + (size_t)s.B * s.D * s.H * p.nsplit * s.d * sizeof(float));
   p.off_pml = off;    if (p.nsplit > 1) off = up256(off + (size_t)s.B * s.D * s.H * p.nsplit * 2 * sizeof(float));
   p.tc = tva_tc_eligible(s);
-  p.tc_nt = p.tc_maxk = p.tc_chmax = p.tc_misc_rows = 0; p.tc_split = 1; p.tc_f32 = p.tc_packed = 0;
+  p.tc_nt = p.tc_maxk = p.tc_chmax = p.tc_misc_rows = 0; p.tc_split = 1; p.tc_f32 = p.tc_general = p.tc_packed = 0;
   p.off_krow = p.off_kmask = p.off_nkeys = p.off_tpo = p.off_tpml = p.off_box = p.off_mode = p.off_misc = p.off_order = p.off_tcnt = p.off_sched = off;
   p.off_selmask = off;
   p.mask_ld = ((p.cand_cap + 31) / 32 + 3) & ~3;

@@ -51,6 +51,7 @@ struct TvaPlan {
   int32_t tc, tc_nt, tc_maxk, tc_chmax;
   int32_t tc_split;                  // chunks a tile may be cut into to fill the device (1: tiles enough)
   int32_t tc_f32;                    // all partial outputs are fp32 (set at the launch)
+  int32_t tc_general;                // the chunking rule of the general instantiation (set at the launch)
   int32_t tc_misc_rows;              // rows of the per-sequence packed buffer
   int32_t tc_packed;                 // the state build has put the entries closed inside the tree into that buffer (set at the launch)
   size_t off_krow, off_kmask, off_nkeys, off_tpo, off_tpml, off_box, off_mode, off_misc, off_order, off_tcnt, off_sched;   // off_sched: the paired kernel's item counter, the pairs that have run out of items

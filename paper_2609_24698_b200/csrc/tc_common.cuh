@@ -126,6 +126,21 @@ __device__ __host__ __forceinline__ void chunking_x(int nk, bool general, int sp
   nch = (nk + CL - 1) / CL;
   if (nch < 1) nch = 1;
 }
+// The record of a tile, which the tile plan leaves and the kernels after it read: {sequence, what, keys, 0}, what = mode (2 bits: 1
+// boxes, 2 gathered) | fp32 partial outputs << 2 | chunk length / 128 << 4 | tile of the sequence << 7 | chunks << 12.  (The chunking is
+// three divisions: by every role of the attention kernel on its own they were 10 KB of its code.)
+__device__ __forceinline__ int4 tile_record(const TvaPlan& pl, int b, int tile, int mode, int nk) {
+  int nch, CL;
+  bool f32;
+  chunking_x(nk, pl.tc_general != 0, pl.tc_split, pl.tc_f32, nch, CL, f32);
+  return make_int4(b, mode | (f32 ? 4 : 0) | (CL / 128) << 4 | tile << 7 | nch << 12, nk, 0);
+}
+static_assert(NCX / 128 < 8 && TSV_MAX_D * 128 / PR <= 32, "fields of a tile's record");
+__device__ __forceinline__ bool rec_gather(const int4& r) { return (r.y & 3) == 2; }
+__device__ __forceinline__ bool rec_f32(const int4& r) { return (r.y & 4) != 0; }
+__device__ __forceinline__ int rec_chunk_keys(const int4& r) { return ((r.y >> 4) & 7) * 128; }
+__device__ __forceinline__ int rec_tile(const int4& r) { return (r.y >> 7) & 31; }
+__device__ __forceinline__ int rec_chunks(const int4& r) { return (int)((uint32_t)r.y >> 12); }
 
 }  // namespace tc
 

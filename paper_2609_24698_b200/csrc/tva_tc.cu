@@ -75,7 +75,7 @@ __device__ __forceinline__ void tc_plan_tile(const tsv_shape& s, const TvaPlan& 
   // thread 0 leaves the tile's record {tile, mode, keys} at that position as soon as it knows the key count
   auto leave_record = [&](int nk, int md) {
     *nkeys = nk; *mode = md;
-    reinterpret_cast<int4*>(ws + pl.off_order)[ntile <= kRankTilesMax ? *ahead_sm : (int)tix] = make_int4((int)tix, md, nk, 0);
+    reinterpret_cast<int4*>(ws + pl.off_order)[ntile <= kRankTilesMax ? *ahead_sm : (int)tix] = tc::tile_record(pl, b, tile, md, nk);
   };
   // The kernel is launched as a programmatic dependent of the selection kernel (itself one of the state build) and runs
   // under those kernels' tails as far as it reads only the caller's inputs and the committed caches: the done flags are
@@ -405,14 +405,10 @@ __global__ void __launch_bounds__(256) tc_combine_pair_kernel(const tsv_shape s,
   // implies that one's.
   const bool early = pl.tc_split == 1;
   if (blockIdx.x == 0 || !early) asm volatile("griddepcontrol.wait;" ::: "memory");
-  const int nk = rec.z, b = (uint32_t)rec.x / (uint32_t)pl.tc_nt, rt = (rec.x - b * pl.tc_nt) * 2 + half;
-  const size_t rix = (size_t)rec.x * 2 + half;
-  if (nk <= 0) return;
-  int nch, CL;
-  bool f32;
-  chunking_x(nk, true, pl.tc_split, pl.tc_f32, nch, CL, f32);
-  if (!ANY32) f32 = false;                                       // (no tile is split, so one with more than one chunk was too long for one: bf16)
-  if (nch <= 1) return;                                          // the paired kernel wrote the output itself
+  const int b = rec.x, rt = rec_tile(rec) * 2 + half, nch = rec_chunks(rec);
+  const size_t rix = (size_t)b * 2 * pl.tc_nt + rt;
+  if (rec.z <= 0 || nch <= 1) return;                            // (one chunk: the paired kernel wrote the output itself)
+  const bool f32 = ANY32 && rec_f32(rec);                        // (where no tile is split, one with more than one chunk was too long for one: bf16)
   const int rows_seq = s.D * s.H, row0 = rt * BM, lane = threadIdx.x & 31;
   const int first = group * 8 * rpw + (threadIdx.x >> 5), last = min(min(BM, rows_seq - row0), (group + 1) * 8 * rpw);
   if (first >= last) return;
@@ -561,6 +557,11 @@ int launch_tva_tc(const tsv_shape& s, const TvaPlan& p_in, const TvaTcPrep& prep
                   void* out, char* ws, int32_t* status, cudaStream_t st, bool with_plan) {
   TvaPlan p = p_in;
   const bool gathered = gathered_tiles_possible(s, p, c);
+  // general: some tile may have more than two chunks of the longest kind, or be gathered; then every multi-chunk tile
+  // leaves bf16 partial outputs for the merge kernel
+  const bool many = (p.tc_maxk + tc::NCX - 1) / tc::NCX > 2 || gathered, general = many || p.tc_split > 1;
+  p.tc_f32 = !many;                                    // (no more than two long chunks a tile: merged without rounding in either instantiation)
+  p.tc_general = general;
   const dim3 pgrid(p.tc_nt + 1, s.B);                                                                              // x: tiles + the packing CTA
   if (with_plan) {
     cudaLaunchConfig_t cfg = {};
@@ -575,10 +576,6 @@ int launch_tva_tc(const tsv_shape& s, const TvaPlan& p_in, const TvaTcPrep& prep
     else cudaLaunchKernelEx(&cfg, tc_plan_kernel<false, 256>, s, p, c, nd, sc, ws);
   }
   count_launch();
-  // general: some tile may have more than two chunks of the longest kind, or be gathered; then every multi-chunk tile
-  // leaves bf16 partial outputs for the merge kernel
-  const bool many = (p.tc_maxk + tc::NCX - 1) / tc::NCX > 2 || gathered, general = many || p.tc_split > 1;
-  p.tc_f32 = !many;                                    // (no more than two long chunks a tile: merged without rounding in either instantiation)
   const int r = launch_tva_tc_pair(s, p, prep, general, nd.q, out, ws, status, st);
   if (r != TSV_OK) return r;
   if (general && p.tc_chmax > 1) {

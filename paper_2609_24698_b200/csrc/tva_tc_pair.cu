@@ -31,10 +31,10 @@ namespace pair {
 using namespace tc;
 
 // Warps: 0, 3, 12-15 producers; 1 MMA issuer; 2 hands out the items; 4-11 softmax and epilogue.  The service warpgroups give
-// registers to the compute warpgroups: 128 x (96 + 160 + 160 + 96) of the 512 x 128 the CTA is launched with.
+// registers to the compute warpgroups: 128 x (120 + 136 + 136 + 120) of the 512 x 128 the CTA is launched with.
 constexpr int TTHREADS = 512;
 constexpr int NPROD = 6;                    // (12 slots: six producers with two each)
-constexpr int REGS_SERVICE = 96, REGS_COMPUTE = 160;
+constexpr int REGS_SERVICE = 120, REGS_COMPUTE = 136;
 static_assert(128 * (2 * REGS_SERVICE + 2 * REGS_COMPUTE) <= TTHREADS * 128, "register split beyond what the CTA is launched with");
 constexpr int BOXB = kBoxRows * 128;       // bytes of one box: kBoxRows rows x 128 bytes
 constexpr float RESCALE_GAP = 16.f;        // log2 units a later piece's row max may exceed the running reference
@@ -65,8 +65,8 @@ struct Ctl {                               // control block at the start of dyna
   uint64_t item_ev;                        // the next item has been handed out
   uint32_t tmem_base;
   int32_t merge_here;                      // set for the CTA that finished a multi-chunk tile last
-  alignas(16) int4 item[2];                // the pair's current and next work: {tile index (-1: no more), mode, keys, chunk}
-  float xch[2][BM];                        // first-slab maxima of the rows, by the two warps that share them
+  alignas(16) int4 item[2];                // the pair's current and next work: the tile's record with the chunk (sequence -1: no more)
+  float xch[2][2][BM];                     // first-slab maxima of the rows, by the two warps that share them (two buffers in turn)
 };
 constexpr int CTLB = 3072;                 // control block bytes; the ring follows (needs a 1024-byte aligned base)
 constexpr int SLOTP = 16384;               // ring slot: every stage of a CTA is at most 16 KiB
@@ -167,12 +167,12 @@ struct Item {
   bool dbl;                // two O buffers: a part is computed while the one before is read out
   bool f32;                // partial outputs are fp32
   bool gather;             // the key list is a list of row codes (array << 30 | row), not of boxes
-  __device__ __forceinline__ Item(int4 r, const TvaPlan& pl, bool general) {
-    tix = r.x; b = r.x / pl.tc_nt; tile = r.x - b * pl.tc_nt;
-    gather = general && r.y == 2;
-    nk = r.z; chunk = r.w;
-    tc::chunking_x(nk, general, pl.tc_split, pl.tc_f32, nch, CL, f32);
-    cbeg = chunk * CL; cend = min(nk, cbeg + CL);
+  __device__ __forceinline__ Item(int4 r, const TvaPlan& pl, bool general) {      // a tile's record, the chunk in its last word
+    b = r.x; tile = rec_tile(r); tix = b * pl.tc_nt + tile;
+    gather = general && rec_gather(r); f32 = general && rec_f32(r);
+    nk = r.z; chunk = r.w; nch = rec_chunks(r);
+    const int stride = rec_chunk_keys(r);
+    cbeg = chunk * stride; cend = min(nk, cbeg + stride);
     CL = max(128, (cend - cbeg + 127) & ~127);           // (the tile's last chunk is as long as what is left)
     npc = (CL + 255) / 256;
     dbl = CL <= 512;
@@ -257,7 +257,7 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
   fence_after();
   const uint32_t tm = sm.tmem_base;
   const int rows_seq = s.D * s.H;
-  // Item n of this pair (tile index -1: no more).  Item 0 is the first chunk of the tile of this pair's rank, which every warp
+  // Item n of this pair (sequence -1: no more).  Item 0 is the first chunk of the tile of this pair's rank, which every warp
   // looks up itself; the others are handed out (warp 2).  The wait is made whatever failed before (a failure skips later
   // waits, never a step of the protocol, so that no warp is left alone at a barrier), and is longer than any other.
   const int own = rec0.z > 0 ? 1 : 0;
@@ -531,10 +531,8 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
           base += tot; w0 += 32;
           n = 0;
           if (w0 + lane < ntile) {
-            int CL;
-            bool f32;
             rec = order[w0 + lane];
-            if (rec.z > 0) { chunking_x(rec.z, GENERAL, pl.tc_split, pl.tc_f32, n, CL, f32); if (w0 + lane < P) --n; }     // (the first chunks of the first P tiles are given)
+            if (rec.z > 0) { n = rec_chunks(rec); if (w0 + lane < P) --n; }     // (the first chunks of the first P tiles are given)
           }
           incl = n;
 #pragma unroll
@@ -585,11 +583,11 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
       if (t0 + lane * P < ntile) rz = order[t0 + lane * P];
       uint32_t zero = __ballot_sync(0xffffffffu, rz.z <= 0);
       while (zero) {
-        const int tix = __shfl_sync(0xffffffffu, rz.x, __ffs(zero) - 1), b = tix / pl.tc_nt, row0 = (tix - b * pl.tc_nt) * PR + (int)rank * BM;
+        const int src = __ffs(zero) - 1, b = __shfl_sync(0xffffffffu, rz.x, src), row0 = __shfl_sync(0xffffffffu, rec_tile(rz), src) * PR + (int)rank * BM;
         zero &= zero - 1;
         uint4* o4 = reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(out_) + ((size_t)b * rows_seq + row0) * DH);
         const int n16 = min(BM, rows_seq - row0) * (DH / 8);
-#pragma unroll 4
+#pragma unroll 1
         for (int i = lane; i < n16; i += 32) o4[i] = make_uint4(0, 0, 0, 0);
       }
     }
@@ -648,22 +646,21 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
     // before: no warp waits for another.  (A two-pass softmax with contiguous halves needed three barriers a piece and
     // read S twice.)
     constexpr uint32_t FULL = 0xffffffffu;
-    uint32_t* xch = reinterpret_cast<uint32_t*>(sm.xch);
+    uint32_t* xch = reinterpret_cast<uint32_t*>(sm.xch) + (it & 1) * 2 * BM;
     auto pair_sync = [&]() { asm volatile("bar.sync %0, 64;" ::"r"(2 + q4) : "memory"); };     // the two warps of these rows
     auto slab_of = [&](int i) { return (i & 1) + ((i & 2) << 1) + 2 * hh; };
-    auto masked = [&](const uint32_t* sv, uint32_t vis, float* v) {      // invisible keys as -inf
-      if (vis == FULL) {
+    // slab i of this warp in the piece whose S begins at column scol: read, invisible keys as -inf; the maximum (unscaled)
+    auto read_slab = [&](uint32_t scol, int i, uint32_t vis, uint32_t (&sv)[32]) {
+      tmem_ld32(scol + slab_of(i) * 32, sv);
+      if (vis != FULL) {
 #pragma unroll
-        for (int t = 0; t < 32; ++t) v[t] = __uint_as_float(sv[t]);
-      } else {
-#pragma unroll
-        for (int t = 0; t < 32; ++t) v[t] = ((vis >> t) & 1u) ? __uint_as_float(sv[t]) : -INFINITY;
+        for (int t = 0; t < 32; ++t) if (!((vis >> t) & 1u)) sv[t] = 0xff800000u;
       }
-    };
-    auto max32 = [&](const float* v) {
-      float mc[4] = {v[0], v[1], v[2], v[3]};
+      float mc[4];
 #pragma unroll
-      for (int t = 4; t < 32; ++t) mc[t & 3] = fmaxf(mc[t & 3], v[t]);
+      for (int c = 0; c < 4; ++c) mc[c] = __uint_as_float(sv[c]);
+#pragma unroll
+      for (int t = 4; t < 32; ++t) mc[t & 3] = fmaxf(mc[t & 3], __uint_as_float(sv[t]));
       return fmaxf(fmaxf(mc[0], mc[1]), fmaxf(mc[2], mc[3]));
     };
     // multiplies this thread's P columns [64 hh of every piece before pc, the first n slabs of piece pc] by f
@@ -686,82 +683,70 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
       for (int c = 0; c < 4; ++c) lp[c] *= f;
     };
     int moved = 0;                                   // this warp changed its reference after the exchange
-    auto do_slab = [&](const uint32_t* sv, uint32_t vis, int pc, int i) {
-      float v[32];
-      uint32_t pk[16];
-      masked(sv, vis, v);
-      const float mc = max32(v) * scale2;
-      if (__any_sync(FULL, mc > m_run + RESCALE_GAP)) {        // (warp-uniform: tensor-memory accesses are warp-collective)
-        const float to = mc > m_run + RESCALE_GAP ? mc : m_run;
-        rescale_p(pc, i, ex2(m_run - to));
-        m_run = to;
-        moved = 1;
-      }
-#pragma unroll
-      for (int t = 0; t < 32; t += 2) {
-        const float p0 = ex2(fmaf(v[t], scale2, -m_run)), p1 = ex2(fmaf(v[t + 1], scale2, -m_run));
-        lp[(t >> 1) & 3] += p0 + p1;
-        const __nv_bfloat162 h2 = __floats2bfloat162_rn(p0, p1);
-        pk[t >> 1] = *reinterpret_cast<const uint32_t*>(&h2);
-      }
-      tmem_st16(tlane + pc * 128 + hh * 64 + i * 16, pk);
-    };
     // Node masks of this lane's keys of a piece, a byte per slab; fetched a piece ahead (fetched when needed they cost the chain a
     // memory latency, 1.3 k cycles per piece after the first).
-    uint8_t km[4];
+    uint32_t km = 0;
     auto fetch_masks = [&](int pc) {
+      km = 0;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const int key = pc * 256 + slab_of(i) * 32 + lane;
-        km[i] = key < CL && w.cbeg + key < w.cend ? __ldg(kmask_g + key) : (uint8_t)0;
+        if (key < CL && w.cbeg + key < w.cend) km |= (uint32_t)__ldg(kmask_g + key) << (8 * i);
       }
     };
     fetch_masks(0);
 #pragma unroll 1
     for (int pc = 0; pc < npc; ++pc) {
       const int ns = CL - pc * 256 >= 256 ? 4 : 2;   // slabs of this warp
-      // visibility, 32 keys per word: the 32 rows of a warp belong to one node (H >= 32 on this path), so one ballot over the
+      const uint32_t km_now = km;
+      // visibility of a slab, a bit per key: the 32 rows of a warp belong to one node (H >= 32 on this path), so one ballot over the
       // keys' node masks gives the word
-      uint32_t vis[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) vis[i] = __ballot_sync(FULL, km[i] & mybit);
+      auto visible = [&](int i) { return __ballot_sync(FULL, (km_now >> (8 * i)) & mybit); };
       if (pc + 1 < npc) fetch_masks(pc + 1);
       if (!fail && !mbar_wait(&sm.acc_ev[pc], (accb >> pc) & 1u)) fail = 1;
       fence_after();
       const uint32_t scol = tlane + (pc == 0 ? 0 : 256);
-      uint32_t sv[2][32];
+      // One slab after the other in a loop of one slab's code: what the two warps of a scheduler leave idle is the other's, and the
+      // instructions of four slabs side by side did not stay in the instruction cache (kernel of 97 KB, a slab 900 cycles; 512 is what
+      // the special-function unit needs for the two warps).
       if (m_run == -INFINITY) {                      // uniform over the two warps of these rows: no visible key so far
-        const int first = vis[0] ? 0 : vis[1] ? 1 : vis[2] ? 2 : vis[3] ? 3 : -1;
-        float mc = -INFINITY;
-        if (first >= 0) {
-          uint32_t s0[32];
-          const uint32_t vw = first == 0 ? vis[0] : first == 1 ? vis[1] : first == 2 ? vis[2] : vis[3];
-          tmem_ld32(scol + slab_of(first) * 32, s0);
-          float v[32];
-          masked(s0, vw, v);
-          mc = max32(v);
-        }
+        int i = 0;
+        uint32_t vis = 0;
+#pragma unroll 1
+        for (; i < ns; ++i) if ((vis = visible(i)) != 0) break;
+        uint32_t sv[32];
+        const float mc = i < ns ? read_slab(scol, i, vis, sv) : -INFINITY;
         xch[hh * BM + row] = __float_as_uint(mc);
         pair_sync();
         m_run = fmaxf(mc, __uint_as_float(xch[(hh ^ 1) * BM + row])) * scale2;
-        pair_sync();                                 // (the exchange words may be written again)
+        if (m_run == -INFINITY) pair_sync();         // (the exchange words will be written again before the next item)
       }
       const bool any = m_run != -INFINITY;
-      tmem_ld32_nowait(scol + slab_of(0) * 32, sv[0]);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        if (i < ns) {
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-          tmem_regs_ready(sv[i & 1]);
-          if (i + 1 < ns) tmem_ld32_nowait(scol + slab_of(i + 1) * 32, sv[(i + 1) & 1]);
-          if (any && vis[i]) do_slab(sv[i & 1], vis[i], pc, i);
-          else {
-            uint32_t z[16];
-#pragma unroll
-            for (int t = 0; t < 16; ++t) z[t] = 0u;
-            tmem_st16(tlane + pc * 128 + hh * 64 + i * 16, z);
+#pragma unroll 1
+      for (int i = 0; i < ns; ++i) {
+        uint32_t pk[16];
+        const uint32_t vis = visible(i);
+        if (any && vis) {
+          uint32_t sv[32];
+          const float mc = read_slab(scol, i, vis, sv) * scale2;
+          if (__any_sync(FULL, mc > m_run + RESCALE_GAP)) {        // (warp-uniform: tensor-memory accesses are warp-collective)
+            const float to = mc > m_run + RESCALE_GAP ? mc : m_run;
+            rescale_p(pc, i, ex2(m_run - to));
+            m_run = to;
+            moved = 1;
           }
+#pragma unroll
+          for (int t = 0; t < 32; t += 2) {
+            const float p0 = ex2(fmaf(__uint_as_float(sv[t]), scale2, -m_run)), p1 = ex2(fmaf(__uint_as_float(sv[t + 1]), scale2, -m_run));
+            lp[(t >> 1) & 3] += p0 + p1;
+            const __nv_bfloat162 h2 = __floats2bfloat162_rn(p0, p1);
+            pk[t >> 1] = *reinterpret_cast<const uint32_t*>(&h2);
+          }
+        } else {
+#pragma unroll
+          for (int t = 0; t < 16; ++t) pk[t] = 0u;
         }
+        tmem_st16(tlane + pc * 128 + hh * 64 + i * 16, pk);
       }
       // the MMA warp waits for the last piece only (and, with three pieces, for piece 1 before it overwrites that
       // piece's S columns); the wait for the stores of a later piece covers the earlier ones
@@ -775,10 +760,14 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
       const uint32_t mine = ring + (uint32_t)NSV * SLOTP + (uint32_t)(warp - 4) * 4096, other = ring + (uint32_t)NSV * SLOTP + (uint32_t)((warp - 4) ^ 4) * 4096;
       auto put = [&](int i, float v) { asm volatile("st.shared.b32 [%0], %1;" ::"r"(mine + (uint32_t)(i * 128 + lane * 4)), "r"(__float_as_uint(v)) : "memory"); };
       auto get = [&](int i) { uint32_t v; asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(other + (uint32_t)(i * 128 + lane * 4)) : "memory"); return __uint_as_float(v); };
-      put(0, l_row); put(1, m_run); put(2, moved ? 1.f : 0.f);
+      // (no reference moved, as nearly always: P is announced before the sums are exchanged)
+      uint32_t any_moved;
+      asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\tbarrier.cta.red.or.pred q, %2, 64, p;\n\tselp.b32 %0, 1, 0, q;\n\t}" : "=r"(any_moved) : "r"(moved), "r"(2 + q4) : "memory");
+      if (!any_moved) p_stored(npc - 1);
+      put(0, l_row); put(1, m_run);
       pair_sync();
       float l_other = get(0);
-      if (moved || get(2) != 0.f) {                  // warp-uniform, and alike in both warps
+      if (any_moved) {                               // (alike in both warps)
         const float m_other = get(1), to = fmaxf(m_run, m_other);
         if (to != -INFINITY) {
           const float f = ex2(m_run - to), fo = ex2(m_other - to);
@@ -787,12 +776,11 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
           l_row *= f; l_other *= fo;
           m_run = to;
         }
+        p_stored(npc - 1);
       }
-      p_stored(npc - 1);
       l_row += l_other;
     }
 
-    const bool rowok = row0 + row < rows_seq;
     const bool full_tile = row0 + BM <= rows_seq;     // whole tile inside the sequence: rows may be stored as 32-row boxes
     const float inv = l_row > 0.f ? 1.f / l_row : 0.f;
     constexpr int cw = OW / 2;                        // columns of the part this thread handles
@@ -802,101 +790,91 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
     for (int part = 0; part < NQ; ++part) {
       if (!fail && !mbar_wait(&sm.acc_ev[3 + part], (accb >> (3 + part)) & 1u)) fail = 1;
       fence_after();
-      do {
-        uint32_t r0[32], r1[32];
-        const uint32_t ocol = tlane + (w.dbl ? 256 + (part & 1) * OW : 384) + hh * cw;
-        tmem_ld32_nowait(ocol, r0);
-        tmem_ld32_nowait(ocol + 32, r1);
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        tmem_regs_ready(r0);
-        tmem_regs_ready(r1);
+      const uint32_t ocol = tlane + (w.dbl ? 256 + (part & 1) * OW : 384) + hh * cw;
+      const int col = part * OW + hh * cw;
+      const bool many = GENERAL && nch > 1;
+      auto read_out = [&]() {                        // in registers: the columns may be overwritten
         fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(map_to_rank(smem_u32(&sm.cmp_ev[3 + part]), 0));   // in registers: the columns may be overwritten
-        const int col = part * OW + hh * cw;
-        const bool many = GENERAL && nch > 1;
-        if ((nch == 1 && full_tile) || many) {
+        if (lane == 0) mbar_arrive_cluster(map_to_rank(smem_u32(&sm.cmp_ev[3 + part]), 0));
+      };
+      auto stage_read = [&]() {                      // the store before has read the staging tile
+        if (stored) {
+          if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+          __syncwarp();
+        }
+        stored = true;
+      };
+      auto stage_store = [&](const CUtensorMap* map, int x, int y) {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) {
+          asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];"
+                       ::"l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(stage) : "memory");
+          asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+        }
+      };
+      if (many && w.f32) {
+        // fp32 partial output: two tiles of 32 rows x 32 columns
+#pragma unroll 1
+        for (int x = 0; x < 2; ++x) {
+          uint32_t r[32];
+          tmem_ld32(ocol + 32 * x, r);
+          if (x) read_out();
+          stage_read();
+#pragma unroll
+          for (int v = 0; v < 8; ++v)
+            asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(stage + lane * 128 + ((v ^ (lane & 7)) << 4)), "f"(__uint_as_float(r[4 * v]) * inv),
+                         "f"(__uint_as_float(r[4 * v + 1]) * inv), "f"(__uint_as_float(r[4 * v + 2]) * inv), "f"(__uint_as_float(r[4 * v + 3]) * inv) : "memory");
+          stage_store(&maps.part32, col + 32 * x, (int)((rix * pl.tc_chmax + chunk) * BM) + q4 * 32);
+        }
+      } else {
+        uint32_t r[64];
+        tmem_ld32_nowait(ocol, r);
+        tmem_ld32_nowait(ocol + 32, r + 32);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        tmem_regs_ready(r);
+        tmem_regs_ready(r + 32);
+        read_out();
+        if (nch == 1 || many) {
           // stage the 32 x 64 bf16 tile in the 128-byte swizzle pattern and store it with one TMA request: into the output,
           // or (multi-chunk tiles, where a merge kernel follows) into the chunk's tile of normalised partial outputs, which a merge kernel
           // combines with the chunks' (max, sum)
-          if (many && w.f32) {               // fp32: two tiles of 32 columns
-#pragma unroll
-            for (int x = 0; x < 2; ++x) {
-              if (stored) {
-                if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-                __syncwarp();
-              }
-              stored = true;
-#pragma unroll
-              for (int v = 0; v < 8; ++v) {
-                float f[4];
-#pragma unroll
-                for (int t = 0; t < 4; ++t) f[t] = __uint_as_float(x ? r1[v * 4 + t] : r0[v * 4 + t]) * inv;
-                asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(stage + lane * 128 + ((v ^ (lane & 7)) << 4)), "f"(f[0]), "f"(f[1]),
-                             "f"(f[2]), "f"(f[3]) : "memory");
-              }
-              asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-              __syncwarp();
-              if (lane == 0) {
-                asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];"
-                             ::"l"(reinterpret_cast<uint64_t>(&maps.part32)), "r"(col + 32 * x), "r"((int)((rix * pl.tc_chmax + chunk) * BM) + q4 * 32), "r"(stage) : "memory");
-                asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-              }
-            }
-            continue;
-          }
-          if (stored) {                                // the store before has read the tile
-            if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-            __syncwarp();
-          }
+          stage_read();
 #pragma unroll
           for (int v = 0; v < 8; ++v) {
-            const uint32_t* src = v < 4 ? r0 + v * 8 : r1 + (v - 4) * 8;
-            uint32_t w[4];
+            uint32_t pk[4];
 #pragma unroll
             for (int t = 0; t < 4; ++t) {
-              const __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(src[2 * t]) * inv, __uint_as_float(src[2 * t + 1]) * inv);
-              w[t] = *reinterpret_cast<const uint32_t*>(&h2);
+              const __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(r[8 * v + 2 * t]) * inv, __uint_as_float(r[8 * v + 2 * t + 1]) * inv);
+              pk[t] = *reinterpret_cast<const uint32_t*>(&h2);
             }
-            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(stage + lane * 128 + ((v ^ (lane & 7)) << 4)), "r"(w[0]), "r"(w[1]),
-                         "r"(w[2]), "r"(w[3]) : "memory");
+            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(stage + lane * 128 + ((v ^ (lane & 7)) << 4)), "r"(pk[0]), "r"(pk[1]), "r"(pk[2]),
+                         "r"(pk[3]) : "memory");
           }
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-          __syncwarp();
-          if (lane == 0) {
-            const CUtensorMap* omap = many ? &maps.part : &maps.out;
-            // (a chunk's bf16 tile lies at the start of the chunk's slot for an fp32 tile: 2 BM rows of 1 KiB per slot)
-            const int orow = many ? (int)((rix * pl.tc_chmax + chunk) * 2 * BM) + q4 * 32 : b * rows_seq + row0 + q4 * 32;
-            asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];"
-                         ::"l"(reinterpret_cast<uint64_t>(omap)), "r"(col), "r"(orow), "r"(stage) : "memory");
-            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-          }
-          stored = true;
-        } else if (nch == 1) {
-          if (rowok) {
-            bf16* orow = reinterpret_cast<bf16*>(out_) + ((size_t)b * rows_seq + row0 + row) * DH + col;
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-              float f[8];
-#pragma unroll
-              for (int t = 0; t < 8; ++t) f[t] = __uint_as_float(r0[v * 8 + t]) * inv;
-              st16(orow + v * 8, f);
-#pragma unroll
-              for (int t = 0; t < 8; ++t) f[t] = __uint_as_float(r1[v * 8 + t]) * inv;
-              st16(orow + 32 + v * 8, f);
+          // (a chunk's bf16 tile lies at the start of the chunk's slot for an fp32 tile: 2 BM rows of 1 KiB per slot)
+          if (many) stage_store(&maps.part, col, (int)((rix * pl.tc_chmax + chunk) * 2 * BM) + q4 * 32);
+          else if (full_tile) stage_store(&maps.out, col, b * rows_seq + row0 + q4 * 32);
+          else {                                     // the rows of this sequence only: plain stores, 64 columns of a row by eight lanes
+            __syncwarp();
+#pragma unroll 1
+            for (int i = lane; i < 32 * 8; i += 32) {
+              const int rr = i >> 3;
+              uint4 v;
+              asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(stage + rr * 128 + (((i ^ rr) & 7) << 4)) : "memory");
+              if (row0 + q4 * 32 + rr < rows_seq)
+                reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(out_) + ((size_t)b * rows_seq + row0 + q4 * 32 + rr) * DH + col)[i & 7] = v;
             }
+            __syncwarp();                            // (the tile is written again)
+            stored = false;
           }
         } else {
           float* po = reinterpret_cast<float*>(ws + pl.off_tpo) + ((rix * pl.tc_chmax + chunk) * BM + row) * DH + col;
 #pragma unroll
-          for (int v = 0; v < 8; ++v) {
-            *reinterpret_cast<float4*>(po + v * 4) = make_float4(__uint_as_float(r0[v * 4]), __uint_as_float(r0[v * 4 + 1]),
-                                                                 __uint_as_float(r0[v * 4 + 2]), __uint_as_float(r0[v * 4 + 3]));
-            *reinterpret_cast<float4*>(po + 32 + v * 4) = make_float4(__uint_as_float(r1[v * 4]), __uint_as_float(r1[v * 4 + 1]),
-                                                                      __uint_as_float(r1[v * 4 + 2]), __uint_as_float(r1[v * 4 + 3]));
-          }
+          for (int v = 0; v < 16; ++v)
+            *reinterpret_cast<float4*>(po + v * 4) = make_float4(__uint_as_float(r[4 * v]), __uint_as_float(r[4 * v + 1]), __uint_as_float(r[4 * v + 2]), __uint_as_float(r[4 * v + 3]));
         }
-      } while (0);
+      }
       if (nch > 1 && part == 0 && hh == 0)
         reinterpret_cast<float2*>(ws + pl.off_tpml)[(rix * pl.tc_chmax + chunk) * BM + row] = make_float2(m_run, l_row);
     }
