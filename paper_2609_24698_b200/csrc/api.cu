@@ -84,6 +84,8 @@ bool make_tva_plan(const tsv_shape& s, TvaPlan& p) {
   p.off_selcnt = off; off = up256(off + (size_t)s.B * s.D * sizeof(int32_t));
   p.off_sel = off;    off = up256(off + (size_t)s.B * s.D * s.topk * sizeof(int32_t));
   p.off_scores = off; if (p.need_scores) off = up256(off + (size_t)s.B * s.D * p.score_ld * sizeof(float));
+  p.ext_ld = (int32_t)((pref + 255) / 256 * 4);
+  p.off_ext = off;    if (p.need_scores) off = up256(off + (size_t)s.B * s.D * p.ext_ld * 2 * sizeof(float));
   p.off_po = off;     if (p.nsplit > 1) off = up256(off + (size_t)s.B * s.D * s.H * p.nsplit * s.d * sizeof(float));
   p.off_pml = off;    if (p.nsplit > 1) off = up256(off + (size_t)s.B * s.D * s.H * p.nsplit * 2 * sizeof(float));
   p.tc = tva_tc_eligible(s);

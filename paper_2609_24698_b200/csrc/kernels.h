@@ -40,13 +40,14 @@ struct AarLayers {
 struct TvaPlan {
   int32_t cand_cap;      // max CSA candidates per node (committed + in-tree)
   int32_t score_ld;      // floats per node row of the score array: cand_cap rounded up to 4 (16-byte rows)
+  int32_t ext_ld;        // ranges (lowest, highest score) kept per node, one per 64 entries (score_rows_kernel)
   int32_t need_scores;   // cand_cap > topk: some node may have to rank its candidates
   int32_t idx_fused;     // ranked nodes score their committed entries inside topk_kernel (short candidate lists: the
                          // separate scoring kernel, which exits at once for every sequence that needs no ranking, is not launched)
   int32_t keys_max;      // max keys one node can attend to
   int32_t ks;            // keys per split (CUDA-core path)
   int32_t nsplit;        // max splits per node
-  size_t off_selcnt, off_sel, off_scores, off_po, off_pml, total;
+  size_t off_selcnt, off_sel, off_scores, off_ext, off_po, off_pml, total;
   // tensor-core path (bf16, d = 512): row tiles per sequence, key-list capacity per tile, max chunks per tile
   int32_t tc, tc_nt, tc_maxk, tc_chmax;
   int32_t tc_split;                  // chunks a tile may be cut into to fill the device (1: tiles enough)

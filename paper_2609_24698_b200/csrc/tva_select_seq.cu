@@ -554,8 +554,10 @@ __global__ void __launch_bounds__(128) score_rows_kernel(const tsv_shape s, cons
   sco.weights(nd.iw + (size_t)b * D * HI, n0, D, HI);
   __syncthreads();
   float* scores = reinterpret_cast<float*>(ws + pl.off_scores) + (size_t)b * D * pl.score_ld;
-  // (the call before on the same workspace may still be read: nothing is written before the kernel before has ended)
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  // No wait before the scores are written: the kernel before is the state build, whose dependents start when it has waited for all
+  // earlier work (the call before on this workspace included), or one that starts its dependents when it has ended.  (With a wait for
+  // the state build's end here four sequences of 128 k tokens began to score 8.6 us after its start instead of XX: YY us a pass.)
+  float lo = INFINITY, hi = -INFINITY;                   // of node n0 + lane / 4, over this warp's entries (a NaN stays in lo)
 #pragma unroll
   for (int st = 0; st < kRowSteps; ++st) {
     const int e = first + st * 64;
@@ -564,12 +566,22 @@ __global__ void __launch_bounds__(128) score_rows_kernel(const tsv_shape s, cons
     sco.score(alo, ahi, qs, bufs[w]);
     const float4 v = *reinterpret_cast<const float4*>(bufs[w] + 4 * lane);
     const int n = n0 + (lane >> 2), i = e + 4 * (lane & 3);            // (rows of the score array are padded to whole float4)
-    if (n < D && i < n_ent) *reinterpret_cast<float4*>(scores + (size_t)n * pl.score_ld + i) = v;
+    if (n < D && i < n_ent) {                            // (entries past the last one are copies of it)
+      *reinterpret_cast<float4*>(scores + (size_t)n * pl.score_ld + i) = v;
+      lo = min_or_nan(min_or_nan(lo, v.x), min_or_nan(min_or_nan(v.y, v.z), v.w));
+      hi = fmaxf(fmaxf(hi, v.x), fmaxf(fmaxf(v.y, v.z), v.w));
+    }
     if (st + 1 < kRowSteps) {
 #pragma unroll
       for (int q = 0; q < 4; ++q) { alo[q] = nlo[q]; ahi[q] = nhi[q]; }
     }
   }
+  // The range of the scores for the selection, which bins them: two passes over the list and a cluster barrier less there.
+#pragma unroll
+  for (int o = 1; o < 4; o <<= 1) { lo = min_or_nan(lo, __shfl_xor_sync(0xffffffffu, lo, o)); hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o)); }
+  if ((lane & 3) == 0 && n0 + (lane >> 2) < D)
+    reinterpret_cast<float2*>(ws + pl.off_ext)[((size_t)b * D + n0 + (lane >> 2)) * pl.ext_ld + blockIdx.x * 4 + w] = make_float2(lo, hi);
+  if (blockIdx.x == 0 && b == 0 && blockIdx.z == 0) asm volatile("griddepcontrol.wait;" ::: "memory");   // (this kernel's completion implies the state build's)
 }
 
 // Selection of one node from the score array by a cluster of eight CTAs: grid (8 D, B).  A CTA keeps its share of the list in
@@ -578,7 +590,6 @@ __global__ void __launch_bounds__(128) score_rows_kernel(const tsv_shape s, cons
 constexpr int kListThreads = 512, kListBins = 1024;
 struct ListSmem {
   int hist[2][kListBins];                                // [0] the intervals; both: the digits of the radix passes
-  float2 ext;
   int cnt[2];                                            // candidates; (entries certainly taken, entries equal to the threshold)
   int eqs;
   float cand_s[ssel::CAP];
@@ -627,40 +638,36 @@ __global__ void __launch_bounds__(kListThreads, 2) topk_list_kernel(const tsv_sh
   uint32_t* bits = reinterpret_cast<uint32_t*>(list + (((pl.score_ld + TSV_MAX_D + CS - 1) / CS + 63) & ~31));
   for (int i = t; i < (len + 31) / 32; i += NT) bits[i] = 0u;
   const float4* src = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(ws + pl.off_scores) + ((size_t)b * D + n) * pl.score_ld + c0);
+  float lo = INFINITY, hi = -INFINITY;                 // the range of the committed entries' scores
+  const float2* ext = reinterpret_cast<const float2*>(ws + pl.off_ext) + ((size_t)b * D + n) * pl.ext_ld;
+  for (int i = t; i < (n_csa + 255) / 256 * 4; i += NT) { const float2 x = __ldcg(ext + i); lo = min_or_nan(lo, x.x); hi = fmaxf(hi, x.y); }
   const int n4 = (min(c1, n_csa) - c0 + 3) >> 2;       // (negative: none)
   for (int i = t; i < n4; i += NT) reinterpret_cast<float4*>(list)[i] = __ldcg(src + i);
   if (c1 > n_csa) {
     ExtraScorer<bf16> ex;
     ex.fetch(s, nd, b, n);
-    ex.score(pe, s, sc, b, [&](int i, float v) { extra[i] = v; });
+    ex.score(pe, s, sc, b, [&](int i, float v) {
+      extra[i] = v;
+      if (v != v && n_csa + i >= c0 && n_csa + i < c1) atomicAdd(&sm.cnt[0], CAP + 1);      // (a NaN: the interval is found overfull, the radix passes follow)
+    });
     __syncthreads();
     for (int i = max(n_csa, c0) + t; i < c1; i += NT) list[i - c0] = extra[i - n_csa];
   }
   __syncthreads();
-  float lo = INFINITY, hi = -INFINITY;
-  for (int i = t; i < len; i += NT) { const float v = list[i]; lo = min_or_nan(lo, v); hi = fmaxf(hi, v); }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) { lo = min_or_nan(lo, __shfl_xor_sync(0xffffffffu, lo, o)); hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o)); }
   if (lane == 0) { sm.red[0][w] = lo; sm.red[1][w] = hi; }
   __syncthreads();
-  if (t == 0) {
-    for (int i = 0; i < NW; ++i) { lo = min_or_nan(lo, sm.red[0][i]); hi = fmaxf(hi, sm.red[1][i]); }
-    sm.ext = make_float2(lo, hi);
-  }
+  lo = sm.red[0][lane % NW]; hi = sm.red[1][lane % NW];
+#pragma unroll
+  for (int o = NW / 2; o > 0; o >>= 1) { lo = min_or_nan(lo, __shfl_xor_sync(0xffffffffu, lo, o)); hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o)); }
   auto peer = [&](const void* p, int r) { return map_to_rank((uint32_t)__cvta_generic_to_shared(p), r); };
   auto peer_i = [&](const int* p, int r) { int v; asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(peer(p, r))); return v; };
   auto peer_f = [&](const float* p, int r) { float v; asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(peer(p, r))); return v; };
   auto meet = [&]() { __syncthreads(); cluster_arrive(); cluster_wait(); };
-  meet();
-  {
-    const int r = lane & 7;
-    lo = peer_f(&sm.ext.x, r); hi = peer_f(&sm.ext.y, r);
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) { lo = min_or_nan(lo, __shfl_xor_sync(0xffffffffu, lo, o)); hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o)); }
-  }
   const float scale = hi > lo ? (float)NB / (hi - lo) : 0.f;
   const bool regular = scale > 0.f && scale < 1e30f;     // (else: all equal, not finite, a NaN among them, or too narrow)
-  auto bin_of = [&](float v) { return min(NB - 1, (int)((v - lo) * scale)); };
+  auto bin_of = [&](float v) { return min(NB - 1, max(0, (int)((v - lo) * scale))); };      // (in-tree entries may lie beyond the range)
   // the interval (of nb in h, over the whole cluster) of the rem-th largest: its number, and what of rem is left in it
   auto locate = [&](const int* h, int nb, int rem, int& bin, int& left) {
     int v[2] = {0, 0};
