@@ -392,9 +392,9 @@ __global__ void __launch_bounds__(NT) tc_plan_kernel(const tsv_shape s, const Tv
 // chunks have said that their rows are stored (it is looked for in the order in which the tiles are worked on), the rest when
 // that kernel has ended: at those 64 sequences a pass of eight layers takes 798 instead of 830 us.  Tiles cut to fill the device
 // all end with that kernel, and looking earlier loses 0.4 us a layer: there the merge waits for it at once.
-// ANY32: some tiles' partial outputs may be fp32 (else all are bf16, and the kernel keeps its registers low).
+// ANY32: some tiles' partial outputs may be fp32 (else all are bf16, and the kernel keeps its registers low).  ROWS: rows merged together.
 constexpr int kMergePolls = 256;       // times a warp looks for its tile's chunks (0.3 us each) before it waits for the whole attention kernel
-template <bool ANY32>
+template <bool ANY32, int ROWS>
 __global__ void __launch_bounds__(256) tc_combine_pair_kernel(const tsv_shape s, const TvaPlan pl, void* __restrict__ out_, const char* __restrict__ ws, const int rpw) {
   using namespace tc;
   constexpr uint32_t FULL = 0xffffffffu;
@@ -423,79 +423,99 @@ __global__ void __launch_bounds__(256) tc_combine_pair_kernel(const tsv_shape s,
     if (done < 8 * nch) asm volatile("griddepcontrol.wait;" ::: "memory");
   }
   const float2* pml = reinterpret_cast<const float2*>(ws + pl.off_tpml) + rix * pl.tc_chmax * BM;
-  auto merge = [&](auto vec) {                                   // vec: 16-byte pieces of a lane's 16 columns
-    constexpr int V = decltype(vec)::value;
+  // vec: 16-byte pieces of a lane's 16 columns; R: rows merged together (their requests are in flight together)
+  auto merge = [&](auto vec, auto rows) {
+    constexpr int V = decltype(vec)::value, R = decltype(rows)::value, U = R > 1 ? 2 : 4;      // U: chunks requested together
     // (a chunk's bf16 tile lies at the start of the chunk's slot of BM x DH floats)
     const uint4* po = reinterpret_cast<const uint4*>(ws + pl.off_tpo) + rix * pl.tc_chmax * BM * (DH / 4) + lane;
 #pragma unroll 1
-    for (int row = first; row < last; row += 8) {
-      const uint4* pr = po + (size_t)row * (DH / (V == 4 ? 4 : 8));
-      float2 x = lane < nch ? __ldcg(pml + (size_t)lane * BM + row) : make_float2(-INFINITY, 0.f);
-      uint4 v[4][V];
+    for (int row = first; row < last; row += 8 * R) {
+      float2 x[R];
+      uint4 v[U][R][V];
+      auto fetch_ml = [&](int c0) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) x[r] = c0 + lane < nch && row + 8 * r < last ? __ldcg(pml + (size_t)(c0 + lane) * BM + row + 8 * r) : make_float2(-INFINITY, 0.f);
+      };
       auto fetch = [&](int c0) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (c0 + u < nch) {
+        for (int u = 0; u < U; ++u)
 #pragma unroll
-            for (int q = 0; q < V; ++q) v[u][q] = __ldcg(pr + (size_t)(c0 + u) * BM * (DH / 4) + 32 * q);
-          }
+          for (int r = 0; r < R; ++r)
+            if (c0 + u < nch && row + 8 * r < last) {
+#pragma unroll
+              for (int q = 0; q < V; ++q) v[u][r][q] = __ldcg(po + (size_t)(row + 8 * r) * (DH / (V == 4 ? 4 : 8)) + (size_t)(c0 + u) * BM * (DH / 4) + 32 * q);
+            }
       };
+      fetch_ml(0);
       fetch(0);
-      float m = x.y > 0.f ? x.x : -INFINITY;
-#pragma unroll 1
-      for (int ch = lane + 32; ch < nch; ch += 32) { const float2 y = __ldcg(pml + (size_t)ch * BM + row); if (y.y > 0.f) m = fmaxf(m, y.x); }
+      float m[R], wt[R], l[R], acc[R][16];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(FULL, m, o));
-      float wt = x.y > 0.f ? x.y * exp2f(x.x - m) : 0.f;         // lane c: weight of chunk c (of the 32 chunks at hand)
-      float l = 0.f, acc[16];
-#pragma unroll
-      for (int k = 0; k < 16; ++k) acc[k] = 0.f;
+      for (int r = 0; r < R; ++r) {
+        m[r] = x[r].y > 0.f ? x[r].x : -INFINITY;
 #pragma unroll 1
-      for (int c0 = 0; c0 < nch; c0 += 4) {
+        for (int ch = lane + 32; ch < nch && row + 8 * r < last; ch += 32) { const float2 y = __ldcg(pml + (size_t)ch * BM + row + 8 * r); if (y.y > 0.f) m[r] = fmaxf(m[r], y.x); }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) m[r] = fmaxf(m[r], __shfl_xor_sync(FULL, m[r], o));
+        wt[r] = x[r].y > 0.f ? x[r].y * exp2f(x[r].x - m[r]) : 0.f;      // lane c: weight of chunk c (of the 32 chunks at hand)
+        l[r] = 0.f;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) acc[r][k] = 0.f;
+      }
+#pragma unroll 1
+      for (int c0 = 0; c0 < nch; c0 += U) {
         if (c0) {
           fetch(c0);
           if ((c0 & 31) == 0) {                                  // (lists of more than 32 chunks)
-            x = c0 + lane < nch ? __ldcg(pml + (size_t)(c0 + lane) * BM + row) : make_float2(-INFINITY, 0.f);
-            wt = x.y > 0.f ? x.y * exp2f(x.x - m) : 0.f;
+            fetch_ml(c0);
+#pragma unroll
+            for (int r = 0; r < R; ++r) wt[r] = x[r].y > 0.f ? x[r].y * exp2f(x[r].x - m[r]) : 0.f;
           }
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const float w = __shfl_sync(FULL, wt, (c0 + u) & 31);
-          if (c0 + u >= nch) continue;
-          l += w;
+        for (int u = 0; u < U; ++u) {
 #pragma unroll
-          for (int q = 0; q < V; ++q) {
-            const uint32_t wd[4] = {v[u][q].x, v[u][q].y, v[u][q].z, v[u][q].w};
+          for (int r = 0; r < R; ++r) {
+            const float w = __shfl_sync(FULL, wt[r], (c0 + u) & 31);
+            if (c0 + u >= nch) continue;
+            l[r] += w;
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              if (V == 4) acc[4 * q + k] = fmaf(__uint_as_float(wd[k]), w, acc[4 * q + k]);
-              else {
-                acc[8 * q + 2 * k] = fmaf(__uint_as_float(wd[k] << 16), w, acc[8 * q + 2 * k]);
-                acc[8 * q + 2 * k + 1] = fmaf(__uint_as_float(wd[k] & 0xFFFF0000u), w, acc[8 * q + 2 * k + 1]);
+            for (int q = 0; q < V; ++q) {
+              const uint32_t wd[4] = {v[u][r][q].x, v[u][r][q].y, v[u][r][q].z, v[u][r][q].w};
+#pragma unroll
+              for (int k = 0; k < 4; ++k) {
+                if (V == 4) acc[r][4 * q + k] = fmaf(__uint_as_float(wd[k]), w, acc[r][4 * q + k]);
+                else {
+                  acc[r][8 * q + 2 * k] = fmaf(__uint_as_float(wd[k] << 16), w, acc[r][8 * q + 2 * k]);
+                  acc[r][8 * q + 2 * k + 1] = fmaf(__uint_as_float(wd[k] & 0xFFFF0000u), w, acc[r][8 * q + 2 * k + 1]);
+                }
               }
             }
           }
         }
       }
-      const float inv = l > 0.f ? 1.f / l : 0.f;
-      uint32_t o[8];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const __nv_bfloat162 h2 = __floats2bfloat162_rn(acc[2 * k] * inv, acc[2 * k + 1] * inv);
-        o[k] = *reinterpret_cast<const uint32_t*>(&h2);
-      }
-      bf16* orow = reinterpret_cast<bf16*>(out_) + ((size_t)b * rows_seq + row0 + row) * DH;
-      if (V == 4) {
+      for (int r = 0; r < R; ++r) {
+        if (row + 8 * r >= last) break;
+        const float inv = l[r] > 0.f ? 1.f / l[r] : 0.f;
+        uint32_t o[8];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) reinterpret_cast<uint2*>(orow)[lane + 32 * q] = make_uint2(o[2 * q], o[2 * q + 1]);
-      } else {
+        for (int k = 0; k < 8; ++k) {
+          const __nv_bfloat162 h2 = __floats2bfloat162_rn(acc[r][2 * k] * inv, acc[r][2 * k + 1] * inv);
+          o[k] = *reinterpret_cast<const uint32_t*>(&h2);
+        }
+        bf16* orow = reinterpret_cast<bf16*>(out_) + ((size_t)b * rows_seq + row0 + row + 8 * r) * DH;
+        if (V == 4) {
 #pragma unroll
-        for (int q = 0; q < 2; ++q) reinterpret_cast<uint4*>(orow)[lane + 32 * q] = make_uint4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
+          for (int q = 0; q < 4; ++q) reinterpret_cast<uint2*>(orow)[lane + 32 * q] = make_uint2(o[2 * q], o[2 * q + 1]);
+        } else {
+#pragma unroll
+          for (int q = 0; q < 2; ++q) reinterpret_cast<uint4*>(orow)[lane + 32 * q] = make_uint4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
+        }
       }
     }
   };
-  if (ANY32 && f32) merge(std::integral_constant<int, 4>()); else merge(std::integral_constant<int, 2>());
+  if (ANY32 && f32) merge(std::integral_constant<int, 4>(), std::integral_constant<int, 1>());
+  else merge(std::integral_constant<int, 2>(), std::integral_constant<int, ROWS>());
 }
 
 bool tva_tc_eligible(const tsv_shape& s) {
@@ -548,8 +568,9 @@ int prepare_tva_tc(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, con
   TSV_PREP((tc_plan_kernel<true, 1024>));
   TSV_PREP((tc_plan_kernel<true, 256>));
   TSV_PREP((tc_plan_kernel<false, 256>));
-  TSV_PREP(tc_combine_pair_kernel<true>);
-  TSV_PREP(tc_combine_pair_kernel<false>);
+  TSV_PREP((tc_combine_pair_kernel<true, 1>));
+  TSV_PREP((tc_combine_pair_kernel<false, 1>));
+  TSV_PREP((tc_combine_pair_kernel<false, 2>));
   return prepare_tva_tc_pair(s, p, c, nd, out, ws, prep);
 }
 
@@ -580,16 +601,20 @@ int launch_tva_tc(const tsv_shape& s, const TvaPlan& p_in, const TvaTcPrep& prep
   if (r != TSV_OK) return r;
   if (general && p.tc_chmax > 1) {
     cudaLaunchConfig_t cfg = {};
-    // rows a warp takes: one while that leaves SMs idle otherwise, up to four
+    // Rows a warp takes: one while that leaves SMs idle otherwise; two, merged together, up to 64 tiles (what is left to merge when the
+    // attention ends is one row's latency then: 32 paged sequences 257 -> 242 us a pass, four rows one after the other before); four
+    // beyond (there the merge runs under the attention's tail, and the registers of two rows at once take a third of the warps:
+    // 64 grown sequences 703 us, with two rows 714-723).
     const int64_t groups = (int64_t)2 * p.tc_nt * s.B * (tc::BM / 8);
-    const int rpw = groups <= 4 * 148 ? 1 : groups <= 8 * 148 ? 2 : 4;
+    const int rpw = groups <= 4 * 148 ? 1 : groups <= 16 * 148 ? 2 : 4;
     cfg.gridDim = dim3(2 * p.tc_nt * s.B * (tc::BM / 8 / rpw)); cfg.blockDim = dim3(256, 1, 1); cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
-    if (p.tc_split > 1 || p.tc_f32) cudaLaunchKernelEx(&cfg, tc_combine_pair_kernel<true>, s, p, out, (const char*)ws, rpw);
-    else cudaLaunchKernelEx(&cfg, tc_combine_pair_kernel<false>, s, p, out, (const char*)ws, rpw);
+    if (p.tc_split > 1 || p.tc_f32) cudaLaunchKernelEx(&cfg, tc_combine_pair_kernel<true, 1>, s, p, out, (const char*)ws, rpw);
+    else if (rpw == 2) cudaLaunchKernelEx(&cfg, tc_combine_pair_kernel<false, 2>, s, p, out, (const char*)ws, rpw);
+    else cudaLaunchKernelEx(&cfg, tc_combine_pair_kernel<false, 1>, s, p, out, (const char*)ws, rpw);
     count_launch();
   }
   return cudaGetLastError() == cudaSuccess ? TSV_OK : TSV_ERR_CUDA;
