@@ -106,7 +106,9 @@ bool make_tva_plan(const tsv_shape& s, TvaPlan& p) {
     int64_t ch = kPairsFor / (int64_t)tiles;
     if (ch > (p.tc_maxk + 127) / 128) ch = (p.tc_maxk + 127) / 128;
     while (ch > p.tc_chmax && up256((size_t)ch * slot) + up256((size_t)ch * slot_ml) > pool) --ch;
-    if (ch >= 4) p.tc_split = (int32_t)ch; else ch = 1;
+    // (the pairs a tile may have, and the chunks it may be cut into: the workspace has slots for those)
+    p.tc_split = (int32_t)(kPairsFor / (int64_t)tiles > 1 ? kPairsFor / (int64_t)tiles : 1);
+    if (ch < 4) ch = 1;
     if (ch > p.tc_chmax) p.tc_chmax = (int32_t)ch;
     p.off_tpo = off_pool;
     p.off_tpml = off_pool + up256((size_t)p.tc_chmax * slot);

@@ -11,7 +11,7 @@ constexpr int DH = 512;             // head dim handled by this path
 constexpr int BM = 128;             // rows per CTA
 constexpr int PR = 256;             // rows per plan tile: two row tiles (one CTA pair) share one key list
 constexpr int NC = 512;             // keys per chunk of a list that is cut into many
-constexpr int NCMIN = 128;          // keys of the shortest chunk worth an SM pair of its own
+constexpr int NCMIN = 256;          // keys of the shortest chunk worth an SM pair of its own
 constexpr uint32_t WAIT_LIMIT = 1u << 14;   // polls before a wait gives up (then no later wait of the thread is attempted)
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -108,16 +108,19 @@ constexpr int NCX = 768;             // max keys per chunk of the TMA kernel: P 
 // general = true: a list that does not fit one chunk is cut into chunks of at most NC keys, whose quarters of O go through two
 // buffers instead of one and which fill the SM pairs better (two chunks of up to NCX instead of three of NC cost 12 % of the
 // attention kernel on 32 paged sequences of 256-4096 tokens, and gained nothing on 64 flat ones).
-// split: chunks a tile may be cut into so that few tiles still use all pairs (1 where there are tiles enough).
+// split: items a tile may be cut into so that few tiles still use all pairs (1 where there are tiles enough).  general: into chunks of
+// at least NCMIN keys, a tile of up to NC keys stays whole.  Then, in both, by columns of the output: 1 << lds items of a chunk
+// compute S and the softmax alike and each its own columns of O, which nobody has to merge.
 // f32: the partial outputs of the tile are fp32 (a tile that is cut for the sake of parallelism alone is not rounded before
 // the merge); f32_all: all multi-chunk tiles are.
-__device__ __host__ __forceinline__ void chunking_x(int nk, bool general, int split, bool f32_all, int& nch, int& CL, bool& f32) {
+__device__ __host__ __forceinline__ void chunking_x(int nk, bool general, int split, int chmax, bool f32_all, int& nch, int& CL, bool& f32, int& lds) {
   nch = (nk + NCX - 1) / NCX;
   if (general && nch > 1) nch = (nk + NC - 1) / NC;
   f32 = f32_all || nch <= 1;
-  if (split > 1) {
+  if (general && split > 1 && nk > NC) {
     int w = (nk + NCMIN - 1) / NCMIN;
     if (w > split) w = split;
+    if (w > chmax) w = chmax;                            // (the workspace has slots for no more)
     if (w > nch) nch = w;
   }
   if (nch < 1) nch = 1;
@@ -125,22 +128,25 @@ __device__ __host__ __forceinline__ void chunking_x(int nk, bool general, int sp
   if (CL < 128) CL = 128;
   nch = (nk + CL - 1) / CL;
   if (nch < 1) nch = 1;
+  lds = 4 * nch <= split ? 2 : 2 * nch <= split ? 1 : 0;
 }
 // The record of a tile, which the tile plan leaves and the kernels after it read: {sequence, what, keys, 0}, what = mode (2 bits: 1
-// boxes, 2 gathered) | fp32 partial outputs << 2 | chunk length / 128 << 4 | tile of the sequence << 7 | chunks << 12.  (The chunking is
-// three divisions: by every role of the attention kernel on its own they were 10 KB of its code.)
+// boxes, 2 gathered) | fp32 partial outputs << 2 | chunk length / 128 << 4 | tile of the sequence << 7 | chunks << 12 | log2 of the
+// items of a chunk << 28.  (The chunking is three divisions: by every role of the attention kernel on its own they were 10 KB of its code.)
 __device__ __forceinline__ int4 tile_record(const TvaPlan& pl, int b, int tile, int mode, int nk) {
-  int nch, CL;
+  int nch, CL, lds;
   bool f32;
-  chunking_x(nk, pl.tc_general != 0, pl.tc_split, pl.tc_f32, nch, CL, f32);
-  return make_int4(b, mode | (f32 ? 4 : 0) | (CL / 128) << 4 | tile << 7 | nch << 12, nk, 0);
+  chunking_x(nk, pl.tc_general != 0, pl.tc_split, pl.tc_chmax, pl.tc_f32, nch, CL, f32, lds);
+  return make_int4(b, mode | (f32 ? 4 : 0) | (CL / 128) << 4 | tile << 7 | nch << 12 | lds << 28, nk, 0);
 }
 static_assert(NCX / 128 < 8 && TSV_MAX_D * 128 / PR <= 32, "fields of a tile's record");
 __device__ __forceinline__ bool rec_gather(const int4& r) { return (r.y & 3) == 2; }
 __device__ __forceinline__ bool rec_f32(const int4& r) { return (r.y & 4) != 0; }
 __device__ __forceinline__ int rec_chunk_keys(const int4& r) { return ((r.y >> 4) & 7) * 128; }
 __device__ __forceinline__ int rec_tile(const int4& r) { return (r.y >> 7) & 31; }
-__device__ __forceinline__ int rec_chunks(const int4& r) { return (int)((uint32_t)r.y >> 12); }
+__device__ __forceinline__ int rec_chunks(const int4& r) { return (r.y >> 12) & 0xFFFF; }
+__device__ __forceinline__ int rec_lds(const int4& r) { return r.y >> 28; }
+__device__ __forceinline__ int rec_items(const int4& r) { return rec_chunks(r) << rec_lds(r); }
 
 }  // namespace tc
 

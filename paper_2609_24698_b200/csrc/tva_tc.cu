@@ -580,8 +580,9 @@ int launch_tva_tc(const tsv_shape& s, const TvaPlan& p_in, const TvaTcPrep& prep
   const bool gathered = gathered_tiles_possible(s, p, c);
   // general: some tile may have more than two chunks of the longest kind, or be gathered; then every multi-chunk tile
   // leaves bf16 partial outputs for the merge kernel
-  const bool many = (p.tc_maxk + tc::NCX - 1) / tc::NCX > 2 || gathered, general = many || p.tc_split > 1;
-  p.tc_f32 = !many;                                    // (no more than two long chunks a tile: merged without rounding in either instantiation)
+  const bool general = (p.tc_maxk + tc::NCX - 1) / tc::NCX > 2 || gathered;
+  p.tc_f32 = !general;                                 // (no more than two long chunks a tile: merged without rounding in the attention kernel)
+  if (general && p.tc_split < 4) p.tc_split = 1;       // (tiles of several chunks: two or three pairs a tile are soon in use)
   p.tc_general = general;
   const dim3 pgrid(p.tc_nt + 1, s.B);                                                                              // x: tiles + the packing CTA
   if (with_plan) {

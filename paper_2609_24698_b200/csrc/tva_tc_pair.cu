@@ -58,7 +58,7 @@ struct Ctl {                               // control block at the start of dyna
   uint64_t fullK[NKS], emptyK[NKS];        // ring of the K stages
   uint64_t fullV[NSV], emptyV[NSV];        // ring of the V stages (starts when the S products are complete)
   uint64_t acc_ev[7];                      // MMA -> other warps, one barrier per event, at most once per item:
-                                           //   [pc] S of piece pc is complete   [3 + p] part p of O is complete
+                                           //   [pc] S of piece pc is complete   [3 + p] the item's part p of O is complete
   uint64_t cmp_ev[7];                      // compute warps -> MMA, likewise:
                                            //   [pc] P of piece pc is in TMEM   [3 + p] part p of O has been read out
   uint64_t stage_free;                     // the item's output tiles have left the staging slots (this CTA's)
@@ -164,21 +164,24 @@ constexpr int NQ = 4, OW = tc::DH / NQ;      // the PV product is computed in NQ
 struct Item {
   int tix, b, tile, nk, chunk, nch, CL, cbeg, cend;
   int npc;                 // S pieces
+  int lds, p0, np;         // log2 of the items of a chunk; this one's parts of O: [p0, p0 + np)
   bool dbl;                // two O buffers: a part is computed while the one before is read out
   bool f32;                // partial outputs are fp32
   bool gather;             // the key list is a list of row codes (array << 30 | row), not of boxes
   __device__ __forceinline__ Item(int4 r, const TvaPlan& pl, bool general) {      // a tile's record, the chunk in its last word
     b = r.x; tile = rec_tile(r); tix = b * pl.tc_nt + tile;
     gather = general && rec_gather(r); f32 = general && rec_f32(r);
-    nk = r.z; chunk = r.w; nch = rec_chunks(r);
+    lds = rec_lds(r);
+    nk = r.z; chunk = r.w >> lds; nch = rec_chunks(r);
+    np = NQ >> lds; p0 = (r.w & ((1 << lds) - 1)) * np;
     const int stride = rec_chunk_keys(r);
     cbeg = chunk * stride; cend = min(nk, cbeg + stride);
     CL = max(128, (cend - cbeg + 127) & ~127);           // (the tile's last chunk is as long as what is left)
     npc = (CL + 255) / 256;
     dbl = CL <= 512;
   }
-  __device__ __forceinline__ uint32_t acc_used() const { return ((1u << npc) - 1u) | (((1u << NQ) - 1u) << 3); }
-  __device__ __forceinline__ uint32_t cmp_used() const { return (1u << (npc - 1)) | (npc == 3 ? 2u : 0u) | (((1u << NQ) - 1u) << 3); }
+  __device__ __forceinline__ uint32_t acc_used() const { return ((1u << npc) - 1u) | (((1u << np) - 1u) << 3); }
+  __device__ __forceinline__ uint32_t cmp_used() const { return (1u << (npc - 1)) | (npc == 3 ? 2u : 0u) | (((1u << np) - 1u) << 3); }
 };
 }  // namespace pair
 
@@ -252,17 +255,18 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
   // The merge kernel, where one follows, may take its places: it waits for this kernel before it does anything.  (Nothing else may
   // start before this kernel has ended: the next call's tile plan would overwrite what is read here.)
   if (GENERAL && pl.tc_chmax > 1) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int4 rec0 = (int)(blockIdx.x >> 1) < s.B * pl.tc_nt ? __ldcg(reinterpret_cast<const int4*>(ws + pl.off_order) + (blockIdx.x >> 1)) : make_int4(-1, 0, 0, 0);
+  // Item 0 of pair p is item p / ntile of tile p % ntile, which every warp looks up itself; the others are handed out (warp 2).
+  const int ntile = s.B * pl.tc_nt, P = gridDim.x >> 1, me = blockIdx.x >> 1, item0 = (uint32_t)me / (uint32_t)ntile;
+  const int4 rec0 = __ldcg(reinterpret_cast<const int4*>(ws + pl.off_order) + (me - item0 * ntile));
   cluster_wait();                                                // barriers of both CTAs exist before anyone signals them
   fence_after();
   const uint32_t tm = sm.tmem_base;
   const int rows_seq = s.D * s.H;
-  // Item n of this pair (sequence -1: no more).  Item 0 is the first chunk of the tile of this pair's rank, which every warp
-  // looks up itself; the others are handed out (warp 2).  The wait is made whatever failed before (a failure skips later
+  // Item n of this pair (sequence -1: no more).  The wait is made whatever failed before (a failure skips later
   // waits, never a step of the protocol, so that no warp is left alone at a barrier), and is longer than any other.
-  const int own = rec0.z > 0 ? 1 : 0;
+  const int own = rec0.z > 0 && item0 < rec_items(rec0) ? 1 : 0;
   auto next_item = [&](int n) {
-    if (n < own) return make_int4(rec0.x, rec0.y, rec0.z, 0);
+    if (n < own) return make_int4(rec0.x, rec0.y, rec0.z, item0);
     bool ok = false;
     for (int i = 0; i < 8 && !ok; ++i) ok = mbar_wait(&sm.item_ev, (uint32_t)(n - own) & 1u);
     int4 r = sm.item[(n - own) & 1];
@@ -306,7 +310,7 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
       const uint32_t box = load_box(w);
       const int CL = w.CL, row0 = w.tile * PR + (int)rank * BM;
       const int nvb = CL / 128;                                    // V stages per part
-      const int NKST = 8 * w.npc, NVST = NQ * nvb;
+      const int NKST = 8 * w.npc, NVST = w.np * nvb;
       // This producer's places of the item are u and u + 6: slots pw + 6 h0 and pw + 6 (1 - h0).
       const int u = (pw + 2 * NPROD - g0) % NPROD, h0 = (g0 + u) % NSV >= NPROD ? 1 : 0;
       const int kpos = (u & 1) ? u >> 1 : 3 + (u >> 1);            // its ring position of the K stages
@@ -387,7 +391,7 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
       if (lane == 0 && !fail && !mbar_wait(&sm.acc_ev[w.npc - 1], (accb >> (w.npc - 1)) & 1u)) fail = 1;
       __syncwarp();
       {
-        int part = 0, kb = u, h = h0;
+        int part = w.p0, kb = u, h = h0;
 #pragma unroll 1
         for (int gv = u; gv < NVST; gv += NPROD) {
           while (kb >= nvb) { kb -= nvb; ++part; }
@@ -439,7 +443,7 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
       // the columns [256, 512) of the item before have been read out
       auto need_pend = [&]() {
 #pragma unroll
-        for (int e = 3 + NQ - 2; e < 3 + NQ; ++e) if (((pend >> e) & 1u) && !fail && !mbar_wait(&sm.cmp_ev[e], (pend_par >> e) & 1u)) fail = 1;
+        for (int e = 3; e < 3 + NQ; ++e) if (((pend >> e) & 1u) && !fail && !mbar_wait(&sm.cmp_ev[e], (pend_par >> e) & 1u)) fail = 1;
         pend = 0;
       };
 #pragma unroll 1
@@ -482,7 +486,7 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
         need_pend();
         sl = g0;                                           // slot of the next V stage
 #pragma unroll 1
-        for (int part = 0; part < NQ; ++part) {
+        for (int part = 0; part < w.np; ++part) {
           const uint32_t ocol = tm + (w.dbl ? 256 + (part & 1) * OW : 384);
           if (part == 0) need_ev(npc - 1);                 // all of P is in TMEM
           else if (!w.dbl || part >= 2) need_ev(3 + part - (w.dbl ? 2 : 1));      // the part before in these columns has been read out
@@ -501,8 +505,8 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
           if (one) mma2_commit(&sm.acc_ev[3 + part]);
         }
         // P (overwritten by the next item's first piece) is free when the last part is complete
-        if (!fail && !mbar_wait(&sm.acc_ev[3 + NQ - 1], (accb >> (3 + NQ - 1)) & 1u)) fail = 1;
-        pend = (w.dbl ? 3u : 2u) << (3 + NQ - 2); pend_par = cmpb;
+        if (!fail && !mbar_wait(&sm.acc_ev[2 + w.np], (accb >> (2 + w.np)) & 1u)) fail = 1;
+        pend = ((1u << w.np) - (1u << max(0, w.np - (w.dbl ? 2 : 1)))) << 3; pend_par = cmpb;      // the last part or two
         accb ^= w.acc_used(); cmpb ^= w.cmp_used();
         g0 = sl;
       }
@@ -510,19 +514,19 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
     __syncwarp();
   } else {
     // ------------------------------------------------------------------ hands out the items
-    // The plan kernel left a record {tile, mode, keys} per tile, most keys first.  The items are the tiles' chunks in that
-    // order; pair p starts with the first chunk of tile p, all others are taken from a counter (items differ in length and in
+    // The plan kernel left a record per tile, longest work items first.  The items are the tiles' chunks (or shares of the columns of
+    // chunks) in that order; pair p starts with the one every warp knows, all others are taken from a counter (items differ in length and in
     // where their rows come from, so a fixed deal leaves pairs idle: 177 k cycles for the slowest of 74 pairs against a mean
-    // of 125 k on 64 sequences of 1-4 k tokens).  The leader's warp takes the next item when all compute warps have stored
-    // the current one's P: every warp of the pair has seen the current one then, and the producers are about to need the next.
-    const int ntile = s.B * pl.tc_nt, P = gridDim.x >> 1, me = blockIdx.x >> 1;
+    // of 125 k on 64 sequences of 1-4 k tokens).  The leader's warp takes the next item when the current one's S is complete and
+    // passes it on when all compute warps have stored its P: every warp of the pair has seen the current one then, and the
+    // producers are about to need the next.
     const int4* order = reinterpret_cast<const int4*>(ws + pl.off_order);
     if (rank == 0) {
       int32_t* counter = reinterpret_cast<int32_t*>(ws + pl.off_sched);
       uint32_t cmpb = 0, accb = 0;
       int base = 0, w0 = -32;                           // window: tiles w0 .. w0 + 31, a lane each; base: items before it
       int4 rec = make_int4(-1, 0, 0, 0);
-      int n = 0, incl = 0, tot = 0;
+      int n = 0, incl = 0, tot = 0, given = 0;          // of the lane's tile: items handed out here, those of the lanes up to it, all lanes'; items given
       auto take = [&]() {                               // the next item of the device
         int q = 0x7fffffff;
         if (lane == 0 && !fail) q = atomicAdd(counter, 1);
@@ -532,7 +536,7 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
           n = 0;
           if (w0 + lane < ntile) {
             rec = order[w0 + lane];
-            if (rec.z > 0) { n = rec_chunks(rec); if (w0 + lane < P) --n; }     // (the first chunks of the first P tiles are given)
+            if (rec.z > 0) { n = rec_items(rec); given = min(n, (P - (w0 + lane) + ntile - 1) / ntile); n -= given; }
           }
           incl = n;
 #pragma unroll
@@ -544,11 +548,11 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
           const uint32_t has = __ballot_sync(0xffffffffu, q - base < incl);
           const int src = __ffs(has) - 1;
           r.x = __shfl_sync(0xffffffffu, rec.x, src); r.y = __shfl_sync(0xffffffffu, rec.y, src); r.z = __shfl_sync(0xffffffffu, rec.z, src);
-          r.w = q - base - (__shfl_sync(0xffffffffu, incl, src) - __shfl_sync(0xffffffffu, n, src)) + (w0 + src < P ? 1 : 0);
+          r.w = q - base - __shfl_sync(0xffffffffu, incl - n - given, src);
         }
         return r;
       };
-      int4 r = own ? make_int4(rec0.x, rec0.y, rec0.z, 0) : take();
+      int4 r = own ? make_int4(rec0.x, rec0.y, rec0.z, item0) : take();
 #pragma unroll 1
       for (int it = 0;; ++it) {
         if (it >= own) {
@@ -787,11 +791,11 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
     const uint32_t stage = ring + (uint32_t)NSV * SLOTP + (uint32_t)(warp - 4) * 4096;   // this warp's tile of 32 rows x 64 columns (bf16)
     bool stored = false;
 #pragma unroll 1
-    for (int part = 0; part < NQ; ++part) {
+    for (int part = 0; part < w.np; ++part) {
       if (!fail && !mbar_wait(&sm.acc_ev[3 + part], (accb >> (3 + part)) & 1u)) fail = 1;
       fence_after();
       const uint32_t ocol = tlane + (w.dbl ? 256 + (part & 1) * OW : 384) + hh * cw;
-      const int col = part * OW + hh * cw;
+      const int col = (w.p0 + part) * OW + hh * cw;
       const bool many = GENERAL && nch > 1;
       auto read_out = [&]() {                        // in registers: the columns may be overwritten
         fence_before();
@@ -875,7 +879,7 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
             *reinterpret_cast<float4*>(po + v * 4) = make_float4(__uint_as_float(r[4 * v]), __uint_as_float(r[4 * v + 1]), __uint_as_float(r[4 * v + 2]), __uint_as_float(r[4 * v + 3]));
         }
       }
-      if (nch > 1 && part == 0 && hh == 0)
+      if (nch > 1 && w.p0 + part == 0 && hh == 0)
         reinterpret_cast<float2*>(ws + pl.off_tpml)[(rix * pl.tc_chmax + chunk) * BM + row] = make_float2(m_run, l_row);
     }
     accb ^= w.acc_used();
@@ -893,7 +897,7 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
       if (warp == 4 && lane == 0) {
         int32_t* cnt = reinterpret_cast<int32_t*>(ws + pl.off_tcnt) + rix;
         const int done = atomicAdd(cnt, 1);
-        sm.merge_here = done == nch - 1;
+        sm.merge_here = done == (nch << w.lds) - 1;
       }
       compute_sync();
       if (sm.merge_here) {
@@ -995,7 +999,7 @@ int prepare_tva_tc_pair(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c
 int launch_tva_tc_pair(const tsv_shape& s, const TvaPlan& p, const TvaTcPrep& prep, bool general, const void* q, void* out, char* ws, int32_t* status, cudaStream_t st) {
   const pair::MapSet& ms = *reinterpret_cast<const pair::MapSet*>(prep.maps);
   cudaLaunchConfig_t cfg = {};
-  const int64_t most = (int64_t)p.tc_nt * s.B * p.tc_chmax;                 // items, if every tile had the most chunks
+  const int64_t most = (int64_t)p.tc_nt * s.B * (p.tc_split > 1 ? (p.tc_chmax > p.tc_split ? p.tc_chmax : p.tc_split) : p.tc_chmax);      // items, if every tile had the most
   cfg.blockDim = dim3(pair::TTHREADS, 1, 1);
   cfg.dynamicSmemBytes = pair::SMEM_X;
   cfg.stream = st;
