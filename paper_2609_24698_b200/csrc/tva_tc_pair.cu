@@ -757,22 +757,24 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
       if (npc == 3 && pc == 1) p_stored(1);
     }
     signal_stored();
-    // The row sums meet (in the output staging area, idle until O is read out); where a warp moved its reference, the two
-    // settle on the larger one first.
+    // The row sums meet (in the words in which the maxima did: the two warps have read those when they are past the barrier below, and
+    // write them next two items on); where a warp moved its reference, the two settle on the larger one first, which the
+    // output staging area carries: no part of O can be complete before both have announced P, which they do after reading it.
     float l_row = (lp[0] + lp[1]) + (lp[2] + lp[3]);
     {
-      const uint32_t mine = ring + (uint32_t)NSV * SLOTP + (uint32_t)(warp - 4) * 4096, other = ring + (uint32_t)NSV * SLOTP + (uint32_t)((warp - 4) ^ 4) * 4096;
-      auto put = [&](int i, float v) { asm volatile("st.shared.b32 [%0], %1;" ::"r"(mine + (uint32_t)(i * 128 + lane * 4)), "r"(__float_as_uint(v)) : "memory"); };
-      auto get = [&](int i) { uint32_t v; asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(other + (uint32_t)(i * 128 + lane * 4)) : "memory"); return __uint_as_float(v); };
+      const uint32_t mine = ring + (uint32_t)NSV * SLOTP + (uint32_t)(warp - 4) * 4096 + lane * 4, other = ring + (uint32_t)NSV * SLOTP + (uint32_t)((warp - 4) ^ 4) * 4096 + lane * 4;
       // (no reference moved, as nearly always: P is announced before the sums are exchanged)
       uint32_t any_moved;
       asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\tbarrier.cta.red.or.pred q, %2, 64, p;\n\tselp.b32 %0, 1, 0, q;\n\t}" : "=r"(any_moved) : "r"(moved), "r"(2 + q4) : "memory");
       if (!any_moved) p_stored(npc - 1);
-      put(0, l_row); put(1, m_run);
+      else asm volatile("st.shared.b32 [%0], %1;" ::"r"(mine), "r"(__float_as_uint(m_run)) : "memory");
+      xch[hh * BM + row] = __float_as_uint(l_row);
       pair_sync();
-      float l_other = get(0);
+      float l_other = __uint_as_float(xch[(hh ^ 1) * BM + row]);
       if (any_moved) {                               // (alike in both warps)
-        const float m_other = get(1), to = fmaxf(m_run, m_other);
+        uint32_t m_bits;
+        asm volatile("ld.shared.b32 %0, [%1];" : "=r"(m_bits) : "r"(other) : "memory");
+        const float m_other = __uint_as_float(m_bits), to = fmaxf(m_run, m_other);
         if (to != -INFINITY) {
           const float f = ex2(m_run - to), fo = ex2(m_other - to);
           const int last = npc - 1;
