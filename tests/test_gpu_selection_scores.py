@@ -83,6 +83,23 @@ def test_nan_scores_select_exactly_topk(form, where, spare):
 
 
 @pytest.mark.parametrize("form", FORMS)
+@pytest.mark.parametrize("sign", [1, -1])
+def test_closed_entries_beyond_the_range_of_the_committed(form, sign):
+    """Entries closed inside the tree score far above or far below every committed entry, whose range the histogram may be laid over; at
+    the threshold committed entries tie."""
+    dtype, D, n, k = form[:4]
+    di = form[4] if len(form) > 4 else 128 if dtype == "bf16" else 64
+    rng = np.random.default_rng(n + 2)
+    ik, tree_ik = np.zeros((n, di), np.float32), np.zeros(di, np.float32)
+    ik[:, 0], tree_ik[1] = rng.integers(1, 200, n), 4096
+    iq = np.zeros((D, 2, di), np.float32)
+    iq[:, 0, 0], iq[:, 1, 1] = 1, 1
+    iw = np.zeros((D, 2), np.float32)
+    iw[:, 0], iw[:, 1] = 1, sign
+    _check(_select(form, 2, ik, tree_ik, iq, iw), form, ik[:, 0].astype(np.float64), 4096.0 * sign)
+
+
+@pytest.mark.parametrize("form", FORMS)
 def test_zeros_of_either_sign_tie(form):
     """All heads of negative weight: the best score is a zero, negative where a product of the two leaves it, positive for an entry
     closed inside the tree.  They tie, and the lower indices win: the committed ones."""
