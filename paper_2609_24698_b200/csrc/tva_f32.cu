@@ -1,16 +1,17 @@
 // tree_verify_attn for fp32 storage with 128-wide rows: one cluster of CTAs per (sequence, node, group of 16 heads).
 //
-// The node's key list (selected CSA entries | committed HCA entries | in-tree HCA entries of the path | window | ancestors-or-self)
-// is split over the CTAs of the cluster; each works through its share in tiles of 64 rows (16-byte asynchronous copies, the next
-// tile's under the arithmetic of this one), and the CTAs merge their (max, sum, O) through distributed shared memory.
+// The node's key list, first the keys that nothing before this kernel decides (committed HCA entries | window | ancestors-or-self),
+// then the others (selected CSA entries | in-tree HCA entries of the path), is split over the CTAs of the cluster, either part evenly;
+// each works through its shares in tiles of 64 rows (16-byte asynchronous copies, the next tile's under the arithmetic of this
+// one), and the CTAs merge their (max, sum, O) through distributed shared memory.
 //
 // Exact fp32 FMAs, so the bound is the shared-memory port or the FMA pipe, whichever the tiling feeds worse (the kernel for all other
 // shapes reads three operands from shared memory per eight FMAs):
 //   S = Q K^T: lane = (4 heads, an eighth of the row); its queries stay in registers for the whole list, a key's row is one
 //              128-byte read for the four lane groups of a warp: 16 reads per 256 FMAs; the eighths meet by 14 shuffles.
 //   O = P K:   warp = (8 heads, a quarter of the tile's keys), lane = 4 columns: three reads per 32 FMAs.
-// All facts of the tree come from the caller's inputs and are worked out, and the queries fetched, before the kernel waits
-// for the selection (it is a programmatic dependent of it).
+// The kernel is a programmatic dependent of the selection and waits for it between the two parts: of 16 sequences of 256-4096 tokens
+// two thirds of the keys are done under the selection (38.5 us a pass before, 35.0 now).
 #include "kernels.h"
 
 namespace tsv {
@@ -44,9 +45,9 @@ __device__ __forceinline__ void cluster_sync() {
 }  // namespace f32a
 
 __global__ void __launch_bounds__(f32a::NT, 2) attn_f32_kernel(const tsv_shape s, const TvaPlan pl, const tsv_cache c, const tsv_nodes nd,
-                                                               const tsv_scratch sc, float* __restrict__ out, char* __restrict__ ws, const int nbuf /* 1: a share is one tile at most */) {
+                                                               const tsv_scratch sc, float* __restrict__ out, char* __restrict__ ws) {
   using namespace f32a;
-  extern __shared__ __align__(16) unsigned char dsm[];               // [nbuf][KT][DH] rows; at the end [4][HG][DH] parts of O
+  extern __shared__ __align__(16) unsigned char dsm[];               // [2][KT][DH] rows; at the end [4][HG][DH] parts of O
   __shared__ TreeMeta tm;
   __shared__ TreeStage tstage;
   __shared__ __align__(16) float P[KT * PP];
@@ -82,125 +83,141 @@ __global__ void __launch_bounds__(f32a::NT, 2) attn_f32_kernel(const tsv_shape s
     if (t == 0) { cnt[0] = __popc(cm); cnt[1] = __popc(hm); cnt[2] = __popc(self); }
   }
   __syncthreads();
-  asm volatile("griddepcontrol.wait;" ::: "memory");                 // the selection, and through it the state build
   if (!live) {                                                        // flagged sequence / padding node: zeros (the whole cluster alike)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (rank == 0)
       for (int i = t; i < nh * DH / 4; i += NT) reinterpret_cast<float4*>(out + row0 * DH)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     return;
   }
-  const int32_t* sel = reinterpret_cast<const int32_t*>(ws + pl.off_sel) + ((size_t)b * D + n) * s.topk;
-  const int n_sel = __ldcg(reinterpret_cast<const int32_t*>(ws + pl.off_selcnt) + (size_t)b * D + n);
+  // The keys in two parts, of each an equal share per CTA: those that neither the selection nor the state build decides
+  // (committed HCA | window | ancestors-or-self), then those that they do (selected CSA | in-tree HCA).
   const int n_hca = tm.n_hca, n_newh = cnt[1], pos = tm.L + tm.depth[n], win_lo = max(0, pos - s.window + 1), n_win = max(0, tm.L - win_lo);
-  const int N = n_sel + n_hca + n_newh + n_win + cnt[2];
-  const int per = (N + cs - 1) / cs, k0 = min(N, rank * per), k1 = min(N, k0 + per);
-  auto key_row = [&](int j) -> const float* {
-    if (j < n_sel) {
-      const int idx = __ldcg(sel + j);
-      if (idx < tm.n_csa) return reinterpret_cast<const float*>(c.csa_kv) + (size_t)csa_rows_of(c, s, b)(idx) * DH;
-      int a = newc[0];
-      for (int i = 0; i < cnt[0]; ++i) if (newc_blk[i] == idx) a = newc[i];
-      return reinterpret_cast<const float*>(sc.new_csa_kv) + ((size_t)b * D + a) * DH;
-    }
-    j -= n_sel;
+  const int32_t* sel = reinterpret_cast<const int32_t*>(ws + pl.off_sel) + ((size_t)b * D + n) * s.topk;
+  int n_sel = 0;
+  int k0 = 0, k1 = 0;                                                 // this CTA's share of the part at hand
+  auto known_row = [&](int j) -> const float* {
     if (j < n_hca) return reinterpret_cast<const float*>(c.hca_kv) + (size_t)hca_rows_of(c, s, b)(j) * DH;
     j -= n_hca;
-    if (j < n_newh) return reinterpret_cast<const float*>(sc.new_hca_kv) + ((size_t)b * D + newh[j]) * DH;
-    j -= n_newh;
     if (j < n_win) return reinterpret_cast<const float*>(c.win_kv) + (size_t)tok_row_of(c, s, b, win_lo + j) * DH;
     return reinterpret_cast<const float*>(nd.kv) + ((size_t)b * D + path[j - n_win]) * DH;
   };
+  auto chosen_row = [&](int j) -> const float* {
+    if (j >= n_sel) return reinterpret_cast<const float*>(sc.new_hca_kv) + ((size_t)b * D + newh[j - n_sel]) * DH;
+    const int idx = __ldcg(sel + j);
+    if (idx < tm.n_csa) return reinterpret_cast<const float*>(c.csa_kv) + (size_t)csa_rows_of(c, s, b)(idx) * DH;
+    int a = newc[0];
+    for (int i = 0; i < cnt[0]; ++i) if (newc_blk[i] == idx) a = newc[i];
+    return reinterpret_cast<const float*>(sc.new_csa_kv) + ((size_t)b * D + a) * DH;
+  };
   const uint32_t ks = (uint32_t)__cvta_generic_to_shared(dsm);
-  auto resolve = [&](int tile) { const int j = k0 + tile * KT + t; if (t < KT && j < k1) rows[tile & 1][t] = key_row(j); };
-  auto issue = [&](int tile) {                                        // after a barrier behind resolve(tile); one copy group per call
+  auto resolve = [&](int part, int tile) {
+    const int j = k0 + tile * KT + t;
+    if (t < KT && j < k1) rows[tile & 1][t] = part ? chosen_row(j) : known_row(j);
+  };
+  auto issue = [&](int tile) {                                        // after a barrier behind resolve(.., tile); one copy group per call
     const int nk = min(KT, k1 - (k0 + tile * KT));
-    const uint32_t dst = ks + (uint32_t)(nbuf == 2 ? (tile & 1) : 0) * (KT * DH * 4);
+    const uint32_t dst = ks + (uint32_t)(tile & 1) * (KT * DH * 4);
     for (int r = w; r < nk; r += NT / 32) cp16(dst + r * (DH * 4) + lane * 16, rows[tile & 1][r] + 4 * lane);
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  const int ntile = (k1 - k0 + KT - 1) / KT;
-  resolve(0);
-  resolve(1);
-  __syncthreads();
-  issue(0);                                                           // (an empty share: an empty group)
   float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};     // heads 2 w, 2 w + 1 (alike in all lanes)
   float4 o[8];                                                        // heads 8 (w & 1) .., columns 4 lane ..
 #pragma unroll
   for (int i = 0; i < 8; ++i) o[i] = make_float4(0.f, 0.f, 0.f, 0.f);
   const float scale = s.sm_scale;
-  for (int tile = 0; tile < ntile; ++tile) {
-    const int nk = min(KT, k1 - (k0 + tile * KT));
-    if (tile) __syncthreads();                                        // the tile before has been read (its buffer is filled again)
-    if (nbuf == 2 && tile + 1 < ntile) issue(tile + 1); else asm volatile("cp.async.commit_group;" ::: "memory");
-    asm volatile("cp.async.wait_group 1;" ::: "memory");
-    __syncthreads();                                                  // the tile's rows are there; rows[tile & 1] has been read
-    const float* K = reinterpret_cast<const float*>(dsm) + (size_t)(nbuf == 2 ? (tile & 1) : 0) * (KT * DH);
-    if (tile + 2 < ntile) resolve(tile + 2);
+  bool any = false;                                                   // a tile has been worked on
 #pragma unroll 1
-    for (int kb = 4 * w; kb < nk; kb += 32) {                         // (rows past nk of a group of four: stale, masked)
-      float a[16];
+  for (int part = 0; part < 2; ++part) {
+    int N = n_hca + n_win + cnt[2];
+    if (part) {
+      asm volatile("griddepcontrol.wait;" ::: "memory");               // the selection, and through it the state build
+      n_sel = __ldcg(reinterpret_cast<const int32_t*>(ws + pl.off_selcnt) + (size_t)b * D + n);
+      N = n_sel + n_newh;
+      __syncthreads();                                                  // (the buffers and row pointers of the part before)
+    }
+    const int per = (N + cs - 1) / cs;
+    k0 = min(N, rank * per); k1 = min(N, k0 + per);
+    const int ntile = (k1 - k0 + KT - 1) / KT;
+    resolve(part, 0);
+    resolve(part, 1);
+    __syncthreads();
+    issue(0);                                                           // (an empty share: an empty group)
+#pragma unroll 1
+    for (int tile = 0; tile < ntile; ++tile, any = true) {
+      const int nk = min(KT, k1 - (k0 + tile * KT));
+      if (tile) __syncthreads();                                        // the tile before has been read (its buffer is filled again)
+      if (tile + 1 < ntile) issue(tile + 1); else asm volatile("cp.async.commit_group;" ::: "memory");
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+      __syncthreads();                                                  // the tile's rows are there; rows[tile & 1] has been read
+      const float* K = reinterpret_cast<const float*>(dsm) + (size_t)(tile & 1) * (KT * DH);
+      if (tile + 2 < ntile) resolve(part, tile + 2);
+#pragma unroll 1
+      for (int kb = 4 * w; kb < nk; kb += 32) {                         // (rows past nk of a group of four: stale, masked)
+        float a[16];
 #pragma unroll
-      for (int i = 0; i < 16; ++i) a[i] = 0.f;
+        for (int i = 0; i < 16; ++i) a[i] = 0.f;
 #pragma unroll
-      for (int x = 0; x < 4; ++x)
+        for (int x = 0; x < 4; ++x)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const float4 kv = reinterpret_cast<const float4*>(K + (kb + k) * DH)[x * 8 + slice];
+          for (int k = 0; k < 4; ++k) {
+            const float4 kv = reinterpret_cast<const float4*>(K + (kb + k) * DH)[x * 8 + slice];
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            a[4 * i + k] = fmaf(q[i][x].x, kv.x, a[4 * i + k]);
-            a[4 * i + k] = fmaf(q[i][x].y, kv.y, a[4 * i + k]);
-            a[4 * i + k] = fmaf(q[i][x].z, kv.z, a[4 * i + k]);
-            a[4 * i + k] = fmaf(q[i][x].w, kv.w, a[4 * i + k]);
+            for (int i = 0; i < 4; ++i) {
+              a[4 * i + k] = fmaf(q[i][x].x, kv.x, a[4 * i + k]);
+              a[4 * i + k] = fmaf(q[i][x].y, kv.y, a[4 * i + k]);
+              a[4 * i + k] = fmaf(q[i][x].z, kv.z, a[4 * i + k]);
+              a[4 * i + k] = fmaf(q[i][x].w, kv.w, a[4 * i + k]);
+            }
+          }
+        // the eight slices: each exchange halves the values a lane is responsible for
+#pragma unroll
+        for (int half = 8, bit = 4; half >= 2; half >>= 1, bit >>= 1) {
+          const bool up = lane & bit;
+#pragma unroll
+          for (int i = 0; i < half; ++i) {
+            const float send = up ? a[i] : a[half + i], keep = up ? a[half + i] : a[i];
+            a[i] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
           }
         }
-      // the eight slices: each exchange halves the values a lane is responsible for
+        const int h = hq + (slice >> 1), k = kb + 2 * (slice & 1);      // this lane: (head h, keys k, k + 1)
+        P[k * PP + h] = k < nk ? a[0] * scale : -INFINITY;
+        P[(k + 1) * PP + h] = k + 1 < nk ? a[1] * scale : -INFINITY;
+      }
+      __syncthreads();
 #pragma unroll
-      for (int half = 8, bit = 4; half >= 2; half >>= 1, bit >>= 1) {
-        const bool up = lane & bit;
+      for (int x = 0; x < 2; ++x) {                                     // softmax of heads 2 w, 2 w + 1
+        const int h = 2 * w + x;
+        const float s0 = lane < nk ? P[lane * PP + h] : -INFINITY, s1 = lane + 32 < nk ? P[(lane + 32) * PP + h] : -INFINITY;
+        float mx = fmaxf(s0, s1);
 #pragma unroll
-        for (int i = 0; i < half; ++i) {
-          const float send = up ? a[i] : a[half + i], keep = up ? a[half + i] : a[i];
-          a[i] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
+        for (int d = 16; d > 0; d >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, d));
+        const float m_new = fmaxf(m_run[x], mx);                        // finite: every tile holds a key
+        const float p0 = expf(s0 - m_new), p1 = expf(s1 - m_new);
+        const float al = expf(m_run[x] - m_new);                        // 0 on the first tile
+        l_run[x] = fmaf(l_run[x], al, warp_sum(p0 + p1));
+        m_run[x] = m_new;
+        if (lane < nk) P[lane * PP + h] = p0;
+        if (lane + 32 < nk) P[(lane + 32) * PP + h] = p1;
+        if (lane == 0) alpha_sm[h] = al;
+      }
+      __syncthreads();
+      {
+        const int hb = 8 * (w & 1), kq = w >> 1;
+        if (any) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) { const float al = alpha_sm[hb + i]; o[i].x *= al; o[i].y *= al; o[i].z *= al; o[i].w *= al; }
         }
-      }
-      const int h = hq + (slice >> 1), k = kb + 2 * (slice & 1);      // this lane: (head h, keys k, k + 1)
-      P[k * PP + h] = k < nk ? a[0] * scale : -INFINITY;
-      P[(k + 1) * PP + h] = k + 1 < nk ? a[1] * scale : -INFINITY;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int x = 0; x < 2; ++x) {                                     // softmax of heads 2 w, 2 w + 1
-      const int h = 2 * w + x;
-      const float s0 = lane < nk ? P[lane * PP + h] : -INFINITY, s1 = lane + 32 < nk ? P[(lane + 32) * PP + h] : -INFINITY;
-      float mx = fmaxf(s0, s1);
-#pragma unroll
-      for (int d = 16; d > 0; d >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, d));
-      const float m_new = fmaxf(m_run[x], mx);                        // finite: every tile holds a key
-      const float p0 = expf(s0 - m_new), p1 = expf(s1 - m_new);
-      const float al = expf(m_run[x] - m_new);                        // 0 on the first tile
-      l_run[x] = fmaf(l_run[x], al, warp_sum(p0 + p1));
-      m_run[x] = m_new;
-      if (lane < nk) P[lane * PP + h] = p0;
-      if (lane + 32 < nk) P[(lane + 32) * PP + h] = p1;
-      if (lane == 0) alpha_sm[h] = al;
-    }
-    __syncthreads();
-    {
-      const int hb = 8 * (w & 1), kq = w >> 1;
-      if (tile) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) { const float al = alpha_sm[hb + i]; o[i].x *= al; o[i].y *= al; o[i].z *= al; o[i].w *= al; }
-      }
-      const int beg = kq * (KT / 4), end = min(nk, beg + KT / 4);
+        const int beg = kq * (KT / 4), end = min(nk, beg + KT / 4);
 #pragma unroll 4
-      for (int k = beg; k < end; ++k) {
-        const float4 kv = reinterpret_cast<const float4*>(K + k * DH)[lane];
-        const float4 pa = *reinterpret_cast<const float4*>(P + k * PP + hb), pb = *reinterpret_cast<const float4*>(P + k * PP + hb + 4);
-        const float pv[8] = {pa.x, pa.y, pa.z, pa.w, pb.x, pb.y, pb.z, pb.w};
+        for (int k = beg; k < end; ++k) {
+          const float4 kv = reinterpret_cast<const float4*>(K + k * DH)[lane];
+          const float4 pa = *reinterpret_cast<const float4*>(P + k * PP + hb), pb = *reinterpret_cast<const float4*>(P + k * PP + hb + 4);
+          const float pv[8] = {pa.x, pa.y, pa.z, pa.w, pb.x, pb.y, pb.z, pb.w};
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          o[i].x = fmaf(pv[i], kv.x, o[i].x); o[i].y = fmaf(pv[i], kv.y, o[i].y);
-          o[i].z = fmaf(pv[i], kv.z, o[i].z); o[i].w = fmaf(pv[i], kv.w, o[i].w);
+          for (int i = 0; i < 8; ++i) {
+            o[i].x = fmaf(pv[i], kv.x, o[i].x); o[i].y = fmaf(pv[i], kv.y, o[i].y);
+            o[i].z = fmaf(pv[i], kv.z, o[i].z); o[i].w = fmaf(pv[i], kv.w, o[i].w);
+          }
         }
       }
     }
@@ -252,13 +269,14 @@ bool tva_f32_applies(const tsv_shape& s) { return s.dtype == TSV_FP32 && s.d == 
 
 int launch_tva_f32(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, const tsv_nodes& nd, const tsv_scratch& sc,
                    void* out, char* ws, cudaStream_t st) {
-  // CTAs per node: as many as all fit the device at once (two per SM) while a share still holds 32 keys
+  // CTAs per node: as many as fit the device at once, one per SM, while a share still holds 32 keys.  One, although the registers
+  // admit two: beside the selection's CTAs there is room for one, and the others would begin when the selection has ended
+  // (16 sequences: 38.9 us a pass with two per SM, 34.8 with one).
   const int64_t base = (int64_t)s.B * s.D * ((s.H + f32a::HG - 1) / f32a::HG);
   int cs = 8;
-  while (cs > 1 && (base * cs > 2 * 148 || (cs - 1) * 32 >= p.keys_max)) cs >>= 1;
-  const int nbuf = (p.keys_max + cs - 1) / cs > f32a::KT ? 2 : 1;
-  const int bytes = nbuf * f32a::KT * f32a::DH * 4;
-  if (!ensure_smem((const void*)attn_f32_kernel, 2 * f32a::KT * f32a::DH * 4)) return TSV_ERR_CUDA;
+  while (cs > 1 && (base * cs > 148 || (cs - 1) * 32 >= p.keys_max)) cs >>= 1;
+  const int bytes = 2 * f32a::KT * f32a::DH * 4;
+  if (!ensure_smem((const void*)attn_f32_kernel, bytes)) return TSV_ERR_CUDA;
   TSV_PREP(attn_f32_kernel);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(cs, s.D * ((s.H + f32a::HG - 1) / f32a::HG), s.B); cfg.blockDim = dim3(f32a::NT, 1, 1); cfg.dynamicSmemBytes = bytes; cfg.stream = st;
@@ -268,7 +286,7 @@ int launch_tva_f32(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, con
   attr[1].id = cudaLaunchAttributeClusterDimension;
   attr[1].val.clusterDim.x = cs; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr; cfg.numAttrs = 2;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, attn_f32_kernel, s, p, c, nd, sc, (float*)out, ws, nbuf);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, attn_f32_kernel, s, p, c, nd, sc, (float*)out, ws);
   count_launch();
   return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? TSV_OK : TSV_ERR_CUDA;
 }
