@@ -108,7 +108,7 @@ bool tva_tc_pair_usable(const tsv_cache& c);
 // Host-side preparation of the tensor-core attention path: everything that can fail on the host (tensor maps, kernel
 // attributes) is done here, before any kernel of the call is enqueued.
 struct TvaTcPrep {
-  alignas(64) unsigned char maps[20 * 128];     // the paired kernel's tensor maps (copied into the launch's parameters)
+  alignas(64) unsigned char maps[18 * 128];     // the paired kernel's tensor maps (copied into the launch's parameters)
 };
 int prepare_tva_tc_pair(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, const tsv_nodes& nd, void* out, char* ws, TvaTcPrep& prep);
 // general: gathered tiles or tiles of more than two chunks may occur (else the instantiation without that code runs)

@@ -13,8 +13,8 @@
 //   warp 1       MMA issuer (leader CTA only): tcgen05.mma.cta_group::2, slot release and accumulator
 //                events by tcgen05.commit multicast to both CTAs
 //   warp 2       hands out the items (leader's counter, both CTAs told)
-//   warps 4-11   one-pass softmax on the CTA's own S rows (TMEM), P written back to TMEM, epilogue of O through
-//                swizzled shared-memory tiles and TMA stores; events to the leader's MMA warp by remote arrive
+//   warps 4-11   one-pass softmax on the CTA's own S rows (TMEM), P written back to TMEM, epilogue of O straight from
+//                registers, or through swizzled shared-memory tiles and TMA stores; events to the leader's MMA warp by remote arrive
 // Stage stream, TMEM column plan, running-max rule and chunking are those described at the kernel.
 #include <cuda.h>
 #include <stdio.h>
@@ -61,7 +61,7 @@ struct Ctl {                               // control block at the start of dyna
                                            //   [pc] S of piece pc is complete   [3 + p] the item's part p of O is complete
   uint64_t cmp_ev[7];                      // compute warps -> MMA, likewise:
                                            //   [pc] P of piece pc is in TMEM   [3 + p] part p of O has been read out
-  uint64_t stage_free;                     // the item's output tiles have left the staging slots (this CTA's)
+  uint64_t stage_free;                     // the item's output tiles have left the staging slots (this CTA's; not used where GENERAL)
   uint64_t item_ev;                        // the next item has been handed out
   uint32_t tmem_base;
   int32_t merge_here;                      // set for the CTA that finished a multi-chunk tile last
@@ -146,13 +146,11 @@ __device__ __forceinline__ void compute_sync() { asm volatile("bar.sync 1, 256;"
 // a stage whose key rows are consecutive rows of one array is fetched by ONE large request.
 struct alignas(64) MapSet {
   CUtensorMap q;          // 128-row boxes
-  CUtensorMap out;        // 32-row boxes (stores)
+  CUtensorMap out;        // 32-row boxes (stores; not used where GENERAL)
   CUtensorMap src[4][3];  // [csa, hca, window, packed misc][32, 64, 128 rows]
   CUtensorMap row[4];     // the same arrays with one-row boxes: gathers of four rows by index
-  CUtensorMap part;       // normalised partial outputs of multi-chunk tiles (bf16, 32-row boxes, stores)
-  CUtensorMap part32;     // the same in fp32, 32-column boxes (tiles cut for the sake of parallelism: no rounding before the merge)
 };
-constexpr int NMAPS = 20;
+constexpr int NMAPS = 18;
 
 constexpr uint32_t OOB_BOX = 0x3FFFFF00u;   // map 0, a row beyond every tensor: the box is zero-filled
 
@@ -328,10 +326,10 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
       auto issue_q = [&](int dk, int slot) {
         if (lane == 0) {
           if (slot < NSV) v_wait(slot >= NPROD);                   // (a V stage of the item before)
-          else if (n_real && !fail && !mbar_wait(&sm.stage_free, (uint32_t)(n_real - 1) & 1u)) fail = 1;
+          else if (!GENERAL && n_real && !fail && !mbar_wait(&sm.stage_free, (uint32_t)(n_real - 1) & 1u)) fail = 1;
           if (rank == 0) mbar_expect_tx(&sm.fullQ[dk], 2 * SLOTP);
           tma_box2(ring + (uint32_t)slot * SLOTP, &maps.q, dk * 64, w.b * rows_seq + row0, map_to_rank(smem_u32(&sm.fullQ[dk]), 0));
-          if (n_real && dk < 2) tma_box_l2(&maps.q, (dk + 6) * 64, w.b * rows_seq + row0);     // (the slots of slices 6 and 7 are free last)
+          if (!GENERAL && n_real && dk < 2) tma_box_l2(&maps.q, (dk + 6) * 64, w.b * rows_seq + row0);     // (the slots of slices 6 and 7 are free last)
         }
         __syncwarp();
       };
@@ -382,7 +380,7 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
       }
       issue_k(kpos);
       if (u & 1) issue_q(3 + (u >> 1), pw + NPROD * (h0 ^ 1));
-      if (u == 2 || u == 4) issue_q(5 + (u >> 1), NSV - 1 + (u >> 1));       // (slots 12 and 13 change hands with the item, when everything before is complete)
+      if (u == 2 || u == 4) issue_q(5 + (u >> 1), NSV - 1 + (u >> 1));       // (slots 12 and 13: free since the S products of the item before, which this warp has awaited, or since its output left them)
 #pragma unroll 1
       for (int gk = kpos + NKS; gk < NKST; gk += NKS) issue_k(gk);
       kcnt ^= w.npc == 1 ? 0x3Cu : w.npc == 2 ? 0x0Fu : 0u;        // (8, 16 or 24 stages over six positions)
@@ -606,15 +604,14 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
     const uint32_t mybit = 1u << ((int)rank * (BM / s.H) + row / s.H);      // node of this row within the pair's plan tile
     const float scale2 = s.sm_scale * 1.4426950408889634f;
     uint32_t accb = 0;                               // parity of the next use of each acc_ev
-    // The merge kernel is told, per warp, that an item's rows are stored.  It costs nothing half an item later, when the stores are
-    // long complete (right after them it is a wait of a memory latency), and the pair's last item is signalled at the end.  Not where
+    // The merge kernel is told, per warp, that an item's rows are stored: half an item later, when the stores are
+    // long complete (right after them the release waits a memory latency for them), and the pair's last item is signalled at the end.  Not where
     // tiles are cut to fill the device: all items end at about the same time there.
     int stored_rix = -1;
     auto signal_stored = [&]() {
-      if (GENERAL && stored_rix >= 0 && lane == 0) {
-        asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
-        asm volatile("fence.proxy.async.global;" ::: "memory");
-        asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(reinterpret_cast<int32_t*>(ws + pl.off_tcnt) + stored_rix) : "memory");
+      if (GENERAL && stored_rix >= 0) {
+        __syncwarp();                                // (the other lanes' stores are before the release)
+        if (lane == 0) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(reinterpret_cast<int32_t*>(ws + pl.off_tcnt) + stored_rix) : "memory");
       }
       stored_rix = -1;
     };
@@ -756,139 +753,168 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
       // piece's S columns); the wait for the stores of a later piece covers the earlier ones
       if (npc == 3 && pc == 1) p_stored(1);
     }
-    signal_stored();
-    // The row sums meet (in the words in which the maxima did: the two warps have read those when they are past the barrier below, and
-    // write them next two items on); where a warp moved its reference, the two settle on the larger one first, which the
-    // output staging area carries: no part of O can be complete before both have announced P, which they do after reading it.
+    // The row sums meet, in the words in which the maxima did (the two warps have read those when they are past the barrier below, and
+    // write them again two items on); where a warp moved its reference, the two settle on the larger one first.
     float l_row = (lp[0] + lp[1]) + (lp[2] + lp[3]);
     {
-      const uint32_t mine = ring + (uint32_t)NSV * SLOTP + (uint32_t)(warp - 4) * 4096 + lane * 4, other = ring + (uint32_t)NSV * SLOTP + (uint32_t)((warp - 4) ^ 4) * 4096 + lane * 4;
       // (no reference moved, as nearly always: P is announced before the sums are exchanged)
       uint32_t any_moved;
       asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\tbarrier.cta.red.or.pred q, %2, 64, p;\n\tselp.b32 %0, 1, 0, q;\n\t}" : "=r"(any_moved) : "r"(moved), "r"(2 + q4) : "memory");
-      if (!any_moved) p_stored(npc - 1);
-      else asm volatile("st.shared.b32 [%0], %1;" ::"r"(mine), "r"(__float_as_uint(m_run)) : "memory");
-      xch[hh * BM + row] = __float_as_uint(l_row);
-      pair_sync();
-      float l_other = __uint_as_float(xch[(hh ^ 1) * BM + row]);
+      auto exchange = [&](float v) {
+        xch[hh * BM + row] = __float_as_uint(v);
+        pair_sync();
+        return __uint_as_float(xch[(hh ^ 1) * BM + row]);
+      };
       if (any_moved) {                               // (alike in both warps)
-        uint32_t m_bits;
-        asm volatile("ld.shared.b32 %0, [%1];" : "=r"(m_bits) : "r"(other) : "memory");
-        const float m_other = __uint_as_float(m_bits), to = fmaxf(m_run, m_other);
+        const float m_other = exchange(m_run), to = fmaxf(m_run, m_other);
         if (to != -INFINITY) {
-          const float f = ex2(m_run - to), fo = ex2(m_other - to);
+          const float f = ex2(m_run - to);
           const int last = npc - 1;
           if (__any_sync(FULL, f != 1.f)) rescale_p(last, CL - last * 256 >= 256 ? 4 : 2, f);
-          l_row *= f; l_other *= fo;
+          l_row *= f;
           m_run = to;
         }
-        p_stored(npc - 1);
+        pair_sync();                                 // (the words are written again)
       }
-      l_row += l_other;
+      p_stored(npc - 1);
+      l_row += exchange(l_row);
     }
+    signal_stored();                                 // (of the item before; after P, which the tensor core waits for)
 
-    const bool full_tile = row0 + BM <= rows_seq;     // whole tile inside the sequence: rows may be stored as 32-row boxes
     const float inv = l_row > 0.f ? 1.f / l_row : 0.f;
     constexpr int cw = OW / 2;                        // columns of the part this thread handles
+    // The output leaves by one of two ways.  GENERAL: straight from registers, so that the next item's last two Q slices need not wait until
+    // staging in their slots has been read (4 x 128 k 103.0 -> 99.7 us, 16 of 512-8192 tokens 3 %).  Else, where most pairs have an item or
+    // two and the code is run through cold, staged for TMA stores, in half the instructions (one short stack 161 us, the other way 164).
+    const bool full_tile = row0 + BM <= rows_seq;     // whole tile inside the sequence: rows may be stored as 32-row boxes
     const uint32_t stage = ring + (uint32_t)NSV * SLOTP + (uint32_t)(warp - 4) * 4096;   // this warp's tile of 32 rows x 64 columns (bf16)
     bool stored = false;
+    // GENERAL: rows of the output, or of the chunk's slot of partial outputs: fp32, or bf16 at the start of the slot, which has room for
+    // fp32; normalised, a merge kernel follows.  Read out so that four lanes share a row; they transpose their 4 x 4 words, and a
+    // warp's store is whole 128-byte lines of eight rows.  (A row per lane, 32 bytes of a line each: 64 short sequences 423 -> 448 us.)
+    const bool p32 = nch > 1 && w.f32;
+    const int quad = lane >> 2, q = lane & 3, rowb = p32 ? DH * 4 : DH * 2;
+    char* dst = nch == 1 ? reinterpret_cast<char*>(out_) + ((size_t)b * rows_seq + row0) * (DH * 2)
+                         : ws + pl.off_tpo + (rix * pl.tc_chmax + chunk) * ((size_t)BM * DH * 4);
+    const bool wide = (reinterpret_cast<uintptr_t>(dst) & 31) == 0;
+    const int nrow = (nch > 1 ? BM : rows_seq - row0) - q4 * 32 - quad;       // rows 8 x of this lane with 8 x < nrow are written
+    dst += (q4 * 32 + quad) * rowb;
+    auto put32 = [&](char* p, const uint32_t (&v)[8]) {
+      if (wide) asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
+      else {                                         // (the caller's output is aligned to 16 bytes)
+        reinterpret_cast<uint4*>(p)[0] = make_uint4(v[0], v[1], v[2], v[3]);
+        reinterpret_cast<uint4*>(p)[1] = make_uint4(v[4], v[5], v[6], v[7]);
+      }
+    };
+    auto transpose4 = [&](uint32_t& v0, uint32_t& v1, uint32_t& v2, uint32_t& v3) {      // lane q's word i <-> lane i's word q
+      const bool h2 = q & 2, h1 = q & 1;
+      const uint32_t a = __shfl_xor_sync(FULL, h2 ? v0 : v2, 2), c = __shfl_xor_sync(FULL, h2 ? v1 : v3, 2);
+      if (h2) { v0 = a; v1 = c; } else { v2 = a; v3 = c; }
+      const uint32_t d = __shfl_xor_sync(FULL, h1 ? v0 : v1, 1), e = __shfl_xor_sync(FULL, h1 ? v2 : v3, 1);
+      if (h1) { v0 = d; v2 = e; } else { v1 = d; v3 = e; }
+    };
 #pragma unroll 1
     for (int part = 0; part < w.np; ++part) {
       if (!fail && !mbar_wait(&sm.acc_ev[3 + part], (accb >> (3 + part)) & 1u)) fail = 1;
       fence_after();
       const uint32_t ocol = tlane + (w.dbl ? 256 + (part & 1) * OW : 384) + hh * cw;
       const int col = (w.p0 + part) * OW + hh * cw;
-      const bool many = GENERAL && nch > 1;
-      auto read_out = [&]() {                        // in registers: the columns may be overwritten
-        fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(map_to_rank(smem_u32(&sm.cmp_ev[3 + part]), 0));
-      };
-      auto stage_read = [&]() {                      // the store before has read the staging tile
-        if (stored) {
+      uint32_t r[64];                                // GENERAL: [half of 16 rows][group of 8 columns][8 rows further][column]: row quad, columns 2 q, 2 q + 1
+      if (GENERAL) {
+        tmem_ld16x256b_x8_nowait(ocol, r);
+        tmem_ld16x256b_x8_nowait(ocol + (16u << 16), r + 32);
+      } else {
+        tmem_ld32_nowait(ocol, r);
+        tmem_ld32_nowait(ocol + 32, r + 32);
+      }
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      tmem_regs_ready(r);
+      tmem_regs_ready(r + 32);
+      fence_before();                                // in registers: the columns may be overwritten
+      __syncwarp();
+      if (lane == 0) mbar_arrive_cluster(map_to_rank(smem_u32(&sm.cmp_ev[3 + part]), 0));
+      if (GENERAL) {
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {                // rows 8 x + quad
+          const float f = __shfl_sync(FULL, inv, 8 * x + quad);
+          const uint32_t* rx = r + 32 * (x >> 1) + 2 * (x & 1);
+          char* p = dst + 8 * x * rowb;
+          uint32_t v[8];
+          if (p32) {
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {            // lane q: the columns of group 4 j + q
+#pragma unroll
+              for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int c = 0; c < 2; ++c) v[2 * i + c] = __float_as_uint(__uint_as_float(rx[4 * (4 * j + i) + c]) * f);
+              transpose4(v[0], v[2], v[4], v[6]);
+              transpose4(v[1], v[3], v[5], v[7]);
+              if (8 * x < nrow) put32(p + (col + 8 * (4 * j + q)) * 4, v);
+            }
+          } else {                                   // lane q: the columns of groups 2 q and 2 q + 1
+#pragma unroll
+            for (int g = 0; g < 8; ++g) {
+              const __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(rx[4 * g]) * f, __uint_as_float(rx[4 * g + 1]) * f);
+              v[4 * (g & 1) + (g >> 1)] = *reinterpret_cast<const uint32_t*>(&h2);
+            }
+            transpose4(v[0], v[1], v[2], v[3]);
+            transpose4(v[4], v[5], v[6], v[7]);
+            if (8 * x < nrow) put32(p + (col + 16 * q) * 2, v);
+          }
+        }
+      } else if (nch == 1) {
+        // stage the 32 x 64 bf16 tile in the 128-byte swizzle pattern and store it with one TMA request
+        if (stored) {                                // the store before has read the staging tile
           if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
           __syncwarp();
         }
         stored = true;
-      };
-      auto stage_store = [&](const CUtensorMap* map, int x, int y) {
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncwarp();
-        if (lane == 0) {
-          asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];"
-                       ::"l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(stage) : "memory");
-          asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-        }
-      };
-      if (many && w.f32) {
-        // fp32 partial output: two tiles of 32 rows x 32 columns
-#pragma unroll 1
-        for (int x = 0; x < 2; ++x) {
-          uint32_t r[32];
-          tmem_ld32(ocol + 32 * x, r);
-          if (x) read_out();
-          stage_read();
 #pragma unroll
-          for (int v = 0; v < 8; ++v)
-            asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(stage + lane * 128 + ((v ^ (lane & 7)) << 4)), "f"(__uint_as_float(r[4 * v]) * inv),
-                         "f"(__uint_as_float(r[4 * v + 1]) * inv), "f"(__uint_as_float(r[4 * v + 2]) * inv), "f"(__uint_as_float(r[4 * v + 3]) * inv) : "memory");
-          stage_store(&maps.part32, col + 32 * x, (int)((rix * pl.tc_chmax + chunk) * BM) + q4 * 32);
+        for (int v = 0; v < 8; ++v) {
+          uint32_t pk[4];
+#pragma unroll
+          for (int t = 0; t < 4; ++t) {
+            const __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(r[8 * v + 2 * t]) * inv, __uint_as_float(r[8 * v + 2 * t + 1]) * inv);
+            pk[t] = *reinterpret_cast<const uint32_t*>(&h2);
+          }
+          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(stage + lane * 128 + ((v ^ (lane & 7)) << 4)), "r"(pk[0]), "r"(pk[1]), "r"(pk[2]),
+                       "r"(pk[3]) : "memory");
+        }
+        if (full_tile) {
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          __syncwarp();
+          if (lane == 0) {
+            asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];"
+                         ::"l"(reinterpret_cast<uint64_t>(&maps.out)), "r"(col), "r"(b * rows_seq + row0 + q4 * 32), "r"(stage) : "memory");
+            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+          }
+        } else {                                     // the rows of this sequence only: plain stores, 64 columns of a row by eight lanes
+          __syncwarp();
+#pragma unroll 1
+          for (int i = lane; i < 32 * 8; i += 32) {
+            const int rr = i >> 3;
+            uint4 v;
+            asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(stage + rr * 128 + (((i ^ rr) & 7) << 4)) : "memory");
+            if (row0 + q4 * 32 + rr < rows_seq)
+              reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(out_) + ((size_t)b * rows_seq + row0 + q4 * 32 + rr) * DH + col)[i & 7] = v;
+          }
+          __syncwarp();                              // (the tile is written again)
+          stored = false;
         }
       } else {
-        uint32_t r[64];
-        tmem_ld32_nowait(ocol, r);
-        tmem_ld32_nowait(ocol + 32, r + 32);
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        tmem_regs_ready(r);
-        tmem_regs_ready(r + 32);
-        read_out();
-        if (nch == 1 || many) {
-          // stage the 32 x 64 bf16 tile in the 128-byte swizzle pattern and store it with one TMA request: into the output,
-          // or (multi-chunk tiles, where a merge kernel follows) into the chunk's tile of normalised partial outputs, which a merge kernel
-          // combines with the chunks' (max, sum)
-          stage_read();
+        float* po = reinterpret_cast<float*>(ws + pl.off_tpo) + ((rix * pl.tc_chmax + chunk) * BM + row) * DH + col;
 #pragma unroll
-          for (int v = 0; v < 8; ++v) {
-            uint32_t pk[4];
-#pragma unroll
-            for (int t = 0; t < 4; ++t) {
-              const __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(r[8 * v + 2 * t]) * inv, __uint_as_float(r[8 * v + 2 * t + 1]) * inv);
-              pk[t] = *reinterpret_cast<const uint32_t*>(&h2);
-            }
-            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(stage + lane * 128 + ((v ^ (lane & 7)) << 4)), "r"(pk[0]), "r"(pk[1]), "r"(pk[2]),
-                         "r"(pk[3]) : "memory");
-          }
-          // (a chunk's bf16 tile lies at the start of the chunk's slot for an fp32 tile: 2 BM rows of 1 KiB per slot)
-          if (many) stage_store(&maps.part, col, (int)((rix * pl.tc_chmax + chunk) * 2 * BM) + q4 * 32);
-          else if (full_tile) stage_store(&maps.out, col, b * rows_seq + row0 + q4 * 32);
-          else {                                     // the rows of this sequence only: plain stores, 64 columns of a row by eight lanes
-            __syncwarp();
-#pragma unroll 1
-            for (int i = lane; i < 32 * 8; i += 32) {
-              const int rr = i >> 3;
-              uint4 v;
-              asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(stage + rr * 128 + (((i ^ rr) & 7) << 4)) : "memory");
-              if (row0 + q4 * 32 + rr < rows_seq)
-                reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(out_) + ((size_t)b * rows_seq + row0 + q4 * 32 + rr) * DH + col)[i & 7] = v;
-            }
-            __syncwarp();                            // (the tile is written again)
-            stored = false;
-          }
-        } else {
-          float* po = reinterpret_cast<float*>(ws + pl.off_tpo) + ((rix * pl.tc_chmax + chunk) * BM + row) * DH + col;
-#pragma unroll
-          for (int v = 0; v < 16; ++v)
-            *reinterpret_cast<float4*>(po + v * 4) = make_float4(__uint_as_float(r[4 * v]), __uint_as_float(r[4 * v + 1]), __uint_as_float(r[4 * v + 2]), __uint_as_float(r[4 * v + 3]));
-        }
+        for (int v = 0; v < 16; ++v)
+          *reinterpret_cast<float4*>(po + v * 4) = make_float4(__uint_as_float(r[4 * v]), __uint_as_float(r[4 * v + 1]), __uint_as_float(r[4 * v + 2]), __uint_as_float(r[4 * v + 3]));
       }
       if (nch > 1 && w.p0 + part == 0 && hh == 0)
         reinterpret_cast<float2*>(ws + pl.off_tpml)[(rix * pl.tc_chmax + chunk) * BM + row] = make_float2(m_run, l_row);
     }
-    accb ^= w.acc_used();
-    if (lane == 0) {                                 // the staging slots are free for the next item's K stages
+    if (!GENERAL && lane == 0) {                     // the staging slots are free for the next item's Q slices
       asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
       asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&sm.stage_free)) : "memory");
     }
+    accb ^= w.acc_used();
     if (GENERAL && nch > 1 && pl.tc_split == 1) stored_rix = (int)rix;
     if (!GENERAL && nch > 1) {
       // Tiles of two chunks where nothing longer can occur: each chunk leaves its unnormalised part of O with (max, sum)
@@ -931,7 +957,7 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
       }
     }
     }
-    if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    if (!GENERAL && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     signal_stored();
     leave();
   }
@@ -949,15 +975,15 @@ static PFN_cuTensorMapEncodeTiled encode_fn() {
   return fn;
 }
 
-// rows x 512 bf16 (or fp32), row-major; boxes of 32 rows x 128 bytes written with the 128-byte swizzle
-static bool make_map(CUtensorMap* m, const void* basep, int64_t rows, int box_rows = kBoxRows, bool f32 = false) {
+// rows x 512 bf16, row-major; boxes of 64 columns in the 128-byte swizzle
+static bool make_map(CUtensorMap* m, const void* basep, int64_t rows, int box_rows) {
   PFN_cuTensorMapEncodeTiled fn = encode_fn();
   if (!fn || rows <= 0 || ((uintptr_t)basep & 15)) return false;
   const cuuint64_t gdim[2] = {(cuuint64_t)tc::DH, (cuuint64_t)rows};
-  const cuuint64_t gstr[1] = {(cuuint64_t)tc::DH * (f32 ? 4 : 2)};
-  const cuuint32_t box[2] = {f32 ? 32u : 64u, (cuuint32_t)box_rows};
+  const cuuint64_t gstr[1] = {(cuuint64_t)tc::DH * 2};
+  const cuuint32_t box[2] = {64u, (cuuint32_t)box_rows};
   const cuuint32_t estr[2] = {1, 1};
-  return fn(m, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(basep), gdim, gstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(basep), gdim, gstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -978,13 +1004,6 @@ int prepare_tva_tc_pair(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c
     for (int k = 0; k < 3 && ok; ++k) ok = make_map(&ms.src[a][k], bases[a], rows[a], 32 << k);
     ok = ok && make_map(&ms.row[a], bases[a], rows[a], 1);
   }
-  // partial outputs: per (128-row tile, chunk) a slot of 128 x 512 fp32 (used so by the instantiation that merges inside
-  // the kernel); the general instantiation stores 128 x 512 bf16 at the start of the slot: as rows of 1 KiB the buffer
-  // has 2 x 128 rows per slot
-  if (p.tc_chmax > 1) ok = ok && make_map(&ms.part, ws + p.off_tpo, (int64_t)s.B * 2 * p.tc_nt * p.tc_chmax * 2 * tc::BM, 32);
-  if (p.tc_split > 1) ok = ok && make_map(&ms.part32, ws + p.off_tpo, (int64_t)s.B * 2 * p.tc_nt * p.tc_chmax * tc::BM, 32, true);
-  else ms.part32 = ms.out;
-  if (p.tc_chmax <= 1) ms.part = ms.out;                                                       // (never used: no tile has more than one chunk)
   if (!ok) {
     fprintf(stderr, "tsv: cuTensorMapEncodeTiled failed\n");
     return TSV_ERR_CUDA;
