@@ -45,7 +45,7 @@ constexpr int NKS = NSX - NQS;             // K stages in flight
 constexpr int NSV = 12;                    // Slots [0, 12) are one FIFO: an item's first six Q slices and its ring of six K stages take the next twelve
                                            // places, its V stages (once the S products are complete) the places from the same start on; so
                                            // the next item's operands land where the V stages are released first.  Slots 12, 13: the last
-                                           // two Q slices, and, when O is read out, the staging of the output (a 4 KiB tile per warp).
+                                           // two Q slices, and, when O is read out, the staging of the output where it is staged (a 4 KiB tile per warp).
 // The FIFO's places of an item, about in the order in which the S products want them: Q0 K0 Q1 K1 Q2 K2 K3 Q3 K4 Q4 K5 Q5 (of places
 // p and p + 6, which are one producer's, one is a Q slice, the other a K stage).  Six stages of operands are requested before the item
 // before is done with; with all of Q and four K stages in the FIFO, and the ring's other two stages waiting for the output's staging,
