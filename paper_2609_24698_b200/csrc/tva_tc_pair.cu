@@ -38,6 +38,7 @@ constexpr int REGS_SERVICE = 120, REGS_COMPUTE = 136;
 static_assert(128 * (2 * REGS_SERVICE + 2 * REGS_COMPUTE) <= TTHREADS * 128, "register split beyond what the CTA is launched with");
 constexpr int BOXB = kBoxRows * 128;       // bytes of one box: kBoxRows rows x 128 bytes
 constexpr float RESCALE_GAP = 16.f;        // log2 units a later piece's row max may exceed the running reference
+constexpr float REF_FLOOR = -3e38f;        // lowest reference: a row whose first visible scores are all -inf gives them the weight zero, not NaN
 
 constexpr int NSX = 14;                    // 16 KiB slots of the staging area
 constexpr int NQS = 8;                     // Q slices of an item (all of d, resident for every piece)
@@ -649,6 +650,11 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
     constexpr uint32_t FULL = 0xffffffffu;
     uint32_t* xch = reinterpret_cast<uint32_t*>(sm.xch) + (it & 1) * 2 * BM;
     auto pair_sync = [&]() { asm volatile("bar.sync %0, 64;" ::"r"(2 + q4) : "memory"); };     // the two warps of these rows
+    auto pair_or = [&](uint32_t x) {                 // the same, and whether x is set in any of their threads
+      uint32_t y;
+      asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\tbarrier.cta.red.or.pred q, %2, 64, p;\n\tselp.b32 %0, 1, 0, q;\n\t}" : "=r"(y) : "r"(x), "r"(2 + q4) : "memory");
+      return y;
+    };
     auto slab_of = [&](int i) { return (i & 1) + ((i & 2) << 1) + 2 * hh; };
     // slab i of this warp in the piece whose S begins at column scol: read, invisible keys as -inf; the maximum (unscaled)
     auto read_slab = [&](uint32_t scol, int i, uint32_t vis, uint32_t (&sv)[32]) {
@@ -683,6 +689,9 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
 #pragma unroll
       for (int c = 0; c < 4; ++c) lp[c] *= f;
     };
+    // A visible key has been found.  The branches that hold warp-collective instructions follow this, which is alike in all threads of
+    // the two warps, and not the rows' references: finite queries and keys can have a product of -inf in one row alone.
+    uint32_t seen = 0;
     int moved = 0;                                   // this warp changed its reference after the exchange
     // Node masks of this lane's keys of a piece, a byte per slab; fetched a piece ahead (fetched when needed they cost the chain a
     // memory latency, 1.3 k cycles per piece after the first).
@@ -710,7 +719,7 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
       // One slab after the other in a loop of one slab's code: what the two warps of a scheduler leave idle is the other's, and the
       // instructions of four slabs side by side did not stay in the instruction cache (kernel of 97 KB, a slab 900 cycles; 512 is what
       // the special-function unit needs for the two warps).
-      if (m_run == -INFINITY) {                      // uniform over the two warps of these rows: no visible key so far
+      if (!seen) {
         int i = 0;
         uint32_t vis = 0;
 #pragma unroll 1
@@ -718,16 +727,14 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
         uint32_t sv[32];
         const float mc = i < ns ? read_slab(scol, i, vis, sv) : -INFINITY;
         xch[hh * BM + row] = __float_as_uint(mc);
-        pair_sync();
-        m_run = fmaxf(mc, __uint_as_float(xch[(hh ^ 1) * BM + row])) * scale2;
-        if (m_run == -INFINITY) pair_sync();         // (the exchange words will be written again before the next item)
+        seen = pair_or(i < ns);                      // (if not, nobody reads the words before they are written again)
+        if (seen) m_run = fmaxf(fmaxf(mc, __uint_as_float(xch[(hh ^ 1) * BM + row])) * scale2, REF_FLOOR);
       }
-      const bool any = m_run != -INFINITY;
 #pragma unroll 1
       for (int i = 0; i < ns; ++i) {
         uint32_t pk[16];
         const uint32_t vis = visible(i);
-        if (any && vis) {
+        if (seen && vis) {
           uint32_t sv[32];
           const float mc = read_slab(scol, i, vis, sv) * scale2;
           if (__any_sync(FULL, mc > m_run + RESCALE_GAP)) {        // (warp-uniform: tensor-memory accesses are warp-collective)
@@ -758,22 +765,18 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
     float l_row = (lp[0] + lp[1]) + (lp[2] + lp[3]);
     {
       // (no reference moved, as nearly always: P is announced before the sums are exchanged)
-      uint32_t any_moved;
-      asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\tbarrier.cta.red.or.pred q, %2, 64, p;\n\tselp.b32 %0, 1, 0, q;\n\t}" : "=r"(any_moved) : "r"(moved), "r"(2 + q4) : "memory");
+      const uint32_t any_moved = pair_or(moved);
       auto exchange = [&](float v) {
         xch[hh * BM + row] = __float_as_uint(v);
         pair_sync();
         return __uint_as_float(xch[(hh ^ 1) * BM + row]);
       };
       if (any_moved) {                               // (alike in both warps)
-        const float m_other = exchange(m_run), to = fmaxf(m_run, m_other);
-        if (to != -INFINITY) {
-          const float f = ex2(m_run - to);
-          const int last = npc - 1;
-          if (__any_sync(FULL, f != 1.f)) rescale_p(last, CL - last * 256 >= 256 ? 4 : 2, f);
-          l_row *= f;
-          m_run = to;
-        }
+        const float m_other = exchange(m_run), to = fmaxf(m_run, m_other), f = ex2(m_run - to);
+        const int last = npc - 1;
+        if (__any_sync(FULL, f != 1.f)) rescale_p(last, CL - last * 256 >= 256 ? 4 : 2, f);
+        l_row *= f;
+        m_run = to;
         pair_sync();                                 // (the words are written again)
       }
       p_stored(npc - 1);
