@@ -80,6 +80,7 @@ bool make_tva_plan(const tsv_shape& s, TvaPlan& p) {
   if (ks < 64) ks = 64;
   p.ks = (int32_t)ks;
   p.nsplit = (int32_t)((p.keys_max + ks - 1) / ks);
+  p.built = 0;
   size_t off = 0;
   p.off_selcnt = off; off = up256(off + (size_t)s.B * s.D * sizeof(int32_t));
   p.off_sel = off;    off = up256(off + (size_t)s.B * s.D * s.topk * sizeof(int32_t));
@@ -173,6 +174,7 @@ static int tva_stages(const tsv_shape& s, const TvaPlan& p_in, const tsv_cache& 
   if (p.tc && !tva_tc_pair_usable(c)) p.tc = 0;       // no row counts for the tensor maps: the CUDA-core path (same workspace)
   if (p.tc && (stages & 6) && (r = prepare_tva_tc(s, p, c, nd, out, ws, prep))) return r;
   if (build != Build::none) {
+    p.built = 1;
     p.tc_packed = p.tc;                               // the attention that follows finds the new entries packed
     if ((r = launch_bsb(s, c, nd, sc, status, build == Build::first_layer, p.tc_packed ? ws + p.off_misc : nullptr, p.tc_misc_rows, st))) return r;
   }

@@ -44,6 +44,7 @@ struct TvaPlan {
   int32_t need_scores;   // cand_cap > topk: some node may have to rank its candidates
   int32_t idx_fused;     // ranked nodes score their committed entries inside topk_kernel (short candidate lists: the
                          // separate scoring kernel, which exits at once for every sequence that needs no ranking, is not launched)
+  int32_t built;         // the kernel before the selection is this call's state build (set at the launch)
   int32_t keys_max;      // max keys one node can attend to
   int32_t ks;            // keys per split (CUDA-core path)
   int32_t nsplit;        // max splits per node

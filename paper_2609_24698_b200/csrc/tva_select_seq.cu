@@ -554,9 +554,11 @@ __global__ void __launch_bounds__(128) score_rows_kernel(const tsv_shape s, cons
   sco.weights(nd.iw + (size_t)b * D * HI, n0, D, HI);
   __syncthreads();
   float* scores = reinterpret_cast<float*>(ws + pl.off_scores) + (size_t)b * D * pl.score_ld;
-  // No wait before the scores are written: the kernel before is the state build, whose dependents start when it has waited for all
-  // earlier work (the call before on this workspace included), or one that starts its dependents when it has ended.  (Without that
-  // wait, and with the ranges kept below, four sequences of 128 k tokens took 103.0 us a pass instead of 107.5.)
+  // No wait before the scores are written where the kernel before is this call's state build, whose dependents start when it has
+  // waited for all earlier work (the call before on this workspace included): without it, and with the ranges kept below, four
+  // sequences of 128 k tokens took 4 % less a pass.  In a call without the state build the kernel before may be any, such as a
+  // selection that signals at its start and still reads scores and ranges.
+  if (!pl.built) asm volatile("griddepcontrol.wait;" ::: "memory");
   float lo = INFINITY, hi = -INFINITY;                   // of node n0 + lane / 4, over this warp's entries (a NaN stays in lo)
 #pragma unroll
   for (int st = 0; st < kRowSteps; ++st) {

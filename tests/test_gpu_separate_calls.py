@@ -40,3 +40,32 @@ def test_tensor_core_shapes(separate_calls, D, lengths, topk, layers, page, defe
 def test_other_shapes(separate_calls, dtype, d, di):
     cfg = synth.Config(f"separate_{dtype}", 217, synth.Shape(dtype, 4, 8, 16, d, 4, 48, 2, di, 32, 40), layers=2, L_min=0, L_max=900, seed=8)
     lockstep(cfg, cycles=2, lengths=[0, 150, 511, 900])
+
+
+@pytest.mark.parametrize("D,L", [(8, 40000), (12, 3000)])
+def test_selections_in_a_row_share_a_workspace(D, L):
+    """The selections of two layers without a state build between them, the way the benchmark times that stage: the next one's scores must
+    not reach the workspace while the one before still reads its own (scores over all SMs, a cluster per node)."""
+    import torch
+    from paper_2609_24698_b200 import binding as tsv, harness as hz
+    sh = synth.Shape("bf16", 4, D, 64, 512, 4, 512, 4, 128, 128, 128)
+    ccap, hcap = hz.capacities(sh, [L] * 4, 2 * D)
+    eng = hz.VerifyEngine(sh, 2, ccap, hcap, L + 2 * D, want_topk=True)
+    gen = torch.Generator(device="cuda").manual_seed(L)
+    inp = hz.InputSet.empty(sh, 2)
+    inp.layers[0].parent.copy_(torch.arange(-1, D - 1).expand(4, D)); inp.layers[0].n_nodes.fill_(D)
+    for c, nd in zip(eng.caches, inp.layers):
+        c.L.fill_(L)
+        for t in (c.csa_ik, nd.ikc, nd.iq, nd.iw):
+            t.normal_(generator=gen)
+    eng.launch_cycle(inp, refresh=False)
+    torch.cuda.synchronize()
+    want = [t.clone() for t in eng.topk_idx]
+    assert int(eng.status.sum()) == 0 and not torch.equal(want[0], want[1])
+    for _ in range(20):
+        for t in eng.topk_idx:
+            t.fill_(-2)
+        for l in range(2):
+            tsv.bench_tree_verify_attn_stages(eng.cshape, eng.caches[l], inp.layers[l], eng.scratch[l], eng.out[l], eng.topk_idx[l], eng.workspace,
+                                              eng.status, tsv.STAGE_SELECT)
+        assert all(torch.equal(a, b) for a, b in zip(eng.topk_idx, want))
