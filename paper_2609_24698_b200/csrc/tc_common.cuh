@@ -141,23 +141,26 @@ __device__ __host__ __forceinline__ void chunking_x(int nk, bool general, int sp
   if (nch < 1) nch = 1;
   lds = 4 * nch <= split ? 2 : 2 * nch <= split ? 1 : 0;
 }
-// The record of a tile, which the tile plan leaves and the kernels after it read: {sequence, what, keys, 0}, what = mode (2 bits: 1
-// boxes, 2 gathered) | fp32 partial outputs << 2 | chunk length / 128 << 4 | tile of the sequence << 7 | chunks << 12 | log2 of the
-// items of a chunk << 28.  (The chunking is three divisions: by every role of the attention kernel on its own they were 10 KB of its code.)
-__device__ __forceinline__ int4 tile_record(const TvaPlan& pl, int b, int tile, int mode, int nk) {
+// The record of a tile, which the tile plan leaves and the kernels after it read: {sequence, what, keys, chunks}, what = mode (2 bits: 1
+// boxes, 2 gathered) | fp32 partial outputs << 2 | chunk length / 128 << 4 | tile of the sequence << 7 | chunks, kManyChunks for that many
+// and more, << 12 | log2 of the items of a chunk << 28.  In the record of a work item the last word is the item: its roles only ask for one
+// chunk, two, or more.  (The chunking is three divisions: by every role of the attention kernel on its own they were 10 KB of its code.)
+constexpr int kManyChunks = 0xFFFF;
+__device__ __host__ __forceinline__ int4 tile_record(const TvaPlan& pl, int b, int tile, int mode, int nk) {
   int nch, CL, lds;
   bool f32;
   chunking_x(nk, pl.tc_general != 0, pl.tc_split, pl.tc_chmax, pl.tc_f32, nch, CL, f32, lds);
-  return make_int4(b, mode | (f32 ? 4 : 0) | (CL / 128) << 4 | tile << 7 | nch << 12 | lds << 28, nk, 0);
+  return make_int4(b, mode | (f32 ? 4 : 0) | (CL / 128) << 4 | tile << 7 | (nch < kManyChunks ? nch : kManyChunks) << 12 | lds << 28, nk, nch);
 }
 static_assert(NCX / 128 < 8 && TSV_MAX_D * 128 / PR <= 32, "fields of a tile's record");
-__device__ __forceinline__ bool rec_gather(const int4& r) { return (r.y & 3) == 2; }
-__device__ __forceinline__ bool rec_f32(const int4& r) { return (r.y & 4) != 0; }
-__device__ __forceinline__ int rec_chunk_keys(const int4& r) { return ((r.y >> 4) & 7) * 128; }
-__device__ __forceinline__ int rec_tile(const int4& r) { return (r.y >> 7) & 31; }
-__device__ __forceinline__ int rec_chunks(const int4& r) { return (r.y >> 12) & 0xFFFF; }
-__device__ __forceinline__ int rec_lds(const int4& r) { return r.y >> 28; }
-__device__ __forceinline__ int rec_items(const int4& r) { return rec_chunks(r) << rec_lds(r); }
+__device__ __host__ __forceinline__ bool rec_gather(const int4& r) { return (r.y & 3) == 2; }
+__device__ __host__ __forceinline__ bool rec_f32(const int4& r) { return (r.y & 4) != 0; }
+__device__ __host__ __forceinline__ int rec_chunk_keys(const int4& r) { return ((r.y >> 4) & 7) * 128; }
+__device__ __host__ __forceinline__ int rec_tile(const int4& r) { return (r.y >> 7) & 31; }
+__device__ __host__ __forceinline__ int rec_chunks_or_many(const int4& r) { return (r.y >> 12) & kManyChunks; }
+__device__ __host__ __forceinline__ int rec_lds(const int4& r) { return r.y >> 28; }
+__device__ __host__ __forceinline__ int rec_chunks(const int4& r) { return r.w; }                    // (of a tile's record)
+__device__ __host__ __forceinline__ int rec_items(const int4& r) { return r.w << rec_lds(r); }       // (likewise)
 
 }  // namespace tc
 

@@ -11,7 +11,7 @@
 //                    rows): the runs as 32-row TMA boxes.  Gathered tiles (selection far from dense, or a paged pool
 //                    whose pages do not hold whole boxes): the CSA run holds only the entries some node of the tile
 //                    selected, and every key is named by array << 30 | row for four-row TMA gathers.
-//                    Each tile CTA leaves its record {tile, mode, keys} at the tile's scheduling position (its rank by
+//                    Each tile CTA leaves its record (tile_record) at the tile's scheduling position (its rank by
 //                    estimated length of its work items, longest first); an extra CTA per sequence packs the small scattered rows.
 //   tc_combine_pair_kernel  merges the chunks of the paired kernel's multi-chunk tiles (fixed order).
 #include <type_traits>
@@ -72,7 +72,7 @@ __device__ __forceinline__ void tc_plan_tile(const tsv_shape& s, const TvaPlan& 
     for (int i = threadIdx.x + blockDim.x; i < ntile; i += blockDim.x)
       est[i] = tile_keys_estimate(s, c.L[i / pl.tc_nt], nd.n_nodes[i / pl.tc_nt], i % pl.tc_nt, npt);
   }
-  // thread 0 leaves the tile's record {tile, mode, keys} at that position as soon as it knows the key count
+  // thread 0 leaves the tile's record at that position as soon as it knows the key count
   auto leave_record = [&](int nk, int md) {
     *nkeys = nk; *mode = md;
     reinterpret_cast<int4*>(ws + pl.off_order)[ntile <= kRankTilesMax ? *ahead_sm : (int)tix] = tc::tile_record(pl, b, tile, md, nk);
@@ -348,7 +348,7 @@ __device__ __forceinline__ void tc_plan_tile(const tsv_shape& s, const TvaPlan& 
   }
 }
 
-// Plan of every (sequence, 256-row tile).  Each tile CTA leaves one 16-byte record {tile, mode, keys} at the tile's
+// Plan of every (sequence, 256-row tile).  Each tile CTA leaves one 16-byte record (tile_record) at the tile's
 // scheduling position: its rank among all tiles by estimated key count, most first, which every CTA works out for itself
 // from the lengths and node counts of all sequences (the paired attention kernel takes the tiles in that order, long
 // ones first and short ones in the tail, and learns all it needs about its tile from one load).  A tile no node of which
@@ -400,7 +400,7 @@ __global__ void __launch_bounds__(256) tc_combine_pair_kernel(const tsv_shape s,
   constexpr uint32_t FULL = 0xffffffffu;
   const int lg = 31 - __clz(BM / 8 / rpw), pos = blockIdx.x >> (lg + 1), half = (blockIdx.x >> lg) & 1, group = blockIdx.x & ((1 << lg) - 1);
   // Launched as a programmatic dependent of the attention kernel, when all CTAs of that have started: the tile plan is complete.
-  const int4 rec = __ldcg(reinterpret_cast<const int4*>(ws + pl.off_order) + pos);     // {tile, mode, keys}
+  const int4 rec = __ldcg(reinterpret_cast<const int4*>(ws + pl.off_order) + pos);
   // (What other kernels wrote is read past the L1.)  One CTA waits for that kernel in any case, so that the completion of this one
   // implies that one's.
   const bool early = pl.tc_split == 1;

@@ -66,7 +66,7 @@ struct Ctl {                               // control block at the start of dyna
   uint64_t item_ev;                        // the next item has been handed out
   uint32_t tmem_base;
   int32_t merge_here;                      // set for the CTA that finished a multi-chunk tile last
-  alignas(16) int4 item[2];                // the pair's current and next work: the tile's record with the chunk (sequence -1: no more)
+  alignas(16) int4 item[2];                // the pair's current and next work: the tile's record with the item in its last word (sequence -1: no more)
   float xch[2][2][BM];                     // first-slab maxima of the rows, by the two warps that share them (two buffers in turn)
 };
 constexpr int CTLB = 3072;                 // control block bytes; the ring follows (needs a 1024-byte aligned base)
@@ -161,17 +161,17 @@ constexpr uint32_t OOB_BOX = 0x3FFFFF00u;   // map 0, a row beyond every tensor:
 namespace pair {
 constexpr int NQ = 4, OW = tc::DH / NQ;      // the PV product is computed in NQ parts of OW columns of d
 struct Item {
-  int tix, b, tile, nk, chunk, nch, CL, cbeg, cend;
+  int tix, b, tile, nk, chunk, nch, CL, cbeg, cend;      // (nch: kManyChunks for more than that)
   int npc;                 // S pieces
   int lds, p0, np;         // log2 of the items of a chunk; this one's parts of O: [p0, p0 + np)
   bool dbl;                // two O buffers: a part is computed while the one before is read out
   bool f32;                // partial outputs are fp32
   bool gather;             // the key list is a list of row codes (array << 30 | row), not of boxes
-  __device__ __forceinline__ Item(int4 r, const TvaPlan& pl, bool general) {      // a tile's record, the chunk in its last word
+  __device__ __forceinline__ Item(int4 r, const TvaPlan& pl, bool general) {      // a tile's record, the item in its last word
     b = r.x; tile = rec_tile(r); tix = b * pl.tc_nt + tile;
     gather = general && rec_gather(r); f32 = general && rec_f32(r);
     lds = rec_lds(r);
-    nk = r.z; chunk = r.w >> lds; nch = rec_chunks(r);
+    nk = r.z; chunk = r.w >> lds; nch = rec_chunks_or_many(r);
     np = NQ >> lds; p0 = (r.w & ((1 << lds) - 1)) * np;
     const int stride = rec_chunk_keys(r);
     cbeg = chunk * stride; cend = min(nk, cbeg + stride);
