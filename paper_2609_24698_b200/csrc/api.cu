@@ -85,10 +85,9 @@ bool make_tva_plan(const tsv_shape& s, TvaPlan& p) {
   p.off_selcnt = off; off = up256(off + (size_t)s.B * s.D * sizeof(int32_t));
   p.off_sel = off;    off = up256(off + (size_t)s.B * s.D * s.topk * sizeof(int32_t));
   p.off_scores = off; if (p.need_scores) off = up256(off + (size_t)s.B * s.D * p.score_ld * sizeof(float));
-  p.ext_ld = (int32_t)((pref + 255) / 256 * 4);
-  p.off_ext = off;    if (p.need_scores) off = up256(off + (size_t)s.B * s.D * p.ext_ld * 2 * sizeof(float));
   p.off_po = off;     if (p.nsplit > 1) off = up256(off + (size_t)s.B * s.D * s.H * p.nsplit * s.d * sizeof(float));
   p.off_pml = off;    if (p.nsplit > 1) off = up256(off + (size_t)s.B * s.D * s.H * p.nsplit * 2 * sizeof(float));
+  size_t off_partials_end = off;
   p.tc = tva_tc_eligible(s);
   p.tc_nt = p.tc_maxk = p.tc_chmax = p.tc_misc_rows = 0; p.tc_split = 1; p.tc_f32 = p.tc_general = p.tc_packed = 0;
   p.off_krow = p.off_kmask = p.off_nkeys = p.off_tpo = p.off_tpml = p.off_box = p.off_mode = p.off_misc = p.off_order = p.off_tcnt = p.off_sched = off;
@@ -104,6 +103,7 @@ bool make_tva_plan(const tsv_shape& s, TvaPlan& p) {
     const size_t slot = 2 * tiles * 128 * s.d * sizeof(float), slot_ml = 2 * tiles * 128 * 2 * sizeof(float);
     if (p.tc_chmax > 1) off = up256(up256(off + p.tc_chmax * slot) + p.tc_chmax * slot_ml);
     const size_t pool = off - off_pool;
+    off_partials_end = off;
     int64_t ch = kPairsFor / (int64_t)tiles;
     if (ch > (p.tc_maxk + 127) / 128) ch = (p.tc_maxk + 127) / 128;
     while (ch > p.tc_chmax && up256((size_t)ch * slot) + up256((size_t)ch * slot_ml) > pool) --ch;
@@ -124,6 +124,11 @@ bool make_tva_plan(const tsv_shape& s, TvaPlan& p) {
     p.off_sched = off; off = up256(off + 2 * sizeof(int32_t));
     p.off_selmask = off; if (p.need_scores) off = up256(off + (size_t)s.B * s.D * p.mask_ld * sizeof(uint32_t));
   }
+  // The ranges of the scores lie where the partial outputs will: the selection has read them when the attention begins.  Where those
+  // take less room (or none), no ranges are kept: the workspace does not grow by them.
+  p.off_ext = p.off_po;
+  p.ext_ld = (int32_t)((pref + 255) / 256 * 4);
+  if (!p.need_scores || (size_t)s.B * s.D * p.ext_ld * 2 * sizeof(float) > off_partials_end - p.off_po) p.ext_ld = 0;
   p.total = off;
   return true;
 }

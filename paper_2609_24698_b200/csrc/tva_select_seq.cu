@@ -578,10 +578,11 @@ __global__ void __launch_bounds__(128) score_rows_kernel(const tsv_shape s, cons
       for (int q = 0; q < 4; ++q) { alo[q] = nlo[q]; ahi[q] = nhi[q]; }
     }
   }
-  // The range of the scores for the selection, which bins them: two passes over the list and a cluster barrier less there.
+  // The range of the scores for the selection, which bins them: two passes over the list and a cluster barrier less there (where there is
+  // no room for the ranges, it makes those).
 #pragma unroll
   for (int o = 1; o < 4; o <<= 1) { lo = min_or_nan(lo, __shfl_xor_sync(0xffffffffu, lo, o)); hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o)); }
-  if ((lane & 3) == 0 && n0 + (lane >> 2) < D)
+  if (pl.ext_ld && (lane & 3) == 0 && n0 + (lane >> 2) < D)
     reinterpret_cast<float2*>(ws + pl.off_ext)[((size_t)b * D + n0 + (lane >> 2)) * pl.ext_ld + blockIdx.x * 4 + w] = make_float2(lo, hi);
   if (blockIdx.x == 0 && b == 0 && blockIdx.z == 0) asm volatile("griddepcontrol.wait;" ::: "memory");   // (this kernel's completion implies the state build's)
 }
@@ -592,6 +593,7 @@ __global__ void __launch_bounds__(128) score_rows_kernel(const tsv_shape s, cons
 constexpr int kListThreads = 512, kListBins = 1024;
 struct ListSmem {
   int hist[2][kListBins];                                // [0] the intervals; both: the digits of the radix passes
+  float2 ext;
   int cnt[2];                                            // candidates; (entries certainly taken, entries equal to the threshold)
   int eqs;
   float cand_s[ssel::CAP];
@@ -642,7 +644,7 @@ __global__ void __launch_bounds__(kListThreads, 2) topk_list_kernel(const tsv_sh
   const float4* src = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(ws + pl.off_scores) + ((size_t)b * D + n) * pl.score_ld + c0);
   float lo = INFINITY, hi = -INFINITY;                 // the range of the committed entries' scores
   const float2* ext = reinterpret_cast<const float2*>(ws + pl.off_ext) + ((size_t)b * D + n) * pl.ext_ld;
-  for (int i = t; i < (n_csa + 255) / 256 * 4; i += NT) { const float2 x = __ldcg(ext + i); lo = min_or_nan(lo, x.x); hi = fmaxf(hi, x.y); }
+  for (int i = t; i < (pl.ext_ld ? (n_csa + 255) / 256 * 4 : 0); i += NT) { const float2 x = __ldcg(ext + i); lo = min_or_nan(lo, x.x); hi = fmaxf(hi, x.y); }
   const int n4 = (min(c1, n_csa) - c0 + 3) >> 2;       // (negative: none)
   for (int i = t; i < n4; i += NT) reinterpret_cast<float4*>(list)[i] = __ldcg(src + i);
   if (c1 > n_csa) {
@@ -656,6 +658,8 @@ __global__ void __launch_bounds__(kListThreads, 2) topk_list_kernel(const tsv_sh
     for (int i = max(n_csa, c0) + t; i < c1; i += NT) list[i - c0] = extra[i - n_csa];
   }
   __syncthreads();
+  if (!pl.ext_ld)                                        // (the range of this CTA's share, the in-tree entries with it)
+    for (int i = t; i < len; i += NT) { const float v = list[i]; lo = min_or_nan(lo, v); hi = fmaxf(hi, v); }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) { lo = min_or_nan(lo, __shfl_xor_sync(0xffffffffu, lo, o)); hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o)); }
   if (lane == 0) { sm.red[0][w] = lo; sm.red[1][w] = hi; }
@@ -667,6 +671,13 @@ __global__ void __launch_bounds__(kListThreads, 2) topk_list_kernel(const tsv_sh
   auto peer_i = [&](const int* p, int r) { int v; asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(peer(p, r))); return v; };
   auto peer_f = [&](const float* p, int r) { float v; asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(peer(p, r))); return v; };
   auto meet = [&]() { __syncthreads(); cluster_arrive(); cluster_wait(); };
+  if (!pl.ext_ld) {                                      // the ranges of all CTAs' shares
+    if (t == 0) sm.ext = make_float2(lo, hi);
+    meet();
+    lo = peer_f(&sm.ext.x, lane & 7); hi = peer_f(&sm.ext.y, lane & 7);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) { lo = min_or_nan(lo, __shfl_xor_sync(0xffffffffu, lo, o)); hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o)); }
+  }
   const float scale = hi > lo ? (float)NB / (hi - lo) : 0.f;
   const bool regular = scale > 0.f && scale < 1e30f;     // (else: all equal, not finite, a NaN among them, or too narrow)
   auto bin_of = [&](float v) { return min(NB - 1, max(0, (int)((v - lo) * scale))); };      // (in-tree entries may lie beyond the range)

@@ -80,3 +80,18 @@ def test_host_errors_return_before_any_launch(lib):
     assert h(C.byref(s), 1, pc, pn, ps, fake, fake, None, fake, fake, fake, None) == tsv.ERR_NULL
     assert tsv._lib.tsv_error_string(tsv.ERR_ALIGN).decode().startswith("a vector pointer")
     assert tsv.version() >= 1000
+
+
+@pytest.mark.parametrize("kw", [
+    dict(dtype=0, B=64, D=8, H=16, d=128, HI=1, di=64, max_L=30208),            # fp32: a cluster per sequence keeps its scores to itself
+    dict(dtype=0, B=16, D=8, H=16, d=128, HI=1, di=64, max_L=102912),
+    dict(B=1, D=5, max_L=91136), dict(B=1, D=5, max_L=93184),                   # scores over all SMs, room for the ranges among the partial outputs
+    dict(B=64, D=5, H=16, d=128, topk=64, max_L=51000),                         # the same, no partial outputs
+])
+def test_shapes_that_the_static_workspace_holds(lib, kw):
+    """Shapes close below the size of the built-in workspace: what the selection keeps beside its scores may not cost them their place."""
+    from paper_2609_24698_b200.binding import CShape, STATIC_WORKSPACE_BYTES
+    lib.tsv_workspace_bytes.restype = C.c_size_t
+    lib.tsv_workspace_bytes.argtypes = [C.POINTER(CShape)]
+    n = lib.tsv_workspace_bytes(C.byref(_shape(**kw)))
+    assert STATIC_WORKSPACE_BYTES * 0.97 < n <= STATIC_WORKSPACE_BYTES

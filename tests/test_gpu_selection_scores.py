@@ -11,9 +11,10 @@ pytestmark = pytest.mark.gpu
 
 # dtype, nodes, committed entries, topk.  One CTA per node (short lists); a cluster per sequence, bf16 and fp32; scores over all SMs
 # and a cluster per node, for more than eight nodes and for a long list; the general kernels (other indexer widths): keys in registers,
-# a cluster per node, a list read again in every pass
+# a cluster per node, a list read again in every pass.  The last: so many heads (the sixth number) that nothing is split and the ranges
+# of the scores over all SMs have no room among partial outputs
 FORMS = [("bf16", 8, 600, 512), ("bf16", 8, 900, 800), ("fp32", 8, 600, 512), ("bf16", 12, 900, 800), ("bf16", 7, 4300, 4200),
-         ("fp32", 8, 900, 800, 16), ("bf16", 8, 2500, 2400, 16), ("fp32", 5, 66000, 65800, 8)]
+         ("fp32", 8, 900, 800, 16), ("bf16", 8, 2500, 2400, 16), ("fp32", 5, 66000, 65800, 8), ("bf16", 20, 900, 800, 128, 256)]
 
 
 def _select(form, HI, ik, tree_ik, iq, iw, room=None, cap=None, status=0):
@@ -23,7 +24,7 @@ def _select(form, HI, ik, tree_ik, iq, iw, room=None, cap=None, status=0):
     from paper_2609_24698_b200 import harness as hz
     dtype, D, n, k = form[:4]
     di = ik.shape[1]
-    sh = synth.Shape(dtype, 1, D, 4, 16, 2, k, HI, di, 64, 64)
+    sh = synth.Shape(dtype, 1, D, form[5] if len(form) > 5 else 4, 16, 2, k, HI, di, 64, 64)
     ccap, hcap = hz.capacities(sh, [2 * n], 2 * D)
     eng = hz.VerifyEngine(sh, 1, ccap, hcap, room or 2 * n + 2 * D, want_topk=True)
     guard = torch.full((D * k + 64,), -2, dtype=torch.int32, device="cuda")
