@@ -901,6 +901,7 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
             if (row0 + q4 * 32 + rr < rows_seq)
               reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(out_) + ((size_t)b * rows_seq + row0 + q4 * 32 + rr) * DH + col)[i & 7] = v;
           }
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");       // (the next item's queries are copied over the tile)
           __syncwarp();                              // (the tile is written again)
           stored = false;
         }

@@ -16,6 +16,7 @@ pytestmark = pytest.mark.gpu
     (14, 6, 600, [90 + 100 * i for i in range(14)]),          # 28 tiles: one chunk by two items, two by one each
     (3, 4, 300, [90, 800, 2600]),                             # three tiles, long lists possible: whole, or cut into chunks of 256 keys
     (76, 2, 300, [100 + 25 * i for i in range(76)]),          # 76 tiles of one to three chunks
+    (150, 3, 600, [40 + 7 * i for i in range(150)]),          # two or three tiles a pair, all ragged: staged rows under the next item's queries
 ])
 def test_shares_of_columns(B, D, topk, lengths):
     cfg = synth.Config(f"few_{B}_{D}", 217, synth.Shape("bf16", B, D, 64, 512, 2, topk, 2, 128, 16, 128), L_min=1, L_max=max(lengths), layers=1, seed=31 + B)
