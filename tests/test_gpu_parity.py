@@ -501,6 +501,15 @@ def test_tc_planted_peaks_reach_rescale_and_merge_paths():
     lockstep(cfg, cycles=1, lengths=[1200, 2040, 1660, 3500, 5000], plant=_plant_peaks(cfg), per_row=True)
 
 
+@pytest.mark.parametrize("topk,lengths", [(512, [2040]), (512, [1200]), (700, [2700]), (512, [2040 - 83 * i for i in range(14)]), (700, [2700 - 90 * i for i in range(14)])])
+def test_tc_planted_peaks_short_capacities(topk, lengths):
+    """The same in capacities that allow two chunks a tile at most and no gathered one (another instantiation of the attention kernel):
+    one sequence, whose tiles are shared by columns among four work items each, and fourteen, shared by two or not at all; one chunk of
+    two or three pieces, or two chunks, which the last work item merges."""
+    cfg = synth.Config(f"tc_peaks_short_{topk}", 86, synth.Shape("bf16", len(lengths), 8, topk=topk, **BENCH_HEADS), L_min=1, L_max=1, seed=8)
+    lockstep(cfg, cycles=1, lengths=lengths, plant=_plant_peaks(cfg), per_row=True)
+
+
 def test_tc_planted_peaks_ranked_tiles():
     """Same planted keys with a small top-k, so that every node ranks: masked-run tiles (n_csa <= 2 topk) and
     gathered tiles, single- and multi-chunk."""
