@@ -10,8 +10,8 @@
 //   S = Q K^T: lane = (4 heads, an eighth of the row); its queries stay in registers for the whole list, a key's row is one
 //              128-byte read for the four lane groups of a warp: 16 reads per 256 FMAs; the eighths meet by 14 shuffles.
 //   O = P K:   warp = (8 heads, a quarter of the tile's keys), lane = 4 columns: three reads per 32 FMAs.
-// The kernel is a programmatic dependent of the selection and waits for it between the two parts: of 16 sequences of 256-4096 tokens
-// two thirds of the keys are done under the selection (38.5 us a pass before, 35.0 now).
+// The kernel is a programmatic dependent of the selection and waits for it between the two parts: of 16 sequences of 256-4096 tokens with
+// 64 selected two thirds of the keys are done under the selection (42.0 us a pass without, 38.0 with).
 #include "kernels.h"
 
 namespace tsv {
@@ -44,6 +44,8 @@ __device__ __forceinline__ void cluster_sync() {
 
 }  // namespace f32a
 
+// EARLY: the keys known before the wait go first.  Else one part, the known keys at its start.
+template <bool EARLY>
 __global__ void __launch_bounds__(f32a::NT, 2) attn_f32_kernel(const tsv_shape s, const TvaPlan pl, const tsv_cache c, const tsv_nodes nd,
                                                                const tsv_scratch sc, float* __restrict__ out, char* __restrict__ ws) {
   using namespace f32a;
@@ -93,6 +95,7 @@ __global__ void __launch_bounds__(f32a::NT, 2) attn_f32_kernel(const tsv_shape s
   // (committed HCA | window | ancestors-or-self), then those that they do (selected CSA | in-tree HCA).
   const int n_hca = tm.n_hca, n_newh = cnt[1], pos = tm.L + tm.depth[n], win_lo = max(0, pos - s.window + 1), n_win = max(0, tm.L - win_lo);
   const int32_t* sel = reinterpret_cast<const int32_t*>(ws + pl.off_sel) + ((size_t)b * D + n) * s.topk;
+  const int lead = EARLY ? 0 : n_hca + n_win + cnt[2];
   int n_sel = 0;
   int k0 = 0, k1 = 0;                                                 // this CTA's share of the part at hand
   auto known_row = [&](int j) -> const float* {
@@ -112,7 +115,10 @@ __global__ void __launch_bounds__(f32a::NT, 2) attn_f32_kernel(const tsv_shape s
   const uint32_t ks = (uint32_t)__cvta_generic_to_shared(dsm);
   auto resolve = [&](int part, int tile) {
     const int j = k0 + tile * KT + t;
-    if (t < KT && j < k1) rows[tile & 1][t] = part ? chosen_row(j) : known_row(j);
+    if (t < KT && j < k1) {
+      if (EARLY) rows[tile & 1][t] = part ? chosen_row(j) : known_row(j);
+      else rows[tile & 1][t] = j < lead ? known_row(j) : chosen_row(j - lead);
+    }
   };
   auto issue = [&](int tile) {                                        // after a barrier behind resolve(.., tile); one copy group per call
     const int nk = min(KT, k1 - (k0 + tile * KT));
@@ -127,12 +133,12 @@ __global__ void __launch_bounds__(f32a::NT, 2) attn_f32_kernel(const tsv_shape s
   const float scale = s.sm_scale;
   bool any = false;                                                   // a tile has been worked on
 #pragma unroll 1
-  for (int part = 0; part < 2; ++part) {
+  for (int part = EARLY ? 0 : 1; part < 2; ++part) {
     int N = n_hca + n_win + cnt[2];
     if (part) {
       asm volatile("griddepcontrol.wait;" ::: "memory");               // the selection, and through it the state build
       n_sel = __ldcg(reinterpret_cast<const int32_t*>(ws + pl.off_selcnt) + (size_t)b * D + n);
-      N = n_sel + n_newh;
+      N = n_sel + n_newh + lead;
       __syncthreads();                                                  // (the buffers and row pointers of the part before)
     }
     const int per = (N + cs - 1) / cs;
@@ -269,15 +275,27 @@ bool tva_f32_applies(const tsv_shape& s) { return s.dtype == TSV_FP32 && s.d == 
 
 int launch_tva_f32(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, const tsv_nodes& nd, const tsv_scratch& sc,
                    void* out, char* ws, cudaStream_t st) {
-  // CTAs per node: as many as fit the device at once, one per SM, while a share still holds 32 keys.  One, although the registers
-  // admit two: beside the selection's CTAs there is room for one, and the others would begin when the selection has ended
-  // (16 sequences: 38.9 us a pass with two per SM, 34.8 with one).
+  // The keys known before the wait go first where some node may rank, which takes the selection long enough to work under it; else they
+  // are a part of the one list, whose shares leave one remainder of a tile instead of two (16 sequences of 2048 tokens with up to 1024
+  // selected: 54.4 us a pass, 56.5 in two parts).
+  const bool early = p.need_scores != 0;
+  const int64_t known = early ? s.max_L / s.m_hca + s.window + s.D : 0, chosen = p.keys_max - known;
+  // CTAs per node: as many as fit the device at once while a share still holds 32 keys.  One per SM where many of the keys precede the
+  // wait: beside the selection's CTAs there is room for one, and the others would begin when the selection has ended (16 sequences of
+  // 256-4096 tokens with 64 selected: 38.0 us, 40.0 with two per SM).  Two, as the registers admit, where two thirds follow it (512
+  // selected: 74.9 us, 85.0 with one), or half if a node would have one CTA only (18 sequences with 256 selected: 50.2, 56.4).  Of
+  // clusters of four and eight 296 CTAs are not resident at once (72 clusters of four: 61 us, 58 of two).
   const int64_t base = (int64_t)s.B * s.D * ((s.H + f32a::HG - 1) / f32a::HG);
-  int cs = 8;
-  while (cs > 1 && (base * cs > 148 || (cs - 1) * 32 >= p.keys_max)) cs >>= 1;
+  auto ctas = [&](int large, int small) {
+    int cs = 8;
+    while (cs > 1 && (base * cs > (cs > 2 ? large : small) || (cs - 1) * 32 >= p.keys_max)) cs >>= 1;
+    return cs;
+  };
+  int cs = ctas(148, 148);
+  if (chosen >= 2 * known || (cs == 1 && chosen >= known)) cs = ctas(256, 296);
   const int bytes = 2 * f32a::KT * f32a::DH * 4;
-  if (!ensure_smem((const void*)attn_f32_kernel, bytes)) return TSV_ERR_CUDA;
-  TSV_PREP(attn_f32_kernel);
+  if (!ensure_smem((const void*)attn_f32_kernel<true>, bytes) || !ensure_smem((const void*)attn_f32_kernel<false>, bytes)) return TSV_ERR_CUDA;
+  TSV_PREP(attn_f32_kernel<true>); TSV_PREP(attn_f32_kernel<false>);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(cs, s.D * ((s.H + f32a::HG - 1) / f32a::HG), s.B); cfg.blockDim = dim3(f32a::NT, 1, 1); cfg.dynamicSmemBytes = bytes; cfg.stream = st;
   cudaLaunchAttribute attr[2];
@@ -286,7 +304,8 @@ int launch_tva_f32(const tsv_shape& s, const TvaPlan& p, const tsv_cache& c, con
   attr[1].id = cudaLaunchAttributeClusterDimension;
   attr[1].val.clusterDim.x = cs; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr; cfg.numAttrs = 2;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, attn_f32_kernel, s, p, c, nd, sc, (float*)out, ws);
+  const cudaError_t e = early ? cudaLaunchKernelEx(&cfg, attn_f32_kernel<true>, s, p, c, nd, sc, (float*)out, ws)
+                              : cudaLaunchKernelEx(&cfg, attn_f32_kernel<false>, s, p, c, nd, sc, (float*)out, ws);
   count_launch();
   return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? TSV_OK : TSV_ERR_CUDA;
 }

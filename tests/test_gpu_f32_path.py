@@ -35,3 +35,14 @@ def test_f32_selection_exact_ties():
 def test_f32_peaked_softmax_over_many_tiles(scale):
     cfg = synth.Config("f32_peaked", 215, synth.Shape("fp32", 8, 8, 64, 128, 2, 500, 1, 64, 32, 128, scale), L_min=0, L_max=3000, seed=5)
     lockstep(cfg, cycles=1, lengths=[3000, 2501, 64, 130, 900, 1027, 2048, 333])
+
+
+# Selections that outweigh the keys known before them: two CTAs an SM, in clusters of eight, four (the most that there are), two; one
+# where there are more nodes than places; capacities in which no node ranks, whose keys are one list, in shares of a few keys and of many
+@pytest.mark.parametrize("B,D,topk,lengths", [
+    (4, 8, 500, [1300, 1041, 90, 0]), (8, 8, 400, [900 + 31 * i for i in range(8)]), (9, 8, 400, [1000 - 7 * i for i in range(9)]),
+    (18, 8, 256, [600 + 20 * i for i in range(18)]), (40, 8, 300, [700 + 9 * i for i in range(40)]), (1, 5, 1000, [700]), (16, 7, 1000, [64 * i + i for i in range(16)]),
+    (40, 8, 600, [25 * i for i in range(40)])])
+def test_f32_selections_that_outweigh_the_rest(B, D, topk, lengths):
+    cfg = synth.Config(f"f32_chosen_{B}_{topk}", 218, synth.Shape("fp32", B, D, 16, 128, 2, topk, 1, 64, 32, 32), L_min=0, L_max=max(lengths), seed=B + topk)
+    lockstep(cfg, cycles=2, lengths=lengths)
