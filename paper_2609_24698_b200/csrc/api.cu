@@ -90,7 +90,7 @@ bool make_tva_plan(const tsv_shape& s, TvaPlan& p) {
   size_t off_partials_end = off;
   p.tc = tva_tc_eligible(s);
   p.tc_nt = p.tc_maxk = p.tc_chmax = p.tc_misc_rows = 0; p.tc_split = 1; p.tc_f32 = p.tc_general = p.tc_packed = 0;
-  p.off_krow = p.off_kmask = p.off_nkeys = p.off_tpo = p.off_tpml = p.off_box = p.off_mode = p.off_misc = p.off_order = p.off_tcnt = p.off_sched = off;
+  p.off_krow = p.off_kmask = p.off_tpo = p.off_tpml = p.off_box = p.off_misc = p.off_order = p.off_tcnt = p.off_sched = off;
   p.off_selmask = off;
   p.mask_ld = ((p.cand_cap + 31) / 32 + 3) & ~3;
   if (p.tc) {
@@ -115,9 +115,7 @@ bool make_tva_plan(const tsv_shape& s, TvaPlan& p) {
     p.off_tpml = off_pool + up256((size_t)p.tc_chmax * slot);
     p.off_krow = off;  off = up256(off + tiles * p.tc_maxk * sizeof(uint32_t));   // row codes of gathered tiles
     p.off_kmask = off; off = up256(off + tiles * p.tc_maxk);
-    p.off_nkeys = off; off = up256(off + tiles * sizeof(int32_t));
     p.off_box = off;   off = up256(off + tiles * (p.tc_maxk / 32) * 2 * sizeof(int32_t));
-    p.off_mode = off;  off = up256(off + tiles * sizeof(int32_t));
     p.off_misc = off;  off = up256(off + (size_t)s.B * p.tc_misc_rows * s.d * 2);
     p.off_order = off; off = up256(off + tiles * 4 * sizeof(int32_t));
     p.off_tcnt = off;  off = up256(off + 2 * tiles * sizeof(int32_t));     // finished chunks per 128-row tile (paired kernel)

@@ -56,7 +56,7 @@ struct TvaPlan {
   int32_t tc_general;                // the chunking rule of the general instantiation (set at the launch)
   int32_t tc_misc_rows;              // rows of the per-sequence packed buffer
   int32_t tc_packed;                 // the state build has put the entries closed inside the tree into that buffer (set at the launch)
-  size_t off_krow, off_kmask, off_nkeys, off_tpo, off_tpml, off_box, off_mode, off_misc, off_order, off_tcnt, off_sched;   // off_sched: the paired kernel's item counter, the pairs that have run out of items
+  size_t off_krow, off_kmask, off_tpo, off_tpml, off_box, off_misc, off_order, off_tcnt, off_sched;   // off_sched: the paired kernel's item counter, the pairs that have run out of items
   // selection as a bit per candidate, one row of mask_ld words per node, written for the nodes that rank: the tile plan combines
   // the rows of a tile's nodes into its per-key node masks (bits, not bytes: the CTA that plans a tile of a long list reads them all)
   size_t off_selmask;

@@ -53,8 +53,6 @@ __device__ __forceinline__ void tc_plan_tile(const tsv_shape& s, const TvaPlan& 
   const size_t tix = (size_t)b * pl.tc_nt + tile;
   uint32_t* krow = reinterpret_cast<uint32_t*>(ws + pl.off_krow) + tix * pl.tc_maxk;    // gathered tiles: array << 30 | row per key
   uint8_t* kmask = reinterpret_cast<uint8_t*>(ws + pl.off_kmask) + tix * pl.tc_maxk;
-  int32_t* nkeys = reinterpret_cast<int32_t*>(ws + pl.off_nkeys) + tix;
-  int32_t* mode = reinterpret_cast<int32_t*>(ws + pl.off_mode) + tix;
   // the cache row offsets are fetched together with the tree scalars (one memory latency for all)
   __shared__ uint8_t cdone[TSV_MAX_D], hdone[TSV_MAX_D];
   __shared__ int64_t row0_sm[2];
@@ -74,7 +72,6 @@ __device__ __forceinline__ void tc_plan_tile(const tsv_shape& s, const TvaPlan& 
   }
   // thread 0 leaves the tile's record at that position as soon as it knows the key count
   auto leave_record = [&](int nk, int md) {
-    *nkeys = nk; *mode = md;
     reinterpret_cast<int4*>(ws + pl.off_order)[ntile <= kRankTilesMax ? *ahead_sm : (int)tix] = tc::tile_record(pl, b, tile, md, nk);
   };
   // The kernel is launched as a programmatic dependent of the selection kernel (itself one of the state build) and runs
@@ -613,7 +610,7 @@ int launch_tva_tc(const tsv_shape& s, const TvaPlan& p_in, const TvaTcPrep& prep
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
-    if (p.tc_split > 1 || p.tc_f32) cudaLaunchKernelEx(&cfg, tc_combine_pair_kernel<true, 1>, s, p, out, (const char*)ws, rpw);
+    if (p.tc_split > 1) cudaLaunchKernelEx(&cfg, tc_combine_pair_kernel<true, 1>, s, p, out, (const char*)ws, rpw);
     else if (rpw == 2) cudaLaunchKernelEx(&cfg, tc_combine_pair_kernel<false, 2>, s, p, out, (const char*)ws, rpw);
     else cudaLaunchKernelEx(&cfg, tc_combine_pair_kernel<false, 1>, s, p, out, (const char*)ws, rpw);
     count_launch();
