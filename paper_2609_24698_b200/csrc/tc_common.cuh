@@ -159,8 +159,10 @@ __device__ __host__ __forceinline__ int rec_chunk_keys(const int4& r) { return (
 __device__ __host__ __forceinline__ int rec_tile(const int4& r) { return (r.y >> 7) & 31; }
 __device__ __host__ __forceinline__ int rec_chunks_or_many(const int4& r) { return (r.y >> 12) & kManyChunks; }
 __device__ __host__ __forceinline__ int rec_lds(const int4& r) { return r.y >> 28; }
-__device__ __host__ __forceinline__ int rec_chunks(const int4& r) { return r.w; }                    // (of a tile's record)
-__device__ __host__ __forceinline__ int rec_items(const int4& r) { return r.w << rec_lds(r); }       // (likewise)
+// Of a tile's record.  (The packed count is read first, the word of its own only where that is saturated: with the word alone the merge
+// kernel was slower, 64 sequences of 1-4 k tokens 755 us a pass, so 743.)
+__device__ __host__ __forceinline__ int rec_chunks(const int4& r) { const int n = rec_chunks_or_many(r); return n < kManyChunks ? n : r.w; }
+__device__ __host__ __forceinline__ int rec_items(const int4& r) { return rec_chunks(r) << rec_lds(r); }
 
 }  // namespace tc
 
