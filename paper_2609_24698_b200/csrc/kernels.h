@@ -51,7 +51,7 @@ struct TvaPlan {
   size_t off_selcnt, off_sel, off_scores, off_ext, off_po, off_pml, total;
   // tensor-core path (bf16, d = 512): row tiles per sequence, key-list capacity per tile, max chunks per tile
   int32_t tc, tc_nt, tc_maxk, tc_chmax;
-  int32_t tc_split;                  // chunks a tile may be cut into to fill the device (1: tiles enough)
+  int32_t tc_split;                  // items a tile may have, to fill the device where tiles are few (1: tiles enough)
   int32_t tc_f32;                    // all partial outputs are fp32 (set at the launch)
   int32_t tc_general;                // the chunking rule of the general instantiation (set at the launch)
   int32_t tc_misc_rows;              // rows of the per-sequence packed buffer

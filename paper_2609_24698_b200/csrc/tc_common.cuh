@@ -11,7 +11,7 @@ constexpr int DH = 512;             // head dim handled by this path
 constexpr int BM = 128;             // rows per CTA
 constexpr int PR = 256;             // rows per plan tile: two row tiles (one CTA pair) share one key list
 constexpr int NC = 512;             // keys per chunk of a list that is cut into many
-constexpr int NCMIN = 256;          // keys of the shortest chunk worth an SM pair of its own
+constexpr int NCMIN = 256;          // keys that are worth an SM pair of their own
 constexpr uint32_t WAIT_LIMIT = 1u << 14;   // polls before a wait gives up (then no later wait of the thread is attempted)
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -119,8 +119,9 @@ constexpr int NCX = 768;             // max keys per chunk of the TMA kernel: P 
 // general = true: a list that does not fit one chunk is cut into chunks of at most NC keys, whose quarters of O go through two
 // buffers instead of one and which fill the SM pairs better (two chunks of up to NCX instead of three of NC cost 12 % of the
 // attention kernel on 32 paged sequences of 256-4096 tokens, and gained nothing on 64 flat ones).
-// split: items a tile may be cut into so that few tiles still use all pairs (1 where there are tiles enough).  general: into chunks of
-// at least NCMIN keys, a tile of up to NC keys stays whole.  Then, in both, by columns of the output: 1 << lds items of a chunk
+// split: items a tile may be cut into so that few tiles still use all pairs (1 where there are tiles enough).  general: a tile of more
+// than NC keys into a chunk for every NCMIN keys or part of them (513 keys: 256, 256 and 1), up to split and to the slots of the
+// workspace; one of up to NC keys stays whole.  Then, in both, by columns of the output: 1 << lds items of a chunk
 // compute S and the softmax alike and each its own columns of O, which nobody has to merge.
 // f32: the partial outputs of the tile are fp32 (a tile that is cut for the sake of parallelism alone is not rounded before
 // the merge); f32_all: all multi-chunk tiles are.

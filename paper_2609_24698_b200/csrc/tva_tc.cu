@@ -381,10 +381,11 @@ __global__ void __launch_bounds__(NT) tc_plan_kernel(const tsv_shape s, const Tv
 // Merge of the paired kernel's multi-chunk tiles (launched with its general instantiation): every chunk left its NORMALISED partial output with
 // the row's (reference max, sum); the row's output is the average of the partial outputs weighted by sum * 2^(max - row max), the
 // chunks accumulated in order.
-// 1-d grid (scheduling position of the tile, its two 128-row halves, groups of 8 * rpw rows): a warp merges rpw rows one after the
-// other, a lane owns 16 columns as 16-byte pieces of the row (coalesced).  Bound by latency and by the L2 and HBM traffic (67 MB read
-// and 34 MB written at 64 sequences of 1-4 k tokens, 15 us): a row's (max, sum) and its first four chunks are requested together
-// (after the maxima had been reduced they cost a third latency), and a CTA lives for several rows (rpw: 1, 2 or 4).
+// 1-d grid (scheduling position of the tile, its two 128-row halves, groups of 8 * rpw rows): a warp merges rpw rows, one after the
+// other or (bf16, rpw = 2) together, a lane owns 16 columns as 16-byte pieces of the row (coalesced).  Bound by latency and by the
+// L2 and HBM traffic (67 MB read and 34 MB written at 64 sequences of 1-4 k tokens, 15 us): a row's (max, sum) and its first four
+// chunks, or those of two rows and their first two chunks, are requested together (after the maxima had been reduced they cost a
+// third latency), and a CTA lives for several rows (rpw: 1, 2 or 4).
 // The CTAs take the places of the attention kernel's as those run out of items, and a tile is merged as soon as all warps of its
 // chunks have said that their rows are stored (it is looked for in the order in which the tiles are worked on), the rest when
 // that kernel has ended: at those 64 sequences a pass of eight layers takes 798 instead of 830 us.  Tiles cut to fill the device
@@ -575,11 +576,14 @@ int launch_tva_tc(const tsv_shape& s, const TvaPlan& p_in, const TvaTcPrep& prep
                   void* out, char* ws, int32_t* status, cudaStream_t st, bool with_plan) {
   TvaPlan p = p_in;
   const bool gathered = gathered_tiles_possible(s, p, c);
-  // general: some tile may have more than two chunks of the longest kind, or be gathered; then every multi-chunk tile
-  // leaves bf16 partial outputs for the merge kernel
+  // general: some tile may have more than two chunks of the longest kind, or be gathered; then every multi-chunk tile leaves
+  // partial outputs for the merge kernel: bf16, or fp32 where the tile would fit one chunk and is cut because tiles are few
   const bool general = (p.tc_maxk + tc::NCX - 1) / tc::NCX > 2 || gathered;
   p.tc_f32 = !general;                                 // (no more than two long chunks a tile: merged without rounding in the attention kernel)
-  if (general && p.tc_split < 4) p.tc_split = 1;       // (tiles of several chunks: two or three pairs a tile are soon in use)
+  // 19-37 general tiles are neither cut nor shared further: mostly of several chunks, they have items enough, and shares fetch the keys
+  // again (not cut and cut, us a pass: 16 sequences of 512-8192 tokens 69.7 and 73.0, 18 of them 75.6 and 80.7, 12 of 16-64 k 180.5 and
+  // 189.4, 10 of 8-32 k 110.0 and 112.0; the other way where lists are short: 12 of 1-4 k 56.4 and 55.7, 14 paged of 256-4096 59.5 and 57.1).
+  if (general && p.tc_split < 4) p.tc_split = 1;
   p.tc_general = general;
   const dim3 pgrid(p.tc_nt + 1, s.B);                                                                              // x: tiles + the packing CTA
   if (with_plan) {
@@ -599,10 +603,10 @@ int launch_tva_tc(const tsv_shape& s, const TvaPlan& p_in, const TvaTcPrep& prep
   if (r != TSV_OK) return r;
   if (general && p.tc_chmax > 1) {
     cudaLaunchConfig_t cfg = {};
-    // Rows a warp takes: one while that leaves SMs idle otherwise; two, merged together, up to 64 tiles (what is left to merge when the
+    // Rows a warp takes: one while that leaves SMs idle otherwise; two, merged together, up to 74 tiles (what is left to merge when the
     // attention ends is one row's latency then: 32 paged sequences 257 -> 242 us a pass, four rows one after the other before); four
     // beyond (there the merge runs under the attention's tail, and the registers of two rows at once take a third of the warps:
-    // 64 grown sequences 703 us, with two rows 714-723).
+    // 64 grown sequences take 2-3 % more with two rows).
     const int64_t groups = (int64_t)2 * p.tc_nt * s.B * (tc::BM / 8);
     const int rpw = groups <= 4 * 148 ? 1 : groups <= 16 * 148 ? 2 : 4;
     cfg.gridDim = dim3(2 * p.tc_nt * s.B * (tc::BM / 8 / rpw)); cfg.blockDim = dim3(256, 1, 1); cfg.stream = st;

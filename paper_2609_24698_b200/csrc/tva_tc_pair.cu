@@ -634,8 +634,8 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(map_to_rank(smem_u32(&sm.cmp_ev[pc]), 0));
     };
-    // The softmax goes over a piece ONCE, in slabs of 32 keys: a slab is read from tensor memory, checked against the row's
-    // reference maximum, exponentiated and stored as P, the next slab's read already on its way.
+    // The softmax goes over a piece ONCE, in slabs of 32 keys, one after the other: a slab is read from tensor memory, checked against
+    // the row's reference maximum, exponentiated and stored as P.
     //
     // Reference: the maximum over the visible keys of the first slab that has any (the two warps of a row, which share
     // its keys, exchange it once).  bf16 and fp32 have the range for weights above 1, so a later slab changes the reference
@@ -788,7 +788,7 @@ tc_attn_pair_kernel(const __grid_constant__ pair::MapSet maps, const tsv_shape s
     constexpr int cw = OW / 2;                        // columns of the part this thread handles
     // The output leaves by one of two ways.  GENERAL: straight from registers, so that the next item's last two Q slices need not wait until
     // staging in their slots has been read (4 x 128 k 103.0 -> 99.7 us, 16 of 512-8192 tokens 3 %).  Else, where most pairs have an item or
-    // two and the code is run through cold, staged for TMA stores, in half the instructions (one short stack 161 us, the other way 164).
+    // two and the code is run through cold, staged for TMA stores, in half the instructions (one short stack takes 2 % more the other way).
     const bool full_tile = row0 + BM <= rows_seq;     // whole tile inside the sequence: rows may be stored as 32-row boxes
     const uint32_t stage = ring + (uint32_t)NSV * SLOTP + (uint32_t)(warp - 4) * 4096;   // this warp's tile of 32 rows x 64 columns (bf16)
     bool stored = false;
